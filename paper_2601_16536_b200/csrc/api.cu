@@ -29,7 +29,9 @@ struct DeviceState {
     void* ws = nullptr;
     size_t ws_bytes = 0;
     bool decode_attr_set[3][2][3][2][2][2] = {};   // [mb][cluster exchange][log2 SG][bf16][symmetric][tensor-copy rows]
-    bool tile_attr_set[5][3][2][2][2] = {};   // [batch-tile index][log2 SG][bf16][symmetric][epilogue]
+    int mid_clusters[16] = {};         // mid_max_clusters, 0 = not asked yet
+    bool mid_attr_set[3][2][2] = {};   // [log2 SG][bf16][symmetric]
+    bool tile_attr_set[2][3][2][2][2] = {};   // [batch-tile index][log2 SG][bf16][symmetric][epilogue]
     // Programmatic dependent launch lets a GEMM kernel prefetch packed weights before the previous
     // kernel in its stream has finished.  The previous kernel of a stream may be a w4a16_pack that
     // writes those weights, so the first GEMM launched on a stream after any pack on the device is a
@@ -233,10 +235,9 @@ int choose_split_decode(int M, int N, int G, int sms) {
 }
 
 // ---- tile-path launch geometry ----------------------------------------------------
-// MT (batch rows per CTA tile = UMMA N) is the smallest of 16, 32, 64, 128, 256 that covers M, else
-// 256.  The unit range (batch tile x column tile x group) is cut into `nchunks` chunks for `ctas`
-// persistent CTAs: balanced chunks, one per CTA, when the caller leaves split_k open; S slices
-// per tile otherwise.
+// MT (batch rows per CTA tile = UMMA N) is 128 up to 128 rows, else 256 (fewer rows go to the kernel above).  The unit
+// range (batch tile x column tile x group) is cut into `nchunks` chunks for `ctas` persistent CTAs: balanced chunks, one
+// per CTA, when the caller leaves split_k open; S slices per tile otherwise.
 struct TileGeom {
     int mt, mt_index, m_tiles, n_tiles, split_k, nchunks, stages, smem_bytes, ctas;
     long tiles;
@@ -246,33 +247,10 @@ constexpr size_t kTileTicketBytes = 131072;   // 16 counters per tile, after the
 constexpr size_t kWsFullHeaderBytes = kWsHeaderBytes + kTileTicketBytes;
 constexpr long kTileMaxTicketTiles = kTileTicketBytes / (sizeof(int) * kTileDequantWarps);
 
-// Batch rows per CTA tile: the smallest of 16 .. 256 that covers M -- except that a narrow weight
-// matrix gives such tiles too few of them for 148 SMs (N = 1536 and M = 64: twelve), and where the Split-K
-// sum is made inside the kernel a twelve-way split costs more than converting the weights once per narrower
-// batch tile: M = 64, N = 1536: 14.5 us with 64-row tiles, 10.1 with 32; M = 32: 10.7 against 9.0 with 16.
-// With 24 tiles or fewer, take the widest narrower tile that gives at least 24.  Tiles of 128 and 256 rows
-// hand that sum to a second kernel, so from twelve column tiles on they stay (us with 64- / 128- / 256-row
-// tiles: M = 256: K = 8192 / N = 2048 19.1 / 17.1 / 16.1, K = 10240 / N = 2048 21.9 / 19.4 / 17.0, K = 8192 /
-// N = 3072 26.8 / 20.9 / 18.6; M = 512, K = 6144 / N = 1536 23.1 / 17.6 / 16.5; M = 128: K = 8192 / N = 2048
-// 13.6 / 13.3 / 15.1, K = 6144 / N = 1536 12.2 / 11.8 / 13.3); with eight column tiles the narrow tile is still
-// ahead (M = 256, K = 4096 / N = 1024: 10.6 / 11.0 / 12.6).
-int tile_mt_index(int M, int N) {
-    const int idx = M <= 16 ? 0 : M <= 32 ? 1 : M <= 64 ? 2 : M <= 128 ? 3 : 4;
-    const long n_tiles = (N + kTileCols - 1) / kTileCols;
-    auto tiles = [&](int i) { return (long)((M + (16 << i) - 1) / (16 << i)) * n_tiles; };
-    if (tiles(idx) > 24) return idx;
-    if (idx >= 3 && n_tiles >= 12) return idx;
-    for (int i = idx - 1; i >= 0; --i) {
-        if (i == 3) continue;   // (128 rows were slower than 64 wherever the narrower tile was taken)
-        if (tiles(i) >= 24) return i;
-    }
-    return 0;   // even 16-row tiles are few: take the most there are
-}
-
 TileGeom tile_geom(int M, int N, int G, int split_k, int sms, int max_smem) {
     TileGeom g;
-    g.mt_index = tile_mt_index(M, N);
-    g.mt = 16 << g.mt_index;
+    g.mt_index = M <= 128 ? 0 : 1;
+    g.mt = 128 << g.mt_index;
     g.m_tiles = (M + g.mt - 1) / g.mt;
     g.n_tiles = (N + kTileCols - 1) / kTileCols;
     g.tiles = (long)g.m_tiles * g.n_tiles;
@@ -283,10 +261,8 @@ TileGeom tile_geom(int M, int N, int G, int split_k, int sms, int max_smem) {
         // an FP32 partial tile behind (store, ticket, reload: the larger the batch tile the dearer, and
         // in mid-stream it stalls the pipeline).  S slices per tile (tiles <= SMs) or whole tiles in
         // waves (tiles > SMs) avoid that at the price of idle SMs.  Cost model in groups per CTA; the
-        // constants are fitted to measurements (K = 11008 / N = 4096, K = 28672 / N = 8192 and
-        // K = N = 8192 with M up to 4096).
-        // (narrow tiles: K = 4096 / N = 12288, M = 16: 96 whole tiles 13.8 us, balanced chunks 16.3)
-        const long penalty = (g.mt <= 32 ? 10 : 6) + g.mt / 8;
+        // constants are fitted to measurements (K = N = 8192 with M up to 4096).
+        const long penalty = 6 + g.mt / 8;
         const long balanced_cost = (g.tiles * G + sms - 1) / sms + penalty;
         int s0 = 1;
         long classic_cost;
@@ -313,16 +289,112 @@ TileGeom tile_geom(int M, int N, int G, int split_k, int sms, int max_smem) {
     const int avail = max_smem - kTileBarBytes - 1024;   // barrier block + alignment slack
     int st = avail / tile_stage_bytes(g.mt);
     if (st > kTileMaxStages) st = kTileMaxStages;
-    if (st > tile_max_slots(g.mt)) st = tile_max_slots(g.mt);   // the ring also lives in tensor memory
-    // parity waits tell a barrier phase only from its neighbour: every issuer has to come back to a slot
-    // on every ring turn and every dequant set on every turn or every second one (kernel_tile.cuh)
-    const int ring_unit = tile_issuers(g.mt) % 2 == 0 ? tile_issuers(g.mt) : 2 * tile_issuers(g.mt);
-    st -= st % ring_unit;                                        // 0 (no valid ring) is refused by the caller
+    if (st > kTileSlots) st = kTileSlots;               // the ring also lives in tensor memory
+    // parity waits tell a barrier phase only from its neighbour: every dequant set has to come back to a slot on
+    // every turn or every second one (kernel_tile.cuh)
+    st -= st % 2;                                                // 0 (no valid ring) is refused by the caller
     g.stages = st;
     g.smem_bytes = kTileBarBytes + 1024 + st * tile_stage_bytes(g.mt);
     // each CTA takes the SM's whole tensor memory: ask for enough shared memory that two never share an SM
     if (g.smem_bytes < 120 * 1024) g.smem_bytes = 120 * 1024;
     return g;
+}
+
+// ---- two-CTAs-per-SM tcgen05 kernel (kernel_mid.cuh): launch geometry --------------
+constexpr int kMidSmemBudget = (228 * 1024) / 2 - 1024;   // dynamic shared memory of one of two CTAs of an SM
+
+struct MidGeom {
+    int mt, m_tiles, n_tiles, split_k, nchunks, wstages, smem_bytes, ctas;
+    long tiles;
+    bool cluster;
+};
+
+// Clusters of `size` CTAs of that kernel (two per SM) that run at the same time.  The SMs of a GPC hold whole clusters
+// only, so this is less than slots / size, and which SMs a GPC has differs from chip to chip: ask, once per device.
+// (The runtime counts one CTA per SM for any kernel that allocates tensor memory, so it is asked about a kernel of the
+// same launch shape without it, which is never launched.  On the chip measured it says 148 / 93 / 71 / 56 / 45 / 37 / 33
+// for 2 .. 8, and calls with one tile more than that take a second wave: 92 tiles in three slices 8.5 us, 96 12.9;
+// 70 in four 7.1, 74 11.4; 32 in eight 6.4, 34 9.8, at K = 2048.)
+__global__ void __launch_bounds__(kMidThreads, 2) mid_shape_probe_kernel(float* out) {
+    extern __shared__ float probe_smem[];
+    out[threadIdx.x] = probe_smem[threadIdx.x];
+}
+int mid_max_clusters(int size) {
+    DeviceState* d = nullptr;
+    if (current_device(&d) != W4A16_OK || !d->is_sm100) return 264 / size;    // (size queries without a device)
+    if (d->mid_clusters[size] != 0) return d->mid_clusters[size];
+    int n = 0;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(size * d->sm_count), 1, 1);
+    cfg.blockDim = dim3(kMidThreads, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)kMidSmemBudget;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(mid_shape_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, d->max_smem_optin) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, mid_shape_probe_kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+    }
+    if (n < 1) n = 1;
+    d->mid_clusters[size] = n;
+    return n;
+}
+
+MidGeom mid_geom(int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg = 1) {
+    MidGeom g;
+    constexpr int kMtc = 64;
+    g.m_tiles = (M + kMtc - 1) / kMtc;
+    g.mt = ((M + g.m_tiles - 1) / g.m_tiles + 15) / 16 * 16;
+    g.n_tiles = (N + kTileCols - 1) / kTileCols;
+    g.tiles = (long)g.m_tiles * g.n_tiles;
+    const int slots = 2 * sms;
+    auto fits = [&](int s) { return mid_smem_bytes(kMtc, g.mt, sg, 2, s) <= kMidSmemBudget; };
+    if (split_k == 0) {
+        // Cost in tenths of a unit's time (0.42 us with one CTA on an SM, a fifth more with two): the longest CTA's
+        // units, 5 per CTA of the cluster for the exchange, 15 where more than half of the slots are taken, so that
+        // the next launch's CTAs do not find room before this one ends.  Measured (us), M = 32: K = N = 4096 four
+        // slices 7.09, eight 7.44; K = 11008 / N = 4096 8 / 6 / 4 slices 11.0 / 11.6 / 13.8; K = 18432 / N = 7168
+        // 5 / 4 21.8 / 22.9; K = 4096 / N = 12288 2 / 1 12.2 / 17.3, three no longer fit at once: 17.5; K = 4096 /
+        // N = 22016 1 / 2 18.7 / 22.6; K = 1024 / N = 3136 4 / 8 4.18 / 5.10.
+        long best = 0;
+        for (int s = 1; s <= kMidMaxCluster && s <= G; ++s) {
+            if (s > 1 && (!allow_cluster || g.tiles > mid_max_clusters(s) || !fits(s))) continue;
+            const long ctas = g.tiles * s;
+            const long units = ((ctas + slots - 1) / slots) * ((G + s - 1) / s);
+            const long cost = units * (ctas > sms ? 12 : 10) + 5 * s + (ctas > sms ? 15 : 0);
+            if (best == 0 || cost < best) { best = cost; split_k = s; }
+        }
+    }
+    g.split_k = split_k;
+    g.cluster = allow_cluster && split_k >= 2 && split_k <= kMidMaxCluster && fits(split_k);
+    g.nchunks = (int)(g.tiles * split_k);
+    g.ctas = g.cluster || g.nchunks < slots ? g.nchunks : slots;
+    int st = kMidMaxWStages;
+    while (st > 2 && mid_smem_bytes(kMtc, g.mt, sg, st, g.cluster ? split_k : 0) > kMidSmemBudget) --st;
+    g.wstages = st;
+    g.smem_bytes = mid_smem_bytes(kMtc, g.mt, sg, st, g.cluster ? split_k : 0);
+    // A CTA takes half of the SM's tensor memory: ask for enough shared memory that no third one, and no CTA of the
+    // wide-tile kernel (which takes all of it), ever shares the SM, so that the allocation never has to wait.
+    if (g.smem_bytes < 108 * 1024) g.smem_bytes = 108 * 1024;
+    return g;
+}
+// Does the tcgen05 path take this shape through that kernel?  Up to 64 rows always; more rows where the weight matrix is
+// so narrow that tiles of 128 and 256 rows leave most SMs idle (24 tiles or fewer, fewer than twelve column tiles).
+bool mid_takes(int M, int N) {
+    if (M <= 64) return true;
+    const int mt = M <= 128 ? 128 : 256;
+    const long n_tiles = (N + kTileCols - 1) / kTileCols;
+    return n_tiles < 12 && ((M + mt - 1) / mt) * n_tiles <= 24;
+}
+
+size_t mid_workspace_bytes(const MidGeom& g) {
+    if (g.split_k == 1) return 0;
+    return round256((size_t)2 * g.nchunks * g.mt * kTileCols * sizeof(float));
 }
 
 // Partial-tile slots of the tile path: two per chunk.  Nothing when every chunk is a whole tile.
@@ -333,6 +405,7 @@ size_t tile_workspace_bytes(const TileGeom& g) {
 
 // Nominal split factor of the tile path's schedule: how many chunks share one tile's K range.
 int choose_split_tile(int M, int N, int G, int sms) {
+    if (mid_takes(M, N)) return mid_geom(M, N, G, 0, sms, true).split_k;
     TileGeom g = tile_geom(M, N, G, 0, sms, 227 * 1024);
     if (g.split_k >= 1) return g.split_k;
     long s = (g.nchunks + g.tiles - 1) / g.tiles;
@@ -359,12 +432,12 @@ EncodeTiledFn encode_tiled_fn() {
     return fn;
 }
 
-// Activations A [M, K] FP16 row-major as a 2-D tensor (k innermost), box = 64 k x mt rows, 128-byte
-// swizzle; rows past M read as zero.
-bool make_act_tensor_map(CUtensorMap* map, const void* A, int M, int K, int mt) {
+// Activations A [M, K] 16-bit row-major as a 2-D tensor (k innermost), box = 64 k x mt rows, 128-byte swizzle; rows past
+// M read as zero.  With stage_k = 128 one copy brings the stage's two boxes.
+bool make_act_tensor_map(CUtensorMap* map, const void* A, int M, int K, int mt, int stage_k) {
     EncodeTiledFn fn = encode_tiled_fn();
     if (fn == nullptr) return false;
-    if (tile_stage_k(mt) == kTileBoxK) {     // one box per stage: plain 2-D tensor, k innermost
+    if (stage_k == kTileBoxK) {     // one box per stage: plain 2-D tensor, k innermost
         const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
         const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
         const cuuint32_t box[2] = {(cuuint32_t)kTileBoxK, (cuuint32_t)mt};
@@ -376,7 +449,7 @@ bool make_act_tensor_map(CUtensorMap* map, const void* A, int M, int K, int mt) 
     // A[M][K] seen as [K / 64][M][64]: one copy brings a stage's 64-k boxes one after the other
     const cuuint64_t dims[3] = {(cuuint64_t)kTileBoxK, (cuuint64_t)M, (cuuint64_t)(K / kTileBoxK)};
     const cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)kTileBoxK * 2};
-    const cuuint32_t box[3] = {(cuuint32_t)kTileBoxK, (cuuint32_t)mt, (cuuint32_t)(tile_stage_k(mt) / kTileBoxK)};
+    const cuuint32_t box[3] = {(cuuint32_t)kTileBoxK, (cuuint32_t)mt, (cuuint32_t)(stage_k / kTileBoxK)};
     const cuuint32_t estr[3] = {1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(A), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -491,8 +564,9 @@ size_t w4a16_workspace_bytes(int M, int N, int K, int group, int split_k) {
         int s = split_k == 0 ? choose_split_decode(M, N, K / kGroup, sm_count_or_default()) : split_k;
         size_t simple = simple_partial_bytes(M, N, s);
         if (simple > need) need = simple;
-        TileGeom tg = tile_geom(M, N, K / kGroup, split_k, sm_count_or_default(), 227 * 1024);
-        if (tile_workspace_bytes(tg) > need) need = tile_workspace_bytes(tg);
+        const size_t tile = mid_takes(M, N) ? mid_workspace_bytes(mid_geom(M, N, K / kGroup, split_k, sm_count_or_default(), true))
+                                         : tile_workspace_bytes(tile_geom(M, N, K / kGroup, split_k, sm_count_or_default(), 227 * 1024));
+        if (tile > need) need = tile;
     }
     return need == 0 ? 0 : kWsFullHeaderBytes + need;
 }
@@ -618,6 +692,29 @@ TileKernel tile_kernel(int mt_index, int sg, bool bf, bool sym, bool epi) {
                                                                        : tile_kernel_f16_sg4(mt_index, sym, epi);
 }
 
+// Split-K sum behind a tcgen05 kernel that only stored its partial tiles (slices of whole tiles).
+int launch_tile_reduce(const float* parts, uint16_t* C, int M, int N, int mt, int n_tiles, long tiles, int split_k, bool bf,
+                       const Epilogue& epi, cudaStream_t st) {
+    const long long quads = (long long)tiles * mt * (kTileCols / 4);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // always behind the GEMM kernel just launched on this stream
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((quads + 255) / 256), 1, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const FastDiv div_mt = fast_div_make((uint32_t)mt), div_nt = fast_div_make((uint32_t)n_tiles);
+    const cudaError_t e = bf ? cudaLaunchKernelEx(&cfg, tile_splitk_reduce_kernel<true>, parts, C, M, N, mt, div_mt, n_tiles, div_nt, split_k, quads, epi)
+                             : cudaLaunchKernelEx(&cfg, tile_splitk_reduce_kernel<false>, parts, C, M, N, mt, div_mt, n_tiles, div_nt, split_k, quads, epi);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return W4A16_ERR_CUDA;
+    }
+    return W4A16_OK;
+}
+
 // The body of every GEMM entry point; the caller holds g_mu.
 int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z, const uint16_t* bias, uint16_t* C,
                 int M, int N, int K, int group, int split_k, int path, int flags, int act, w4a16_stream_t stream) {
@@ -675,6 +772,74 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         return W4A16_OK;
     }
 
+    if (path == W4A16_PATH_TILE && mid_takes(M, N)) {
+        const MidGeom g = mid_geom(M, N, G, split_k, d->sm_count, d->cluster_ok, sg);
+        if (g.smem_bytes > d->max_smem_optin) return W4A16_ERR_PATH;
+        if (g.split_k != 1 && ws_body_bytes < mid_workspace_bytes(g)) return W4A16_ERR_WORKSPACE;
+        if ((long long)g.tiles * (g.split_k > g.mt ? g.split_k : g.mt) >= (1ll << 31)) return W4A16_ERR_SHAPE;   // (32-bit chunk arithmetic)
+        CUtensorMap tmap;
+        if (!make_act_tensor_map(&tmap, A, M, K, g.mt, mid_stage_k(64))) return W4A16_ERR_CUDA;
+        MidParams p;
+        p.Wq = static_cast<const uint32_t*>(Wq);
+        p.S = static_cast<const uint16_t*>(S);
+        p.Z = Zw;
+        p.C = C;
+        p.ws = reinterpret_cast<float*>(ws_body);
+        p.M = M; p.N = N; p.K = K; p.G = G;
+        p.n_tiles = g.n_tiles;
+        p.mt = g.mt;
+        p.split_k = g.split_k;
+        p.nchunks = g.nchunks;
+        p.wstages = g.wstages;
+        p.cluster = g.cluster ? 1 : 0;
+        p.div_split = fast_div_make((uint32_t)g.split_k);
+        p.div_ntiles = fast_div_make((uint32_t)g.n_tiles);
+        p.slice_base = G / g.split_k;
+        p.slice_rem = G % g.split_k;
+        p.epi = epi;
+        MidKernel kern = bf ? mid_kernel_bf16(sg, sym) : mid_kernel_f16(sg, sym);
+        bool& attr_set = d->mid_attr_set[log2_sg(sg)][bf ? 1 : 0][sym ? 1 : 0];
+        if (!attr_set) {
+            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, d->max_smem_optin) != cudaSuccess) {
+                cudaGetLastError();
+                return W4A16_ERR_CUDA;
+            }
+            attr_set = true;
+        }
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(g.ctas, 1, 1);
+        cfg.blockDim = dim3(kMidThreads, 1, 1);
+        cfg.dynamicSmemBytes = (size_t)g.smem_bytes;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[2];
+        int n_attr = 0;
+        if (g.cluster) {   // the slices of a tile are one cluster (consecutive blockIdx.x)
+            attr[n_attr].id = cudaLaunchAttributeClusterDimension;
+            attr[n_attr].val.clusterDim.x = (unsigned)g.split_k;
+            attr[n_attr].val.clusterDim.y = 1;
+            attr[n_attr].val.clusterDim.z = 1;
+            ++n_attr;
+        }
+        if (d->pdl_allowed(st)) {
+            attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
+            ++n_attr;
+        }
+        cfg.attrs = attr;
+        cfg.numAttrs = n_attr;
+        if (cudaLaunchKernelEx(&cfg, kern, tmap, p) != cudaSuccess) {
+            cudaGetLastError();
+            if (g.cluster) {   // (see the warp-MMA kernel below)
+                d->cluster_ok = false;
+                return gemm_locked(A, Wq, S, Z, bias, C, M, N, K, group, split_k, path_asked, flags, act, stream);
+            }
+            return W4A16_ERR_CUDA;
+        }
+        if (g.split_k > 1 && !g.cluster)
+            return launch_tile_reduce(p.ws, C, M, N, g.mt, g.n_tiles, g.tiles, g.split_k, bf, epi, st);
+        return W4A16_OK;
+    }
+
     if (path == W4A16_PATH_TILE) {
         TileGeom g = tile_geom(M, N, G, split_k, d->sm_count, d->max_smem_optin);
         if (g.stages < 2) return W4A16_ERR_PATH;
@@ -685,7 +850,7 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         // (the kernel's chunk arithmetic is 32-bit)
         if ((long long)g.tiles * G >= (1ll << 31)) return W4A16_ERR_SHAPE;
         CUtensorMap tmap;
-        if (!make_act_tensor_map(&tmap, A, M, K, g.mt)) return W4A16_ERR_CUDA;
+        if (!make_act_tensor_map(&tmap, A, M, K, g.mt, kTileStageK)) return W4A16_ERR_CUDA;
         TileParams p;
         p.Wq = static_cast<const uint32_t*>(Wq);
         p.S = static_cast<const uint16_t*>(S);
@@ -705,9 +870,8 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         // bias / activation) is a second, GPU-wide kernel behind this one (kernels_basic.cuh).  Balanced
         // chunks, whose pieces belong to different tiles, keep the reduce inside the kernel.
         // Measured (us, in the kernel / second kernel): M = 256: K = 10240 / N = 4608 (four slices) 31.9 / 24.6,
-        // K = 16384 / N = 4096 39.2 / 32.9, K = N = 8192 (two slices) 34.1 / 33.3; 64-row tiles are level (16.6 /
-        // 16.5 at K = 11008 / N = 4096) and 32-row tiles lose the extra launch (12.9 / 13.7): from 128 rows on.
-        const bool defer = g.split_k >= 2 && g.mt >= 128;
+        // K = 16384 / N = 4096 39.2 / 32.9, K = N = 8192 (two slices) 34.1 / 33.3.
+        const bool defer = g.split_k >= 2;
         p.defer_reduce = defer ? 1 : 0;
         const bool has_epi = !defer && (bias != nullptr || act != W4A16_ACT_NONE);
         TileKernel kern = tile_kernel(g.mt_index, sg, bf, sym, has_epi);
@@ -724,7 +888,7 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         // tail of the previous kernel in the stream; it orders itself with griddepcontrol.wait
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(g.ctas, 1, 1);
-        cfg.blockDim = dim3(tile_threads(g.mt), 1, 1);
+        cfg.blockDim = dim3(kTileThreads, 1, 1);
         cfg.dynamicSmemBytes = (size_t)g.smem_bytes;
         cfg.stream = st;
         cudaLaunchAttribute attr[1];
@@ -736,25 +900,7 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
             cudaGetLastError();
             return W4A16_ERR_CUDA;
         }
-        if (defer) {
-            const long long quads = (long long)g.tiles * g.mt * (kTileCols / 4);
-            cudaLaunchConfig_t rcfg = {};
-            rcfg.gridDim = dim3((unsigned)((quads + 255) / 256), 1, 1);
-            rcfg.blockDim = dim3(256, 1, 1);
-            rcfg.stream = st;
-            rcfg.attrs = attr;      // always behind the GEMM kernel just launched on this stream
-            rcfg.numAttrs = 1;
-            const float* parts = p.ws;
-            const int mt_log2 = 4 + g.mt_index;
-            cudaError_t e = bf ? cudaLaunchKernelEx(&rcfg, tile_splitk_reduce_kernel<true>, parts, C, M, N, mt_log2, g.n_tiles,
-                                                    g.split_k, quads, epi)
-                               : cudaLaunchKernelEx(&rcfg, tile_splitk_reduce_kernel<false>, parts, C, M, N, mt_log2, g.n_tiles,
-                                                    g.split_k, quads, epi);
-            if (e != cudaSuccess) {
-                cudaGetLastError();
-                return W4A16_ERR_CUDA;
-            }
-        }
+        if (defer) return launch_tile_reduce(p.ws, C, M, N, g.mt, g.n_tiles, g.tiles, g.split_k, bf, epi, st);
         return W4A16_OK;
     }
 
@@ -984,6 +1130,7 @@ int w4a16_device_status(int* status_out) {
     }
     // every translation unit that holds kernels has a status word of its own
     const int words[] = {status_take_this_unit(),     status_take_decode_f16(),   status_take_decode_bf16(),
+                         status_take_mid_f16(),        status_take_mid_bf16(),
                          status_take_tile_f16_sg1(),  status_take_tile_f16_sg2(), status_take_tile_f16_sg4(),
                          status_take_tile_bf16_sg1(), status_take_tile_bf16_sg2(), status_take_tile_bf16_sg4()};
     int v = 0;

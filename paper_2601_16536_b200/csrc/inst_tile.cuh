@@ -8,9 +8,7 @@ template <bool SYM, bool EPI>
 TileKernel pick(int mt_index) {
     constexpr bool BF = W4A16_INST_BF;
     constexpr int SG = W4A16_INST_SG;
-    return mt_index == 0 ? gemm_tile_kernel<16, SG, BF, SYM, EPI> : mt_index == 1 ? gemm_tile_kernel<32, SG, BF, SYM, EPI>
-         : mt_index == 2 ? gemm_tile_kernel<64, SG, BF, SYM, EPI> : mt_index == 3 ? gemm_tile_kernel<128, SG, BF, SYM, EPI>
-                                                                                   : gemm_tile_kernel<256, SG, BF, SYM, EPI>;
+    return mt_index == 0 ? gemm_tile_kernel<128, SG, BF, SYM, EPI> : gemm_tile_kernel<256, SG, BF, SYM, EPI>;
 }
 }  // namespace
 

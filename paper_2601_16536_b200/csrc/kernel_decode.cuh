@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) gemm_decode_kernel(const __gri
                     if (lane == 0)
                         asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(xbar0) : "memory");
                 } else {
-                    if (!mbar_wait_cluster(xbar, 0u)) return;   // status recorded
+                    if (!mbar_wait_cluster(smem_u32(xbar), 0u)) return;   // status recorded
                     for (int idx = threadIdx.x; idx < rows * kTileN; idx += kDecConsumers) {
                         const int n = idx & (kTileN - 1), m = idx >> 6;
                         float v = red[m * kDecRedStride + n];

@@ -28,18 +28,12 @@
 // No warp ever waits for another CTA, and the order of the sum is fixed, so results are
 // bit-identical from run to run.
 //
-// One pipeline stage is a whole group (128 k, eight MMAs) for batch tiles of up to 64 rows and half
-// a group (64 k, four MMAs) above: narrow tiles are bound by per-stage work other than the MMAs
-// (the dequant warps' instruction streams, the control warps' loops), wide ones by the tensor pipe.
-// A ring of R slots holds, per slot, the stage's activation boxes in shared memory and its
-// dequantized weights in tensor memory (32 or 64 columns; six or eight slots fit beside the
-// accumulators); the MMAs of a stage release both with one commit.  Four sets of four dequant
-// warps take stages round-robin; inside a set warp w owns TMEM lanes 32 (w % 4) .. + 31.  Each
-// thread keeps the packed words of its next two or three stages in registers (loads issued that
-// far ahead, pointers stepped, no register copies).  Tiles of up to 32 rows have three MMA-issuing
-// warps that take the stages round-robin, each summing into an accumulator of its own (the epilogue
-// adds them in stage order); the others have one issuer, and two accumulators that alternate
-// between segments (MT = 16, 64, 128), so one drains while the next fills.  The packed weights do not depend on the
+// Batch tiles of 128 and 256 rows (17 to 64 rows: kernel_mid.cuh).  One pipeline stage is half a group (64 k, four MMAs).
+// A ring of R slots holds, per slot, the stage's activation box in shared memory and its dequantized weights in tensor
+// memory (32 columns; eight slots fit beside the accumulators).  Four sets of four dequant warps take stages round-robin;
+// inside a set warp w owns TMEM lanes 32 (w % 4) .. + 31.  Each thread keeps the packed words of its next three stages in
+// registers (loads issued that far ahead, pointers stepped, no register copies).  With MT = 128 two accumulators alternate
+// between segments, so one drains while the next fills.  The packed weights do not depend on the
 // previous kernel in the stream: under programmatic dependent launch the dequant warps load and
 // convert weights until the TMEM ring is full before anything waits for that kernel; only
 // activations, C and the workspace are touched after griddepcontrol.wait.
@@ -59,34 +53,20 @@ namespace w4a16 {
 
 constexpr int kTileCols = 128;                      // n per CTA tile = UMMA M
 constexpr int kTileBoxK = 64;                       // k per activation TMA box (one 128-byte swizzle row)
-// k per pipeline stage: a whole group for narrow batch tiles (twice the MMAs per barrier round: the
-// issuing lane and the per-stage synchronisation are what bounds them), half a group otherwise
-__host__ __device__ constexpr int tile_stage_k(int mt) { return mt <= 64 ? 128 : 64; }
+constexpr int kTileStageK = 64;                     // k per pipeline stage
 constexpr int kTileDequantWarps = 16;               // four sets of four (one warp per TMEM lane quarter)
 constexpr int kTileSets = kTileDequantWarps / 4;
-// MMA-issuing warps.  With narrow batch tiles one issuing warp is busy nearly all the time (a lone
-// warp of dependent scalar code beside sixteen busy dequant warps needs 600 to 700 clocks per stage,
-// of which the eight MMAs are about 100), so for tiles of up to 32 rows the stages are dealt to three
-// issuers, each with an accumulator of its own; the epilogue adds the accumulators in issuer order.
-// Measured at K = 11008, N = 4096: 14.0 -> 13.0 us at M = 16; 64-row tiles are faster with one issuer
-// and two alternating accumulators (16.9 against 18.3 us), so the split stops at 32 rows.
-// An issuer must meet every phase of the `full` barriers it waits on, and a dequant set every phase
-// of its `retired` barriers: the ring size has to be an even multiple of the issuer count (host).
-__host__ __device__ constexpr int tile_issuers(int mt) { return mt <= 32 ? 3 : 1; }
-// producer, issuers, dequant / epilogue warps
-__host__ __device__ constexpr int tile_threads(int mt) { return (1 + tile_issuers(mt) + kTileDequantWarps) * 32; }
-// accumulators per issuer that alternate between segments, and the TMEM columns between accumulators
-__host__ __device__ constexpr int tile_dbufs(int mt) { return mt <= 16 ? 2 : mt <= 32 ? 1 : mt <= 128 ? 2 : 1; }
-__host__ __device__ constexpr int tile_d_stride(int mt) { return mt <= 64 ? mt : 128; }
-constexpr int kTileMaxStages = 8;                   // ring slots: activation boxes + stage_k / 2 TMEM columns each
-// TMEM columns: the accumulators first (two of up to 128 columns, or one of 256), then the operand ring
-__host__ __device__ constexpr int tile_a_col_base(int mt) { return mt <= 64 ? 128 : 256; }
-__host__ __device__ constexpr int tile_max_slots(int mt) { return (512 - tile_a_col_base(mt)) / (tile_stage_k(mt) / 2); }
-// stages of packed words a dequant thread holds in registers (loads issued that far ahead)
-__host__ __device__ constexpr int tile_prefetch(int mt) { return mt <= 64 ? 2 : 3; }
+constexpr int kTileThreads = (2 + kTileDequantWarps) * 32;   // producer, issuer, dequant / epilogue warps
+// accumulators that alternate between segments
+__host__ __device__ constexpr int tile_dbufs(int mt) { return mt <= 128 ? 2 : 1; }
+constexpr int kTileMaxStages = 8;                   // ring slots: activation box + stage_k / 2 TMEM columns each
+// TMEM columns: the accumulators first (two of 128 columns, or one of 256), then the operand ring
+constexpr int kTileACol = 256;
+constexpr int kTileSlots = (512 - kTileACol) / (kTileStageK / 2);
+constexpr int kTilePrefetch = 3;                    // stages of packed words a dequant thread holds in registers
 constexpr int kTileBarBytes = 1024;
 
-__host__ __device__ constexpr int tile_stage_bytes(int mt) { return mt * tile_stage_k(mt) * 2; }
+__host__ __device__ constexpr int tile_stage_bytes(int mt) { return mt * kTileStageK * 2; }
 
 struct TileParams {
     const uint32_t* Wq;
@@ -124,10 +104,10 @@ inline void tile_fill_chunk_math(TileParams& p) {
 // ------------------------------------------------------------------ tcgen05 / TMA wrappers
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
+__device__ __forceinline__ void tc_commit(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ void tc_commit(uint64_t* bar) { tc_commit(smem_u32(bar)); }
 // D(tmem) (+)= A(tmem) . B(shared descriptor); `accumulate` == 0 overwrites D.
 __device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
                                           uint32_t accumulate) {
@@ -138,33 +118,12 @@ __device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// 32 consecutive 32-bit TMEM columns of this thread's lane <- registers.
-__device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
-        "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"
-        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]),
-        "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]),
-        "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
-        : "memory");
-}
+// 16 consecutive 32-bit TMEM columns of this thread's lane <- registers.
 __device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
         ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
         "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-        : "memory");
-}
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
-        "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr)
         : "memory");
 }
 __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
@@ -174,12 +133,6 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
           "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr)
         : "memory");
-}
-__device__ __forceinline__ void tc_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr)
-                 : "memory");
 }
 __device__ __forceinline__ void tc_ld4(uint32_t taddr, uint32_t (&r)[4]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
@@ -352,7 +305,7 @@ struct StageRegs {
 // no Z buffer); EPI = bias / activation fused into the final cast.  (Both compiled in: decided at run time
 // they cost 5 to 10 % on narrow tiles and 9 % at M = 256.)
 template <int MT, int SG, bool BF, bool SYM, bool EPI>
-__global__ void __launch_bounds__(tile_threads(MT), 1)
+__global__ void __launch_bounds__(kTileThreads, 1)
 gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte alignment of the stage buffers (the swizzle atom) regardless of where the
@@ -361,15 +314,13 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
     constexpr int kStageBytes = tile_stage_bytes(MT);
     constexpr uint32_t kIdesc = tile_idesc(MT, BF);
     constexpr int kCW = MT / kTileSets;                  // accumulator columns (batch rows) per epilogue warp
-    constexpr int kNI = tile_issuers(MT);                // MMA-issuing warps, one accumulator (set) each
-    constexpr int kDBufs = tile_dbufs(MT);               // accumulators per issuer: accumulator (b, i) sits
-    constexpr int kDStride = tile_d_stride(MT);          // at column (b * kNI + i) * kDStride
-    constexpr int kStageK = tile_stage_k(MT);            // k per ring slot
+    constexpr int kDBufs = tile_dbufs(MT);               // accumulator b sits at column 128 b
+    constexpr int kStageK = kTileStageK;                 // k per ring slot
     constexpr int kSPU = kGroup / kStageK;               // stages per unit
     constexpr int kSlotCols = kStageK / 2;               // TMEM columns of one operand slot
-    constexpr int kACol = tile_a_col_base(MT);
+    constexpr int kACol = kTileACol;
     constexpr int kNW = kStageK / 32;                    // 16-byte chunks of a thread's column per stage
-    constexpr int kPF = tile_prefetch(MT);
+    constexpr int kPF = kTilePrefetch;
     constexpr int kNR = SG / kSPU > 0 ? SG / kSPU : 1;   // scale rows one stage touches
     constexpr bool sym = SYM;
 
@@ -391,7 +342,7 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
             mbar_init(&retired[kTileMaxStages + i], 1);
         }
         for (int i = 0; i < 2; ++i) {
-            mbar_init(&d_full[i], kNI);      // every issuer reports once per segment
+            mbar_init(&d_full[i], 1);
             mbar_init(&d_empty[i], kTileDequantWarps);
         }
         flags[0] = 0;
@@ -426,12 +377,8 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
             for (int j = 0; j < nst; ++j) {
                 if (r.turn != 0u && !wait_slot_free(retired, r)) { ok = false; break; }
                 if (elect_one()) {
-                    // one copy per stage: kStageK / 64 boxes of MT rows x 64 k, box b at b * MT * 128 bytes
                     mbar_expect_tx(&full[r.slot], (uint32_t)kStageBytes);
-                    if constexpr (kStageK == kTileBoxK)
-                        tma_load_2d(stage0 + (size_t)r.slot * kStageBytes, &tmap_a, kb * kTileBoxK, m, &full[r.slot]);
-                    else
-                        tma_load_3d(stage0 + (size_t)r.slot * kStageBytes, &tmap_a, 0, m, kb, &full[r.slot]);
+                    tma_load_2d(stage0 + (size_t)r.slot * kStageBytes, &tmap_a, kb * kTileBoxK, m, &full[r.slot]);
                 }
                 __syncwarp();
                 kb += kStageK / kTileBoxK;
@@ -443,56 +390,40 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
             flags[1] = (int)n;
             if (!ok) *abort_flag = 1;
         }
-    } else if (warp <= kNI) {
-        // ------------------------------------------------------------ MMA issuer `iss`: the stages whose
-        // index in this CTA is = iss (mod kNI), summed into this issuer's own accumulator
-        const int iss = warp - 1;
+    } else if (warp == 1) {
+        // ------------------------------------------------------------ MMA issuer
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        uint32_t n_seg = 0, n_prev = 0;
+        uint32_t n_seg = 0;
         bool ok = true;
         RingPos r{0, 0u, 0u};
         for (SegWalk w(p, kSPU); w.valid() && ok; w.next(), ++n_seg) {
             const int dbuf = n_seg % kDBufs;
-            // the epilogue of the segment that used this accumulator before must have drained it (an
-            // issuer without a stage in this segment waits too, so that its report below cannot land
-            // in the barrier phase of that earlier segment)
+            // the epilogue of the segment that used this accumulator before must have drained it
             if (!mbar_wait(&d_empty[dbuf], ((n_seg / kDBufs) & 1u) ^ 1u)) { ok = false; break; }
-            const uint32_t d_t = tmem_base + (dbuf * kNI + iss) * kDStride;
+            const uint32_t d_t = tmem_base + dbuf * 128;
             const int nst = w.stages_in_seg();
-            int j = kNI == 1 ? 0 : (int)(((uint32_t)(iss + kNI) - w.n0 % kNI) % kNI);
-            if (j >= nst) {
-                if (elect_one()) mbar_arrive(&d_full[dbuf]);     // nothing of mine in this segment
-                __syncwarp();
-                continue;
-            }
             uint32_t acc = 0u;                                   // the segment's first MMA overwrites
-            for (; j < nst; j += kNI) {
-                const uint32_t n = w.n0 + (uint32_t)j;
-                r.advance((int)(n - n_prev), R);
-                n_prev = n;
+            for (int j = 0; j < nst; ++j) {
                 if (!mbar_wait(&full[r.slot], r.ph)) { ok = false; break; }
                 tc_fence_after();
                 if (elect_one()) {
                     const uint64_t bdesc = smem_desc_sw128(smem_u32(stage0 + (size_t)r.slot * kStageBytes));
                     const uint32_t a_t = tmem_base + kACol + r.slot * kSlotCols;
 #pragma unroll
-                    for (int kk = 0; kk < kStageK / 16; ++kk) {
-                        // 16 k per instruction: 8 TMEM columns of A; in B 32 bytes along the swizzled rows of
-                        // a 64-k box, the next box MT * 128 bytes further
-                        const uint64_t bd = bdesc + (uint64_t)((kk / 4) * (MT * 128 / 16) + (kk % 4) * 2);
-                        tc_mma_ts(d_t, a_t + kk * 8, bd, kIdesc, kk == 0 ? acc : 1u);
-                    }
+                    for (int kk = 0; kk < kStageK / 16; ++kk)    // 16 k: 8 TMEM columns of A, 32 bytes along B's swizzled rows
+                        tc_mma_ts(d_t, a_t + kk * 8, bdesc + (uint64_t)(kk * 2), kIdesc, kk == 0 ? acc : 1u);
                     tc_commit(retired_bar(retired, r));
-                    if (j + kNI >= nst) tc_commit(&d_full[dbuf]);
+                    if (j + 1 == nst) tc_commit(&d_full[dbuf]);
                 }
                 __syncwarp();
                 acc = 1u;
+                r.advance(1, R);
             }
         }
         if (!ok && lane == 0) *abort_flag = 1;
     } else {
         // ------------------------------------------------------------ dequant + epilogue warps
-        const int dw = warp - (1 + kNI);       // 0..15
+        const int dw = warp - 2;               // 0..15
         const int set = dw >> 2;               // takes the stages whose index in this CTA is = set (mod 4)
         const int quarter = warp & 3;          // TMEM lanes this warp may touch
         const int row = quarter * 32 + lane;   // column n inside the CTA tile = TMEM lane
@@ -563,11 +494,11 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
         };
         point();
         // register ring of prefetched stages, written out so that no slot is ever copied
-        static_assert(kPF == 2 || kPF == 3, "the ring below has two or three slots");
+        static_assert(kPF == 3, "the ring below has three slots");
         StageRegs<kNW, kNR> pf0, pf1, pf2;
         fetch(pf0);
         fetch(pf1);
-        if (kPF == 3) fetch(pf2);
+        fetch(pf2);
         // Converting weights into the TMEM ring touches nothing the previous kernel may still be writing,
         // so it starts at once and runs until the ring is full; the dependency wait comes before this
         // warp's first write to global memory (the first epilogue).
@@ -615,11 +546,8 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
                 n_prev = n;
                 // convert ring slot pi, then refill it with the stage kPF ahead
                 if (pi == 0) { ok = convert(pf0, n); fetch(pf0); pi = 1; }
-                else if (kPF == 2 || pi == 1) { ok = convert(pf1, n); fetch(pf1); pi = (kPF == 3) ? 2 : 0; }
-                else {
-                    if constexpr (kPF == 3) { ok = convert(pf2, n); fetch(pf2); }
-                    pi = 0;
-                }
+                else if (pi == 1) { ok = convert(pf1, n); fetch(pf1); pi = 2; }
+                else { ok = convert(pf2, n); fetch(pf2); pi = 0; }
                 if (!ok) break;
                 tc_wait_st();
                 tc_fence_before();
@@ -639,38 +567,17 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
             const int T = w.t;
             const int n = w.nt * kTileCols + row;
             const int m_base = w.mt_i * MT + set * kCW;     // first batch row of this warp's columns
-            const uint32_t d_t = tmem_base + lane_addr + (dbuf * kNI) * kDStride + set * kCW;
-            // first stage of each issuer inside this segment: an issuer with none has no sum to add
-            const int iss0 = (int)(w.n0 % kNI);
+            const uint32_t d_t = tmem_base + lane_addr + dbuf * 128 + set * kCW;
             const long long tile_u0 = (long long)T * p.G;
             const bool whole = w.whole_tile();
             // first segment of a chunk -> slot 2 ci, its continuation into a later tile -> 2 ci + 1
             float* part = p.ws + ((size_t)(2 * w.ci + (w.first ? 0 : 1)) * MT + set * kCW) * kTileCols + row;
-            constexpr int kStep = kCW >= 16 ? 16 : kCW;
+            constexpr int kStep = 16;
 #pragma unroll 1
             for (int cc = 0; cc < kCW; cc += kStep) {
                 uint32_t v[kStep];
-                if constexpr (kNI == 1) {
-                    if constexpr (kStep == 16) tc_ld16(d_t + cc, v);
-                    else if constexpr (kStep == 8) tc_ld8(d_t + cc, v);
-                    else tc_ld4(d_t + cc, v);
-                    tc_wait_ld();
-                }
-                // several issuers: add their sums in stage order (issuer iss0 took the segment's first stage)
-#pragma unroll
-                for (int ii = 0; ii < (kNI == 1 ? 0 : kNI); ++ii) {
-                    if (ii >= nst) break;                        // warp-uniform
-                    int i = iss0 + ii;
-                    if (i >= kNI) i -= kNI;
-                    uint32_t t[kStep];
-                    if constexpr (kStep == 16) tc_ld16(d_t + i * kDStride + cc, t);
-                    else if constexpr (kStep == 8) tc_ld8(d_t + i * kDStride + cc, t);
-                    else tc_ld4(d_t + i * kDStride + cc, t);
-                    tc_wait_ld();
-#pragma unroll
-                    for (int q = 0; q < kStep; ++q)
-                        v[q] = ii == 0 ? t[q] : __float_as_uint(__uint_as_float(v[q]) + __uint_as_float(t[q]));
-                }
+                tc_ld16(d_t + cc, v);
+                tc_wait_ld();
                 if (whole) {
                     if (n < p.N) {
 #pragma unroll

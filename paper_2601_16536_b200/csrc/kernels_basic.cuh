@@ -243,19 +243,18 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ ws, uint16_t* __r
 // of a 32 us launch at M = 256); here the whole GPU does it at once.
 template <bool BF>
 __global__ void __launch_bounds__(256)
-tile_splitk_reduce_kernel(const float* __restrict__ ws, uint16_t* __restrict__ C, int M, int N, int mt_log2, int n_tiles,
-                          int split_k, long long quads, Epilogue epi) {
+tile_splitk_reduce_kernel(const float* __restrict__ ws, uint16_t* __restrict__ C, int M, int N, int mt, FastDiv div_mt,
+                          int n_tiles, FastDiv div_ntiles, int split_k, long long quads, Epilogue epi) {
     // the next kernel of the stream may start its prologue; the partial tiles are the previous kernel's output
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= quads) return;
-    const int mt = 1 << mt_log2;
     const int nq = (int)(q & 31);                       // which four of the tile's 128 columns
-    const long long r = q >> 5;
-    const int m_local = (int)(r & (mt - 1));
-    const int T = (int)(r >> mt_log2);                  // tile = batch tile * n_tiles + column tile
-    const int mt_i = T / n_tiles, nt = T - mt_i * n_tiles;
+    const int r = (int)(q >> 5);                        // (tiles * mt < 2^31: the caller checks)
+    const int T = fast_div(r, div_mt);                  // tile = batch tile * n_tiles + column tile
+    const int m_local = r - T * mt;
+    const int mt_i = fast_div(T, div_ntiles), nt = T - mt_i * n_tiles;
     const int m = mt_i * mt + m_local, n = nt * 128 + nq * 4;
     if (m >= M || n >= N) return;
     const size_t slot = (size_t)2 * mt * 128;           // floats between the slots of neighbouring slices
