@@ -605,13 +605,12 @@ int w4a16_quantize(const uint16_t* W16, uint32_t* Wq_raw, uint16_t* S_raw, uint8
     DeviceState* d = nullptr;
     if ((rc = current_device(&d)) != W4A16_OK) return rc;
     if (!d->is_sm100) return W4A16_ERR_ARCH;
-    const int G = K / group;
-    const size_t total = (size_t)G * N;
-    const unsigned blocks = (unsigned)((total + 127) / 128);
+    const int G = K / kGroup, sg = kGroup / group;
+    const unsigned blocks = (unsigned)((long long)G * (N / kTileN));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     uint8_t* z = sym ? nullptr : Z_raw;
-    if (bf) quantize_kernel<true><<<blocks, 128, 0, st>>>(W16, Wq_raw, S_raw, z, N, G, group, sym ? 1 : 0);
-    else quantize_kernel<false><<<blocks, 128, 0, st>>>(W16, Wq_raw, S_raw, z, N, G, group, sym ? 1 : 0);
+    if (bf) quantize_kernel<true><<<blocks, kBlockKernelThreads, 0, st>>>(W16, Wq_raw, S_raw, z, N, G, sg, sym ? 1 : 0);
+    else quantize_kernel<false><<<blocks, kBlockKernelThreads, 0, st>>>(W16, Wq_raw, S_raw, z, N, G, sg, sym ? 1 : 0);
     return cudaGetLastError() == cudaSuccess ? W4A16_OK : W4A16_ERR_CUDA;
 }
 
@@ -631,11 +630,10 @@ int w4a16_pack_fmt(const uint32_t* Wq_raw, const uint16_t* S_raw, const uint8_t*
     if (!d->is_sm100) return W4A16_ERR_ARCH;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int G = K / kGroup, sg = kGroup / group;
-    size_t words = (size_t)K * N / 8, sc = (size_t)G * sg * N, zw = sc / 8;
-    pack_wq_kernel<<<(unsigned)((words + 255) / 256), 256, 0, st>>>(Wq_raw, static_cast<uint32_t*>(Wq), N, G, words);
-    pack_s_kernel<<<(unsigned)((sc + 255) / 256), 256, 0, st>>>(S_raw, static_cast<uint16_t*>(S), N, G, sg, sc);
-    if (!sym)
-        pack_z_kernel<<<(unsigned)((zw + 255) / 256), 256, 0, st>>>(Z_raw, static_cast<uint32_t*>(Z), N, G, sg, zw);
+    const int blocks = (int)((long long)G * (N / kTileN)), per = kBlockKernelThreads / 32;
+    pack_kernel<<<(unsigned)((blocks + per - 1) / per), kBlockKernelThreads, 0, st>>>(
+        Wq_raw, S_raw, sym ? nullptr : Z_raw, static_cast<uint32_t*>(Wq), static_cast<uint16_t*>(S),
+        sym ? nullptr : static_cast<uint8_t*>(Z), N, G, sg, blocks);
     ++d->pack_epoch;
     return cudaGetLastError() == cudaSuccess ? W4A16_OK : W4A16_ERR_CUDA;
 }
@@ -658,16 +656,16 @@ int w4a16_dequant_fmt(const void* Wq, const void* S, const void* Z, uint16_t* W1
     DeviceState* d = nullptr;
     if ((rc = current_device(&d)) != W4A16_OK) return rc;
     if (!d->is_sm100) return W4A16_ERR_ARCH;
-    size_t words = (size_t)K * N / 8;
+    const int blocks = (int)((long long)(K / kGroup) * (N / kTileN)), per = kBlockKernelThreads / 32;
+    const unsigned grid = (unsigned)((blocks + per - 1) / per);
     const uint32_t* z = sym ? nullptr : static_cast<const uint32_t*>(Z);
-    const unsigned blocks = (unsigned)((words + 255) / 256);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (bf)
-        dequant_kernel<true><<<blocks, 256, 0, st>>>(static_cast<const uint32_t*>(Wq), static_cast<const uint16_t*>(S), z,
-                                                     W16, N, K / kGroup, kGroup / group, words);
+        dequant_kernel<true><<<grid, kBlockKernelThreads, 0, st>>>(static_cast<const uint32_t*>(Wq), static_cast<const uint16_t*>(S),
+                                                                   z, W16, N, K / kGroup, kGroup / group, blocks);
     else
-        dequant_kernel<false><<<blocks, 256, 0, st>>>(static_cast<const uint32_t*>(Wq), static_cast<const uint16_t*>(S), z,
-                                                      W16, N, K / kGroup, kGroup / group, words);
+        dequant_kernel<false><<<grid, kBlockKernelThreads, 0, st>>>(static_cast<const uint32_t*>(Wq), static_cast<const uint16_t*>(S),
+                                                                    z, W16, N, K / kGroup, kGroup / group, blocks);
     return cudaGetLastError() == cudaSuccess ? W4A16_OK : W4A16_ERR_CUDA;
 }
 

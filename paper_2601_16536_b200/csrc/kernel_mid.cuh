@@ -9,7 +9,7 @@
 //     CTAs find room beside the last ones of this launch (programmatic dependent launch);
 //   - packed weights through a shared-memory ring filled by TMA bulk copies, 2 units (2 x 128 k) of the tile's two
 //     64-column blocks per stage, six copies by a warp of its own: the eight dequant warps issue no global loads and
-//     keep no addresses (20.5 M warp instructions for K = 28672 / N = 8192, the conversion itself is 11.7 M of them);
+//     keep no addresses (21.0 M warp instructions for K = 28672 / N = 8192, the conversion itself is 12 M of them);
 //   - ten warps and not eleven, so that 96 registers a thread fit twice on an SM: at 80 the stage loop spends a
 //     quarter of its instructions on moving and re-making addresses (39.1 against 33.5 us at M = 32 on that shape);
 //   - S slices of a tile's K range as a cluster of S CTAs.  Every CTA finishes 1 / S of the tile's batch rows: it

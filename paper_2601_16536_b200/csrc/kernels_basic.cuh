@@ -6,66 +6,53 @@
 
 namespace w4a16 {
 
+// The three kernels below work on whole blocks (64 columns x 128 k), numbered with the column tile fastest, so that the
+// CTAs that run together touch neighbouring columns of the same rows.  They are bound by HBM.
+constexpr int kBlockKernelThreads = 128;
+struct BlockPos {
+    int t, g;        // column tile, k block
+    size_t blk;      // position in the packed buffers
+    __device__ __forceinline__ BlockPos(int b, int T, int G) : t(b % T), g(b / T), blk((size_t)t * G + g) {}
+};
+
 // ------------------------------------------------------------------ pack
-// Decode a packed word's position: idx -> block, column inside the tile, first k inside the block.
-__device__ __forceinline__ void word_position(size_t idx, size_t& blk, int& col, int& kw) {
-    const int within = (int)(idx & 1023);
-    blk = idx >> 10;
-    const int c = within >> 9, rb = (within >> 6) & 7, i = (within >> 5) & 1, slot = (within >> 2) & 7;
-    col = rb * 8 + ((slot - 4 * i) & 7);
-    kw = c * 8 + i * 4 + (within & 3);
+// Raw word (nibble i = k + i) -> packed word (even k in the low half, odd k in the high half, ascending).
+__device__ __forceinline__ uint32_t pack_word(uint32_t r) {
+    const uint32_t e = r & 0x0f0f0f0fu, o = (r >> 4) & 0x0f0f0f0fu;
+    return __byte_perm(e | (e >> 4), o | (o >> 4), 0x6420);
 }
 
-// One thread per packed word.  Pure bit moves (Section 2.2 storage packing): the word's eight k
-// are one raw word of the same column; only the nibble order inside the word changes.
-__global__ void pack_wq_kernel(const uint32_t* __restrict__ raw, uint32_t* __restrict__ out, int N, int G,
-                               size_t total_words) {
-    size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= total_words) return;
-    size_t blk;
-    int col, kw;
-    word_position(idx, blk, col, kw);
-    const int t = (int)(blk / G), g = (int)(blk % G);
-    const uint32_t r = raw[(size_t)(g * (kGroup / 8) + kw) * N + (size_t)t * kTileN + col];
-    uint32_t w = 0;
+// One warp per block.  A lane reads four consecutive k-words of one column (32 columns: 128 bytes a row) and writes them
+// as the column's 16-byte chunk: eight columns make up a 128-byte line.  Scales and zero points of the block go along in
+// the same launch.  K = 11008 / N = 4096: three kernels with a thread per word 36 us together, this one
+// 12.4 us (HBM floor 6.9).
+__global__ void __launch_bounds__(kBlockKernelThreads)
+pack_kernel(const uint32_t* __restrict__ Wq_raw, const uint16_t* __restrict__ S_raw, const uint8_t* __restrict__ Z_raw,
+            uint32_t* __restrict__ Wq, uint16_t* __restrict__ S, uint8_t* __restrict__ Z, int N, int G, int sg, int blocks) {
+    const int b = blockIdx.x * (kBlockKernelThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (b >= blocks) return;
+    const BlockPos pos(b, N / kTileN, G);
+    const uint32_t* src = Wq_raw + (size_t)pos.g * (kGroup / 8) * N + (size_t)pos.t * kTileN + lane;
+    uint32_t r[2][16];
 #pragma unroll
-    for (int p = 0; p < 8; ++p) {
-        const int off = 2 * (p & 3) + (p >> 2);  // k offset held by nibble p
-        w |= ((r >> (4 * off)) & 15u) << (4 * p);
+    for (int kw = 0; kw < 16; ++kw)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) r[h][kw] = __ldg(src + (size_t)kw * N + 32 * h);
+    __syncwarp();                        // (all 32 loads stay ahead of the first store)
+    uint4* dst = reinterpret_cast<uint4*>(Wq + pos.blk * kBlockWords);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)      // k-words 4 q .. 4 q + 3
+            dst[block_word_index(32 * h + lane, 4 * q) / 4] = make_uint4(pack_word(r[h][4 * q]), pack_word(r[h][4 * q + 1]),
+                                                                         pack_word(r[h][4 * q + 2]), pack_word(r[h][4 * q + 3]));
+    // positions 2 lane, 2 lane + 1 of a row of scales / zero points belong to columns c0, c0 + 8 (sz_perm)
+    const int c0 = (lane & 16) * 2 + ((lane >> 1) & 7) + (lane & 1) * 16;
+    for (int j = 0; j < sg; ++j) {
+        const size_t in = (size_t)(pos.g * sg + j) * N + (size_t)pos.t * kTileN + c0, row = pos.blk * sg + j;
+        reinterpret_cast<uint32_t*>(S + row * kSBlockHalves)[lane] = (uint32_t)S_raw[in] | ((uint32_t)S_raw[in + 8] << 16);
+        if (Z_raw != nullptr) Z[row * (kZBlockWords * 4) + lane] = (uint8_t)((Z_raw[in] & 15u) | (Z_raw[in + 8] << 4));
     }
-    out[idx] = w;
-}
-
-// Scales: packed position idx = ((blk * sg + j) * 64 + sz_perm(col)); one thread per raw scale.
-__global__ void pack_s_kernel(const uint16_t* __restrict__ raw, uint16_t* __restrict__ out, int N, int G, int sg,
-                              size_t total) {
-    size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;   // over (t, g, j, col)
-    if (idx >= total) return;
-    const int col = (int)(idx & 63);
-    const size_t row = idx >> 6;                 // (t * G + g) * sg + j
-    const int j = (int)(row % sg);
-    const size_t blk = row / sg;
-    const int t = (int)(blk / G), g = (int)(blk % G);
-    out[row * kSBlockHalves + sz_perm(col)] = raw[(size_t)(g * sg + j) * N + (size_t)t * kTileN + col];
-}
-
-// Zero points: one thread per packed word (eight permuted positions of one row).
-__global__ void pack_z_kernel(const uint8_t* __restrict__ raw, uint32_t* __restrict__ out, int N, int G, int sg,
-                              size_t total_words) {
-    size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= total_words) return;
-    const int wi = (int)(idx & 7);
-    const size_t row = idx >> 3;
-    const int j = (int)(row % sg);
-    const size_t blk = row / sg;
-    const int t = (int)(blk / G), g = (int)(blk % G);
-    uint32_t w = 0;
-    for (int col = 0; col < kTileN; ++col) {
-        const int p = sz_perm(col);
-        if ((p >> 3) == wi)
-            w |= (uint32_t)(raw[(size_t)(g * sg + j) * N + (size_t)t * kTileN + col] & 15u) << (4 * (p & 7));
-    }
-    out[idx] = w;
 }
 
 // Scale (16-bit pattern) and zero point of column `col` for the k-word kw (0..15) of block blk.
@@ -96,68 +83,163 @@ __device__ __forceinline__ float group_scale(float num, float den, uint16_t& bit
 }
 
 template <bool BF>
-__global__ void quantize_kernel(const uint16_t* __restrict__ W16, uint32_t* __restrict__ Wq, uint16_t* __restrict__ S,
-                                uint8_t* __restrict__ Z, int N, int G, int group, int symmetric) {
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;   // (g, n), n fastest
-    if (idx >= (size_t)G * N) return;
-    const int n = (int)(idx % (size_t)N), g = (int)(idx / (size_t)N);
-    const uint16_t* col = W16 + (size_t)g * group * N + n;
-    float lo = INFINITY, hi = -INFINITY, amax = 0.0f;
-    for (int k = 0; k < group; ++k) {
-        const float x = widen<BF>(col[(size_t)k * N]);
-        lo = x < lo ? x : lo;
-        hi = x > hi ? x : hi;
-        amax = fabsf(x) > amax ? fabsf(x) : amax;
-    }
-    uint16_t sb;
-    float s;
-    int z;
-    if (symmetric) {
-        s = group_scale<BF>(amax, 7.0f, sb);
-        z = kSymZero;
-    } else {
-        s = group_scale<BF>(__fsub_rn(hi, lo), 15.0f, sb);
-        const float zf = rintf(__fdiv_rn(-lo, s));
-        z = zf < 0.0f ? 0 : zf > 15.0f ? 15 : (int)zf;
-    }
-    S[idx] = sb;
-    if (Z != nullptr) Z[idx] = (uint8_t)z;
-    for (int kw = 0; kw < group / 8; ++kw) {
-        uint32_t w = 0;
+__device__ __forceinline__ uint32_t min2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    if constexpr (BF) asm("min.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    else asm("min.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+template <bool BF>
+__device__ __forceinline__ uint32_t max2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    if constexpr (BF) asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    else asm("max.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
+// One code of the definition above.
+__device__ __forceinline__ uint32_t quantize_exact(float x, float s, int z) {
+    const float r = __fadd_rn(rintf(__fdiv_rn(x, s)), (float)z);
+    return (uint32_t)(r < 0.0f ? 0 : r > 15.0f ? 15 : (int)r);
+}
+
+// One CTA per 64 columns x 128 k, each of its four warps 32 k: a lane keeps its two columns' 32 rows in registers (128
+// bytes a row and warp, every weight read once), warps of the same group exchange minimum and maximum through shared
+// memory.  Codes
+// without a division: u = x * (1 / s) + 768 in one FMA is the quotient rounded to a multiple of 2^-14 (where it is below
+// 256; beyond 16 every code is clamped anyway), and that has the same nearest integer, ties to even, as the definition's
+// fl(x / s): x = X 2^a and s = T 2^b have 11-bit significands, so x - h s for a half-integer h is zero or at least
+// 2^min(a, b - 1), which with |h| >= 1/2 (hence a >= b - 2) is more than 2^-13 of s.  The reciprocal, the FMA and the
+// definition's own division are off by less than 2^-19, the grid by at most 2^-15: a tie lands on the half exactly,
+// anything else stays on its side of it.  (Scales whose reciprocal is not a normal number take the divisions.)
+// K = 11008 / N = 4096: a thread per (group, column), two passes and a division per weight 96 us, this form 29 us (HBM floor 17).
+template <bool BF>
+__global__ void __launch_bounds__(kBlockKernelThreads)
+quantize_kernel(const uint16_t* __restrict__ W16, uint32_t* __restrict__ Wq, uint16_t* __restrict__ S,
+                uint8_t* __restrict__ Z, int N, int G, int sg, int symmetric) {
+    __shared__ uint32_t part_lo[4][32], part_hi[4][32];
+    const BlockPos pos(blockIdx.x, N / kTileN, G);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const size_t n = (size_t)pos.t * kTileN + 2 * lane;
+    const uint16_t* src = W16 + (size_t)(pos.g * kGroup + warp * 32) * N + n;
+    uint32_t v[32];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float x = widen<BF>(col[(size_t)(kw * 8 + i) * N]);
-            const float r = __fadd_rn(rintf(__fdiv_rn(x, s)), (float)z);
-            const int q = r < 0.0f ? 0 : r > 15.0f ? 15 : (int)r;
-            w |= (uint32_t)q << (4 * i);
+    for (int k = 0; k < 32; ++k) v[k] = __ldg(reinterpret_cast<const uint32_t*>(src + (size_t)k * N));
+    uint32_t lo = BF ? 0x7f807f80u : 0x7c007c00u, hi = lo | 0x80008000u;     // +inf, -inf
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+        lo = min2<BF>(lo, v[k]);
+        hi = max2<BF>(hi, v[k]);
+    }
+    const int wpg = 4 / sg, first = warp / wpg * wpg;    // warps that share a group, the first of them
+    part_lo[warp][lane] = lo;
+    part_hi[warp][lane] = hi;
+    __syncthreads();
+    for (int i = 0; i < wpg; ++i) {
+        lo = min2<BF>(lo, part_lo[first + i][lane]);
+        hi = max2<BF>(hi, part_hi[first + i][lane]);
+    }
+    constexpr float kGrid = 768.0f;                      // 1.5 * 2^9: neighbours 2^-14 apart
+    constexpr float kMagic = 12582912.0f;                // 1.5 * 2^23, bits 0x4b400000: neighbours 1 apart
+    uint16_t sb[2];
+    float s[2], rinv[2], least[2], most[2];
+    int z[2];
+    bool slow[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const float l = widen<BF>((uint16_t)(lo >> (16 * c))), h = widen<BF>((uint16_t)(hi >> (16 * c)));
+        if (symmetric) {
+            s[c] = group_scale<BF>(fmaxf(fabsf(l), fabsf(h)), 7.0f, sb[c]);
+            z[c] = kSymZero;
+        } else {
+            s[c] = group_scale<BF>(__fsub_rn(h, l), 15.0f, sb[c]);
+            const float zf = rintf(__fdiv_rn(-l, s[c]));
+            z[c] = zf < 0.0f ? 0 : zf > 15.0f ? 15 : (int)zf;
         }
-        Wq[((size_t)g * (group / 8) + kw) * N + n] = w;
+        rinv[c] = __frcp_rn(s[c]);
+        least[c] = kMagic - (float)z[c];                 // codes 0 and 15
+        most[c] = kMagic + (float)(15 - z[c]);
+        slow[c] = !(s[c] > 1e-30f && s[c] < 1e30f);
+    }
+    const size_t out = (size_t)(pos.g * sg + warp / wpg) * N + n;
+    if (warp == first) {
+        *reinterpret_cast<uint32_t*>(S + out) = (uint32_t)sb[0] | ((uint32_t)sb[1] << 16);
+        if (Z != nullptr) *reinterpret_cast<uint16_t*>(Z + out) = (uint16_t)(z[0] | (z[1] << 8));
+    }
+    uint32_t* dst = Wq + (size_t)(pos.g * (kGroup / 8) + warp * 4) * N + n;
+#pragma unroll
+    for (int kw = 0; kw < 4; ++kw) {
+        uint32_t w[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            uint32_t acc = 0u;
+#pragma unroll
+            for (int i = 7; i >= 0; --i) {
+                const float u = __fmaf_rn(widen<BF>((uint16_t)(v[8 * kw + i] >> (16 * c))), rinv[c], kGrid);
+                const float y = __fadd_rn(u, kMagic - kGrid);          // low bits: round(x / s)
+                acc = acc * 16u + __float_as_uint(fminf(fmaxf(y, least[c]), most[c]));
+            }
+            w[c] = acc + ((uint32_t)z[c] - 0x4b400000u) * 0x11111111u; // + z in each digit, the constant's copies out again
+            if (slow[c]) {
+                w[c] = 0u;
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    w[c] |= quantize_exact(widen<BF>((uint16_t)(v[8 * kw + i] >> (16 * c))), s[c], z[c]) << (4 * i);
+            }
+        }
+        *reinterpret_cast<uint2*>(dst + (size_t)kw * N) = make_uint2(w[0], w[1]);
     }
 }
 
 // ------------------------------------------------------------------ dequant
-// Algorithm 1, Phase 1 as a standalone kernel: one thread per packed word, eight results
-// w16 = rn((q - z) * s) in the 16-bit format: (q - z) is formed exactly and multiplied by s with one
-// multiply (round-to-nearest-even, subnormals kept).  Z == nullptr: symmetric format, z = 8.
+// Algorithm 1, Phase 1 as a standalone kernel: w16 = rn((q - z) * s) in the 16-bit format: (q - z) is formed exactly and
+// multiplied by s with one multiply (round-to-nearest-even, subnormals kept).  Z == nullptr: symmetric format, z = 8.
+// One warp per block: a lane takes 8 neighbouring columns x 32 k (eight 16-byte loads in flight), swaps the halves of
+// neighbouring columns' registers and stores 16 bytes of a row at a time, eight lanes one 128-byte line of the row.
+// K = N = 8192: a thread per word with 2-byte stores 68 us, this form 31 us (HBM floor 25.6).
 template <bool BF>
-__global__ void dequant_kernel(const uint32_t* __restrict__ Wq, const uint16_t* __restrict__ S,
-                               const uint32_t* __restrict__ Z, uint16_t* __restrict__ W16, int N, int G, int sg,
-                               size_t total_words) {
-    size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= total_words) return;
-    size_t blk;
-    int col, kw;
-    word_position(idx, blk, col, kw);
-    const int t = (int)(blk / G), g = (int)(blk % G);
-    uint16_t s;
-    uint32_t z;
-    load_sz(S, Z, blk, sg, col, kw, s, z);
-    const Pack8 f = dequant_word<BF>(Wq[idx], zconst_lo<BF>(z), zconst_hi<BF>(z), (uint32_t)s * 0x00010001u);
-    uint16_t* p = W16 + (size_t)(g * kGroup + kw * 8) * N + (size_t)t * kTileN + col;
+__global__ void __launch_bounds__(kBlockKernelThreads)
+dequant_kernel(const uint32_t* __restrict__ Wq, const uint16_t* __restrict__ S, const uint32_t* __restrict__ Z,
+               uint16_t* __restrict__ W16, int N, int G, int sg, int blocks) {
+    const int b = blockIdx.x * (kBlockKernelThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (b >= blocks) return;
+    const BlockPos pos(b, N / kTileN, G);
+    const int rb = lane & 7, kq = lane >> 3;      // columns 8 rb .. + 7, k = 32 kq .. + 31 of the block
+    const uint4* src = reinterpret_cast<const uint4*>(Wq + pos.blk * kBlockWords);
+    uint4 w[8];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        p[(size_t)(2 * j) * N] = (uint16_t)(f.h[j] & 0xffffu);
-        p[(size_t)(2 * j + 1) * N] = (uint16_t)(f.h[j] >> 16);
+    for (int c = 0; c < 8; ++c) w[c] = __ldg(src + block_word_index(8 * rb + c, 4 * kq) / 4);
+    const size_t row = pos.blk * sg + kq * sg / 4;
+    // column 8 rb + c sits at position p0 + 4 c of a row of scales / zero points
+    const int p0 = sz_perm(8 * rb);
+    uint4 zz = make_uint4(0u, 0u, 0u, 0u);
+    if (Z != nullptr) zz = __ldg(reinterpret_cast<const uint4*>(Z + row * kZBlockWords) + (p0 >> 5));
+    const uint32_t zw[4] = {zz.x, zz.y, zz.z, zz.w};
+    uint32_t s2[8], zlo[8], zhi[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        s2[c] = (uint32_t)__ldg(S + row * kSBlockHalves + p0 + 4 * c) * 0x00010001u;
+        const uint32_t z = Z == nullptr ? (uint32_t)kSymZero : ((zw[c >> 1] >> (16 * (c & 1) + 4 * (p0 & 3))) & 15u);
+        zlo[c] = zconst_lo<BF>(z);
+        zhi[c] = zconst_hi<BF>(z);
+    }
+    uint16_t* dst = W16 + (size_t)(pos.g * kGroup + 32 * kq) * N + (size_t)pos.t * kTileN + 8 * rb;
+#pragma unroll
+    for (int kw = 0; kw < 4; ++kw) {
+        Pack8 f[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const uint32_t word = kw == 0 ? w[c].x : kw == 1 ? w[c].y : kw == 2 ? w[c].z : w[c].w;
+            f[c] = dequant_word<BF>(word, zlo[c], zhi[c], s2[c]);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            uint16_t* p = dst + (size_t)(8 * kw + 2 * j) * N;
+            *reinterpret_cast<uint4*>(p) = make_uint4(__byte_perm(f[0].h[j], f[1].h[j], 0x5410), __byte_perm(f[2].h[j], f[3].h[j], 0x5410),
+                                                      __byte_perm(f[4].h[j], f[5].h[j], 0x5410), __byte_perm(f[6].h[j], f[7].h[j], 0x5410));
+            *reinterpret_cast<uint4*>(p + N) = make_uint4(__byte_perm(f[0].h[j], f[1].h[j], 0x7632), __byte_perm(f[2].h[j], f[3].h[j], 0x7632),
+                                                          __byte_perm(f[4].h[j], f[5].h[j], 0x7632), __byte_perm(f[6].h[j], f[7].h[j], 0x7632));
+        }
     }
 }
 

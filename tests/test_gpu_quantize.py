@@ -41,6 +41,30 @@ def test_quantize_is_bit_exact(group, symmetric, bf16):
         assert np.array_equal(Z.cpu().numpy(), z)
 
 
+@pytest.mark.parametrize("group", [32, 128])
+@pytest.mark.parametrize("symmetric", [False, True])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_quantize_is_bit_exact_on_ties_and_extreme_scales(group, symmetric, bf16):
+    """Quotients that are exact half-integers (weights k/2 times a short scale), groups far from zero (every quotient
+    large), and column magnitudes from the format's subnormals to its largest numbers: the integers still are the ones
+    of the definition's binary32 division."""
+    K, N = 256, 128
+    r = np.random.Generator(np.random.PCG64([group, 21]))
+    x = (r.integers(-15, 16, size=(K, N)) * 0.5 * 2.0 ** r.integers(-6, 3, size=(1, N))).astype(np.float64)
+    x[:, 1::4] = r.standard_normal((K, N // 4)) * 1e-3 + 100.0
+    x[:, 2::4] = r.standard_normal((K, N // 4)) * 2.0 ** np.linspace(-120 if bf16 else -23, 100 if bf16 else 11, N // 4)
+    x[:, 3::4] = r.integers(-255, 256, size=(K, N // 4)) * 0.125
+    bits = wl._bits16(x.astype(np.float32), bf16)
+    flags = (B.FLAG_SYMMETRIC if symmetric else 0) | (B.FLAG_BF16 if bf16 else 0)
+    W = torch.from_numpy(bits.view(np.int16)).cuda().view(torch.bfloat16 if bf16 else torch.float16)
+    Wq, S, Z = B.w4a16_quantize(W, group, flags)
+    torch.cuda.synchronize()
+    wq, s, z = oracle.quantize(bits, K, N, group, symmetric=symmetric, bf16=bf16)
+    assert np.array_equal(Wq.cpu().numpy().view(np.uint32), wq)
+    assert np.array_equal(S.view(torch.int16).cpu().numpy().view(np.uint16), s)
+    assert symmetric or np.array_equal(Z.cpu().numpy(), z)
+
+
 @pytest.mark.parametrize("M,symmetric", [(4, False), (4, True), (48, False)])
 def test_quantize_pack_gemm_chain(M, symmetric):
     K, N, group = 2048, 512, 128
