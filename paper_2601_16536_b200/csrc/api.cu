@@ -30,8 +30,8 @@ struct DeviceState {
     size_t ws_bytes = 0;
     bool decode_attr_set[3][2][3][2][2][2] = {};   // [mb][cluster exchange][log2 SG][bf16][symmetric][tensor-copy rows]
     int mid_clusters[16] = {};         // mid_max_clusters, 0 = not asked yet
-    bool mid_attr_set[3][2][2] = {};   // [log2 SG][bf16][symmetric]
-    bool tile_attr_set[2][3][2][2][2] = {};   // [batch-tile index][log2 SG][bf16][symmetric][epilogue]
+    bool mid_attr_set[2][3][2][2] = {};   // [64 / 128 rows][log2 SG][bf16][symmetric]
+    bool tile_attr_set[3][2][2][2] = {};   // [log2 SG][bf16][symmetric][epilogue]
     // Programmatic dependent launch lets a GEMM kernel prefetch packed weights before the previous
     // kernel in its stream has finished.  The previous kernel of a stream may be a w4a16_pack that
     // writes those weights, so the first GEMM launched on a stream after any pack on the device is a
@@ -235,45 +235,52 @@ int choose_split_decode(int M, int N, int G, int sms) {
 }
 
 // ---- tile-path launch geometry ----------------------------------------------------
-// MT (batch rows per CTA tile = UMMA N) is 128 up to 128 rows, else 256 (fewer rows go to the kernel above).  The unit
-// range (batch tile x column tile x group) is cut into `nchunks` chunks for `ctas` persistent CTAs: balanced chunks, one
-// per CTA, when the caller leaves split_k open; S slices per tile otherwise.
+// The unit range (batch tile x column tile x group) is cut into `nchunks` chunks for `ctas` persistent CTAs: balanced
+// chunks, one per CTA, when the caller leaves split_k open and slices would leave too many SMs idle; S slices per tile or
+// whole tiles otherwise.
 struct TileGeom {
-    int mt, mt_index, m_tiles, n_tiles, split_k, nchunks, stages, smem_bytes, ctas;
-    long tiles;
+    int mt, m_tiles, n_tiles, split_k, nchunks, stages, smem_bytes, ctas;
+    long tiles, cost;
 };
 
 constexpr size_t kTileTicketBytes = 131072;   // 16 counters per tile, after the 16 KiB of the small-M kernel
 constexpr size_t kWsFullHeaderBytes = kWsHeaderBytes + kTileTicketBytes;
 constexpr long kTileMaxTicketTiles = kTileTicketBytes / (sizeof(int) * kTileDequantWarps);
 
-TileGeom tile_geom(int M, int N, int G, int split_k, int sms, int max_smem) {
+// Activation ring of a CTA: beyond about 200 KiB of shared memory the L1 that the weight loads pass through gets too small
+// (148 whole tiles of K = 16384, 208 rows: eight slots 120 us, six 100; 256 rows have six either way).
+constexpr int kTileSmem = 200 * 1024;
+
+// What a launch costs, in ns, and how its units are cut.  A unit takes 400 + 1.85 mt ns (148 whole tiles of K = 16384: 80
+// rows 74 us, 128 83, 160 90, 208 100, 256 111), a launch 3.5 us beside its units, K slices 5.5 us more for storing
+// partial tiles and the kernel that sums them.
+TileGeom tile_geom_rows(int mt, int M, int N, int G, int split_k, int sms) {
     TileGeom g;
-    g.mt_index = M <= 128 ? 0 : 1;
-    g.mt = 128 << g.mt_index;
-    g.m_tiles = (M + g.mt - 1) / g.mt;
+    g.mt = mt;
+    g.m_tiles = (M + mt - 1) / mt;
     g.n_tiles = (N + kTileCols - 1) / kTileCols;
     g.tiles = (long)g.m_tiles * g.n_tiles;
     // more tiles than ticket counters: whole tiles only (no partial tiles, no tickets)
     if (split_k == 0 && g.tiles > kTileMaxTicketTiles) split_k = 1;
+    const long unit_ns = 400 + mt * 37 / 20;
+    g.cost = 0;
     if (split_k == 0) {
         // Balanced chunks use every SM to the end, but a chunk that starts or ends inside a tile leaves
         // an FP32 partial tile behind (store, ticket, reload: the larger the batch tile the dearer, and
         // in mid-stream it stalls the pipeline).  S slices per tile (tiles <= SMs) or whole tiles in
-        // waves (tiles > SMs) avoid that at the price of idle SMs.  Cost model in groups per CTA; the
-        // constants are fitted to measurements (K = N = 8192 with M up to 4096).
-        const long penalty = 6 + g.mt / 8;
-        const long balanced_cost = (g.tiles * G + sms - 1) / sms + penalty;
+        // waves (tiles > SMs) avoid that at the price of idle SMs.  Constants fitted to K = N = 8192 with M up to 4096.
+        const long balanced = ((g.tiles * G + sms - 1) / sms + 6 + mt / 8) * unit_ns;
         int s0 = 1;
-        long classic_cost;
+        long classic;
         if (g.tiles <= sms) {
             s0 = sms / (int)g.tiles;
             if (s0 > G) s0 = G;
-            classic_cost = (G + s0 - 1) / s0;
+            classic = (G + s0 - 1) / s0 * unit_ns + (s0 > 1 ? 5500 : 0);
         } else {
-            classic_cost = ((g.tiles + sms - 1) / sms) * G;
+            classic = ((g.tiles + sms - 1) / sms) * G * unit_ns;
         }
-        if (classic_cost <= balanced_cost) split_k = s0;
+        if (classic <= balanced) split_k = s0;
+        g.cost = 3500 + (classic < balanced ? classic : balanced);
     }
     g.split_k = split_k;
     if (split_k == 0) {
@@ -286,26 +293,37 @@ TileGeom tile_geom(int M, int N, int G, int split_k, int sms, int max_smem) {
         g.nchunks = (int)(g.tiles * split_k);
     }
     g.ctas = g.nchunks < sms ? g.nchunks : sms;
-    const int avail = max_smem - kTileBarBytes - 1024;   // barrier block + alignment slack
-    int st = avail / tile_stage_bytes(g.mt);
+    int st = (kTileSmem - kTileBarBytes - 1024) / tile_stage_bytes(mt);   // (barrier block + alignment slack)
     if (st > kTileMaxStages) st = kTileMaxStages;
     if (st > kTileSlots) st = kTileSlots;               // the ring also lives in tensor memory
     // parity waits tell a barrier phase only from its neighbour: every dequant set has to come back to a slot on
     // every turn or every second one (kernel_tile.cuh)
-    st -= st % 2;                                                // 0 (no valid ring) is refused by the caller
+    st -= st % 2;
     g.stages = st;
-    g.smem_bytes = kTileBarBytes + 1024 + st * tile_stage_bytes(g.mt);
+    g.smem_bytes = kTileBarBytes + 1024 + st * tile_stage_bytes(mt);
     // each CTA takes the SM's whole tensor memory: ask for enough shared memory that two never share an SM
     if (g.smem_bytes < 120 * 1024) g.smem_bytes = 120 * 1024;
     return g;
+}
+
+// Batch rows per tile (the MMA's N): M in equal parts of at most 256 rows, rounded up to 16 -- the fewest parts, or one or
+// two more where that fills the last wave of tiles better.  M = 777, N = 22016: 4 x 208 rows 126 us, 4 x 256 131.
+TileGeom tile_geom(int M, int N, int G, int split_k, int sms) {
+    const int least = (M + 255) / 256;
+    TileGeom best = {};
+    for (int parts = least; parts < least + 3; ++parts) {
+        const TileGeom g = tile_geom_rows(((M + parts - 1) / parts + 15) / 16 * 16, M, N, G, 0, sms);
+        if (parts == least || g.cost < best.cost) best = g;
+    }
+    return split_k == 0 ? best : tile_geom_rows(best.mt, M, N, G, split_k, sms);
 }
 
 // ---- two-CTAs-per-SM tcgen05 kernel (kernel_mid.cuh): launch geometry --------------
 constexpr int kMidSmemBudget = (228 * 1024) / 2 - 1024;   // dynamic shared memory of one of two CTAs of an SM
 
 struct MidGeom {
-    int mt, m_tiles, n_tiles, split_k, nchunks, wstages, smem_bytes, ctas;
-    long tiles;
+    int mtc, mt, m_tiles, n_tiles, split_k, nchunks, wstages, smem_bytes, ctas;
+    long tiles, cost;
     bool cluster;
 };
 
@@ -319,55 +337,64 @@ __global__ void __launch_bounds__(kMidThreads, 2) mid_shape_probe_kernel(float* 
     extern __shared__ float probe_smem[];
     out[threadIdx.x] = probe_smem[threadIdx.x];
 }
-int mid_max_clusters(int size) {
+const int* mid_max_clusters() {     // [size]
+    static const int without_device[kMidMaxCluster + 1] = {0, 296, 148, 93, 71, 56, 45, 37, 33};   // (size queries on a host)
     DeviceState* d = nullptr;
-    if (current_device(&d) != W4A16_OK || !d->is_sm100) return 264 / size;    // (size queries without a device)
-    if (d->mid_clusters[size] != 0) return d->mid_clusters[size];
-    int n = 0;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)size;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(size * d->sm_count), 1, 1);
-    cfg.blockDim = dim3(kMidThreads, 1, 1);
-    cfg.dynamicSmemBytes = (size_t)kMidSmemBudget;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaFuncSetAttribute(mid_shape_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, d->max_smem_optin) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, mid_shape_probe_kernel, &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        n = 0;
+    if (current_device(&d) != W4A16_OK || !d->is_sm100) return without_device;
+    if (d->mid_clusters[1] != 0) return d->mid_clusters;
+    const bool ok = cudaFuncSetAttribute(mid_shape_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         d->max_smem_optin) == cudaSuccess;
+    for (int size = 2; size <= kMidMaxCluster; ++size) {
+        int n = 0;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)size;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(size * d->sm_count), 1, 1);
+        cfg.blockDim = dim3(kMidThreads, 1, 1);
+        cfg.dynamicSmemBytes = (size_t)kMidSmemBudget;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (!ok || cudaOccupancyMaxActiveClusters(&n, mid_shape_probe_kernel, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        d->mid_clusters[size] = n;
     }
-    if (n < 1) n = 1;
-    d->mid_clusters[size] = n;
-    return n;
+    d->mid_clusters[1] = 2 * d->sm_count;
+    return d->mid_clusters;
 }
 
-MidGeom mid_geom(int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg = 1) {
+// mtc: most batch rows of a tile, 64 or 128.  Cost model in ns, fitted to the figures below: a unit takes a CTA 400 + 0.7 mt
+// ns when it has the SM to itself and 480 + 2 mt when two share it (64-row build), 500 + 2 mt and 640 + 3.2 mt (128 rows);
+// a launch 4 us beside its units, and 0.7 us more where more than half of the slots are taken, so that the next launch's
+// CTAs do not find room before this one ends; the exchange inside a cluster of s 600 + 150 s (4300 + 300 s).
+// Measured (us), M = 32: K = N = 4096 four slices 7.09, eight 7.44; K = 11008 / N = 4096 8 / 6 / 4 slices 11.0 / 11.6 /
+// 13.8; K = 18432 / N = 7168 5 / 4 21.8 / 22.9; K = 4096 / N = 12288 2 / 1 12.2 / 17.3, three no longer fit at once: 17.5;
+// K = 4096 / N = 22016 1 / 2 18.7 / 22.6; K = 1024 / N = 3136 4 / 8 4.18 / 5.10.
+MidGeom mid_geom(int mtc, int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg = 1) {
     MidGeom g;
-    constexpr int kMtc = 64;
-    g.m_tiles = (M + kMtc - 1) / kMtc;
+    g.mtc = mtc;
+    g.m_tiles = (M + g.mtc - 1) / g.mtc;
     g.mt = ((M + g.m_tiles - 1) / g.m_tiles + 15) / 16 * 16;
     g.n_tiles = (N + kTileCols - 1) / kTileCols;
     g.tiles = (long)g.m_tiles * g.n_tiles;
     const int slots = 2 * sms;
-    auto fits = [&](int s) { return mid_smem_bytes(kMtc, g.mt, sg, 2, s) <= kMidSmemBudget; };
+    auto fits = [&](int s) { return mid_smem_bytes(g.mtc, g.mt, sg, 2, s) <= kMidSmemBudget; };
+    g.cost = 0;
     if (split_k == 0) {
-        // Cost in tenths of a unit's time (0.42 us with one CTA on an SM, a fifth more with two): the longest CTA's
-        // units, 5 per CTA of the cluster for the exchange, 15 where more than half of the slots are taken, so that
-        // the next launch's CTAs do not find room before this one ends.  Measured (us), M = 32: K = N = 4096 four
-        // slices 7.09, eight 7.44; K = 11008 / N = 4096 8 / 6 / 4 slices 11.0 / 11.6 / 13.8; K = 18432 / N = 7168
-        // 5 / 4 21.8 / 22.9; K = 4096 / N = 12288 2 / 1 12.2 / 17.3, three no longer fit at once: 17.5; K = 4096 /
-        // N = 22016 1 / 2 18.7 / 22.6; K = 1024 / N = 3136 4 / 8 4.18 / 5.10.
-        long best = 0;
+        const int* max_clusters = mid_max_clusters();
+        const bool wide = mtc > 64;
+        const long alone = wide ? 500 + 2 * g.mt : 400 + g.mt * 7 / 10, shared = wide ? 640 + g.mt * 16 / 5 : 480 + 2 * g.mt;
         for (int s = 1; s <= kMidMaxCluster && s <= G; ++s) {
-            if (s > 1 && (!allow_cluster || g.tiles > mid_max_clusters(s) || !fits(s))) continue;
+            if (s > 1 && (!allow_cluster || g.tiles > max_clusters[s] || !fits(s))) continue;
             const long ctas = g.tiles * s;
             const long units = ((ctas + slots - 1) / slots) * ((G + s - 1) / s);
-            const long cost = units * (ctas > sms ? 12 : 10) + 5 * s + (ctas > sms ? 15 : 0);
-            if (best == 0 || cost < best) { best = cost; split_k = s; }
+            const long cost = 4000 + units * (ctas > sms ? shared : alone) + (ctas > sms ? 700 : 0) +
+                              (s > 1 ? (wide ? 4300 + 300 * s : 600 + 150 * s) : 0);
+            if (g.cost == 0 || cost < g.cost) { g.cost = cost; split_k = s; }
         }
     }
     g.split_k = split_k;
@@ -375,23 +402,14 @@ MidGeom mid_geom(int M, int N, int G, int split_k, int sms, bool allow_cluster, 
     g.nchunks = (int)(g.tiles * split_k);
     g.ctas = g.cluster || g.nchunks < slots ? g.nchunks : slots;
     int st = kMidMaxWStages;
-    while (st > 2 && mid_smem_bytes(kMtc, g.mt, sg, st, g.cluster ? split_k : 0) > kMidSmemBudget) --st;
+    while (st > 2 && mid_smem_bytes(g.mtc, g.mt, sg, st, g.cluster ? split_k : 0) > kMidSmemBudget) --st;
     g.wstages = st;
-    g.smem_bytes = mid_smem_bytes(kMtc, g.mt, sg, st, g.cluster ? split_k : 0);
+    g.smem_bytes = mid_smem_bytes(g.mtc, g.mt, sg, st, g.cluster ? split_k : 0);
     // A CTA takes half of the SM's tensor memory: ask for enough shared memory that no third one, and no CTA of the
     // wide-tile kernel (which takes all of it), ever shares the SM, so that the allocation never has to wait.
     if (g.smem_bytes < 108 * 1024) g.smem_bytes = 108 * 1024;
     return g;
 }
-// Does the tcgen05 path take this shape through that kernel?  Up to 64 rows always; more rows where the weight matrix is
-// so narrow that tiles of 128 and 256 rows leave most SMs idle (24 tiles or fewer, fewer than twelve column tiles).
-bool mid_takes(int M, int N) {
-    if (M <= 64) return true;
-    const int mt = M <= 128 ? 128 : 256;
-    const long n_tiles = (N + kTileCols - 1) / kTileCols;
-    return n_tiles < 12 && ((M + mt - 1) / mt) * n_tiles <= 24;
-}
-
 size_t mid_workspace_bytes(const MidGeom& g) {
     if (g.split_k == 1) return 0;
     return round256((size_t)2 * g.nchunks * g.mt * kTileCols * sizeof(float));
@@ -403,12 +421,42 @@ size_t tile_workspace_bytes(const TileGeom& g) {
     return round256((size_t)2 * g.nchunks * g.mt * kTileCols * sizeof(float));
 }
 
-// Nominal split factor of the tile path's schedule: how many chunks share one tile's K range.
+// The tcgen05 path's kernel for a shape: up to 64 rows the 64-row build of kernel_mid.cuh; above, the cheapest by the cost
+// models of it (several batch tiles), its 128-row build and kernel_tile.cuh.  Measured (us, in that order), the first column
+// decides: M = 128: K = N = 4096 10.4 / 14.8 / 13.0, K = 11008 / N = 4096 17.6 / 21.0 / 20.8, K = N = 8192 23.5 / 24.4 /
+// 26.6, K = 4096 / N = 22016 38.5 / 33.3 / 35.8; M = 256: K = N = 2048 8.0 / 12.2 / 11.7, K = 16384 / N = 4096 40.6 / 38.3 /
+// 32.9; M = 300, K = 4096 / N = 12288 - / 33.5 / 45.0; M = 512 - / 62.7 / 48.5; M = 1024, K = N = 8192 - / 128 / 102.
+struct WidePlan {
+    bool use_mid;
+    MidGeom mid;
+    TileGeom tile;
+    size_t workspace_bytes() const { return use_mid ? mid_workspace_bytes(mid) : tile_workspace_bytes(tile); }
+};
+WidePlan wide_plan(int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg = 1) {
+    WidePlan w;
+    w.use_mid = true;
+    if (M <= 64) {
+        w.mid = mid_geom(64, M, N, G, split_k, sms, allow_cluster, sg);
+        return w;
+    }
+    w.mid = mid_geom(64, M, N, G, 0, sms, allow_cluster, sg);
+    const MidGeom m128 = mid_geom(128, M, N, G, 0, sms, allow_cluster, sg);
+    if (m128.cost < w.mid.cost) w.mid = m128;
+    w.tile = tile_geom(M, N, G, 0, sms);
+    w.use_mid = w.mid.cost < w.tile.cost;
+    if (split_k != 0) {
+        if (w.use_mid) w.mid = mid_geom(w.mid.mtc, M, N, G, split_k, sms, allow_cluster, sg);
+        else w.tile = tile_geom(M, N, G, split_k, sms);
+    }
+    return w;
+}
+
+// Nominal split factor of the tcgen05 path's schedule: how many chunks share one tile's K range.
 int choose_split_tile(int M, int N, int G, int sms) {
-    if (mid_takes(M, N)) return mid_geom(M, N, G, 0, sms, true).split_k;
-    TileGeom g = tile_geom(M, N, G, 0, sms, 227 * 1024);
-    if (g.split_k >= 1) return g.split_k;
-    long s = (g.nchunks + g.tiles - 1) / g.tiles;
+    const WidePlan w = wide_plan(M, N, G, 0, sms, true);
+    if (w.use_mid) return w.mid.split_k;
+    if (w.tile.split_k >= 1) return w.tile.split_k;
+    long s = (w.tile.nchunks + w.tile.tiles - 1) / w.tile.tiles;
     if (s < 1) s = 1;
     if (s > G) s = G;
     return (int)s;
@@ -564,9 +612,10 @@ size_t w4a16_workspace_bytes(int M, int N, int K, int group, int split_k) {
         int s = split_k == 0 ? choose_split_decode(M, N, K / kGroup, sm_count_or_default()) : split_k;
         size_t simple = simple_partial_bytes(M, N, s);
         if (simple > need) need = simple;
-        const size_t tile = mid_takes(M, N) ? mid_workspace_bytes(mid_geom(M, N, K / kGroup, split_k, sm_count_or_default(), true))
-                                         : tile_workspace_bytes(tile_geom(M, N, K / kGroup, split_k, sm_count_or_default(), 227 * 1024));
-        if (tile > need) need = tile;
+        for (bool clusters : {true, false}) {
+            const size_t tile = wide_plan(M, N, K / kGroup, split_k, sm_count_or_default(), clusters).workspace_bytes();
+            if (tile > need) need = tile;
+        }
     }
     return need == 0 ? 0 : kWsFullHeaderBytes + need;
 }
@@ -683,11 +732,11 @@ namespace {
 DecodeKernel decode_kernel(int mb, bool cluster, int sg, bool bf, bool sym, bool a_box) {
     return bf ? decode_kernel_bf16(mb, cluster, sg, sym, a_box) : decode_kernel_f16(mb, cluster, sg, sym, a_box);
 }
-TileKernel tile_kernel(int mt_index, int sg, bool bf, bool sym, bool epi) {
-    if (bf) return sg == 1 ? tile_kernel_bf16_sg1(mt_index, sym, epi) : sg == 2 ? tile_kernel_bf16_sg2(mt_index, sym, epi)
-                                                                                : tile_kernel_bf16_sg4(mt_index, sym, epi);
-    return sg == 1 ? tile_kernel_f16_sg1(mt_index, sym, epi) : sg == 2 ? tile_kernel_f16_sg2(mt_index, sym, epi)
-                                                                       : tile_kernel_f16_sg4(mt_index, sym, epi);
+TileKernel tile_kernel(int sg, bool bf, bool sym, bool epi) {
+    if (bf) return sg == 1 ? tile_kernel_bf16_sg1(sym, epi) : sg == 2 ? tile_kernel_bf16_sg2(sym, epi)
+                                                                                : tile_kernel_bf16_sg4(sym, epi);
+    return sg == 1 ? tile_kernel_f16_sg1(sym, epi) : sg == 2 ? tile_kernel_f16_sg2(sym, epi)
+                                                                       : tile_kernel_f16_sg4(sym, epi);
 }
 
 // Split-K sum behind a tcgen05 kernel that only stored its partial tiles (slices of whole tiles).
@@ -770,13 +819,15 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         return W4A16_OK;
     }
 
-    if (path == W4A16_PATH_TILE && mid_takes(M, N)) {
-        const MidGeom g = mid_geom(M, N, G, split_k, d->sm_count, d->cluster_ok, sg);
+    WidePlan plan = {};
+    if (path == W4A16_PATH_TILE) plan = wide_plan(M, N, G, split_k, d->sm_count, d->cluster_ok, sg);
+    if (path == W4A16_PATH_TILE && plan.use_mid) {
+        const MidGeom& g = plan.mid;
         if (g.smem_bytes > d->max_smem_optin) return W4A16_ERR_PATH;
         if (g.split_k != 1 && ws_body_bytes < mid_workspace_bytes(g)) return W4A16_ERR_WORKSPACE;
         if ((long long)g.tiles * (g.split_k > g.mt ? g.split_k : g.mt) >= (1ll << 31)) return W4A16_ERR_SHAPE;   // (32-bit chunk arithmetic)
         CUtensorMap tmap;
-        if (!make_act_tensor_map(&tmap, A, M, K, g.mt, mid_stage_k(64))) return W4A16_ERR_CUDA;
+        if (!make_act_tensor_map(&tmap, A, M, K, g.mt, mid_stage_k(g.mtc))) return W4A16_ERR_CUDA;
         MidParams p;
         p.Wq = static_cast<const uint32_t*>(Wq);
         p.S = static_cast<const uint16_t*>(S);
@@ -795,8 +846,8 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         p.slice_base = G / g.split_k;
         p.slice_rem = G % g.split_k;
         p.epi = epi;
-        MidKernel kern = bf ? mid_kernel_bf16(sg, sym) : mid_kernel_f16(sg, sym);
-        bool& attr_set = d->mid_attr_set[log2_sg(sg)][bf ? 1 : 0][sym ? 1 : 0];
+        MidKernel kern = bf ? mid_kernel_bf16(g.mtc, sg, sym) : mid_kernel_f16(g.mtc, sg, sym);
+        bool& attr_set = d->mid_attr_set[g.mtc <= 64 ? 0 : 1][log2_sg(sg)][bf ? 1 : 0][sym ? 1 : 0];
         if (!attr_set) {
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, d->max_smem_optin) != cudaSuccess) {
                 cudaGetLastError();
@@ -839,8 +890,8 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
     }
 
     if (path == W4A16_PATH_TILE) {
-        TileGeom g = tile_geom(M, N, G, split_k, d->sm_count, d->max_smem_optin);
-        if (g.stages < 2) return W4A16_ERR_PATH;
+        const TileGeom& g = plan.tile;
+        if (g.smem_bytes > d->max_smem_optin) return W4A16_ERR_PATH;
         if (g.split_k != 1) {
             if (g.tiles > kTileMaxTicketTiles) return W4A16_ERR_SPLITK;
             if (ws_body_bytes < tile_workspace_bytes(g)) return W4A16_ERR_WORKSPACE;
@@ -857,6 +908,7 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         p.tickets = reinterpret_cast<int*>(d->ws ? static_cast<unsigned char*>(d->ws) + kWsHeaderBytes : nullptr);
         p.ws = reinterpret_cast<float*>(ws_body);
         p.M = M; p.N = N; p.K = K; p.G = G;
+        p.mt = g.mt;
         p.n_tiles = g.n_tiles;
         p.m_tiles = g.m_tiles;
         p.split_k = g.split_k;
@@ -870,10 +922,9 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         // Measured (us, in the kernel / second kernel): M = 256: K = 10240 / N = 4608 (four slices) 31.9 / 24.6,
         // K = 16384 / N = 4096 39.2 / 32.9, K = N = 8192 (two slices) 34.1 / 33.3.
         const bool defer = g.split_k >= 2;
-        p.defer_reduce = defer ? 1 : 0;
         const bool has_epi = !defer && (bias != nullptr || act != W4A16_ACT_NONE);
-        TileKernel kern = tile_kernel(g.mt_index, sg, bf, sym, has_epi);
-        bool& attr_set = d->tile_attr_set[g.mt_index][log2_sg(sg)][bf ? 1 : 0][sym ? 1 : 0][has_epi ? 1 : 0];
+        TileKernel kern = tile_kernel(sg, bf, sym, has_epi);
+        bool& attr_set = d->tile_attr_set[log2_sg(sg)][bf ? 1 : 0][sym ? 1 : 0][has_epi ? 1 : 0];
         if (!attr_set) {
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, d->max_smem_optin) !=
                 cudaSuccess) {

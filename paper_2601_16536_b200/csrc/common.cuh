@@ -357,4 +357,13 @@ __device__ __forceinline__ uint16_t finish(float v, int n, const Epilogue& e) {
     return cast_out<BF>(v);
 }
 
+// The same with the column's bias at hand.
+template <bool BF>
+__device__ __forceinline__ uint16_t finish_col(float v, bool has_bias, float bias, int act) {
+    if (has_bias) v += bias;
+    if (act == kActRelu) v = fmaxf(v, 0.f);
+    else if (act == kActSilu) v = v / (1.f + __expf(-v));
+    return cast_out<BF>(v);
+}
+
 }  // namespace w4a16

@@ -4,18 +4,19 @@
 
 namespace w4a16 {
 namespace {
-template <int SG>
-MidKernel pick(bool sym) {
+template <int MTC>
+MidKernel pick(int sg, bool sym) {
     constexpr bool BF = W4A16_INST_BF;
-    return sym ? gemm_mid_kernel<64, SG, BF, true> : gemm_mid_kernel<64, SG, BF, false>;
+    if (sym) return sg == 1 ? gemm_mid_kernel<MTC, 1, BF, true> : sg == 2 ? gemm_mid_kernel<MTC, 2, BF, true> : gemm_mid_kernel<MTC, 4, BF, true>;
+    return sg == 1 ? gemm_mid_kernel<MTC, 1, BF, false> : sg == 2 ? gemm_mid_kernel<MTC, 2, BF, false> : gemm_mid_kernel<MTC, 4, BF, false>;
 }
 }  // namespace
 
 #define W4A16_CAT2(a, b) a##b
 #define W4A16_CAT(a, b) W4A16_CAT2(a, b)
 
-MidKernel W4A16_CAT(mid_kernel_, W4A16_INST_NAME)(int sg, bool sym) {
-    return sg == 1 ? pick<1>(sym) : sg == 2 ? pick<2>(sym) : pick<4>(sym);
+MidKernel W4A16_CAT(mid_kernel_, W4A16_INST_NAME)(int mtc, int sg, bool sym) {
+    return mtc <= 64 ? pick<64>(sg, sym) : pick<128>(sg, sym);
 }
 int W4A16_CAT(status_take_mid_, W4A16_INST_NAME)() { return status_take_this_unit(); }
 

@@ -52,9 +52,10 @@ __host__ __device__ constexpr int mid_wstage_bytes(int sg) {
 }
 // Partial sums a CTA of a cluster of S receives: S - 1 slots of its share of the rows, in groups of four rows.
 __host__ __device__ inline int mid_xch_slot_bytes(int mt, int S) { return (mt / 4 + S - 1) / S * (kTileCols * 16); }
-inline int mid_xch_bytes(int mt, int S) { return S > 1 ? (S - 1) * mid_xch_slot_bytes(mt, S) : 0; }
+// Up to 64 rows they have a buffer of their own; above, they lie on top of the (by then idle) rings.
+inline int mid_xch_bytes(int mtc, int mt, int S) { return mtc <= 64 && S > 1 ? (S - 1) * mid_xch_slot_bytes(mt, S) : 0; }
 inline int mid_smem_bytes(int mtc, int mt, int sg, int wstages, int cluster) {
-    return 1024 + mid_slots(mtc) * mt * mid_stage_k(mtc) * 2 + wstages * mid_wstage_bytes(sg) + mid_xch_bytes(mt, cluster) +
+    return 1024 + mid_slots(mtc) * mt * mid_stage_k(mtc) * 2 + wstages * mid_wstage_bytes(sg) + mid_xch_bytes(mtc, mt, cluster) +
            kMidBarBytes;
 }
 
@@ -89,14 +90,6 @@ struct MidChunk {
     }
 };
 
-template <bool BF>
-__device__ __forceinline__ uint16_t finish_col(float v, bool has_bias, float bias, int act) {
-    if (has_bias) v += bias;
-    if (act == kActRelu) v = fmaxf(v, 0.f);
-    else if (act == kActSilu) v = v / (1.f + __expf(-v));
-    return cast_out<BF>(v);
-}
-
 template <int OFF>
 __device__ __forceinline__ uint4 mid_lds128(uint32_t addr) {
     uint4 v;
@@ -117,6 +110,7 @@ gemm_mid_kernel(const __grid_constant__ CUtensorMap tmap_a, const MidParams p) {
     constexpr int kSPU = kGroup / kStageK;            // operand slots per unit
     constexpr int R = mid_slots(MTC);
     constexpr int kSlotCols = kStageK / 2;
+    constexpr bool kOverlay = MTC > 64;               // exchange buffer on top of the rings
     constexpr int kWStage = mid_wstage_bytes(SG);
     constexpr int kWS = 2 * kMidWUnits * kBlockBytes;                       // scale rows of a weight stage
     constexpr int kWZ = kWS + 2 * kMidWUnits * SG * kSBlockHalves * 2;      // zero-point rows
@@ -128,10 +122,10 @@ gemm_mid_kernel(const __grid_constant__ CUtensorMap tmap_a, const MidParams p) {
     const uint32_t act0 = smem_u32(smem);
     const uint32_t w0 = act0 + (uint32_t)(R * abytes);
     const uint32_t w_end = (uint32_t)(p.wstages * kWStage);                 // ring size in bytes
-    const uint32_t xch = w0 + w_end;
+    const uint32_t xch = kOverlay ? act0 : w0 + w_end;
     const int xslot = mid_xch_slot_bytes(mt, p.split_k);
     // slot i: full (activation box landed, operand stored) at bars + 16 i, retired (the MMAs that read it) 8 further
-    const uint32_t bars = xch + (uint32_t)(p.cluster ? (p.split_k - 1) * xslot : 0);
+    const uint32_t bars = w0 + w_end + (uint32_t)(!kOverlay && p.cluster ? (p.split_k - 1) * xslot : 0);
     const uint32_t d_full = bars + 16u * R, d_empty = d_full + 8u, xbar = d_full + 16u;   // xbar: the other slices' sums have landed
     unsigned char* misc = smem + (bars - act0) + 16 * R + 24;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc);
@@ -166,8 +160,13 @@ gemm_mid_kernel(const __grid_constant__ CUtensorMap tmap_a, const MidParams p) {
     const uint32_t tmem_base = *tmem_slot;
     // Every CTA of a cluster must be running, its barriers initialised, before anyone writes to its shared memory: all
     // threads arrive here and each waits once, later, where the guarantee is needed.
-    bool cl_waited = p.cluster == 0;
-    if (p.cluster) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    // (With the exchange on top of the rings the guarantee needed is that every CTA has done with its rings: they arrive
+    // when they have.)
+    bool cl_arrived = p.cluster == 0, cl_waited = p.cluster == 0;
+    if (!kOverlay && p.cluster) {
+        asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+        cl_arrived = true;
+    }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (warp == kMidDequantWarps) {
@@ -401,6 +400,10 @@ gemm_mid_kernel(const __grid_constant__ CUtensorMap tmap_a, const MidParams p) {
             }
             // Cluster: rows 4 q .. 4 q + 3 are finished by CTA owner(q); quads = mt / 4 in S equal runs (the last may
             // be shorter).  Slot of slice s at CTA d: s - (s > d).
+            if (kOverlay) {
+                asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+                cl_arrived = true;
+            }
             asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
             cl_waited = true;
             const int S = p.split_k, rank = c.slice;
@@ -463,6 +466,7 @@ gemm_mid_kernel(const __grid_constant__ CUtensorMap tmap_a, const MidParams p) {
         if (!ok && lane == 0) flags[0] = 1;
     }
     __syncwarp();
+    if (!cl_arrived) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     if (!cl_waited) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
     // ---------------------------------------------------------------- teardown

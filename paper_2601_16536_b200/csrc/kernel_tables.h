@@ -16,14 +16,15 @@ typedef void (*MidKernel)(const CUtensorMap, const MidParams);
 // a_box: activation rows of a stage as one tensor copy
 DecodeKernel decode_kernel_f16(int mb, bool cluster, int sg, bool sym, bool a_box);
 DecodeKernel decode_kernel_bf16(int mb, bool cluster, int sg, bool sym, bool a_box);
-MidKernel mid_kernel_f16(int sg, bool sym);
-MidKernel mid_kernel_bf16(int sg, bool sym);
-TileKernel tile_kernel_f16_sg1(int mt_index, bool sym, bool epi);
-TileKernel tile_kernel_f16_sg2(int mt_index, bool sym, bool epi);
-TileKernel tile_kernel_f16_sg4(int mt_index, bool sym, bool epi);
-TileKernel tile_kernel_bf16_sg1(int mt_index, bool sym, bool epi);
-TileKernel tile_kernel_bf16_sg2(int mt_index, bool sym, bool epi);
-TileKernel tile_kernel_bf16_sg4(int mt_index, bool sym, bool epi);
+// mtc: most batch rows of a tile (64, 128)
+MidKernel mid_kernel_f16(int mtc, int sg, bool sym);
+MidKernel mid_kernel_bf16(int mtc, int sg, bool sym);
+TileKernel tile_kernel_f16_sg1(bool sym, bool epi);
+TileKernel tile_kernel_f16_sg2(bool sym, bool epi);
+TileKernel tile_kernel_f16_sg4(bool sym, bool epi);
+TileKernel tile_kernel_bf16_sg1(bool sym, bool epi);
+TileKernel tile_kernel_bf16_sg2(bool sym, bool epi);
+TileKernel tile_kernel_bf16_sg4(bool sym, bool epi);
 
 int status_take_decode_f16();
 int status_take_decode_bf16();

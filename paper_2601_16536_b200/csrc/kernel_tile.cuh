@@ -24,16 +24,16 @@
 // The part of a chunk inside one tile is a segment: the accumulator is zeroed at its first MMA and
 // drained after its last.  A segment that covers a whole tile is cast to FP16 and stored; any other
 // segment leaves as an FP32 partial tile in the workspace, and the warp that draws the last ticket
-// of its 32-column x MT/4-row region adds the partial regions in ascending K order (Phase 3).
+// of its 32-column region (its 16-row steps) adds the partial regions in ascending K order (Phase 3).
 // No warp ever waits for another CTA, and the order of the sum is fixed, so results are
 // bit-identical from run to run.
 //
-// Batch tiles of 128 and 256 rows (17 to 64 rows: kernel_mid.cuh).  One pipeline stage is half a group (64 k, four MMAs).
+// Batch tiles of up to 256 rows, a run-time multiple of 16 (MT; which shapes come here and which go to kernel_mid.cuh is
+// the host's choice by cost).  One pipeline stage is half a group (64 k, four MMAs).
 // A ring of R slots holds, per slot, the stage's activation box in shared memory and its dequantized weights in tensor
-// memory (32 columns; eight slots fit beside the accumulators).  Four sets of four dequant warps take stages round-robin;
-// inside a set warp w owns TMEM lanes 32 (w % 4) .. + 31.  Each thread keeps the packed words of its next three stages in
-// registers (loads issued that far ahead, pointers stepped, no register copies).  With MT = 128 two accumulators alternate
-// between segments, so one drains while the next fills.  The packed weights do not depend on the
+// memory (32 columns; eight slots fit beside the accumulator).  Four sets of four dequant warps take stages round-robin;
+// inside a set warp w owns TMEM lanes 32 (w % 4) .. + 31.  Each thread keeps the packed words of its next two stages in
+// registers (loads issued that far ahead, pointers stepped, no register copies).  The packed weights do not depend on the
 // previous kernel in the stream: under programmatic dependent launch the dequant warps load and
 // convert weights until the TMEM ring is full before anything waits for that kernel; only
 // activations, C and the workspace are touched after griddepcontrol.wait.
@@ -57,13 +57,11 @@ constexpr int kTileStageK = 64;                     // k per pipeline stage
 constexpr int kTileDequantWarps = 16;               // four sets of four (one warp per TMEM lane quarter)
 constexpr int kTileSets = kTileDequantWarps / 4;
 constexpr int kTileThreads = (2 + kTileDequantWarps) * 32;   // producer, issuer, dequant / epilogue warps
-// accumulators that alternate between segments
-__host__ __device__ constexpr int tile_dbufs(int mt) { return mt <= 128 ? 2 : 1; }
 constexpr int kTileMaxStages = 8;                   // ring slots: activation box + stage_k / 2 TMEM columns each
-// TMEM columns: the accumulators first (two of 128 columns, or one of 256), then the operand ring
+// TMEM columns: the accumulator first, then the operand ring
 constexpr int kTileACol = 256;
 constexpr int kTileSlots = (512 - kTileACol) / (kTileStageK / 2);
-constexpr int kTilePrefetch = 3;                    // stages of packed words a dequant thread holds in registers
+constexpr int kTilePrefetch = 2;                    // stages of packed words a dequant thread holds in registers
 constexpr int kTileBarBytes = 1024;
 
 __host__ __device__ constexpr int tile_stage_bytes(int mt) { return mt * kTileStageK * 2; }
@@ -76,12 +74,12 @@ struct TileParams {
     float* ws;       // partial tiles: [2 * nchunks slots][MT][128] FP32
     int* tickets;    // zeroed counters: [tile][16 epilogue warps]
     int M, N, K, G;
+    int mt;          // batch rows of a tile: multiple of 16, at most 256
     int n_tiles;     // NT = ceil(N / 128)
     int m_tiles;     // ceil(M / MT)
     int split_k;     // 0: balanced chunks; S >= 1: classic Split-K
     int nchunks;
     int stages;
-    int defer_reduce;   // 1: partial tiles are only stored; tile_splitk_reduce_kernel sums them (classic slices)
     // chunk arithmetic, prepared by the host (tile_fill_chunk_math); units = m_tiles n_tiles G < 2^31
     FastDiv div_G, div_split, div_nchunks, div_ntiles;
     int slice_base, slice_rem;   // classic: G / split_k, G % split_k
@@ -174,24 +172,18 @@ __device__ __forceinline__ int tile_chunk_begin(const TileParams& p, int i) {
     const int t = fast_div(i, p.div_split), s = i - t * p.split_k;
     return t * p.G + s * p.slice_base + min(s, p.slice_rem);
 }
-// The chunk that holds unit u.  (Out of line and with scalar arguments -- a reference to the kernel's parameter
-// block would be copied to local memory for every call; only the Split-K epilogue of balanced chunks comes here.)
-static __device__ __noinline__ int tile_chunk_of_s(int split_k, int G, int nchunks, long long units, long long u) {
-    if (split_k == 0) return (int)(((u + 1) * nchunks - 1) / units);
-    const int t = (int)(u / G), g = (int)(u - (long long)t * G);
-    const int base = G / split_k, rem = G % split_k;
-    const int s = (g < rem * (base + 1)) ? g / (base + 1) : rem + (g - rem * (base + 1)) / max(base, 1);
-    return t * split_k + s;
+// The balanced chunk that holds unit u.  (Out of line: only the epilogue of partial tiles comes here.)
+static __device__ __noinline__ int tile_chunk_of_s(int nchunks, long long units, long long u) {
+    return (int)(((u + 1) * nchunks - 1) / units);
 }
 __device__ __forceinline__ int tile_chunk_of(const TileParams& p, long long u) {
-    return tile_chunk_of_s(p.split_k, p.G, p.nchunks, (long long)p.m_tiles * p.n_tiles * p.G, u);
+    return tile_chunk_of_s(p.nchunks, (long long)p.m_tiles * p.n_tiles * p.G, u);
 }
 
 // Where chunk ci (or the next non-empty one of this CTA, stepping by `stride`) starts.
 struct ChunkStart {
     int ci;        // the chunk found (>= nchunks: none left)
     int t;         // tile = batch tile * NT + column tile
-    int nt, mt_i;  // t % NT, t / NT
     int g0;        // first group inside the tile
     int len;       // units of the chunk
 };
@@ -208,8 +200,6 @@ __device__ __forceinline__ ChunkStart tile_chunk_start(const TileParams& p, int 
     c.len = len;
     c.t = fast_div(u0, p.div_G);
     c.g0 = u0 - c.t * p.G;
-    c.mt_i = fast_div(c.t, p.div_ntiles);
-    c.nt = c.t - c.mt_i * p.n_tiles;
     return c;
 }
 
@@ -222,7 +212,6 @@ struct SegWalk {
     const TileParams& p;
     int ci;            // current chunk
     int t;             // tile = batch tile * NT + column tile
-    int nt, mt_i;      // t % NT, t / NT
     int g0;            // first group of the segment inside the tile
     int units;         // groups in the segment
     int left;          // units of the chunk after this segment
@@ -230,7 +219,7 @@ struct SegWalk {
     uint32_t n0;       // stages of this CTA before the segment (ring positions derive from it)
     const int spu;     // stages per unit (group): 1 or 2
     __device__ __forceinline__ SegWalk(const TileParams& p_, int spu_)
-        : p(p_), ci((int)blockIdx.x), t(0), nt(0), mt_i(0), g0(0), units(0), left(0), first(true), n0(0), spu(spu_) {
+        : p(p_), ci((int)blockIdx.x), t(0), g0(0), units(0), left(0), first(true), n0(0), spu(spu_) {
         load_chunk();
     }
     __device__ __forceinline__ void load_chunk() {
@@ -239,8 +228,6 @@ struct SegWalk {
         if (ci >= p.nchunks) return;
         t = c.t;
         g0 = c.g0;
-        mt_i = c.mt_i;
-        nt = c.nt;
         units = min(c.len, p.G - g0);
         left = c.len - units;
         first = true;
@@ -254,12 +241,14 @@ struct SegWalk {
             return;
         }
         ++t;
-        if (++nt == p.n_tiles) { nt = 0; ++mt_i; }
         g0 = 0;
         units = min(left, p.G);
         left -= units;
         first = false;
     }
+    // (batch tile and column tile: asked once per segment, and two registers fewer than kept)
+    __device__ __forceinline__ int mt_i() const { return fast_div(t, p.div_ntiles); }
+    __device__ __forceinline__ int nt() const { return t - mt_i() * p.n_tiles; }
     __device__ __forceinline__ int stages_in_seg() const { return spu * units; }
     __device__ __forceinline__ bool whole_tile() const { return g0 == 0 && units == p.G; }
 };
@@ -300,21 +289,19 @@ struct StageRegs {
     uint32_t zw[NR];    // zero-point words that hold the column's nibble
 };
 
-// MT = batch rows per tile; SG = scale / zero-point rows per 128-k block (quantization group 128 / SG);
+// SG = scale / zero-point rows per 128-k block (quantization group 128 / SG);
 // BF = BF16 instead of FP16 activations, scales, weights and output; SYM = symmetric format (zero point 8,
 // no Z buffer); EPI = bias / activation fused into the final cast.  (Both compiled in: decided at run time
-// they cost 5 to 10 % on narrow tiles and 9 % at M = 256.)
-template <int MT, int SG, bool BF, bool SYM, bool EPI>
+// they cost 9 % at M = 256.)
+template <int SG, bool BF, bool SYM, bool EPI>
 __global__ void __launch_bounds__(kTileThreads, 1)
 gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte alignment of the stage buffers (the swizzle atom) regardless of where the
     // dynamic segment starts
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    constexpr int kStageBytes = tile_stage_bytes(MT);
-    constexpr uint32_t kIdesc = tile_idesc(MT, BF);
-    constexpr int kCW = MT / kTileSets;                  // accumulator columns (batch rows) per epilogue warp
-    constexpr int kDBufs = tile_dbufs(MT);               // accumulator b sits at column 128 b
+    const int mt = p.mt;
+    const int stage_bytes = tile_stage_bytes(mt);
     constexpr int kStageK = kTileStageK;                 // k per ring slot
     constexpr int kSPU = kGroup / kStageK;               // stages per unit
     constexpr int kSlotCols = kStageK / 2;               // TMEM columns of one operand slot
@@ -326,9 +313,9 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
 
     uint64_t* full = reinterpret_cast<uint64_t*>(smem);          // [R]  activation box landed AND operand stored in TMEM
     uint64_t* retired = full + kTileMaxStages;                   // [2][R]  the stage's MMAs retired: slot free
-    uint64_t* d_full = retired + 2 * kTileMaxStages;             // [2]  accumulator complete
-    uint64_t* d_empty = d_full + 2;                              // [2]  accumulator drained by the epilogue
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(d_empty + 2);
+    uint64_t* d_full = retired + 2 * kTileMaxStages;             // accumulator complete
+    uint64_t* d_empty = d_full + 1;                              // accumulator drained by the epilogue
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(d_empty + 1);
     int* flags = reinterpret_cast<int*>(tmem_slot + 1);          // [0] a bounded wait ran out, [1] stages issued
     unsigned char* stage0 = smem + kTileBarBytes;
 
@@ -341,10 +328,8 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
             mbar_init(&retired[i], 1);
             mbar_init(&retired[kTileMaxStages + i], 1);
         }
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&d_full[i], 1);
-            mbar_init(&d_empty[i], kTileDequantWarps);
-        }
+        mbar_init(d_full, 1);
+        mbar_init(d_empty, kTileDequantWarps);
         flags[0] = 0;
         flags[1] = 0;
         fence_mbar_init();
@@ -372,13 +357,13 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
         uint32_t n = 0;
         for (SegWalk w(p, kSPU); w.valid() && ok; w.next()) {
             int kb = w.g0 * (kGroup / kTileBoxK);            // 64-k box index along K
-            const int m = w.mt_i * MT;
+            const int m = w.mt_i() * mt;
             const int nst = w.stages_in_seg();
             for (int j = 0; j < nst; ++j) {
                 if (r.turn != 0u && !wait_slot_free(retired, r)) { ok = false; break; }
                 if (elect_one()) {
-                    mbar_expect_tx(&full[r.slot], (uint32_t)kStageBytes);
-                    tma_load_2d(stage0 + (size_t)r.slot * kStageBytes, &tmap_a, kb * kTileBoxK, m, &full[r.slot]);
+                    mbar_expect_tx(&full[r.slot], (uint32_t)stage_bytes);
+                    tma_load_2d(stage0 + r.slot * stage_bytes, &tmap_a, kb * kTileBoxK, m, &full[r.slot]);
                 }
                 __syncwarp();
                 kb += kStageK / kTileBoxK;
@@ -393,27 +378,26 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
         asm volatile("griddepcontrol.wait;" ::: "memory");
+        const uint32_t idesc = tile_idesc(mt, BF);
         uint32_t n_seg = 0;
         bool ok = true;
         RingPos r{0, 0u, 0u};
         for (SegWalk w(p, kSPU); w.valid() && ok; w.next(), ++n_seg) {
-            const int dbuf = n_seg % kDBufs;
-            // the epilogue of the segment that used this accumulator before must have drained it
-            if (!mbar_wait(&d_empty[dbuf], ((n_seg / kDBufs) & 1u) ^ 1u)) { ok = false; break; }
-            const uint32_t d_t = tmem_base + dbuf * 128;
+            // the epilogue of the segment before must have drained the accumulator
+            if (!mbar_wait(d_empty, (n_seg & 1u) ^ 1u)) { ok = false; break; }
             const int nst = w.stages_in_seg();
             uint32_t acc = 0u;                                   // the segment's first MMA overwrites
             for (int j = 0; j < nst; ++j) {
                 if (!mbar_wait(&full[r.slot], r.ph)) { ok = false; break; }
                 tc_fence_after();
                 if (elect_one()) {
-                    const uint64_t bdesc = smem_desc_sw128(smem_u32(stage0 + (size_t)r.slot * kStageBytes));
+                    const uint64_t bdesc = smem_desc_sw128(smem_u32(stage0 + r.slot * stage_bytes));
                     const uint32_t a_t = tmem_base + kACol + r.slot * kSlotCols;
 #pragma unroll
                     for (int kk = 0; kk < kStageK / 16; ++kk)    // 16 k: 8 TMEM columns of A, 32 bytes along B's swizzled rows
-                        tc_mma_ts(d_t, a_t + kk * 8, bdesc + (uint64_t)(kk * 2), kIdesc, kk == 0 ? acc : 1u);
+                        tc_mma_ts(tmem_base, a_t + kk * 8, bdesc + (uint64_t)(kk * 2), idesc, kk == 0 ? acc : 1u);
                     tc_commit(retired_bar(retired, r));
-                    if (j + 1 == nst) tc_commit(&d_full[dbuf]);
+                    if (j + 1 == nst) tc_commit(d_full);
                 }
                 __syncwarp();
                 acc = 1u;
@@ -429,23 +413,22 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
         const int row = quarter * 32 + lane;   // column n inside the CTA tile = TMEM lane
         const int half = row >> 6, col = row & 63;
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
-        // word offsets of this thread's two 16-byte chunks inside a block's 64-k half
-        const int wo0 = (col >> 3) * 64 + (col & 7) * 4;
-        const int wo1 = (col >> 3) * 64 + 32 + (((col & 7) + 4) & 7) * 4;
+        // 16-byte index of this thread's two chunks inside a block's 64-k half
+        const int wo0 = (col >> 3) * 16 + (col & 7);
+        const int wo1 = (col >> 3) * 16 + 8 + (((col & 7) + 4) & 7);
         const int zp = sz_perm(col);         // position of this column's scale / zero point inside a row
         const int zsh = 4 * (zp & 7);
 
         // this set's first stage inside a segment
         auto first_own = [&](const SegWalk& w) { return (int)(((uint32_t)set - w.n0) & 3u); };
         // Load cursor: runs kPF of this set's stages ahead of the compute loop.  Inside a segment this
-        // set's stages are kTileSets apart (kTileSets / kSPU groups on, same part of the group), so the
-        // three pointers just step; they are recomputed only when the cursor enters a new segment.
+        // set's stages are kTileSets apart, so its position steps; it is recomputed only when the cursor enters a new
+        // segment.  (One 32-bit position instead of three pointers: the loop runs at the register limit.)
+        static_assert(kSPU == 2, "a stage is one 64-k half of a packed block");
         SegWalk wl(p, kSPU);
         int jl = 0;
         bool l_in = false;                      // this thread's column exists (not past the matrix edge)
-        const uint32_t* lw = nullptr;           // the stage's first word of this thread's 8-column block
-        const uint16_t* ls = nullptr;
-        const uint32_t* lz = nullptr;
+        uint32_t hb = 0u;                       // 64-k half block: 2 * packed block + half
         auto point = [&]() {                    // cursor entered a new segment: settle on a stage, set pointers
             while (wl.valid()) {
                 jl = first_own(wl);
@@ -453,28 +436,23 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
                 wl.next();
             }
             if (!wl.valid()) return;
-            const int t64 = 2 * wl.nt + half;   // 64-column packed tile
+            const int t64 = 2 * wl.nt() + half;   // 64-column packed tile
             l_in = t64 * kTileN < p.N;
-            const size_t blk = (size_t)t64 * p.G + (wl.g0 + jl / kSPU);
-            lw = p.Wq + blk * kBlockWords + (jl % kSPU) * 512;
-            // first scale row of the stage: a 64-k stage of a block with SG >= 2 rows starts at row (SG / 2) * half
-            const size_t row = blk * SG + (SG >= kSPU ? (jl % kSPU) * (SG / kSPU) : 0);
-            ls = p.S + row * kSBlockHalves + zp;
-            lz = sym ? nullptr : p.Z + row * kZBlockWords + (zp >> 3);
+            hb = 2u * (uint32_t)(t64 * p.G + wl.g0) + (uint32_t)jl;
         };
         // load the cursor's stage (zeros past the matrix edge) and advance the cursor
         auto fetch = [&](StageRegs<kNW, kNR>& r) {
             if (!wl.valid()) return;
             if (l_in) {
-#pragma unroll
-                for (int h = 0; h < kNW / 2; ++h) {
-                    r.w[2 * h] = __ldg(reinterpret_cast<const uint4*>(lw + h * 512 + wo0));
-                    r.w[2 * h + 1] = __ldg(reinterpret_cast<const uint4*>(lw + h * 512 + wo1));
-                }
+                const uint4* w = reinterpret_cast<const uint4*>(p.Wq) + (size_t)hb * (kBlockWords / 8);
+                r.w[0] = __ldg(w + wo0);
+                r.w[1] = __ldg(w + wo1);
+                // first scale row of the stage: a 64-k half of a block with SG >= 2 rows starts at row (SG / 2) * half
+                const size_t sr = SG >= 2 ? (size_t)hb * (SG / 2) : (size_t)(hb >> 1);
 #pragma unroll
                 for (int i = 0; i < kNR; ++i) {
-                    r.s[i] = __ldg(ls + i * kSBlockHalves);
-                    r.zw[i] = sym ? 0u : __ldg(lz + i * kZBlockWords);
+                    r.s[i] = __ldg(p.S + (sr + i) * kSBlockHalves + zp);
+                    r.zw[i] = sym ? 0u : __ldg(p.Z + (sr + i) * kZBlockWords + (zp >> 3));
                 }
             } else {
 #pragma unroll
@@ -484,9 +462,7 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
             }
             jl += kTileSets;
             if (jl < wl.stages_in_seg()) {
-                lw += (kTileSets / kSPU) * kBlockWords;
-                ls += (kTileSets / kSPU) * (SG * kSBlockHalves);
-                if (!sym) lz += (kTileSets / kSPU) * (SG * kZBlockWords);
+                hb += kTileSets;
             } else {
                 wl.next();
                 point();
@@ -494,11 +470,10 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
         };
         point();
         // register ring of prefetched stages, written out so that no slot is ever copied
-        static_assert(kPF == 3, "the ring below has three slots");
-        StageRegs<kNW, kNR> pf0, pf1, pf2;
+        static_assert(kPF == 2, "the ring below has two slots");
+        StageRegs<kNW, kNR> pf0, pf1;
         fetch(pf0);
         fetch(pf1);
-        fetch(pf2);
         // Converting weights into the TMEM ring touches nothing the previous kernel may still be writing,
         // so it starts at once and runs until the ring is full; the dependency wait comes before this
         // warp's first write to global memory (the first epilogue).
@@ -546,8 +521,7 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
                 n_prev = n;
                 // convert ring slot pi, then refill it with the stage kPF ahead
                 if (pi == 0) { ok = convert(pf0, n); fetch(pf0); pi = 1; }
-                else if (pi == 1) { ok = convert(pf1, n); fetch(pf1); pi = 2; }
-                else { ok = convert(pf2, n); fetch(pf2); pi = 0; }
+                else { ok = convert(pf1, n); fetch(pf1); pi = 0; }
                 if (!ok) break;
                 tc_wait_st();
                 tc_fence_before();
@@ -557,24 +531,25 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
             if (!ok) break;
 
             // ---------------------------------------------------- epilogue of this segment
-            const int dbuf = n_seg % kDBufs;
-            if (!mbar_wait(&d_full[dbuf], (n_seg / kDBufs) & 1u)) { ok = false; break; }
+            if (!mbar_wait(d_full, n_seg & 1u)) { ok = false; break; }
             tc_fence_after();
             if (!dep_waited) {
                 asm volatile("griddepcontrol.wait;" ::: "memory");
                 dep_waited = true;
             }
             const int T = w.t;
-            const int n = w.nt * kTileCols + row;
-            const int m_base = w.mt_i * MT + set * kCW;     // first batch row of this warp's columns
-            const uint32_t d_t = tmem_base + lane_addr + dbuf * 128 + set * kCW;
+            const int n = w.nt() * kTileCols + row;
+            const int m_base = w.mt_i() * mt;
+            const uint32_t d_t = tmem_base + lane_addr;
+            const bool has_bias = EPI && p.epi.bias != nullptr;
+            const float bias = has_bias && n < p.N ? widen<BF>(p.epi.bias[n]) : 0.f;
             const long long tile_u0 = (long long)T * p.G;
             const bool whole = w.whole_tile();
             // first segment of a chunk -> slot 2 ci, its continuation into a later tile -> 2 ci + 1
-            float* part = p.ws + ((size_t)(2 * w.ci + (w.first ? 0 : 1)) * MT + set * kCW) * kTileCols + row;
+            float* part = p.ws + ((size_t)(2 * w.ci + (w.first ? 0 : 1)) * mt) * kTileCols + row;
             constexpr int kStep = 16;
 #pragma unroll 1
-            for (int cc = 0; cc < kCW; cc += kStep) {
+            for (int cc = kStep * set; cc < mt; cc += kStep * kTileSets) {      // rows 16 at a time to the sets
                 uint32_t v[kStep];
                 tc_ld16(d_t + cc, v);
                 tc_wait_ld();
@@ -583,7 +558,7 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
 #pragma unroll
                         for (int q = 0; q < kStep; ++q) {
                             const int m = m_base + cc + q;
-                            if (m < p.M) p.C[(size_t)m * p.N + n] = (EPI ? finish<BF>(__uint_as_float(v[q]), n, p.epi) : cast_out<BF>(__uint_as_float(v[q])));
+                            if (m < p.M) p.C[(size_t)m * p.N + n] = EPI ? finish_col<BF>(__uint_as_float(v[q]), has_bias, bias, p.epi.act) : cast_out<BF>(__uint_as_float(v[q]));
                         }
                     }
                 } else {
@@ -594,15 +569,13 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
             // accumulator drained: a later segment's first MMA may overwrite it
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&d_empty[dbuf]);
+            if (lane == 0) mbar_arrive(d_empty);
 
-            if (!whole && p.defer_reduce == 0) {
-                // Split-K reduce (Algorithm 1, Phase 3), per warp region (32 columns n x MT/4 rows m)
+            if (!whole && p.split_k == 0) {
+                // Split-K reduce (Algorithm 1, Phase 3), per warp region (its 32 columns n x its rows m)
                 __threadfence();
                 __syncwarp();
-                // (classic slices: no division on the way to the ticket)
-                const int c_first = p.split_k > 0 ? T * p.split_k : tile_chunk_of(p, tile_u0);
-                const int c_last = p.split_k > 0 ? c_first + p.split_k - 1 : tile_chunk_of(p, tile_u0 + p.G - 1);
+                const int c_first = tile_chunk_of(p, tile_u0), c_last = tile_chunk_of(p, tile_u0 + p.G - 1);
                 int* ticket = p.tickets + ((size_t)T * kTileDequantWarps + dw);
                 int last = 0;
                 if (lane == 0) {
@@ -616,31 +589,16 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
                     // contributors in ascending K: chunk c_first (its first segment if it starts at the tile's
                     // first unit, else its continuation), then the first segments of the others.  Rows are
                     // summed kStep at a time so that many loads are in flight.
-                    const size_t slot_elems = (size_t)MT * kTileCols;
-                    const float* base = p.ws + (size_t)(set * kCW) * kTileCols + row;
-                    const size_t first_slot =
-                        2 * (size_t)c_first + ((p.split_k > 0 || tile_chunk_begin(p, c_first) == tile_u0) ? 0 : 1);
+                    const size_t slot_elems = (size_t)mt * kTileCols;
+                    const float* base = p.ws + row;
+                    const size_t first_slot = 2 * (size_t)c_first + (tile_chunk_begin(p, c_first) == tile_u0 ? 0 : 1);
 #pragma unroll 1
-                    for (int m0 = 0; m0 < kCW; m0 += kStep) {
+                    for (int m0 = kStep * set; m0 < mt; m0 += kStep * kTileSets) {
                         float acc[kStep];
 #pragma unroll
                         for (int q = 0; q < kStep; ++q)
                             acc[q] = __ldcg(base + first_slot * slot_elems + (size_t)(m0 + q) * kTileCols);
-                        // two contributors' loads in flight at a time (one per round trip would make
-                        // the tail S - 1 trips long); the additions keep the ascending order
-                        int c = c_first + 1;
-                        for (; c + 1 <= c_last; c += 2) {
-                            const float* src = base + (size_t)(2 * c) * slot_elems + (size_t)m0 * kTileCols;
-                            float x0[kStep], x1[kStep];
-#pragma unroll
-                            for (int q = 0; q < kStep; ++q) {
-                                x0[q] = __ldcg(src + (size_t)q * kTileCols);
-                                x1[q] = __ldcg(src + 2 * slot_elems + (size_t)q * kTileCols);
-                            }
-#pragma unroll
-                            for (int q = 0; q < kStep; ++q) { acc[q] += x0[q]; acc[q] += x1[q]; }
-                        }
-                        if (c <= c_last) {
+                        for (int c = c_first + 1; c <= c_last; ++c) {
                             const float* src = base + (size_t)(2 * c) * slot_elems + (size_t)m0 * kTileCols;
 #pragma unroll
                             for (int q = 0; q < kStep; ++q) acc[q] += __ldcg(src + (size_t)q * kTileCols);
@@ -649,7 +607,7 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
 #pragma unroll
                             for (int q = 0; q < kStep; ++q) {
                                 const int m = m_base + m0 + q;
-                                if (m < p.M) p.C[(size_t)m * p.N + n] = (EPI ? finish<BF>(acc[q], n, p.epi) : cast_out<BF>(acc[q]));
+                                if (m < p.M) p.C[(size_t)m * p.N + n] = EPI ? finish_col<BF>(acc[q], has_bias, bias, p.epi.act) : cast_out<BF>(acc[q]);
                             }
                         }
                     }

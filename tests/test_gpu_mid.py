@@ -1,4 +1,4 @@
-"""GPU: the tcgen05 kernel for 17 to 64 batch rows (two CTAs per SM) at the sizes where it can go wrong: batch rows at the
+"""GPU: the tcgen05 kernel with two CTAs per SM at the sizes where it can go wrong: batch rows at the
 edges of its 16-row steps, slices that share a tile's rows unevenly or outnumber them, slices inside a cluster (up to
 eight) and beyond one (summed by a second kernel), odd unit counts per slice, a 64-column tail tile, several chunks per
 CTA, several batch tiles.  Inputs are exactly representable, so every schedule has to give the closed form's bits."""
@@ -30,4 +30,28 @@ def test_exact_inputs_bit_equal_for_every_schedule(M, K, N, splits):
         torch.cuda.synchronize()
         assert B.w4a16_device_status() == 0
         assert np.array_equal(c_bits(C), want), "split_k=%d" % split_k
+    del ws
+
+
+@pytest.mark.parametrize("M,K,N,splits", [
+    # batch tiles of 96, 112, 128 rows in the two-CTA kernel (exchange on top of its rings), several of them, a ragged last one
+    (96, 640, 21952, (0, 1, 2)), (128, 1152, 11072, (0, 3)), (300, 1024, 12288, (0, 2)), (128, 384, 22016, (0, 3)),
+    # batch tiles of the wide-tile kernel that are not a power of two: 176, 208, 240 rows, whole tiles, slices, balanced chunks
+    (176, 2048, 3200, (0, 1, 3)), (777, 512, 5696, (0, 1, 2)), (470, 1536, 8256, (0, 1, 4)), (600, 1024, 8192, (0, 1))])
+def test_batch_tiles_above_64_rows_bit_equal(M, K, N, splits):
+    d = wl.make_exact_problem(M, K, N, seed=8100 + M)
+    n0 = N - 192        # the last columns: a 64-column tail tile where there is one
+    want = oracle.gemm_int(d["A_int"], d["Wq"][:, n0:].copy(), d["E"][:, n0:].copy(), d["Z"][:, n0:].copy(), M, 192, K, 128)
+    pw = pack_problem(d, N, K)
+    A = to_dev(d["A"])
+    ws = ensure_ws(M, N, K, splits)
+    first = None
+    for split_k in splits:
+        C = torch.full((M, N), float("nan"), dtype=torch.float16, device="cuda")
+        B.w4a16_gemm(A, pw, C=C, split_k=split_k, path=B.PATH_TILE)
+        torch.cuda.synchronize()
+        assert B.w4a16_device_status() == 0
+        assert np.array_equal(c_bits(C)[:, n0:], want), "split_k=%d" % split_k
+        first = C if first is None else first
+        assert torch.equal(first, C), "split_k=%d" % split_k
     del ws
