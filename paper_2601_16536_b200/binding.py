@@ -104,7 +104,11 @@ def _check(rc: int, what: str):
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    """Raw handle of the current stream of the current device.  (Through the two C functions that
+    ``torch.cuda.current_stream()`` ends in: 0.2 us, where the stream object it builds costs 3.1 us of a call's 8.5.)"""
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t: Optional[torch.Tensor]) -> int:
