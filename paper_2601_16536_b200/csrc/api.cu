@@ -45,6 +45,12 @@ struct DeviceState {
     int stream_evict = 0;
     bool cluster_ok = true;   // cleared when a cluster launch is refused (fewer SMs than usual, MPS limits ...)
 
+    // Has a GEMM been launched on `st` since the last pack?
+    bool packs_seen(cudaStream_t st) const {
+        for (int i = 0; i < kStreamSlots; ++i)
+            if (streams[i].epoch != 0 && streams[i].stream == st) return streams[i].epoch == pack_epoch;
+        return false;
+    }
     // May this launch on `st` overlap the previous kernel of the stream?  Records the launch.
     bool pdl_allowed(cudaStream_t st) {
         for (int i = 0; i < kStreamSlots; ++i) {
@@ -762,6 +768,32 @@ int launch_tile_reduce(const float* parts, uint16_t* C, int M, int N, int mt, in
     return W4A16_OK;
 }
 
+constexpr size_t kStageMaxBytes = 4u << 20;   // (w4a16_gemm_host)
+
+int stage_activations(const void* host, void* dev, int n16, cudaStream_t st) {
+    std::lock_guard<std::mutex> lock(g_mu);
+    DeviceState* d = nullptr;
+    const int rc = current_device(&d);
+    if (rc != W4A16_OK) return rc;
+    if (!d->is_sm100) return W4A16_ERR_ARCH;
+    const int want = (n16 + kStageThreads - 1) / kStageThreads;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(want < 4 * d->sm_count ? want : 4 * d->sm_count), 1, 1);
+    cfg.blockDim = dim3(kStageThreads, 1, 1);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    // (behind a pack a plain launch: the GEMM that follows asks for packed weights while this kernel runs)
+    cfg.numAttrs = d->packs_seen(st) ? 1 : 0;
+    if (cudaLaunchKernelEx(&cfg, stage_activations_kernel, static_cast<const uint4*>(host), static_cast<uint4*>(dev), n16) != cudaSuccess) {
+        cudaGetLastError();
+        return W4A16_ERR_CUDA;
+    }
+    return W4A16_OK;
+}
+
 // The body of every GEMM entry point; the caller holds g_mu.
 int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z, const uint16_t* bias, uint16_t* C,
                 int M, int N, int K, int group, int split_k, int path, int flags, int act, w4a16_stream_t stream) {
@@ -1055,23 +1087,29 @@ int w4a16_gemm_host(const uint16_t* A_host, uint16_t* A_dev, const void* Wq, con
     if (!A_host || !A_dev || !C_dev || !C_host) return W4A16_ERR_NULL;
     if (M < 1 || K < 1 || N < 1) return W4A16_ERR_SHAPE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (cudaMemcpyAsync(A_dev, A_host, (size_t)M * K * 2, cudaMemcpyHostToDevice, st) != cudaSuccess) {
+    // Page-locked host memory that the device can address: the kernels read and write it themselves (each element of C is
+    // written once, by whoever finishes its sum), which saves two copies, their runtime calls and the waits between copy
+    // engine and SMs.  Anything else goes through the staging buffers and the copy engine; so do activations of more than
+    // kStageMaxBytes.  us a call on one stream, K = 11008 / N = 4096, copy engine / kernel: M = 1 25.4 / 17.7, 8 34.9 / 22.4,
+    // 64 68 / 55, 190 143 / 138, 256 182 / 182: bound by PCIe there, so the SMs are left alone.
+    auto addressable = [](const void* p) -> void* {
+        cudaPointerAttributes attr;
+        if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return attr.type == cudaMemoryTypeHost && attr.devicePointer != nullptr && aligned16(attr.devicePointer) ? attr.devicePointer : nullptr;
+    };
+    const size_t a_bytes = (size_t)M * K * 2;
+    const void* a_direct = a_bytes <= kStageMaxBytes && a_bytes % 16 == 0 && aligned16(A_dev) ? addressable(A_host) : nullptr;
+    if (a_direct != nullptr) {
+        const int rc = stage_activations(a_direct, A_dev, (int)(a_bytes / 16), st);
+        if (rc != W4A16_OK) return rc;
+    } else if (cudaMemcpyAsync(A_dev, A_host, a_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess) {
         cudaGetLastError();
         return W4A16_ERR_CUDA;
     }
-    // Page-locked host memory that the device can address takes the result straight from the kernel's stores
-    // (each element of C is written once, by whoever finishes its sum): one copy and one runtime call less.
-    // Anything else goes through C_dev and a copy.
-    uint16_t* c_direct = nullptr;
-    {
-        cudaPointerAttributes attr;
-        if (cudaPointerGetAttributes(&attr, C_host) == cudaSuccess) {
-            if (attr.type == cudaMemoryTypeHost && attr.devicePointer != nullptr && aligned16(attr.devicePointer))
-                c_direct = static_cast<uint16_t*>(attr.devicePointer);
-        } else {
-            cudaGetLastError();
-        }
-    }
+    uint16_t* const c_direct = static_cast<uint16_t*>(addressable(C_host));
     int rc = w4a16_gemm(A_dev, Wq, S, Z, c_direct ? c_direct : C_dev, M, N, K, group, split_k, stream);
     if (rc != W4A16_OK) return rc;
     if (!c_direct && cudaMemcpyAsync(C_host, C_dev, (size_t)M * N * 2, cudaMemcpyDeviceToHost, st) != cudaSuccess) {

@@ -73,6 +73,36 @@ def test_gemm_on_a_non_default_stream_matches_the_default_stream(path, M):
     del ws
 
 
+@pytest.mark.parametrize("M,K,N", [(3, 256, 256), (16, 1152, 1152), (200, 11008, 256)])
+def test_host_buffer_calls_are_ordered_on_their_stream(M, K, N):
+    """Pinned activations staged by a kernel (up to 4 MiB) and by the copy engine: one staging buffer shared by calls that
+    follow each other, and, where K = N, a result buffer that is the next call's activations."""
+    d = wl.make_problem(M, K, N, seed=3400 + M)
+    ws = ensure_ws(M, N, K, 0)
+    raw = [to_dev(d[k]) for k in ("Wq", "S", "Z")]
+    A2 = wl.draw_activations(M, K, 3401)
+    hosts = [torch.from_numpy(a.view(np.float16)).pin_memory() for a in (d["A"], A2)]
+    outs = [torch.zeros((M, N), dtype=torch.float16).pin_memory() for _ in range(3)]
+    A_dev = torch.empty((M, K), dtype=torch.float16, device="cuda")
+    C_dev = torch.empty((M, N), dtype=torch.float16, device="cuda")
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        for _ in range(3):
+            pw = B.w4a16_pack(raw[0], raw[1], raw[2], N, K)       # the first call behind a pack must see it complete
+            B.w4a16_gemm_host(hosts[0], A_dev, pw, C_dev, outs[0])
+            B.w4a16_gemm_host(hosts[1], A_dev, pw, C_dev, outs[1])
+            if K == N:
+                B.w4a16_gemm_host(outs[1], A_dev, pw, C_dev, outs[2])
+    torch.cuda.synchronize()
+    assert B.w4a16_device_status() == 0
+    for host, out in zip(hosts, outs):
+        assert np.array_equal(out.numpy().view(np.uint16), c_bits(B.w4a16_gemm(host.cuda(), pw)))
+    if K == N:
+        assert np.array_equal(outs[2].numpy().view(np.uint16), c_bits(B.w4a16_gemm(outs[1].cuda(), pw)))
+    del ws
+
+
 def test_a_wait_that_runs_out_is_reported_and_the_library_keeps_working():
     M, K, N = 8, 1152, 256
     d = wl.make_problem(M, K, N, seed=3300)
