@@ -128,6 +128,7 @@ struct DecodeGeom {
     int prefetch;      // stages whose weights are requested before the wait for the previous kernel
     bool a_box;        // activation rows of a stage as one tensor copy (kernel_decode.cuh)
     int cps;       // CTAs per SM the launch is sized for (2 or 3)
+    long cost;     // ns by the cost model (automatic schedules)
     bool cluster;  // one thread-block cluster of split_k CTAs per tile: partial tiles meet in shared memory
     int split_k;   // what the kernel runs: 0 = balanced chunks, S >= 1 = S slices per tile
 };
@@ -138,6 +139,8 @@ struct DecodeGeom {
 // row the two are within 1 % (9.15 / 9.09 there, 32.6 / 32.8 at K = 28672 / N = 8192, 14.9 / 15.2 at K = 4096 /
 // N = 22016: the box takes 8 KiB of a slot whatever M is, and long shapes want the ring stage that costs).
 constexpr int kDecABoxMinRows = 2;
+
+const int* mid_max_clusters();
 
 DecodeGeom decode_geom(int M, int N, int G, int split_k, int sms, bool allow_cluster = true, int sg = 1) {
     DecodeGeom g;
@@ -151,42 +154,43 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, int sms, bool allow_clu
     // against 15.8 at N = 22016.  The kernel keeps the template parameter.)
     g.cps = 2;
     long slots = (long)g.cps * sms;
+    g.cost = 0;
     if (split_k == 0) {
-        // How the unit range is cut when the caller leaves it open.  Balanced chunks use every CTA
-        // slot, but a chunk that crosses a tile boundary goes through the workspace exchange in
-        // mid-stream.  S slices per tile keep every chunk inside one tile, and their exchange is
-        // cheaper: none at S = 1, through the cluster for S <= 6, at the end of the stream otherwise.
-        // Slices are sized for 7/8 of the slots: a launch that fills every slot cannot start (and
-        // prefetch its weights) before the launch in front of it has drained (K = 10240 / N = 4608,
-        // 72 tiles: three slices 10.7 us, four 13.2).  Costs in units per CTA, exchanges priced from
-        // measurements: none 0, cluster 4, workspace at the end of a slice 9, workspace in mid-stream
-        // 13 (1.3 / 2.8 / about 4 us at 0.3 us per unit).  K = 4096 / N = 22016: whole tiles 15.0 us,
-        // balanced 18.1; K = 28672 / N = 8192: two slices 33.8, balanced 34.3; K = 11008 / N = 4096:
-        // four slices 9.7, three 10.5, two 13.5; K = 6144 / N = 1536: six slices in a cluster 4.8,
-        // twelve through the workspace 6.5.  Equal chunks over every slot also run 8 % longer than their
-        // share of the units says (SMs finish the same work up to 8 % apart, and with every slot taken there
-        // is no slack): K = 28672 / N = 8192 balanced 32.4 / two slices in a cluster 31.7 us at M = 1, 40.6 /
-        // 38.7 at M = 16; K = 22016 / N = 8192 26.6 / 25.1; but K = 8192 / N = 10240 balanced 16.5 / whole 18.7.
-        long best = (units * 27 / 25 + slots - 1) / slots + 13;
-        int best_s = 0;
-        if (T > slots) {
-            // more tiles than CTAs: whole tiles dealt round-robin; the CTAs of an SM share its issue
-            // slots, so uneven tile counts cost less than the longest CTA suggests (15 % allowed)
-            const long whole_cost = (units * 23 / 20 + slots - 1) / slots;
-            if (whole_cost <= best) { best = whole_cost; best_s = 1; }
-        } else {
-            int s0 = (int)((slots * 7 / 8) / T);
-            if (s0 < 1) s0 = 1;
-            if (s0 > G) s0 = G;
-            const long ws_cost = (G + s0 - 1) / s0 + (s0 == 1 ? 0 : 9);
-            if (ws_cost <= best) { best = ws_cost; best_s = s0; }
-            if (allow_cluster && g.mchunks == 1 && s0 >= 2) {
-                const int sc = s0 < kDecMaxCluster ? s0 : kDecMaxCluster;   // fewer, longer slices that fit a cluster
-                const long cl_cost = (G + sc - 1) / sc + 4;
-                if (cl_cost <= best) { best = cl_cost; best_s = sc; }
+        // How the unit range is cut when the caller leaves it open.  Balanced chunks use every CTA slot, but a chunk that
+        // crosses a tile boundary goes through the workspace exchange in mid-stream.  S slices per tile keep every chunk
+        // inside one tile, and their exchange is cheaper: none at S = 1, through the cluster for S <= 6 (if that many
+        // clusters run at once: a second wave doubles the time), through the workspace at the end of the stream otherwise.
+        // Costs in ns: a unit takes a CTA 288 with 8 rows and 330 with 16 (two CTAs on some SM set the pace whatever the
+        // count: 64 units of 134 whole tiles 17.8 us, of 160 18.6), the rest is what a launch shows beside its units; 500
+        // more with nine tenths of the slots taken, because then the next launch cannot start before this one ends.
+        // us, measured: K = 8192 / N = 8576 two slices 11.3, whole tiles 17.8, balanced 14.9; N = 10240 (320 slices do not
+        // fit) balanced 16.5, whole 18.6; K = 4096 / N = 12288 whole 10.2, balanced 12.1; K = 11008 / N = 4096 four slices
+        // 8.6, three 10.5; K = 23168 / N = 4416 four 15.0, three 18.0; K = 6144 / N = 1536 six in a cluster 4.3, twelve
+        // through the workspace 6.5; K = 28672 / N = 8192 two 31.2, balanced 32.4; K = 4096 / N = 22016 (344 whole tiles on
+        // 296 CTAs, whose pairs share the SM's issue slots: 15 % over the mean) 14.4, balanced 18.4.
+        const long unit_ns = g.mb == 1 ? 288 : 330, wide = g.mb == 1 ? 0 : 700;
+        const int* max_clusters = mid_max_clusters();      // (two CTAs per SM, like that kernel)
+        auto take = [&](int s, long cost) {
+            if (g.cost == 0 || cost < g.cost) { g.cost = cost; split_k = s; }
+        };
+        take(1, 1500 + wide + unit_ns * (T > slots ? (units * 23 / 20 + slots - 1) / slots : (long)G));
+        if (allow_cluster && g.mchunks == 1) {
+            // Clusters of 3 and 5 (and 6, a little) fit the SMs that the launch in front leaves free badly: with most slots
+            // taken a short launch waits for a place (K = 8192, 86 .. 91 tiles in three slices 13 to 14 us, in two 11.0; 52
+            // in five 9.9, in four 7.2; 43 in six 6.8, in five 6.5), a long one hardly (K = 21760, 86 tiles in three 18.0,
+            // balanced 20.5; but 90 in three 22.4, balanced 21.0).  Two and four keep their time up to the last tile that fits (69 tiles in four 7.9, in three 8.7).
+            for (int s = 2; s <= kDecMaxCluster && s <= G; ++s) {
+                if (T + 2 > max_clusters[s]) continue;
+                const long u = (G + s - 1) / s, ctas = (long)T * s;
+                long wait = s % 2 != 0 && ctas * 37 > slots * 30 ? 5000 - 60 * u : s == 6 && ctas * 37 > slots * 32 ? 1250 - 15 * u : 0;
+                if (wait < 0) wait = 0;
+                if (s % 2 != 0 && 10 * ctas > 9 * slots && wait < 3500) wait = 3500;
+                take(s, (s == 2 ? 1700 : 2150) + wide * 7 / 4 + unit_ns * u + (10 * ctas > 9 * slots ? 500 : 0) + wait);
             }
         }
-        split_k = best_s;
+        const int s0 = (int)(slots * 7 / 8 / T < G ? slots * 7 / 8 / T : G);
+        if (s0 > kDecMaxCluster || (s0 >= 2 && !(allow_cluster && g.mchunks == 1))) take(s0, 4200 + wide + unit_ns * ((G + s0 - 1) / s0));
+        take(0, 5700 + wide + unit_ns * ((units * 27 / 25 + slots - 1) / slots));
     }
     g.split_k = split_k;
     if (split_k == 0) {
