@@ -461,6 +461,17 @@ WidePlan wide_plan(int M, int N, int G, int split_k, int sms, bool allow_cluster
     return w;
 }
 
+// 9 to 16 rows with path and split_k left open: the warp-MMA kernel runs its 16-row build, which converts every weight for
+// two MMAs; the two-CTA tcgen05 kernel is ahead on long shapes and level on short ones.  Its cost model, fitted to 32 and 64
+// rows, is 2 us too high here.  us, warp-MMA / tcgen05, M = 16: K = 28672 / N = 8192 38.6 / 32.1, K = 18432 / N = 7168 26.4 /
+// 21.3, K = 4096 / N = 12288 12.7 / 11.1, N = 22016 18.8 / 18.0, K = 8192 / N = 8192 13.3 / 12.5, K = 1024 / N = 3136 5.0 /
+// 3.9, K = 11008 / N = 4096 10.9 / 10.4; K = N = 4096 6.1 / 6.8, K = 2048 / N = 8192 5.9 / 6.5, K = 6144 / N = 1536 6.0 / 6.0.
+bool small_batch_takes_mid(int M, int N, int G, int sms, bool allow_cluster, int sg) {
+    if (M < 9 || M > 16) return false;
+    const long mid = mid_geom(64, M, N, G, 0, sms, allow_cluster, sg).cost - 2000;
+    return mid * 20 < decode_geom(M, N, G, 0, sms, allow_cluster, sg).cost * 19;
+}
+
 // Nominal split factor of the tcgen05 path's schedule: how many chunks share one tile's K range.
 int choose_split_tile(int M, int N, int G, int sms) {
     const WidePlan w = wide_plan(M, N, G, 0, sms, true);
@@ -528,12 +539,10 @@ bool make_decode_tensor_map(CUtensorMap* map, const void* A, int M, int K, int m
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Path taken when the caller does not force one.  Measured on B200 (us, warp-MMA kernel / tcgen05 kernel): up to
-// 16 batch rows the warp-MMA kernel is ahead or level everywhere, with or without a cluster exchange (M = 16:
-// K = 11008 / N = 4096 10.8 / 12.2, K = N = 4096 6.0 / 7.9, K = 4096 / N = 12288 12.5 / 13.1, K = 4096 /
-// N = 22016 18.8 / 21.7, K = 28672 / N = 8192 40.6 / 41.2, K = 18432 / N = 7168 26.4 / 26.7); from 17 rows on it
-// needs a second pass over the weights and the tcgen05 kernel wins by 1.4 to 2 times (M = 24: 22.5 / 12.8 and
-// 75.8 / 42.2 on the first and the last of those shapes).
+// Path taken when the caller does not force one: up to 16 batch rows the warp-MMA kernel (with 9 to 16, long shapes go to
+// the tcgen05 kernel all the same: small_batch_takes_mid), above that the tcgen05 kernels; the warp-MMA kernel would need a
+// second pass over the weights (M = 24, when that was measured: 22.5 us against 12.8 and 75.8 against 42.2 at K = 11008 /
+// N = 4096 and K = 28672 / N = 8192).
 int resolve_path(int M, int path) {
     if (path != W4A16_PATH_AUTO) return path;
     return M <= 16 ? W4A16_PATH_DECODE : W4A16_PATH_TILE;
@@ -594,7 +603,10 @@ int w4a16_choose_split_k_ex(int M, int N, int K, int group, int path) {
     if (check_weight_shape(N, K, group) != W4A16_OK || M < 1) return 1;
     int G = K / kGroup;
     switch (resolve_path(M, path)) {
-        case W4A16_PATH_DECODE: return choose_split_decode(M, N, G, sm_count_or_default());
+        case W4A16_PATH_DECODE:
+            if (path == W4A16_PATH_AUTO && small_batch_takes_mid(M, N, G, sm_count_or_default(), true, kGroup / group))
+                return choose_split_tile(M, N, G, sm_count_or_default());
+            return choose_split_decode(M, N, G, sm_count_or_default());
         case W4A16_PATH_TILE: return choose_split_tile(M, N, G, sm_count_or_default());
         default: return 1;
     }
@@ -856,6 +868,9 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
     }
 
     WidePlan plan = {};
+    if (path_asked == W4A16_PATH_AUTO && split_k == 0 && path == W4A16_PATH_DECODE &&
+        small_batch_takes_mid(M, N, G, d->sm_count, d->cluster_ok, sg))
+        path = W4A16_PATH_TILE;
     if (path == W4A16_PATH_TILE) plan = wide_plan(M, N, G, split_k, d->sm_count, d->cluster_ok, sg);
     if (path == W4A16_PATH_TILE && plan.use_mid) {
         const MidGeom& g = plan.mid;
