@@ -151,6 +151,36 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsign
     return mbar_wait(smem_u32(bar), parity, limit_ns);
 }
 
+// The same wait with its slow path in line and in PTX, for the weight producer and the issuer of kernel_mid.cuh: a call
+// costs them 1 to 4 % of a launch (M = 64: K = 4096 / N = 22016 20.8 -> 20.0 us, N = 12288 14.3 -> 13.9; M = 32: K = N = 4096
+// 7.08 -> 6.81, K = 28672 / N = 8192 33.6 -> 33.1).  In that kernel's dequant warps, and in kernel_tile.cuh, it takes
+// registers from the conversion loop and loses 1 to 5 %.
+__device__ __forceinline__ bool mbar_wait_inline(uint32_t addr, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p, q;\n\t"
+        ".reg .u64 t0, t1;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@p bra DONE;\n\t"
+        "mov.u64 t0, %%globaltimer;\n\t"
+        "AGAIN:\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 20000;\n\t"
+        "@p bra DONE;\n\t"
+        "mov.u64 t1, %%globaltimer;\n\t"
+        "sub.u64 t1, t1, t0;\n\t"
+        "setp.lt.u64 q, t1, %3;\n\t"
+        "@q bra AGAIN;\n\t"
+        "DONE:\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t"
+        "}"
+        : "=r"(ok)
+        : "r"(addr), "r"(parity), "n"(kWaitLimitNs)
+        : "memory");
+    if (!ok) report_status(kStatusMbarTimeout);
+    return ok != 0;
+}
+
 // The same bounded wait with cluster-scope acquire: for a barrier that CTAs of the cluster arrive on
 // after writing this CTA's shared memory.
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity) {

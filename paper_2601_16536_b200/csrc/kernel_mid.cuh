@@ -182,7 +182,7 @@ gemm_mid_kernel(const __grid_constant__ CUtensorMap tmap_a, const MidParams p) {
                 size_t blk = (size_t)t64 * p.G + c.g0;
                 for (int left = c.units; left > 0; left -= kMidWUnits, blk += kMidWUnits, ++n) {
                     const uint32_t st = w0 + woff;
-                    if (n >= p.wstages && !mbar_wait(st + kWEmpty, ph ^ 1u)) { ok = false; break; }
+                    if (n >= p.wstages && !mbar_wait_inline(st + kWEmpty, ph ^ 1u)) { ok = false; break; }
                     const int gc = min(left, kMidWUnits);
                     mbar_expect_tx(st + kWFull, (uint32_t)(halves * gc * (kBlockBytes + SG * kSBlockHalves * 2 + (SYM ? 0 : SG * kZBlockWords * 4))));
                     for (int h = 0; h < halves; ++h) {
@@ -239,12 +239,12 @@ gemm_mid_kernel(const __grid_constant__ CUtensorMap tmap_a, const MidParams p) {
         const uint32_t box_step = (uint32_t)(mt * 128 / 16);     // the next 64-k box, in descriptor units
         for (int ci = blockIdx.x; ci < p.nchunks && ok; ci += gridDim.x, ++seg) {
             const MidChunk c(p, ci);
-            if (seg != 0 && !mbar_wait(d_empty, (seg - 1u) & 1u)) { ok = false; break; }
+            if (seg != 0 && !mbar_wait_inline(d_empty, (seg - 1u) & 1u)) { ok = false; break; }
             tc_fence_after();
             const int nst = c.units * kSPU;
             for (int j = 0; j < nst; ++j) {
                 const uint32_t bar = bars + 16u * slot;
-                if (!mbar_wait(bar, ph)) { ok = false; break; }
+                if (!mbar_wait_inline(bar, ph)) { ok = false; break; }
                 tc_fence_after();
                 if (elect_one()) {
                     const uint64_t bdesc = smem_desc_sw128(act0 + (uint32_t)(slot * abytes));
@@ -259,7 +259,7 @@ gemm_mid_kernel(const __grid_constant__ CUtensorMap tmap_a, const MidParams p) {
                 }
                 __syncwarp();
                 if (prev != 0u) {
-                    if (!mbar_wait(prev + 8u, prev_ph)) { ok = false; break; }
+                    if (!mbar_wait_inline(prev + 8u, prev_ph)) { ok = false; break; }
                     next_act();
                 }
                 prev = bar;
