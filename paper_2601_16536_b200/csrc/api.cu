@@ -468,6 +468,9 @@ WidePlan wide_plan(int M, int N, int G, int split_k, int sms, bool allow_cluster
 // 3.9, K = 11008 / N = 4096 10.9 / 10.4; K = N = 4096 6.1 / 6.8, K = 2048 / N = 8192 5.9 / 6.5, K = 6144 / N = 1536 6.0 / 6.0.
 bool small_batch_takes_mid(int M, int N, int G, int sms, bool allow_cluster, int sg) {
     if (M < 9 || M > 16) return false;
+    // (more 64-column tiles than CTA slots: K = 4096 / N = 22016 18.8 / 18.0 by itself, and behind or in front of a cluster
+    // launch, as between a block's projections, 23.4 / 18.0: some SMs get four tiles)
+    if (N / kTileN > 2 * sms) return true;
     const long mid = mid_geom(64, M, N, G, 0, sms, allow_cluster, sg).cost - 2000;
     return mid * 20 < decode_geom(M, N, G, 0, sms, allow_cluster, sg).cost * 19;
 }
