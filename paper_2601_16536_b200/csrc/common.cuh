@@ -378,12 +378,21 @@ __device__ __forceinline__ float widen(uint16_t v) {
     return r;
 }
 
+// x / (1 + exp(-x)) by the hardware reciprocal (1 ulp; exp(-x) = inf gives 0): the result is rounded to 16 bits next, and
+// __expf's own error (2 ulp and more) is the larger one.  With the IEEE division M = 777, K = 4096 / N = 22016 took 159 us, with
+// this 147 (without bias and SiLU 121); M = 128 38.3 and 34.7, M = 64 23.4 and 21.9.
+__device__ __forceinline__ float silu(float x) {
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(1.f + __expf(-x)));
+    return x * r;
+}
+
 // The final value of C[m, n] from its FP32 sum.
 template <bool BF>
 __device__ __forceinline__ uint16_t finish(float v, int n, const Epilogue& e) {
     if (e.bias != nullptr) v += widen<BF>(e.bias[n]);
     if (e.act == kActRelu) v = fmaxf(v, 0.f);
-    else if (e.act == kActSilu) v = v / (1.f + __expf(-v));
+    else if (e.act == kActSilu) v = silu(v);
     return cast_out<BF>(v);
 }
 
@@ -392,7 +401,7 @@ template <bool BF>
 __device__ __forceinline__ uint16_t finish_col(float v, bool has_bias, float bias, int act) {
     if (has_bias) v += bias;
     if (act == kActRelu) v = fmaxf(v, 0.f);
-    else if (act == kActSilu) v = v / (1.f + __expf(-v));
+    else if (act == kActSilu) v = silu(v);
     return cast_out<BF>(v);
 }
 
