@@ -253,44 +253,43 @@ struct TileGeom {
     long tiles, cost;
 };
 
-constexpr size_t kTileTicketBytes = 131072;   // 16 counters per tile, after the 16 KiB of the small-M kernel
-constexpr size_t kWsFullHeaderBytes = kWsHeaderBytes + kTileTicketBytes;
-constexpr long kTileMaxTicketTiles = kTileTicketBytes / (sizeof(int) * kTileDequantWarps);
+constexpr size_t kWsFullHeaderBytes = W4A16_WORKSPACE_HEADER_BYTES;   // (the small-M kernel's tickets, the rest reserved)
 
 // Activation ring of a CTA: beyond about 200 KiB of shared memory the L1 that the weight loads pass through gets too small
 // (148 whole tiles of K = 16384, 208 rows: eight slots 120 us, six 100; 256 rows have six either way).
 constexpr int kTileSmem = 200 * 1024;
 
-// What a launch costs, in ns, and how its units are cut.  A unit takes 400 + 1.85 mt ns (148 whole tiles of K = 16384: 80
-// rows 74 us, 128 83, 160 90, 208 100, 256 111), a launch 3.5 us beside its units, K slices 5.5 us more for storing
-// partial tiles and the kernel that sums them.
+// What a launch costs, in ns, and how its units are cut.  A unit takes 400 + 1.85 mt ns with every SM busy (148 whole tiles
+// of K = 16384: 80 rows 74 us, 128 83, 160 90, 208 100, 256 111), 40 % less with few (the L2 that brings the activations is
+// what they share), a launch 3.5 us beside its units, K slices 4 us more for the partial tiles and the kernel that sums them.
 TileGeom tile_geom_rows(int mt, int M, int N, int G, int split_k, int sms) {
     TileGeom g;
     g.mt = mt;
     g.m_tiles = (M + mt - 1) / mt;
     g.n_tiles = (N + kTileCols - 1) / kTileCols;
     g.tiles = (long)g.m_tiles * g.n_tiles;
-    // more tiles than ticket counters: whole tiles only (no partial tiles, no tickets)
-    if (split_k == 0 && g.tiles > kTileMaxTicketTiles) split_k = 1;
     const long unit_ns = 400 + mt * 37 / 20;
     g.cost = 0;
     if (split_k == 0) {
-        // Balanced chunks use every SM to the end, but a chunk that starts or ends inside a tile leaves
-        // an FP32 partial tile behind (store, ticket, reload: the larger the batch tile the dearer, and
-        // in mid-stream it stalls the pipeline).  S slices per tile (tiles <= SMs) or whole tiles in
-        // waves (tiles > SMs) avoid that at the price of idle SMs.  Constants fitted to K = N = 8192 with M up to 4096.
-        const long balanced = ((g.tiles * G + sms - 1) / sms + 6 + mt / 8) * unit_ns;
+        // Balanced chunks use every SM to the end, but a chunk that starts or ends inside a tile leaves an FP32 partial tile
+        // behind, whose store stalls the pipeline in mid-stream: 12 us in all, 17.5 where chunks span several tiles.  S
+        // slices per tile (tiles <= SMs) or whole tiles in waves (tiles > SMs) avoid that at the price of idle SMs.
+        // us, slices or waves / balanced: M = 256: K = 16384 / N = 4096 30.5 / 32.1, K = N = 8192 29.6 / 32.0; M = 600, K = N =
+        // 8192 83.3 / 82.7; M = 777, K = 4096 / N = 22016 119 / 140; M = 1024, K = N = 8192 99 / 112; M = 256, K = 8192 /
+        // N = 20480 (160 tiles) 86.5 / 78.8.
+        auto busy = [&](long ctas, long u) { return u * unit_ns * (6 * sms + 4 * ctas) / (10 * sms); };
+        const long balanced = (g.tiles * G + sms - 1) / sms * unit_ns + (g.tiles <= sms ? 12000 : 17500);
         int s0 = 1;
         long classic;
         if (g.tiles <= sms) {
             s0 = sms / (int)g.tiles;
             if (s0 > G) s0 = G;
-            classic = (G + s0 - 1) / s0 * unit_ns + (s0 > 1 ? 5500 : 0);
+            classic = busy(g.tiles * s0, (G + s0 - 1) / s0) + (s0 > 1 ? 7500 : 3500);
         } else {
-            classic = ((g.tiles + sms - 1) / sms) * G * unit_ns;
+            classic = busy(sms, g.tiles / sms * G) + (g.tiles % sms != 0 ? busy(g.tiles % sms, G) : 0) + 3500;
         }
         if (classic <= balanced) split_k = s0;
-        g.cost = 3500 + (classic < balanced ? classic : balanced);
+        g.cost = classic < balanced ? classic : balanced;
     }
     g.split_k = split_k;
     if (split_k == 0) {
@@ -378,7 +377,7 @@ const int* mid_max_clusters() {     // [size]
 }
 
 // mtc: most batch rows of a tile, 64 or 128.  Cost model in ns, fitted to the figures below: a unit takes a CTA 400 + 0.7 mt
-// ns when it has the SM to itself and 480 + 2 mt when two share it (64-row build), 500 + 2 mt and 640 + 3.2 mt (128 rows);
+// ns when it has the SM to itself and 470 + 1.6 mt when two share it (64-row build), 500 + 2 mt and 560 + 2.8 mt (128 rows);
 // a launch 4 us beside its units, and 0.7 us more where more than half of the slots are taken, so that the next launch's
 // CTAs do not find room before this one ends; the exchange inside a cluster of s 600 + 150 s (4300 + 300 s).
 // Measured (us), M = 32: K = N = 4096 four slices 7.09, eight 7.44; K = 11008 / N = 4096 8 / 6 / 4 slices 11.0 / 11.6 /
@@ -397,7 +396,7 @@ MidGeom mid_geom(int mtc, int M, int N, int G, int split_k, int sms, bool allow_
     if (split_k == 0) {
         const int* max_clusters = mid_max_clusters();
         const bool wide = mtc > 64;
-        const long alone = wide ? 500 + 2 * g.mt : 400 + g.mt * 7 / 10, shared = wide ? 640 + g.mt * 16 / 5 : 480 + 2 * g.mt;
+        const long alone = wide ? 500 + 2 * g.mt : 400 + g.mt * 7 / 10, shared = wide ? 560 + g.mt * 14 / 5 : 470 + g.mt * 8 / 5;
         for (int s = 1; s <= kMidMaxCluster && s <= G; ++s) {
             if (s > 1 && (!allow_cluster || g.tiles > max_clusters[s] || !fits(s))) continue;
             const long ctas = g.tiles * s;
@@ -463,7 +462,7 @@ WidePlan wide_plan(int M, int N, int G, int split_k, int sms, bool allow_cluster
 
 // 9 to 16 rows with path and split_k left open: the warp-MMA kernel runs its 16-row build, which converts every weight for
 // two MMAs; the two-CTA tcgen05 kernel is ahead on long shapes and level on short ones.  Its cost model, fitted to 32 and 64
-// rows, is 2 us too high here.  us, warp-MMA / tcgen05, M = 16: K = 28672 / N = 8192 38.6 / 32.1, K = 18432 / N = 7168 26.4 /
+// rows, is 1.7 us too high here.  us, warp-MMA / tcgen05, M = 16: K = 28672 / N = 8192 38.6 / 32.1, K = 18432 / N = 7168 26.4 /
 // 21.3, K = 4096 / N = 12288 12.7 / 11.1, N = 22016 18.8 / 18.0, K = 8192 / N = 8192 13.3 / 12.5, K = 1024 / N = 3136 5.0 /
 // 3.9, K = 11008 / N = 4096 10.9 / 10.4; K = N = 4096 6.1 / 6.8, K = 2048 / N = 8192 5.9 / 6.5, K = 6144 / N = 1536 6.0 / 6.0.
 bool small_batch_takes_mid(int M, int N, int G, int sms, bool allow_cluster, int sg) {
@@ -471,7 +470,7 @@ bool small_batch_takes_mid(int M, int N, int G, int sms, bool allow_cluster, int
     // (more 64-column tiles than CTA slots: K = 4096 / N = 22016 18.8 / 18.0 by itself, and behind or in front of a cluster
     // launch, as between a block's projections, 23.4 / 18.0: some SMs get four tiles)
     if (N / kTileN > 2 * sms) return true;
-    const long mid = mid_geom(64, M, N, G, 0, sms, allow_cluster, sg).cost - 2000;
+    const long mid = mid_geom(64, M, N, G, 0, sms, allow_cluster, sg).cost - 1700;
     return mid * 20 < decode_geom(M, N, G, 0, sms, allow_cluster, sg).cost * 19;
 }
 
@@ -657,7 +656,7 @@ int w4a16_set_workspace(void* dev_ptr, size_t bytes) {
     }
     if ((reinterpret_cast<uintptr_t>(dev_ptr) & 255u) != 0) return W4A16_ERR_ALIGN;
     if (bytes < kWsFullHeaderBytes) return W4A16_ERR_WORKSPACE;
-    // both kernels' ticket blocks start at zero (and leave zeros behind after every call)
+    // the ticket counters start at zero (and are zero again after every call)
     if (cudaMemset(dev_ptr, 0, kWsFullHeaderBytes) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
         cudaGetLastError();
         return W4A16_ERR_CUDA;
@@ -764,22 +763,31 @@ TileKernel tile_kernel(int sg, bool bf, bool sym, bool epi) {
                                                                        : tile_kernel_f16_sg4(sym, epi);
 }
 
-// Split-K sum behind a tcgen05 kernel that only stored its partial tiles (slices of whole tiles).
-int launch_tile_reduce(const float* parts, uint16_t* C, int M, int N, int mt, int n_tiles, long tiles, int split_k, bool bf,
-                       const Epilogue& epi, cudaStream_t st) {
-    const long long quads = (long long)tiles * mt * (kTileCols / 4);
+// Split-K sum behind a tcgen05 kernel that stored its partial tiles: S slices per tile, or (split_k == 0) balanced chunks.
+int launch_tile_reduce(const float* parts, uint16_t* C, int M, int N, int G, int mt, int n_tiles, long tiles, int split_k,
+                       int nchunks, bool bf, const Epilogue& epi, cudaStream_t st) {
+    TileReduce p;
+    p.M = M; p.N = N; p.G = G;
+    p.mt = mt;
+    p.n_tiles = n_tiles;
+    p.split_k = split_k;
+    p.nchunks = nchunks;
+    p.bal_q = (int)((long long)tiles * G / nchunks);
+    p.bal_r = (int)((long long)tiles * G % nchunks);
+    p.div_mt = fast_div_make((uint32_t)mt);
+    p.div_ntiles = fast_div_make((uint32_t)n_tiles);
+    p.epi = epi;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // always behind the GEMM kernel just launched on this stream
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((quads + 255) / 256), 1, 1);
+    cfg.gridDim = dim3((unsigned)(tiles * mt / 8), 1, 1);
     cfg.blockDim = dim3(256, 1, 1);
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const FastDiv div_mt = fast_div_make((uint32_t)mt), div_nt = fast_div_make((uint32_t)n_tiles);
-    const cudaError_t e = bf ? cudaLaunchKernelEx(&cfg, tile_splitk_reduce_kernel<true>, parts, C, M, N, mt, div_mt, n_tiles, div_nt, split_k, quads, epi)
-                             : cudaLaunchKernelEx(&cfg, tile_splitk_reduce_kernel<false>, parts, C, M, N, mt, div_mt, n_tiles, div_nt, split_k, quads, epi);
+    const cudaError_t e = bf ? cudaLaunchKernelEx(&cfg, tile_splitk_reduce_kernel<true>, parts, C, p)
+                             : cudaLaunchKernelEx(&cfg, tile_splitk_reduce_kernel<false>, parts, C, p);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return W4A16_ERR_CUDA;
@@ -840,7 +848,7 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
     Epilogue epi;
     epi.bias = bias;
     epi.act = act;
-    // registered workspace: [16 KiB small-M tickets][128 KiB tile tickets][partial results]
+    // registered workspace: [small-M tickets and reserve: the documented header][partial results]
     unsigned char* ws_body = d->ws ? static_cast<unsigned char*>(d->ws) + kWsFullHeaderBytes : nullptr;
     const size_t ws_body_bytes = d->ws_bytes > kWsFullHeaderBytes ? d->ws_bytes - kWsFullHeaderBytes : 0;
 
@@ -939,7 +947,7 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
             return W4A16_ERR_CUDA;
         }
         if (g.split_k > 1 && !g.cluster)
-            return launch_tile_reduce(p.ws, C, M, N, g.mt, g.n_tiles, g.tiles, g.split_k, bf, epi, st);
+            return launch_tile_reduce(p.ws, C, M, N, G, g.mt, g.n_tiles, g.tiles, g.split_k, g.nchunks, bf, epi, st);
         return W4A16_OK;
     }
 
@@ -947,7 +955,6 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         const TileGeom& g = plan.tile;
         if (g.smem_bytes > d->max_smem_optin) return W4A16_ERR_PATH;
         if (g.split_k != 1) {
-            if (g.tiles > kTileMaxTicketTiles) return W4A16_ERR_SPLITK;
             if (ws_body_bytes < tile_workspace_bytes(g)) return W4A16_ERR_WORKSPACE;
         }
         // (the kernel's chunk arithmetic is 32-bit)
@@ -959,7 +966,6 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         p.S = static_cast<const uint16_t*>(S);
         p.Z = Zw;
         p.C = C;
-        p.tickets = reinterpret_cast<int*>(d->ws ? static_cast<unsigned char*>(d->ws) + kWsHeaderBytes : nullptr);
         p.ws = reinterpret_cast<float*>(ws_body);
         p.M = M; p.N = N; p.K = K; p.G = G;
         p.mt = g.mt;
@@ -970,13 +976,10 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         p.stages = g.stages;
         tile_fill_chunk_math(p);
         p.epi = epi;
-        // Slices of whole tiles on CTAs of their own: the sum of the partial tiles (and with it the optional
-        // bias / activation) is a second, GPU-wide kernel behind this one (kernels_basic.cuh).  Balanced
-        // chunks, whose pieces belong to different tiles, keep the reduce inside the kernel.
-        // Measured (us, in the kernel / second kernel): M = 256: K = 10240 / N = 4608 (four slices) 31.9 / 24.6,
-        // K = 16384 / N = 4096 39.2 / 32.9, K = N = 8192 (two slices) 34.1 / 33.3.
-        const bool defer = g.split_k >= 2;
-        const bool has_epi = !defer && (bias != nullptr || act != W4A16_ACT_NONE);
+        // Partial tiles are summed (and get the optional bias / activation) by a second, GPU-wide kernel behind this one
+        // (kernels_basic.cuh).  Measured (us, in the kernel / second kernel), M = 256: K = 10240 / N = 4608 (four slices)
+        // 31.9 / 24.6, K = 16384 / N = 4096 39.2 / 32.9, K = N = 8192 (two slices) 34.1 / 33.3.
+        const bool has_epi = g.split_k < 2 && (bias != nullptr || act != W4A16_ACT_NONE);
         TileKernel kern = tile_kernel(sg, bf, sym, has_epi);
         bool& attr_set = d->tile_attr_set[log2_sg(sg)][bf ? 1 : 0][sym ? 1 : 0][has_epi ? 1 : 0];
         if (!attr_set) {
@@ -1003,7 +1006,8 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
             cudaGetLastError();
             return W4A16_ERR_CUDA;
         }
-        if (defer) return launch_tile_reduce(p.ws, C, M, N, g.mt, g.n_tiles, g.tiles, g.split_k, bf, epi, st);
+        if (g.split_k != 1)
+            return launch_tile_reduce(p.ws, C, M, N, G, g.mt, g.n_tiles, g.tiles, g.split_k, g.nchunks, bf, epi, st);
         return W4A16_OK;
     }
 

@@ -8,7 +8,7 @@
 //   registers --tcgen05.st--> TMEM (A operand, one column n per lane, k packed along columns)
 //   HBM --TMA tensor (128B swizzle)--> shared (activation tile, MT rows m x 64 k): B operand
 //   tcgen05.mma.kind::f16  D[128 n x MT m] (FP32, TMEM) += A(TMEM) . B(shared)   one elected lane
-//   TMEM --tcgen05.ld--> registers -> FP16 C, or FP32 partial tile + ticket (Split-K)
+//   TMEM --tcgen05.ld--> registers -> FP16 C, or FP32 partial tile (Split-K)
 //
 // so packed weights go from HBM straight to registers, dequantized weights never touch shared or
 // global memory (Algorithm 1's Phase 1 output stays on chip), and the activation tile is re-used
@@ -23,10 +23,9 @@
 //     (Algorithm 1, Phase 2), chunks dealt round-robin.
 // The part of a chunk inside one tile is a segment: the accumulator is zeroed at its first MMA and
 // drained after its last.  A segment that covers a whole tile is cast to FP16 and stored; any other
-// segment leaves as an FP32 partial tile in the workspace, and the warp that draws the last ticket
-// of its 32-column region (its 16-row steps) adds the partial regions in ascending K order (Phase 3).
-// No warp ever waits for another CTA, and the order of the sum is fixed, so results are
-// bit-identical from run to run.
+// segment leaves as an FP32 partial tile in the workspace, for the kernel launched behind this one that adds them in
+// ascending K order (Phase 3, tile_splitk_reduce_kernel).  No warp ever waits for another CTA, and the order of the sum is
+// fixed, so results are bit-identical from run to run.
 //
 // Batch tiles of up to 256 rows, a run-time multiple of 16 (MT; which shapes come here and which go to kernel_mid.cuh is
 // the host's choice by cost).  One pipeline stage is half a group (64 k, four MMAs).
@@ -42,7 +41,7 @@
 // out records a status code and the CTA drains and exits (TMEM is always released).
 //
 // Which schedule a shape gets when the caller leaves split_k open is the host's choice (api.cu):
-// partial tiles are dear (FP32 store, ticket, reload; in mid-chunk they also stall the pipeline), so
+// partial tiles are dear (FP32 store, reload; in mid-chunk they also stall the pipeline), so
 // balanced chunks are used only where the SMs left idle by whole slices or whole tiles cost more.
 #pragma once
 
@@ -72,7 +71,6 @@ struct TileParams {
     const uint32_t* Z;   // nullptr: symmetric format, zero point 8
     uint16_t* C;
     float* ws;       // partial tiles: [2 * nchunks slots][MT][128] FP32
-    int* tickets;    // zeroed counters: [tile][16 epilogue warps]
     int M, N, K, G;
     int mt;          // batch rows of a tile: multiple of 16, at most 256
     int n_tiles;     // NT = ceil(N / 128)
@@ -172,14 +170,6 @@ __device__ __forceinline__ int tile_chunk_begin(const TileParams& p, int i) {
     const int t = fast_div(i, p.div_split), s = i - t * p.split_k;
     return t * p.G + s * p.slice_base + min(s, p.slice_rem);
 }
-// The balanced chunk that holds unit u.  (Out of line: only the epilogue of partial tiles comes here.)
-static __device__ __noinline__ int tile_chunk_of_s(int nchunks, long long units, long long u) {
-    return (int)(((u + 1) * nchunks - 1) / units);
-}
-__device__ __forceinline__ int tile_chunk_of(const TileParams& p, long long u) {
-    return tile_chunk_of_s(p.nchunks, (long long)p.m_tiles * p.n_tiles * p.G, u);
-}
-
 // Where chunk ci (or the next non-empty one of this CTA, stepping by `stride`) starts.
 struct ChunkStart {
     int ci;        // the chunk found (>= nchunks: none left)
@@ -407,8 +397,7 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
         if (!ok && lane == 0) *abort_flag = 1;
     } else {
         // ------------------------------------------------------------ dequant + epilogue warps
-        const int dw = warp - 2;               // 0..15
-        const int set = dw >> 2;               // takes the stages whose index in this CTA is = set (mod 4)
+        const int set = (warp - 2) >> 2;       // takes the stages whose index in this CTA is = set (mod 4)
         const int quarter = warp & 3;          // TMEM lanes this warp may touch
         const int row = quarter * 32 + lane;   // column n inside the CTA tile = TMEM lane
         const int half = row >> 6, col = row & 63;
@@ -537,13 +526,11 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
                 asm volatile("griddepcontrol.wait;" ::: "memory");
                 dep_waited = true;
             }
-            const int T = w.t;
             const int n = w.nt() * kTileCols + row;
             const int m_base = w.mt_i() * mt;
             const uint32_t d_t = tmem_base + lane_addr;
             const bool has_bias = EPI && p.epi.bias != nullptr;
             const float bias = has_bias && n < p.N ? widen<BF>(p.epi.bias[n]) : 0.f;
-            const long long tile_u0 = (long long)T * p.G;
             const bool whole = w.whole_tile();
             // first segment of a chunk -> slot 2 ci, its continuation into a later tile -> 2 ci + 1
             float* part = p.ws + ((size_t)(2 * w.ci + (w.first ? 0 : 1)) * mt) * kTileCols + row;
@@ -570,49 +557,6 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(d_empty);
-
-            if (!whole && p.split_k == 0) {
-                // Split-K reduce (Algorithm 1, Phase 3), per warp region (its 32 columns n x its rows m)
-                __threadfence();
-                __syncwarp();
-                const int c_first = tile_chunk_of(p, tile_u0), c_last = tile_chunk_of(p, tile_u0 + p.G - 1);
-                int* ticket = p.tickets + ((size_t)T * kTileDequantWarps + dw);
-                int last = 0;
-                if (lane == 0) {
-                    const int old = atomicAdd(ticket, 1);
-                    last = (old == c_last - c_first);
-                    if (last) *ticket = 0;   // every contributor has arrived: zero for the next call
-                }
-                last = __shfl_sync(0xffffffffu, last, 0);
-                if (last) {
-                    __threadfence();
-                    // contributors in ascending K: chunk c_first (its first segment if it starts at the tile's
-                    // first unit, else its continuation), then the first segments of the others.  Rows are
-                    // summed kStep at a time so that many loads are in flight.
-                    const size_t slot_elems = (size_t)mt * kTileCols;
-                    const float* base = p.ws + row;
-                    const size_t first_slot = 2 * (size_t)c_first + (tile_chunk_begin(p, c_first) == tile_u0 ? 0 : 1);
-#pragma unroll 1
-                    for (int m0 = kStep * set; m0 < mt; m0 += kStep * kTileSets) {
-                        float acc[kStep];
-#pragma unroll
-                        for (int q = 0; q < kStep; ++q)
-                            acc[q] = __ldcg(base + first_slot * slot_elems + (size_t)(m0 + q) * kTileCols);
-                        for (int c = c_first + 1; c <= c_last; ++c) {
-                            const float* src = base + (size_t)(2 * c) * slot_elems + (size_t)m0 * kTileCols;
-#pragma unroll
-                            for (int q = 0; q < kStep; ++q) acc[q] += __ldcg(src + (size_t)q * kTileCols);
-                        }
-                        if (n < p.N) {
-#pragma unroll
-                            for (int q = 0; q < kStep; ++q) {
-                                const int m = m_base + m0 + q;
-                                if (m < p.M) p.C[(size_t)m * p.N + n] = EPI ? finish_col<BF>(acc[q], has_bias, bias, p.epi.act) : cast_out<BF>(acc[q]);
-                            }
-                        }
-                    }
-                }
-            }
         }
         if (!ok && lane == 0) *abort_flag = 1;
     }

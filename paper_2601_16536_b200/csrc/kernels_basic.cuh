@@ -317,49 +317,68 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ ws, uint16_t* __r
     C[i] = finish<BF>(acc, (int)(i % (size_t)N), epi);
 }
 
-// Algorithm 1, Phase 3 for the tcgen05 kernel when every column tile is cut into `split_k` slices of its own
-// CTAs: that kernel only stores its FP32 partial tiles (slot 2 (T split_k + s) of [batch row in tile][128
-// columns]) and this one, launched behind it, sums them in ascending s, applies the optional bias /
-// activation and rounds once.  A thread takes four neighbouring columns of one batch row.  Inside the GEMM
-// kernel the same sum was a chain of L2 round trips in the one CTA per tile that finished last (5 to 10 us
-// of a 32 us launch at M = 256); here the whole GPU does it at once.
+// Algorithm 1, Phase 3 for the tcgen05 kernels whose partial tiles went to the workspace (FP32, [batch row in tile][128
+// columns]; the first segment of chunk c in slot 2 c, its continuation into a later tile in slot 2 c + 1): this kernel,
+// launched behind, sums them in ascending K, applies the optional bias / activation and rounds once.  A thread takes four
+// neighbouring columns of one batch row, a block eight rows of one tile.  Inside the GEMM kernel the same sum was a chain of
+// L2 round trips in the one CTA per tile that finished last (5 to 10 us of a 32 us launch at M = 256); here the whole GPU
+// does it at once.
+struct TileReduce {
+    int M, N, G, mt, n_tiles;
+    int split_k;                 // S >= 2: S slices per tile; 0: balanced chunks
+    int nchunks, bal_q, bal_r;   // balanced: units = bal_q nchunks + bal_r
+    FastDiv div_mt, div_ntiles;
+    Epilogue epi;
+};
 template <bool BF>
 __global__ void __launch_bounds__(256)
-tile_splitk_reduce_kernel(const float* __restrict__ ws, uint16_t* __restrict__ C, int M, int N, int mt, FastDiv div_mt,
-                          int n_tiles, FastDiv div_ntiles, int split_k, long long quads, Epilogue epi) {
+tile_splitk_reduce_kernel(const float* __restrict__ ws, uint16_t* __restrict__ C, const TileReduce p) {
+    __shared__ int chunks[3];                           // first and last contributor, slot of the first
     // the next kernel of the stream may start its prologue; the partial tiles are the previous kernel's output
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int r = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5);   // (tiles * mt < 2^31: the caller checks)
+    const int T = fast_div(r, p.div_mt);                // tile = batch tile * n_tiles + column tile; mt % 16 == 0: one per block
+    if (threadIdx.x == 0) {
+        if (p.split_k > 0) {
+            chunks[0] = T * p.split_k;
+            chunks[1] = chunks[0] + p.split_k - 1;
+            chunks[2] = 2 * chunks[0];
+        } else {
+            const long long units = (long long)p.bal_q * p.nchunks + p.bal_r, u0 = (long long)T * p.G;
+            const int c0 = (int)(((u0 + 1) * p.nchunks - 1) / units);
+            chunks[0] = c0;
+            chunks[1] = (int)(((u0 + p.G) * p.nchunks - 1) / units);
+            chunks[2] = 2 * c0 + ((long long)c0 * p.bal_q + (long long)c0 * p.bal_r / p.nchunks == u0 ? 0 : 1);
+        }
+    }
+    __syncthreads();
+    const int c_first = chunks[0], c_last = chunks[1];
+    if (c_first == c_last) return;                      // one chunk has the whole tile and has written it
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= quads) return;
-    const int nq = (int)(q & 31);                       // which four of the tile's 128 columns
-    const int r = (int)(q >> 5);                        // (tiles * mt < 2^31: the caller checks)
-    const int T = fast_div(r, div_mt);                  // tile = batch tile * n_tiles + column tile
-    const int m_local = r - T * mt;
-    const int mt_i = fast_div(T, div_ntiles), nt = T - mt_i * n_tiles;
-    const int m = mt_i * mt + m_local, n = nt * 128 + nq * 4;
-    if (m >= M || n >= N) return;
-    const size_t slot = (size_t)2 * mt * 128;           // floats between the slots of neighbouring slices
-    const float* src = ws + ((size_t)T * split_k) * slot + (size_t)m_local * 128 + nq * 4;
-    float4 acc = __ldcg(reinterpret_cast<const float4*>(src));
-    int s = 1;
-    for (; s + 3 < split_k; s += 4) {                   // four slices' loads in flight, added in order
-        const float4 x0 = __ldcg(reinterpret_cast<const float4*>(src + (size_t)s * slot));
-        const float4 x1 = __ldcg(reinterpret_cast<const float4*>(src + (size_t)(s + 1) * slot));
-        const float4 x2 = __ldcg(reinterpret_cast<const float4*>(src + (size_t)(s + 2) * slot));
-        const float4 x3 = __ldcg(reinterpret_cast<const float4*>(src + (size_t)(s + 3) * slot));
+    const int m_local = r - T * p.mt;
+    const int mt_i = fast_div(T, p.div_ntiles), nt = T - mt_i * p.n_tiles;
+    const int m = mt_i * p.mt + m_local, n = nt * 128 + (int)(threadIdx.x & 31) * 4;
+    if (m >= p.M || n >= p.N) return;
+    const size_t slot = (size_t)p.mt * 128, step = 2 * slot;   // floats of a slot; between the first segments of neighbouring chunks
+    const float* base = ws + (size_t)m_local * 128 + (threadIdx.x & 31) * 4;
+    float4 acc = __ldcg(reinterpret_cast<const float4*>(base + (size_t)chunks[2] * slot));
+    const float* src = base + (size_t)(c_first + 1) * step;
+    int c = c_first + 1;
+    for (; c + 2 <= c_last; c += 3, src += 3 * step) {  // three contributors' loads in flight, added in order
+        const float4 x0 = __ldcg(reinterpret_cast<const float4*>(src));
+        const float4 x1 = __ldcg(reinterpret_cast<const float4*>(src + step));
+        const float4 x2 = __ldcg(reinterpret_cast<const float4*>(src + 2 * step));
         acc.x += x0.x; acc.y += x0.y; acc.z += x0.z; acc.w += x0.w;
         acc.x += x1.x; acc.y += x1.y; acc.z += x1.z; acc.w += x1.w;
         acc.x += x2.x; acc.y += x2.y; acc.z += x2.z; acc.w += x2.w;
-        acc.x += x3.x; acc.y += x3.y; acc.z += x3.z; acc.w += x3.w;
     }
-    for (; s < split_k; ++s) {
-        const float4 x = __ldcg(reinterpret_cast<const float4*>(src + (size_t)s * slot));
+    for (; c <= c_last; ++c, src += step) {
+        const float4 x = __ldcg(reinterpret_cast<const float4*>(src));
         acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
     }
-    const uint32_t lo = (uint32_t)finish<BF>(acc.x, n, epi) | ((uint32_t)finish<BF>(acc.y, n + 1, epi) << 16);
-    const uint32_t hi = (uint32_t)finish<BF>(acc.z, n + 2, epi) | ((uint32_t)finish<BF>(acc.w, n + 3, epi) << 16);
-    *reinterpret_cast<uint2*>(C + (size_t)m * N + n) = make_uint2(lo, hi);
+    const uint32_t lo = (uint32_t)finish<BF>(acc.x, n, p.epi) | ((uint32_t)finish<BF>(acc.y, n + 1, p.epi) << 16);
+    const uint32_t hi = (uint32_t)finish<BF>(acc.z, n + 2, p.epi) | ((uint32_t)finish<BF>(acc.w, n + 3, p.epi) << 16);
+    *reinterpret_cast<uint2*>(C + (size_t)m * p.N + n) = make_uint2(lo, hi);
 }
 
 // Activations from page-locked host memory into the staging buffer, ahead of the GEMM (w4a16_gemm_host).  The copy engine
