@@ -272,7 +272,9 @@ TileGeom tile_geom_rows(int mt, int M, int N, int G, int split_k, int sms) {
     g.cost = 0;
     if (split_k == 0) {
         // Balanced chunks use every SM to the end, but a chunk that starts or ends inside a tile leaves an FP32 partial tile
-        // behind, whose store stalls the pipeline in mid-stream: 12 us in all, 17.5 where chunks span several tiles.  S
+        // behind, whose store stalls the pipeline in mid-stream: 12 us in all, 17.5 where chunks span two tiles, and never from two
+        // waves on (the CTAs no longer read the same activations at the same time: M = 2787, K = 4224 / N = 13824 319 us, in
+        // waves 290).  S
         // slices per tile (tiles <= SMs) or whole tiles in waves (tiles > SMs) avoid that at the price of idle SMs.
         // us, slices or waves / balanced: M = 256: K = 16384 / N = 4096 30.5 / 32.1, K = N = 8192 29.6 / 32.0; M = 600, K = N =
         // 8192 83.3 / 82.7; M = 777, K = 4096 / N = 22016 119 / 140; M = 1024, K = N = 8192 99 / 112; M = 256, K = 8192 /
@@ -288,8 +290,9 @@ TileGeom tile_geom_rows(int mt, int M, int N, int G, int split_k, int sms) {
         } else {
             classic = busy(sms, g.tiles / sms * G) + (g.tiles % sms != 0 ? busy(g.tiles % sms, G) : 0) + 3500;
         }
-        if (classic <= balanced) split_k = s0;
-        g.cost = classic < balanced ? classic : balanced;
+        const bool waves = classic <= balanced || g.tiles >= 2 * sms;
+        if (waves) split_k = s0;
+        g.cost = waves ? classic : balanced;
     }
     g.split_k = split_k;
     if (split_k == 0) {
