@@ -806,13 +806,17 @@ int stage_activations(const void* host, void* dev, int n16, cudaStream_t st) {
     const int rc = current_device(&d);
     if (rc != W4A16_OK) return rc;
     if (!d->is_sm100) return W4A16_ERR_ARCH;
-    const int want = (n16 + kStageThreads - 1) / kStageThreads;
+    // Larger copies as single warps, so that the reads in flight are spread over more SMs: us a call, K = 11008 / N = 4096,
+    // 128 / 32 threads: M = 8 (11,008 pieces of 16 bytes) 27.1 / 22.6, M = 16 34.4 / 25.5; M = 1 (1,376) 18.0 / 18.8, and
+    // K = 4096 (512) 11.1 / 12.7.
+    const int threads = n16 < 8192 ? kStageThreads : 32;
+    const int want = (n16 + threads - 1) / threads;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(want < 4 * d->sm_count ? want : 4 * d->sm_count), 1, 1);
-    cfg.blockDim = dim3(kStageThreads, 1, 1);
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
     cfg.stream = st;
     cfg.attrs = attr;
     // (behind a pack a plain launch: the GEMM that follows asks for packed weights while this kernel runs)

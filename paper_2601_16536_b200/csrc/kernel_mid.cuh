@@ -1,4 +1,5 @@
-// tcgen05 kernel for 17 to 64 batch rows: two small CTAs per SM, Split-K inside a thread-block cluster.
+// tcgen05 kernel for batch tiles of up to 64 or 128 rows (M = 9 to a few hundred; the host chooses by cost): two small CTAs
+// per SM, Split-K inside a thread-block cluster.
 //
 // Same product as kernel_tile.cuh (transposed, C^T = W16^T . A^T, dequantized weights as the 128-row A operand in
 // tensor memory, FP32 accumulator in tensor memory).  What bounds these calls is neither HBM nor the tensor pipe

@@ -384,13 +384,13 @@ tile_splitk_reduce_kernel(const float* __restrict__ ws, uint16_t* __restrict__ C
 // Activations from page-locked host memory into the staging buffer, ahead of the GEMM (w4a16_gemm_host).  The copy engine
 // would need a semaphore each way and 5.5 us of host time a call; a kernel reads the same bytes over PCIe, and the GEMM
 // behind it starts its prologue and weight requests meanwhile (programmatic dependent launch).
-constexpr int kStageThreads = 128;
+constexpr int kStageThreads = 128;       // at most
 __global__ void __launch_bounds__(kStageThreads)
 stage_activations_kernel(const uint4* __restrict__ host, uint4* __restrict__ dev, int n16) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // the staging buffer may still be read, and the host buffer written, by what comes before on the stream
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (int i = blockIdx.x * kStageThreads + threadIdx.x; i < n16; i += gridDim.x * kStageThreads) dev[i] = __ldcv(host + i);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += gridDim.x * blockDim.x) dev[i] = __ldcv(host + i);
 }
 
 // Diagnostic: one warp waits on a barrier that nobody ever arrives on, with a limit of `limit_ns`.  The wait
