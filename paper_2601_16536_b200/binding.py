@@ -20,6 +20,7 @@ LIB_PATH = os.path.join(_HERE, "libw4a16.so")
 PATH_AUTO, PATH_SIMPLE, PATH_DECODE, PATH_TILE = 0, 1, 2, 3
 FLAG_SYMMETRIC, FLAG_BF16 = 1, 2
 ACT_NONE, ACT_RELU, ACT_SILU = 0, 1, 2
+KERNEL_SIMPLE, KERNEL_DECODE, KERNEL_TILE, KERNEL_MID64, KERNEL_MID128 = 1, 2, 3, 4, 5
 GROUP = 128
 WS_HEADER_BYTES = 16384 + 131072   # W4A16_WORKSPACE_HEADER_BYTES
 
@@ -29,9 +30,17 @@ EXPORTS = (
     "w4a16_choose_split_k_ex", "w4a16_choose_path", "w4a16_pack", "w4a16_dequant", "w4a16_gemm", "w4a16_gemm_ex",
     "w4a16_gemm_host", "w4a16_gemm_static_ws", "w4a16_device_status", "w4a16_selftest_wait_timeout",
     "w4a16_pack_fmt", "w4a16_dequant_fmt", "w4a16_gemm_fmt", "w4a16_quantize",
+    "w4a16_gemm_plan",
 )
 
 _lib = None
+
+
+class Plan(ctypes.Structure):
+    """``w4a16_plan``: kernel (KERNEL_*), batch rows of a tile, slices per tile (0 = balanced chunks), whether they meet
+    in a cluster, workspace bytes that the call asks for."""
+    _fields_ = [("kernel", ctypes.c_int), ("tile_rows", ctypes.c_int), ("split_k", ctypes.c_int), ("cluster", ctypes.c_int),
+                ("workspace_bytes", ctypes.c_size_t)]
 
 
 class W4A16Error(RuntimeError):
@@ -64,6 +73,8 @@ def load():
     L.w4a16_choose_split_k.argtypes = [i, i, i, i]
     L.w4a16_choose_path.restype = i
     L.w4a16_choose_path.argtypes = [i, i, i, i]
+    L.w4a16_gemm_plan.restype = i
+    L.w4a16_gemm_plan.argtypes = [i, i, i, i, i, i, ctypes.POINTER(Plan)]
     L.w4a16_choose_split_k_ex.restype = i
     L.w4a16_choose_split_k_ex.argtypes = [i, i, i, i, i]
     L.w4a16_pack.restype = i
@@ -138,6 +149,13 @@ def w4a16_choose_split_k(M: int, N: int, K: int, group: int = GROUP, path: int =
 
 def w4a16_choose_path(M: int, N: int, K: int, group: int = GROUP) -> int:
     return load().w4a16_choose_path(M, N, K, group)
+
+
+def w4a16_gemm_plan(M: int, N: int, K: int, group: int = GROUP, split_k: int = 0, path: int = PATH_AUTO) -> Plan:
+    """What ``w4a16_gemm`` runs for these arguments on the current device (a B200 where there is none)."""
+    p = Plan()
+    _check(load().w4a16_gemm_plan(M, N, K, group, split_k, path, ctypes.byref(p)), "w4a16_gemm_plan")
+    return p
 
 
 def w4a16_set_workspace(ws: Optional[torch.Tensor]) -> None:

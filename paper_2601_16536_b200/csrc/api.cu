@@ -110,10 +110,15 @@ bool flags_ok(int flags) { return (flags & ~(W4A16_FLAG_SYMMETRIC | W4A16_FLAG_B
 
 size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 
+// For the size and schedule queries, which also answer on a host without a device.
 int sm_count_or_default() {
     DeviceState* d = nullptr;
     if (current_device(&d) == W4A16_OK) return d->sm_count;
     return 148;
+}
+bool clusters_ok() {
+    DeviceState* d = nullptr;
+    return current_device(&d) != W4A16_OK || d->cluster_ok;
 }
 
 // ---- decode-path launch geometry ------------------------------------------------
@@ -142,7 +147,7 @@ constexpr int kDecABoxMinRows = 2;
 
 const int* mid_max_clusters();
 
-DecodeGeom decode_geom(int M, int N, int G, int split_k, int sms, bool allow_cluster = true, int sg = 1) {
+DecodeGeom decode_geom(int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg) {
     DecodeGeom g;
     g.mb = decode_mb(M);
     g.mchunks = (M + 8 * g.mb - 1) / (8 * g.mb);
@@ -234,8 +239,8 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, int sms, bool allow_clu
 }
 
 // Nominal split factor of the balanced schedule: how many CTAs share one column tile's K range.
-int choose_split_decode(int M, int N, int G, int sms) {
-    DecodeGeom g = decode_geom(M, N, G, 0, sms);
+int choose_split_decode(int M, int N, int G, int sms, bool allow_cluster, int sg) {
+    DecodeGeom g = decode_geom(M, N, G, 0, sms, allow_cluster, sg);
     if (g.split_k >= 1) return g.split_k;
     const int T = N / kTileN;
     int s = (g.ctas + T - 1) / T;
@@ -386,7 +391,7 @@ const int* mid_max_clusters() {     // [size]
 // Measured (us), M = 32: K = N = 4096 four slices 7.09, eight 7.44; K = 11008 / N = 4096 8 / 6 / 4 slices 11.0 / 11.6 /
 // 13.8; K = 18432 / N = 7168 5 / 4 21.8 / 22.9; K = 4096 / N = 12288 2 / 1 12.2 / 17.3, three no longer fit at once: 17.5;
 // K = 4096 / N = 22016 1 / 2 18.7 / 22.6; K = 1024 / N = 3136 4 / 8 4.18 / 5.10.
-MidGeom mid_geom(int mtc, int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg = 1) {
+MidGeom mid_geom(int mtc, int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg) {
     MidGeom g;
     g.mtc = mtc;
     g.m_tiles = (M + g.mtc - 1) / g.mtc;
@@ -444,7 +449,7 @@ struct WidePlan {
     TileGeom tile;
     size_t workspace_bytes() const { return use_mid ? mid_workspace_bytes(mid) : tile_workspace_bytes(tile); }
 };
-WidePlan wide_plan(int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg = 1) {
+WidePlan wide_plan(int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg) {
     WidePlan w;
     w.use_mid = true;
     if (M <= 64) {
@@ -478,8 +483,8 @@ bool small_batch_takes_mid(int M, int N, int G, int sms, bool allow_cluster, int
 }
 
 // Nominal split factor of the tcgen05 path's schedule: how many chunks share one tile's K range.
-int choose_split_tile(int M, int N, int G, int sms) {
-    const WidePlan w = wide_plan(M, N, G, 0, sms, true);
+int choose_split_tile(int M, int N, int G, int sms, bool allow_cluster, int sg) {
+    const WidePlan w = wide_plan(M, N, G, 0, sms, allow_cluster, sg);
     if (w.use_mid) return w.mid.split_k;
     if (w.tile.split_k >= 1) return w.tile.split_k;
     long s = (w.tile.nchunks + w.tile.tiles - 1) / w.tile.tiles;
@@ -562,6 +567,39 @@ size_t decode_partial_bytes(const DecodeGeom& g) {
     return round256((size_t)g.mchunks * 2 * (size_t)g.nchunks * (8 * g.mb) * kTileN * sizeof(float));
 }
 
+// What a GEMM call runs: kernel, schedule and the workspace behind the header that it asks for (0: none).  The entry points
+// and the queries all come here, with the group's scale rows per block (sg): whether a cluster's exchange buffer fits, and
+// with it the number of slices, depends on them.
+struct GemmPlan {
+    int kernel;          // W4A16_KERNEL_*
+    int split_simple;
+    DecodeGeom dec;
+    WidePlan wide;
+    size_t workspace;
+};
+GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, int sms, bool allow_cluster) {
+    GemmPlan p;
+    int path = resolve_path(M, path_asked);
+    if (path_asked == W4A16_PATH_AUTO && split_k == 0 && path == W4A16_PATH_DECODE &&
+        small_batch_takes_mid(M, N, G, sms, allow_cluster, sg))
+        path = W4A16_PATH_TILE;
+    if (path == W4A16_PATH_SIMPLE) {
+        p.kernel = W4A16_KERNEL_SIMPLE;
+        p.split_simple = split_k == 0 ? choose_split_decode(M, N, G, sms, true, sg) : split_k;
+        p.workspace = p.split_simple > 1 ? simple_partial_bytes(M, N, p.split_simple) : 0;
+    } else if (path == W4A16_PATH_DECODE) {
+        p.kernel = W4A16_KERNEL_DECODE;
+        p.dec = decode_geom(M, N, G, split_k, sms, allow_cluster, sg);
+        // (the cluster exchange does not touch the workspace, but the contract stays the same for every schedule)
+        p.workspace = p.dec.split_k != 1 ? decode_partial_bytes(p.dec) : 0;
+    } else {
+        p.wide = wide_plan(M, N, G, split_k, sms, allow_cluster, sg);
+        p.kernel = !p.wide.use_mid ? W4A16_KERNEL_TILE : p.wide.mid.mtc <= 64 ? W4A16_KERNEL_MID64 : W4A16_KERNEL_MID128;
+        p.workspace = p.wide.workspace_bytes();
+    }
+    return p;
+}
+
 // ---- built-in scratch for w4a16_gemm_static_ws -------------------------------------
 // Lives in the library's device image: every GPU that loads the library holds these bytes until
 // the process exits.  In host code `g_static_ws` is only a handle for cudaGetSymbolAddress; the
@@ -606,13 +644,14 @@ size_t w4a16_packed_z_bytes(int N, int K, int group) {   // asymmetric formats; 
 int w4a16_choose_split_k_ex(int M, int N, int K, int group, int path) {
     std::lock_guard<std::mutex> lock(g_mu);
     if (check_weight_shape(N, K, group) != W4A16_OK || M < 1) return 1;
-    int G = K / kGroup;
+    const int G = K / kGroup, sg = kGroup / group, sms = sm_count_or_default();
+    const bool clusters = clusters_ok();
     switch (resolve_path(M, path)) {
         case W4A16_PATH_DECODE:
-            if (path == W4A16_PATH_AUTO && small_batch_takes_mid(M, N, G, sm_count_or_default(), true, kGroup / group))
-                return choose_split_tile(M, N, G, sm_count_or_default());
-            return choose_split_decode(M, N, G, sm_count_or_default());
-        case W4A16_PATH_TILE: return choose_split_tile(M, N, G, sm_count_or_default());
+            if (path == W4A16_PATH_AUTO && small_batch_takes_mid(M, N, G, sms, clusters, sg))
+                return choose_split_tile(M, N, G, sms, clusters, sg);
+            return choose_split_decode(M, N, G, sms, clusters, sg);
+        case W4A16_PATH_TILE: return choose_split_tile(M, N, G, sms, clusters, sg);
         default: return 1;
     }
 }
@@ -628,23 +667,39 @@ int w4a16_choose_split_k(int M, int N, int K, int group) {
 size_t w4a16_workspace_bytes(int M, int N, int K, int group, int split_k) {
     std::lock_guard<std::mutex> lock(g_mu);
     if (check_weight_shape(N, K, group) != W4A16_OK || M < 1 || split_k < 0 || split_k > K / kGroup) return 0;
-    // enough for whichever path w4a16_gemm / w4a16_gemm_ex may take with this split_k
-    size_t need = 0;
-    if (split_k != 1) {
-        // the schedule differs between a device that places clusters and one that refused them: cover both
-        DecodeGeom g = decode_geom(M, N, K / kGroup, split_k, sm_count_or_default(), true);
-        DecodeGeom g2 = decode_geom(M, N, K / kGroup, split_k, sm_count_or_default(), false);
-        need = decode_partial_bytes(g);
-        if (g2.split_k != 1 && decode_partial_bytes(g2) > need) need = decode_partial_bytes(g2);
-        int s = split_k == 0 ? choose_split_decode(M, N, K / kGroup, sm_count_or_default()) : split_k;
-        size_t simple = simple_partial_bytes(M, N, s);
-        if (simple > need) need = simple;
-        for (bool clusters : {true, false}) {
-            const size_t tile = wide_plan(M, N, K / kGroup, split_k, sm_count_or_default(), clusters).workspace_bytes();
-            if (tile > need) need = tile;
+    if (split_k == 1) return 0;
+    // enough for whichever path w4a16_gemm / w4a16_gemm_ex may take with this split_k, on a device that places clusters
+    // and on one that refused them (the schedule differs)
+    const int G = K / kGroup, sg = kGroup / group, sms = sm_count_or_default();
+    size_t need = simple_partial_bytes(M, N, split_k == 0 ? choose_split_decode(M, N, G, sms, true, sg) : split_k);
+    const size_t whole = decode_partial_bytes(decode_geom(M, N, G, split_k, sms, true, sg));   // (asked for by whole tiles too)
+    if (whole > need) need = whole;
+    for (bool clusters : {true, false})
+        for (int path : {W4A16_PATH_AUTO, W4A16_PATH_SIMPLE, W4A16_PATH_DECODE, W4A16_PATH_TILE}) {
+            const size_t n = gemm_plan(M, N, G, sg, split_k, path, sms, clusters).workspace;
+            if (n > need) need = n;
         }
+    return kWsFullHeaderBytes + need;
+}
+
+int w4a16_gemm_plan(int M, int N, int K, int group, int split_k, int path, w4a16_plan* out) {
+    std::lock_guard<std::mutex> lock(g_mu);
+    if (!out) return W4A16_ERR_NULL;
+    const int rc = check_weight_shape(N, K, group);
+    if (rc != W4A16_OK) return rc;
+    if (M < 1) return W4A16_ERR_SHAPE;
+    if (split_k < 0 || split_k > K / kGroup) return W4A16_ERR_SPLITK;
+    if (path < W4A16_PATH_AUTO || path > W4A16_PATH_TILE) return W4A16_ERR_PATH;
+    const GemmPlan g = gemm_plan(M, N, K / kGroup, kGroup / group, split_k, path, sm_count_or_default(), clusters_ok());
+    out->kernel = g.kernel;
+    out->workspace_bytes = g.workspace == 0 ? 0 : kWsFullHeaderBytes + g.workspace;
+    switch (g.kernel) {
+        case W4A16_KERNEL_SIMPLE: out->tile_rows = kSimpleMB; out->split_k = g.split_simple; out->cluster = 0; break;
+        case W4A16_KERNEL_DECODE: out->tile_rows = 8 * g.dec.mb; out->split_k = g.dec.split_k; out->cluster = g.dec.cluster ? 1 : 0; break;
+        case W4A16_KERNEL_TILE: out->tile_rows = g.wide.tile.mt; out->split_k = g.wide.tile.split_k; out->cluster = 0; break;
+        default: out->tile_rows = g.wide.mid.mt; out->split_k = g.wide.mid.split_k; out->cluster = g.wide.mid.cluster ? 1 : 0;
     }
-    return need == 0 ? 0 : kWsFullHeaderBytes + need;
+    return W4A16_OK;
 }
 
 int w4a16_set_workspace(void* dev_ptr, size_t bytes) {
@@ -847,9 +902,8 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
     if ((rc = current_device(&d)) != W4A16_OK) return rc;
     if (!d->is_sm100) return W4A16_ERR_ARCH;
 
-    const int path_asked = path;
-    path = resolve_path(M, path);
     if (split_k > 65535) return W4A16_ERR_SPLITK;
+    const GemmPlan plan = gemm_plan(M, N, G, sg, split_k, path, d->sm_count, d->cluster_ok);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint32_t* Zw = sym ? nullptr : static_cast<const uint32_t*>(Z);
     Epilogue epi;
@@ -859,9 +913,9 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
     unsigned char* ws_body = d->ws ? static_cast<unsigned char*>(d->ws) + kWsFullHeaderBytes : nullptr;
     const size_t ws_body_bytes = d->ws_bytes > kWsFullHeaderBytes ? d->ws_bytes - kWsFullHeaderBytes : 0;
 
-    if (path == W4A16_PATH_SIMPLE) {
-        if (split_k == 0) split_k = choose_split_decode(M, N, G, d->sm_count);
-        if (split_k > 1 && ws_body_bytes < simple_partial_bytes(M, N, split_k)) return W4A16_ERR_WORKSPACE;
+    if (plan.kernel == W4A16_KERNEL_SIMPLE) {
+        split_k = plan.split_simple;
+        if (ws_body_bytes < plan.workspace) return W4A16_ERR_WORKSPACE;
         int mchunks = (M + kSimpleMB - 1) / kSimpleMB;
         if (mchunks > 65535) return W4A16_ERR_PATH;
         float* partials = reinterpret_cast<float*>(ws_body);
@@ -885,15 +939,10 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         return W4A16_OK;
     }
 
-    WidePlan plan = {};
-    if (path_asked == W4A16_PATH_AUTO && split_k == 0 && path == W4A16_PATH_DECODE &&
-        small_batch_takes_mid(M, N, G, d->sm_count, d->cluster_ok, sg))
-        path = W4A16_PATH_TILE;
-    if (path == W4A16_PATH_TILE) plan = wide_plan(M, N, G, split_k, d->sm_count, d->cluster_ok, sg);
-    if (path == W4A16_PATH_TILE && plan.use_mid) {
-        const MidGeom& g = plan.mid;
+    if (plan.kernel == W4A16_KERNEL_MID64 || plan.kernel == W4A16_KERNEL_MID128) {
+        const MidGeom& g = plan.wide.mid;
         if (g.smem_bytes > d->max_smem_optin) return W4A16_ERR_PATH;
-        if (g.split_k != 1 && ws_body_bytes < mid_workspace_bytes(g)) return W4A16_ERR_WORKSPACE;
+        if (ws_body_bytes < plan.workspace) return W4A16_ERR_WORKSPACE;
         if ((long long)g.tiles * (g.split_k > g.mt ? g.split_k : g.mt) >= (1ll << 31)) return W4A16_ERR_SHAPE;   // (32-bit chunk arithmetic)
         CUtensorMap tmap;
         if (!make_act_tensor_map(&tmap, A, M, K, g.mt, mid_stage_k(g.mtc))) return W4A16_ERR_CUDA;
@@ -949,7 +998,7 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
             cudaGetLastError();
             if (g.cluster) {   // (see the warp-MMA kernel below)
                 d->cluster_ok = false;
-                return gemm_locked(A, Wq, S, Z, bias, C, M, N, K, group, split_k, path_asked, flags, act, stream);
+                return gemm_locked(A, Wq, S, Z, bias, C, M, N, K, group, split_k, path, flags, act, stream);
             }
             return W4A16_ERR_CUDA;
         }
@@ -958,12 +1007,10 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         return W4A16_OK;
     }
 
-    if (path == W4A16_PATH_TILE) {
-        const TileGeom& g = plan.tile;
+    if (plan.kernel == W4A16_KERNEL_TILE) {
+        const TileGeom& g = plan.wide.tile;
         if (g.smem_bytes > d->max_smem_optin) return W4A16_ERR_PATH;
-        if (g.split_k != 1) {
-            if (ws_body_bytes < tile_workspace_bytes(g)) return W4A16_ERR_WORKSPACE;
-        }
+        if (ws_body_bytes < plan.workspace) return W4A16_ERR_WORKSPACE;
         // (the kernel's chunk arithmetic is 32-bit)
         if ((long long)g.tiles * G >= (1ll << 31)) return W4A16_ERR_SHAPE;
         CUtensorMap tmap;
@@ -1018,12 +1065,11 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         return W4A16_OK;
     }
 
-    // W4A16_PATH_DECODE
-    DecodeGeom g = decode_geom(M, N, G, split_k, d->sm_count, d->cluster_ok, sg);
+    // W4A16_KERNEL_DECODE
+    const DecodeGeom& g = plan.dec;
     if (g.mchunks > 65535 || (long)g.mchunks * (N / kTileN) > kMaxTickets) return W4A16_ERR_PATH;
     if (g.smem_bytes > d->max_smem_optin) return W4A16_ERR_PATH;
-    // (the cluster exchange does not touch the workspace, but the contract stays the same for every schedule)
-    if (g.split_k != 1 && ws_body_bytes < decode_partial_bytes(g)) return W4A16_ERR_WORKSPACE;
+    if (ws_body_bytes < plan.workspace) return W4A16_ERR_WORKSPACE;
     DecodeParams p;
     p.A = A;
     p.Wq = static_cast<const uint32_t*>(Wq);
@@ -1085,7 +1131,7 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
             // the device would not place the clusters: from now on the workspace exchange (and the path
             // rule that goes with it), starting with this call
             d->cluster_ok = false;
-            return gemm_locked(A, Wq, S, Z, bias, C, M, N, K, group, split_k, path_asked, flags, act, stream);
+            return gemm_locked(A, Wq, S, Z, bias, C, M, N, K, group, split_k, path, flags, act, stream);
         }
         return W4A16_ERR_CUDA;
     }

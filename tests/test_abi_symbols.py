@@ -2,6 +2,7 @@
 arguments on the host before touching a device (no compute calls here)."""
 import ctypes
 import os
+import random
 import re
 
 import pytest
@@ -126,6 +127,28 @@ def test_path_and_schedule_rules_at_the_benchmark_shapes(lib):
     assert split(4096, 8192, 8192) == 1
     # unsupported shapes are refused, not guessed
     assert lib.w4a16_choose_path(1, 100, 4096, 128) < 0
+
+
+def test_workspace_query_covers_what_every_call_asks_for(lib):
+    """Host logic, sizes drawn over the supported range: the size that w4a16_workspace_bytes reports is enough for the
+    call on every path, whatever the group, and w4a16_choose_split_k reports the split that runs.  (The exchange buffer of a
+    cluster shares its room with scale rows, so the number of slices depends on the group.)"""
+    rng = random.Random(20)
+    shapes = [(64, 2560, 5120), (64, 3008, 5120), (51, 1024, 1536), (50, 3072, 19200), (9, 22016, 4096)]
+    for _ in range(1500):
+        shapes.append((rng.choice([1, 8, 16, 32, rng.randint(1, 64), rng.randint(49, 64), rng.randint(65, 256), rng.randint(257, 4096)]),
+                       64 * rng.randint(1, 448), 128 * rng.randint(1, 224)))
+    for M, N, K in shapes:
+        for group in (32, 64, 128):
+            for split in {0, min(2, K // 128), min(rng.randint(2, 12), K // 128), K // 128}:
+                size = lib.w4a16_workspace_bytes(M, N, K, group, split)
+                for path in (0, 1, 2, 3):
+                    p = B.w4a16_gemm_plan(M, N, K, group, split, path)
+                    assert p.workspace_bytes <= size, (M, N, K, group, split, path)
+                    if split != 0:
+                        assert p.split_k == split
+                    elif path != B.PATH_SIMPLE and p.split_k != 0:
+                        assert lib.w4a16_choose_split_k_ex(M, N, K, group, path) == p.split_k, (M, N, K, group, path)
 
 
 def test_argument_errors_are_reported_before_any_device_work(lib):
