@@ -353,8 +353,9 @@ tile_splitk_reduce_kernel(const float* __restrict__ ws, uint16_t* __restrict__ C
     }
     __syncthreads();
     const int c_first = chunks[0], c_last = chunks[1];
-    if (c_first == c_last) return;                      // one chunk has the whole tile and has written it
+    // Every CTA waits, also one without work: the launch behind this kernel counts on this grid not ending before the GEMM.
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (c_first == c_last) return;                      // one chunk has the whole tile and has written it
     const int m_local = r - T * p.mt;
     const int mt_i = fast_div(T, p.div_ntiles), nt = T - mt_i * p.n_tiles;
     const int m = mt_i * p.mt + m_local, n = nt * 128 + (int)(threadIdx.x & 31) * 4;
