@@ -213,8 +213,9 @@ int w4a16_quantize(const uint16_t *W16, uint32_t *Wq_raw, uint16_t *S_raw, uint8
  * C_host is page-locked host memory that the device can address (cudaHostAlloc /
  * cudaHostRegister, 16-byte aligned), the kernel stores the result there itself: the
  * copy is skipped and C_dev is not written.  Page-locked A_host of up to 4 MiB is copied
- * by a kernel instead of the copy engine (the whole buffer must be page-locked).  The host buffers must stay valid until the
- * stream has run them.  Weights stay resident on the device (they are the model's
+ * by a kernel instead of the copy engine.  (A host buffer that is page-locked in part goes to the copy
+ * engine, which refuses it: W4A16_ERR_CUDA.)  The host buffers must stay valid until the stream has run
+ * them.  Weights stay resident on the device (they are the model's
  * parameters, packed once). */
 int w4a16_gemm_host(const uint16_t *A_host, uint16_t *A_dev, const void *Wq, const void *S,
                     const void *Z, uint16_t *C_dev, uint16_t *C_host, int M, int N, int K,

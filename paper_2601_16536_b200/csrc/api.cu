@@ -855,6 +855,37 @@ int launch_tile_reduce(const float* parts, uint16_t* C, int M, int N, int G, int
 
 constexpr size_t kStageMaxBytes = 4u << 20;   // (w4a16_gemm_host)
 
+// Can kernels reach all `bytes` of this host memory, by the same address?  Not if it is pageable, or page-locked in part: a
+// copy call then deals with it or refuses it.  The driver tells the extent of one registration, so neighbouring ones are
+// walked; 50 ns each.
+bool device_reaches(const void* host, size_t bytes) {
+    typedef CUresult (*GetAttributesFn)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+    static const GetAttributesFn get = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult qr;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &f, cudaEnableDefault, &qr) != cudaSuccess || qr != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<GetAttributesFn>(f);
+    }();
+    if (get == nullptr || !aligned16(host)) return false;
+    CUdeviceptr at = reinterpret_cast<CUdeviceptr>(host);
+    const CUdeviceptr end = at + bytes;
+    while (at < end) {
+        unsigned int type = 0, managed = 0;
+        CUdeviceptr dev = 0, start = 0;
+        size_t size = 0;
+        CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                      CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+        void* out[] = {&type, &managed, &dev, &start, &size};
+        if (get(5, what, out, at) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || managed != 0 || dev != at || start > at || start + size <= at)
+            return false;
+        at = start + size;
+    }
+    return true;
+}
+
 int stage_activations(const void* host, void* dev, int n16, cudaStream_t st) {
     std::lock_guard<std::mutex> lock(g_mu);
     DeviceState* d = nullptr;
@@ -1171,25 +1202,16 @@ int w4a16_gemm_host(const uint16_t* A_host, uint16_t* A_dev, const void* Wq, con
     // engine and SMs.  Anything else goes through the staging buffers and the copy engine; so do activations of more than
     // kStageMaxBytes.  us a call on one stream, K = 11008 / N = 4096, copy engine / kernel: M = 1 25.4 / 17.7, 8 34.9 / 22.4,
     // 64 68 / 55, 190 143 / 138, 256 182 / 182: bound by PCIe there, so the SMs are left alone.
-    auto addressable = [](const void* p) -> void* {
-        cudaPointerAttributes attr;
-        if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        return attr.type == cudaMemoryTypeHost && attr.devicePointer != nullptr && aligned16(attr.devicePointer) ? attr.devicePointer : nullptr;
-    };
     const size_t a_bytes = (size_t)M * K * 2;
-    const void* a_direct = a_bytes <= kStageMaxBytes && a_bytes % 16 == 0 && aligned16(A_dev) ? addressable(A_host) : nullptr;
-    if (a_direct != nullptr) {
-        const int rc = stage_activations(a_direct, A_dev, (int)(a_bytes / 16), st);
+    if (a_bytes <= kStageMaxBytes && a_bytes % 16 == 0 && aligned16(A_dev) && device_reaches(A_host, a_bytes)) {
+        const int rc = stage_activations(A_host, A_dev, (int)(a_bytes / 16), st);
         if (rc != W4A16_OK) return rc;
     } else if (cudaMemcpyAsync(A_dev, A_host, a_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess) {
         cudaGetLastError();
         return W4A16_ERR_CUDA;
     }
-    uint16_t* const c_direct = static_cast<uint16_t*>(addressable(C_host));
-    int rc = w4a16_gemm(A_dev, Wq, S, Z, c_direct ? c_direct : C_dev, M, N, K, group, split_k, stream);
+    const bool c_direct = device_reaches(C_host, (size_t)M * N * 2);
+    int rc = w4a16_gemm(A_dev, Wq, S, Z, c_direct ? C_host : C_dev, M, N, K, group, split_k, stream);
     if (rc != W4A16_OK) return rc;
     if (!c_direct && cudaMemcpyAsync(C_host, C_dev, (size_t)M * N * 2, cudaMemcpyDeviceToHost, st) != cudaSuccess) {
         cudaGetLastError();

@@ -5,6 +5,8 @@ finished (programmatic dependent launch), so the library has to order the first 
 after a w4a16_pack enqueued on that stream.  The status path (a bounded wait that runs out) is
 exercised with the library's diagnostic kernel: nothing faults, the context stays usable.
 """
+import mmap
+
 import numpy as np
 import pytest
 import torch
@@ -100,6 +102,49 @@ def test_host_buffer_calls_are_ordered_on_their_stream(M, K, N):
         assert np.array_equal(out.numpy().view(np.uint16), c_bits(B.w4a16_gemm(host.cuda(), pw)))
     if K == N:
         assert np.array_equal(outs[2].numpy().view(np.uint16), c_bits(B.w4a16_gemm(outs[1].cuda(), pw)))
+    del ws
+
+
+@pytest.mark.parametrize("which", ["A", "C"])
+def test_host_buffer_that_is_page_locked_in_part_is_refused(which):
+    """Only the first page of the buffer is registered: no kernel may touch it by its address.  The copy engine refuses such
+    a buffer; with its second part registered too, every byte is reachable and the call works."""
+    M, K, N = 4, 1152, 1088                      # 9,216 and 8,704 bytes: three pages each
+    d = wl.make_problem(M, K, N, seed=3400)
+    pw = pack_problem(d, N, K)
+    A = to_dev(d["A"])
+    ws = ensure_ws(M, N, K, 0)
+    want = c_bits(B.w4a16_gemm(A, pw)).copy()
+    page = mmap.PAGESIZE
+    memory = mmap.mmap(-1, 3 * page)
+    cols, bits = (K, d["A"]) if which == "A" else (N, None)
+    buf = torch.frombuffer(memory, dtype=torch.float16)[:M * cols].view(M, cols)
+    A_host = torch.from_numpy(d["A"].view(np.float16)).pin_memory()
+    C_host = torch.zeros((M, N), dtype=torch.float16).pin_memory()
+    if bits is not None:
+        buf.copy_(A_host)
+        A_host = buf
+    else:
+        C_host = buf
+    A_dev, C_dev = torch.empty((M, K), dtype=torch.float16, device="cuda"), torch.empty((M, N), dtype=torch.float16, device="cuda")
+    rt, base = torch.cuda.cudart(), buf.data_ptr()
+    assert base % page == 0
+    assert int(rt.cudaHostRegister(base, page, 0)) == 0
+    try:
+        with pytest.raises(B.W4A16Error) as e:
+            B.w4a16_gemm_host(A_host, A_dev, pw, C_dev, C_host)
+        assert e.value.code == -6
+        torch.cuda.synchronize()
+        assert int(rt.cudaHostRegister(base + page, 2 * page, 0)) == 0
+        try:
+            B.w4a16_gemm_host(A_host, A_dev, pw, C_dev, C_host)
+            torch.cuda.synchronize()
+            assert B.w4a16_device_status() == 0
+            assert np.array_equal(C_host.numpy().view(np.uint16), want)
+        finally:
+            rt.cudaHostUnregister(base + page)
+    finally:
+        rt.cudaHostUnregister(base)
     del ws
 
 
