@@ -157,8 +157,11 @@ int w4a16_dequant(const void *Wq, const void *S, const void *Z, uint16_t *W16,
  *             and return W4A16_ERR_SPLITK beyond their cap)
  * Results are bit-identical from run to run for fixed arguments (with split_k == 0 the schedule,
  * and with it the order of the FP32 sums, is the library's choice for this entry point and device;
- * it changes once, for good, if the device refuses a thread-block-cluster launch).  If the chosen
- * split needs workspace and too little is registered: W4A16_ERR_WORKSPACE.
+ * it changes once, for good, if the device refuses a thread-block-cluster launch, and it depends
+ * on whether the registered workspace is large enough).  If the chosen split needs workspace and too
+ * little is registered: W4A16_ERR_WORKSPACE; with split_k == 0 that is where the library's choice is
+ * K slices that meet in the workspace (slices that meet in a cluster need none, and chunks that
+ * cross tile boundaries give way to whole tiles).
  * Ordering: A, C and the workspace are touched in stream order.  The packed buffers Wq, S, Z
  * may be read (prefetched) while the previous kernel of the stream is still running, so
  * they must not be written by in-flight work other than a w4a16_pack enqueued earlier on the

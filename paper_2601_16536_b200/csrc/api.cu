@@ -5,6 +5,7 @@
 
 #include <cuda_runtime.h>
 
+#include <stdint.h>
 #include <string.h>
 
 #include <mutex>
@@ -567,6 +568,11 @@ size_t decode_partial_bytes(const DecodeGeom& g) {
     return round256((size_t)g.mchunks * 2 * (size_t)g.nchunks * (8 * g.mb) * kTileN * sizeof(float));
 }
 
+// Workspace that the warp-MMA kernel's schedule asks for, given the caller's split_k.
+size_t decode_scratch(const DecodeGeom& g, int split_k) {
+    return g.split_k == 1 || (split_k == 0 && g.cluster) ? 0 : decode_partial_bytes(g);
+}
+
 // What a GEMM call runs: kernel, schedule and the workspace behind the header that it asks for (0: none).  The entry points
 // and the queries all come here, with the group's scale rows per block (sg): whether a cluster's exchange buffer fits, and
 // with it the number of slices, depends on them.
@@ -577,7 +583,9 @@ struct GemmPlan {
     WidePlan wide;
     size_t workspace;
 };
-GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, int sms, bool allow_cluster) {
+// An explicit split_k > 1 asks for its workspace on every kernel, used or not.  With split_k == 0 slices that meet in a cluster
+// ask for none, and balanced chunks, which cross tile boundaries, give way to whole tiles where `ws_bytes` does not hold them.
+GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, int sms, bool allow_cluster, size_t ws_bytes = SIZE_MAX) {
     GemmPlan p;
     int path = resolve_path(M, path_asked);
     if (path_asked == W4A16_PATH_AUTO && split_k == 0 && path == W4A16_PATH_DECODE &&
@@ -590,12 +598,19 @@ GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, int
     } else if (path == W4A16_PATH_DECODE) {
         p.kernel = W4A16_KERNEL_DECODE;
         p.dec = decode_geom(M, N, G, split_k, sms, allow_cluster, sg);
-        // (the cluster exchange does not touch the workspace, but the contract stays the same for every schedule)
-        p.workspace = p.dec.split_k != 1 ? decode_partial_bytes(p.dec) : 0;
+        p.workspace = decode_scratch(p.dec, split_k);
+        if (p.workspace > ws_bytes && p.dec.split_k == 0) {
+            p.dec = decode_geom(M, N, G, 1, sms, allow_cluster, sg);
+            p.workspace = 0;
+        }
     } else {
         p.wide = wide_plan(M, N, G, split_k, sms, allow_cluster, sg);
         p.kernel = !p.wide.use_mid ? W4A16_KERNEL_TILE : p.wide.mid.mtc <= 64 ? W4A16_KERNEL_MID64 : W4A16_KERNEL_MID128;
-        p.workspace = p.wide.workspace_bytes();
+        p.workspace = split_k == 0 && p.wide.use_mid && p.wide.mid.cluster ? 0 : p.wide.workspace_bytes();
+        if (p.workspace > ws_bytes && !p.wide.use_mid && p.wide.tile.split_k == 0) {
+            p.wide.tile = tile_geom(M, N, G, 1, sms);
+            p.workspace = 0;
+        }
     }
     return p;
 }
@@ -934,16 +949,15 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
     if (!d->is_sm100) return W4A16_ERR_ARCH;
 
     if (split_k > 65535) return W4A16_ERR_SPLITK;
-    const GemmPlan plan = gemm_plan(M, N, G, sg, split_k, path, d->sm_count, d->cluster_ok);
+    // registered workspace: [small-M tickets and reserve: the documented header][partial results]
+    unsigned char* ws_body = d->ws ? static_cast<unsigned char*>(d->ws) + kWsFullHeaderBytes : nullptr;
+    const size_t ws_body_bytes = d->ws_bytes > kWsFullHeaderBytes ? d->ws_bytes - kWsFullHeaderBytes : 0;
+    const GemmPlan plan = gemm_plan(M, N, G, sg, split_k, path, d->sm_count, d->cluster_ok, ws_body_bytes);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint32_t* Zw = sym ? nullptr : static_cast<const uint32_t*>(Z);
     Epilogue epi;
     epi.bias = bias;
     epi.act = act;
-    // registered workspace: [small-M tickets and reserve: the documented header][partial results]
-    unsigned char* ws_body = d->ws ? static_cast<unsigned char*>(d->ws) + kWsFullHeaderBytes : nullptr;
-    const size_t ws_body_bytes = d->ws_bytes > kWsFullHeaderBytes ? d->ws_bytes - kWsFullHeaderBytes : 0;
-
     if (plan.kernel == W4A16_KERNEL_SIMPLE) {
         split_k = plan.split_simple;
         if (ws_body_bytes < plan.workspace) return W4A16_ERR_WORKSPACE;
@@ -1236,7 +1250,10 @@ int w4a16_gemm_static_ws(const uint16_t* A, const void* Wq, const void* S, const
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return W4A16_ERR_CUDA;
 
-    const DecodeGeom g = decode_geom(M, N, G, split_k, d->sm_count, false, sg);   // no clusters here: this entry point keeps the path it was built with
+    DecodeGeom g = decode_geom(M, N, G, split_k, d->sm_count, false, sg);   // no clusters here: this entry point keeps the path it was built with
+    // (balanced chunks give way to whole tiles, as in gemm_plan)
+    if (g.split_k == 0 && kWsHeaderBytes + decode_partial_bytes(g) > (size_t)W4A16_STATIC_WS_BYTES)
+        g = decode_geom(M, N, G, 1, d->sm_count, false, sg);
     if (g.mchunks > 65535 || (long)g.mchunks * (N / kTileN) > kMaxTickets) return W4A16_ERR_PATH;
     if (g.smem_bytes > d->max_smem_optin) return W4A16_ERR_PATH;
     // the whole scratch need of this shape must fit the built-in array, or nothing is launched (a schedule of

@@ -125,6 +125,40 @@ def test_workspace_errors():
     torch.cuda.synchronize()
 
 
+# Schedules that the library picks itself where whole tiles would leave SMs idle: slices that meet in a cluster (each kernel)
+# never touch the workspace; balanced chunks give way to whole tiles when there is none.
+@pytest.mark.parametrize("M,K,N,kernel,cluster", [
+    (4, 1792, 8576, B.KERNEL_DECODE, 1), (16, 4096, 12288, B.KERNEL_MID64, 1), (32, 1280, 12288, B.KERNEL_MID64, 1),
+    (65, 5632, 6464, B.KERNEL_MID128, 1), (129, 6016, 9984, B.KERNEL_TILE, 0)])
+def test_automatic_schedules_without_a_workspace(M, K, N, kernel, cluster):
+    plan = B.w4a16_gemm_plan(M, N, K)
+    assert (plan.kernel, plan.cluster) == (kernel, cluster) and (cluster or plan.split_k == 0)
+    d = wl.make_exact_problem(M, K, N, seed=4100 + M)
+    n0 = N - 128
+    want = oracle.gemm_int(d["A_int"], d["Wq"][:, n0:].copy(), d["E"][:, n0:].copy(), d["Z"][:, n0:].copy(), M, 128, K, 128)
+    pw = pack_problem(d, N, K)
+    B.w4a16_set_workspace(None)
+    C = B.w4a16_gemm(to_dev(d["A"]), pw)
+    torch.cuda.synchronize()
+    assert B.w4a16_device_status() == 0
+    assert np.array_equal(c_bits(C)[:, n0:], want)
+    ws = ensure_ws(M, N, K, 0)
+    assert torch.equal(C, B.w4a16_gemm(to_dev(d["A"]), pw))     # (exact inputs: the same bits from every schedule)
+    del ws
+
+
+def test_static_scratch_schedule_gives_way_to_whole_tiles():
+    # 24 rows, 139 column tiles: balanced chunks would need more than the built-in array
+    M, K, N = 24, 3584, 8896
+    d = wl.make_exact_problem(M, K, N, seed=4200)
+    pw = pack_problem(d, N, K)
+    A = to_dev(d["A"])
+    C = B.w4a16_gemm_static_ws(A, pw)
+    torch.cuda.synchronize()
+    assert B.w4a16_device_status() == 0
+    assert torch.equal(C, B.w4a16_gemm_static_ws(A, pw, split_k=1))
+
+
 # Host result buffer: page-locked memory takes the kernel's stores directly (the device staging buffer is then
 # left alone), ordinary pageable memory gets the result through the staging buffer and a copy.  Both on the
 # warp-MMA kernel (M = 8) and the tcgen05 kernel (M = 40).
