@@ -168,35 +168,51 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, int sms, bool allow_clu
         // clusters run at once: a second wave doubles the time), through the workspace at the end of the stream otherwise.
         // Costs in ns: a unit takes a CTA 288 with 8 rows and 330 with 16 (two CTAs on some SM set the pace whatever the
         // count: 64 units of 134 whole tiles 17.8 us, of 160 18.6), the rest is what a launch shows beside its units; 500
-        // more with nine tenths of the slots taken, because then the next launch cannot start before this one ends.
+        // more with nine tenths of the slots taken, because then the next launch cannot start before this one ends; 80 per four
+        // rows for every chunk of a tile that the last one to arrive adds (16 rows, four tiles of K = 7296 in 8 / 16 / 24 / 57
+        // slices: 7.9 / 9.8 / 13.5 / 23.6 us, six in a cluster 5.0).
         // us, measured: K = 8192 / N = 8576 two slices 11.3, whole tiles 17.8, balanced 14.9; N = 10240 (320 slices do not
         // fit) balanced 16.5, whole 18.6; K = 4096 / N = 12288 whole 10.2, balanced 12.1; K = 11008 / N = 4096 four slices
         // 8.6, three 10.5; K = 23168 / N = 4416 four 15.0, three 18.0; K = 6144 / N = 1536 six in a cluster 4.3, twelve
         // through the workspace 6.5; K = 28672 / N = 8192 two 31.2, balanced 32.4; K = 4096 / N = 22016 (344 whole tiles on
         // 296 CTAs, whose pairs share the SM's issue slots: 15 % over the mean) 14.4, balanced 18.4.
-        const long unit_ns = g.mb == 1 ? 288 : 330, wide = g.mb == 1 ? 0 : 700;
+        const long unit_ns = g.mb == 1 ? 288 : 330, wide = g.mb == 1 ? 0 : 700, add_ns = ((M < 8 * g.mb ? M : 8 * g.mb) + 3) / 4 * 80;
         const int* max_clusters = mid_max_clusters();      // (two CTAs per SM, like that kernel)
         auto take = [&](int s, long cost) {
             if (g.cost == 0 || cost < g.cost) { g.cost = cost; split_k = s; }
         };
         take(1, 1500 + wide + unit_ns * (T > slots ? (units * 23 / 20 + slots - 1) / slots : (long)G));
         if (allow_cluster && g.mchunks == 1) {
-            // Clusters of 3 and 5 (and 6, a little) fit the SMs that the launch in front leaves free badly: with most slots
-            // taken a short launch waits for a place (K = 8192, 86 .. 91 tiles in three slices 13 to 14 us, in two 11.0; 52
-            // in five 9.9, in four 7.2; 43 in six 6.8, in five 6.5), a long one hardly (K = 21760, 86 tiles in three 18.0,
-            // balanced 20.5; but 90 in three 22.4, balanced 21.0).  Two and four keep their time up to the last tile that fits (69 tiles in four 7.9, in three 8.7).
+            // The last clusters that fit find a place late, while the launch in front still holds its SMs: from 7/8 or 8/9 of them
+            // on with 5 or 3 CTAs (us, M = 8, K = 7296: 48 / 49 / 50 / 52 tiles in five 5.8 / 6.2 / 8.5 / 9.2, in four 6.7; 82 / 84 /
+            // 86 / 90 in three 8.1 / 8.6 / 11.5 / 12.8, in two 9.8), a few tiles before the end with 4 and 6 (K = 2048: 66 / 68 /
+            // 69 / 70 in four 4.0 / 4.4 / 4.9 / 5.1, in two 4.2; 41 / 42 / 43 / 44 in six 3.8 / 4.0 / 4.4 / 4.8, in five 3.5), not
+            // with 2.  A long launch hardly notices (K = 28672: 50 in five 14.9; K = 10880: 42 in six 7.0, in five 7.7).  Of equal
+            // slices the even count is ahead (20 tiles of K = 3200, M = 16: 4.4 in six, 4.9 in five).
             for (int s = 2; s <= kDecMaxCluster && s <= G; ++s) {
-                if (T + 2 > max_clusters[s]) continue;
+                const int room = max_clusters[s];
+                if (T + 2 > room) continue;
                 const long u = (G + s - 1) / s, ctas = (long)T * s;
-                long wait = s % 2 != 0 && ctas * 37 > slots * 30 ? 5000 - 60 * u : s == 6 && ctas * 37 > slots * 32 ? 1250 - 15 * u : 0;
+                long wait = 0;
+                if (s == 3 || s == 5) {
+                    const int over = s == 3 ? T - room * 8 / 9 : T - room * 7 / 8;
+                    if (over >= 0 && s == 5) wait = over == 0 ? 800 - 40 * u : 2000L * over;
+                    if (over >= 0 && s == 3) wait = g.mb == 1 ? 960L * over - 450 : 1500L * (over + 1);   // (M = 16, K = 4096: 80 tiles 6.9, 82 9.8)
+                    if (wait > 5000 - 60 * u) wait = 5000 - 60 * u;
+                    if (10 * ctas > 9 * slots && wait < 3500) wait = 3500;
+                } else if (s == 4 || s == 6) {
+                    const int over = T + 4 - room;
+                    if (over > 0) wait = s == 4 ? 500 * over - 15 * u : 700 * over - 45 * u;
+                }
                 if (wait < 0) wait = 0;
-                if (s % 2 != 0 && 10 * ctas > 9 * slots && wait < 3500) wait = 3500;
-                take(s, (s == 2 ? 1700 : 2150) + wide * 7 / 4 + unit_ns * u + (10 * ctas > 9 * slots ? 500 : 0) + wait);
+                take(s, (s == 2 ? 1700 : 2150) + (s % 2 != 0 && u > 3 ? 150 : 0) + wide * 7 / 4 + unit_ns * u + (10 * ctas > 9 * slots ? 500 : 0) + wait);
             }
         }
         const int s0 = (int)(slots * 7 / 8 / T < G ? slots * 7 / 8 / T : G);
-        if (s0 > kDecMaxCluster || (s0 >= 2 && !(allow_cluster && g.mchunks == 1))) take(s0, 4200 + wide + unit_ns * ((G + s0 - 1) / s0));
-        take(0, 5700 + wide + unit_ns * ((units * 27 / 25 + slots - 1) / slots));
+        if (s0 > kDecMaxCluster || (s0 >= 2 && !(allow_cluster && g.mchunks == 1)))
+            take(s0, 4000 + wide + add_ns * s0 + unit_ns * ((G + s0 - 1) / s0));
+        const long share = slots / T > 3 ? slots / T - 3 : 0;      // (contributors of a tile, beyond what the constant holds)
+        take(0, 5700 + wide + add_ns * share + unit_ns * ((units * 27 / 25 + slots - 1) / slots));
     }
     g.split_k = split_k;
     if (split_k == 0) {

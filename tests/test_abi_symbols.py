@@ -151,6 +151,16 @@ def test_workspace_query_covers_what_every_call_asks_for(lib):
                         assert lib.w4a16_choose_split_k_ex(M, N, K, group, path) == p.split_k, (M, N, K, group, path)
 
 
+def test_slices_of_few_column_tiles_meet_in_a_cluster(lib):
+    """Up to 16 rows and few column tiles: the sum through the workspace costs time for every slice and every row, so many
+    slices are not taken because each is short (us, six in a cluster / the slices named): M = 10, K = 4480 4.6 / 35 14.1;
+    M = 11, K = 6016 5.4 / 18 10.7; M = 16, K = 5632 6.2 / 15 11.6.  With one row and a long K they are ahead."""
+    for M, N, K, group in [(10, 384, 4480, 32), (10, 384, 4224, 64), (11, 896, 6016, 128), (9, 768, 5888, 32), (16, 1088, 5632, 32)]:
+        p = B.w4a16_gemm_plan(M, N, K, group, 0, B.PATH_DECODE)
+        assert (p.split_k, p.cluster) == (6, 1), (M, N, K, group)
+    assert B.w4a16_gemm_plan(2, 640, 19072, 64).split_k == 25        # 7.9 us; six in a cluster 9.3
+
+
 def test_argument_errors_are_reported_before_any_device_work(lib):
     buf = (ctypes.c_uint8 * 4096)()
     p = ctypes.addressof(buf)
