@@ -115,8 +115,8 @@ int w4a16_choose_split_k_ex(int M, int N, int K, int group, int path);
  * kernel; forcing the path forces the kernel.) */
 int w4a16_choose_path(int M, int N, int K, int group);
 
-/* What w4a16_gemm_ex runs for these arguments on the current device (on a host without one: what a B200 would run).
- * For tests, benchmarks and logs; returns W4A16_OK or the error that the call itself would return for these arguments. */
+/* What w4a16_gemm_fmt runs for these arguments on the current device (on a host without one: what a B200 would run),
+ * without a bias and an activation or (with_epilogue != 0) with either.  For tests, benchmarks and logs; returns W4A16_OK or the error that the call itself would return for these arguments. */
 enum {
     W4A16_KERNEL_SIMPLE = 1, /* plain FP32-FMA kernel */
     W4A16_KERNEL_DECODE = 2, /* warp-MMA kernel */
@@ -131,7 +131,7 @@ typedef struct {
     int cluster;            /* 1: the slices of a tile meet in a thread-block cluster */
     size_t workspace_bytes; /* workspace that has to be registered for the call; 0 = none */
 } w4a16_plan;
-int w4a16_gemm_plan(int M, int N, int K, int group, int split_k, int path, w4a16_plan *out);
+int w4a16_gemm_plan(int M, int N, int K, int group, int split_k, int path, int with_epilogue, w4a16_plan *out);
 
 /* Offline reorder of the raw nibbles, scales and zero points into the packed layout
  * (pure data movement, a bijection; Section 2.2 storage packing).  Reads the three raw

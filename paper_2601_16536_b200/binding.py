@@ -74,7 +74,7 @@ def load():
     L.w4a16_choose_path.restype = i
     L.w4a16_choose_path.argtypes = [i, i, i, i]
     L.w4a16_gemm_plan.restype = i
-    L.w4a16_gemm_plan.argtypes = [i, i, i, i, i, i, ctypes.POINTER(Plan)]
+    L.w4a16_gemm_plan.argtypes = [i, i, i, i, i, i, i, ctypes.POINTER(Plan)]
     L.w4a16_choose_split_k_ex.restype = i
     L.w4a16_choose_split_k_ex.argtypes = [i, i, i, i, i]
     L.w4a16_pack.restype = i
@@ -151,10 +151,12 @@ def w4a16_choose_path(M: int, N: int, K: int, group: int = GROUP) -> int:
     return load().w4a16_choose_path(M, N, K, group)
 
 
-def w4a16_gemm_plan(M: int, N: int, K: int, group: int = GROUP, split_k: int = 0, path: int = PATH_AUTO) -> Plan:
-    """What ``w4a16_gemm`` runs for these arguments on the current device (a B200 where there is none)."""
+def w4a16_gemm_plan(M: int, N: int, K: int, group: int = GROUP, split_k: int = 0, path: int = PATH_AUTO,
+                    with_epilogue: bool = False) -> Plan:
+    """What ``w4a16_gemm`` runs for these arguments on the current device (a B200 where there is none), without or with a
+    bias or an activation."""
     p = Plan()
-    _check(load().w4a16_gemm_plan(M, N, K, group, split_k, path, ctypes.byref(p)), "w4a16_gemm_plan")
+    _check(load().w4a16_gemm_plan(M, N, K, group, split_k, path, int(with_epilogue), ctypes.byref(p)), "w4a16_gemm_plan")
     return p
 
 

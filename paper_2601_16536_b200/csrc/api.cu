@@ -5,6 +5,7 @@
 
 #include <cuda_runtime.h>
 
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -175,13 +176,14 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, int sms, bool allow_clu
         // fit) balanced 16.5, whole 18.6; K = 4096 / N = 12288 whole 10.2, balanced 12.1; K = 11008 / N = 4096 four slices
         // 8.6, three 10.5; K = 23168 / N = 4416 four 15.0, three 18.0; K = 6144 / N = 1536 six in a cluster 4.3, twelve
         // through the workspace 6.5; K = 28672 / N = 8192 two 31.2, balanced 32.4; K = 4096 / N = 22016 (344 whole tiles on
-        // 296 CTAs, whose pairs share the SM's issue slots: 15 % over the mean) 14.4, balanced 18.4.
+        // 296 CTAs, whose pairs share the SM's issue slots: 15 % over the mean, with 16 rows 30) 14.4, balanced 18.4.
         const long unit_ns = g.mb == 1 ? 288 : 330, wide = g.mb == 1 ? 0 : 700, add_ns = ((M < 8 * g.mb ? M : 8 * g.mb) + 3) / 4 * 80;
         const int* max_clusters = mid_max_clusters();      // (two CTAs per SM, like that kernel)
         auto take = [&](int s, long cost) {
             if (g.cost == 0 || cost < g.cost) { g.cost = cost; split_k = s; }
         };
-        take(1, 1500 + wide + unit_ns * (T > slots ? (units * 23 / 20 + slots - 1) / slots : (long)G));
+        if (T > slots) take(1, g.mb == 1 ? 1500 + unit_ns * ((units * 23 / 20 + slots - 1) / slots) : 4000 + unit_ns * units * 13 / (10 * slots));
+        else take(1, 1500 + wide + unit_ns * G);
         if (allow_cluster && g.mchunks == 1) {
             // The last clusters that fit find a place late, while the launch in front still holds its SMs: from 7/8 or 8/9 of them
             // on with 5 or 3 CTAs (us, M = 8, K = 7296: 48 / 49 / 50 / 52 tiles in five 5.8 / 6.2 / 8.5 / 9.2, in four 6.7; 82 / 84 /
@@ -197,7 +199,7 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, int sms, bool allow_clu
                 if (s == 3 || s == 5) {
                     const int over = s == 3 ? T - room * 8 / 9 : T - room * 7 / 8;
                     if (over >= 0 && s == 5) wait = over == 0 ? 800 - 40 * u : 2000L * over;
-                    if (over >= 0 && s == 3) wait = g.mb == 1 ? 960L * over - 450 : 1500L * (over + 1);   // (M = 16, K = 4096: 80 tiles 6.9, 82 9.8)
+                    if (over >= (g.mb == 1 ? 0 : -1) && s == 3) wait = g.mb == 1 ? 960L * over - 450 : 1500L * (over + 2);   // (M = 16, K = 4096: 80 tiles 6.9, 82 9.8)
                     if (wait > 5000 - 60 * u) wait = 5000 - 60 * u;
                     if (10 * ctas > 9 * slots && wait < 3500) wait = 3500;
                 } else if (s == 4 || s == 6) {
@@ -212,7 +214,7 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, int sms, bool allow_clu
         if (s0 > kDecMaxCluster || (s0 >= 2 && !(allow_cluster && g.mchunks == 1)))
             take(s0, 4000 + wide + add_ns * s0 + unit_ns * ((G + s0 - 1) / s0));
         const long share = slots / T > 3 ? slots / T - 3 : 0;      // (contributors of a tile, beyond what the constant holds)
-        take(0, 5700 + wide + add_ns * share + unit_ns * ((units * 27 / 25 + slots - 1) / slots));
+        take(0, (g.mb == 1 ? 5700 : 7500) + add_ns * share + unit_ns * ((units * 27 / 25 + slots - 1) / slots));
     }
     g.split_k = split_k;
     if (split_k == 0) {
@@ -281,40 +283,60 @@ constexpr size_t kWsFullHeaderBytes = W4A16_WORKSPACE_HEADER_BYTES;   // (the sm
 // (148 whole tiles of K = 16384, 208 rows: eight slots 120 us, six 100; 256 rows have six either way).
 constexpr int kTileSmem = 200 * 1024;
 
-// What a launch costs, in ns, and how its units are cut.  A unit takes 400 + 1.85 mt ns with every SM busy (148 whole tiles
-// of K = 16384: 80 rows 74 us, 128 83, 160 90, 208 100, 256 111), 40 % less with few (the L2 that brings the activations is
-// what they share), a launch 3.5 us beside its units, K slices 4 us more for the partial tiles and the kernel that sums them.
+// What the host needs to issue a GEMM and the kernel that sums its slices, in ns: no shorter schedule is worth them.
+constexpr long kTwoLaunches = 6300;
+
+// What a launch costs, in ns, and how its units are cut.  Here and below the constants are least-squares fits of the relative
+// error to calls timed back to back, 12,700 schedules of 840 shapes drawn over M = 17 to 1500 (FP16, groups of 128): 3 to 6 %
+// off; the schedules they choose take 1.4 % longer than the best ones timed.  A unit takes a CTA 0.50 us with 80 rows and 0.57 with
+// 256 while few SMs are busy (the ring's hand-offs) and up to 0.79 with all of them (the L2 that brings the activations); the
+// rest is what a launch shows beside its units, the epilogue's rows among it, and for slices the second kernel, the partial
+// tiles and 79 ns for every slice that it adds.
 TileGeom tile_geom_rows(int mt, int M, int N, int G, int split_k, int sms) {
     TileGeom g;
     g.mt = mt;
     g.m_tiles = (M + mt - 1) / mt;
     g.n_tiles = (N + kTileCols - 1) / kTileCols;
     g.tiles = (long)g.m_tiles * g.n_tiles;
-    const long unit_ns = 400 + mt * 37 / 20;
     g.cost = 0;
     if (split_k == 0) {
         // Balanced chunks use every SM to the end, but a chunk that starts or ends inside a tile leaves an FP32 partial tile
-        // behind, whose store stalls the pipeline in mid-stream: 12 us in all, 17.5 where chunks span two tiles, and never from two
-        // waves on (the CTAs no longer read the same activations at the same time: M = 2787, K = 4224 / N = 13824 319 us, in
-        // waves 290).  S
-        // slices per tile (tiles <= SMs) or whole tiles in waves (tiles > SMs) avoid that at the price of idle SMs.
+        // behind, whose store stalls the pipeline in mid-stream; dearer from two waves on (the CTAs no longer read the same
+        // activations at the same time) and never from three (M = 2787, K = 4224 / N = 13824 319 us, in waves 290; but 2.2 waves of
+        // 256 rows, M = 1454, K = 13056 / N = 6912 205 us, in waves 240).  S slices per tile (tiles <= SMs)
+        // or whole tiles in waves (tiles > SMs) avoid that at the price of idle SMs.
         // us, slices or waves / balanced: M = 256: K = 16384 / N = 4096 30.5 / 32.1, K = N = 8192 29.6 / 32.0; M = 600, K = N =
         // 8192 83.3 / 82.7; M = 777, K = 4096 / N = 22016 119 / 140; M = 1024, K = N = 8192 99 / 112; M = 256, K = 8192 /
         // N = 20480 (160 tiles) 86.5 / 78.8.
-        auto busy = [&](long ctas, long u) { return u * unit_ns * (6 * sms + 4 * ctas) / (10 * sms); };
-        const long balanced = (g.tiles * G + sms - 1) / sms * unit_ns + (g.tiles <= sms ? 12000 : 17500);
-        int s0 = 1;
-        long classic;
+        auto take = [&](int s, long cost) {
+            if (g.cost == 0 || cost < g.cost) { g.cost = cost; split_k = s; }
+        };
+        const long balanced = (g.tiles * G + sms - 1) / sms;
+        // percent; activations of half the L2 and more do not stay in it when the CTAs read different parts of them (M = 2509,
+        // K = 22144 / N = 3392, 111 MB: 370 us, in waves 290)
+        const int dearer = ((long)M * G * (2 * kGroup) > (56l << 20) ? 113 : 100) * (g.tiles < 2 * sms ? 100 : 113) / 100;
         if (g.tiles <= sms) {
-            s0 = sms / (int)g.tiles;
-            if (s0 > G) s0 = G;
-            classic = busy(g.tiles * s0, (G + s0 - 1) / s0) + (s0 > 1 ? 7500 : 3500);
+            const int tiles = (int)g.tiles;
+            take(1, 1965 + 12 * mt + tiles * 149 / 20 + (long)G * (476 + mt * (400 + 3 * tiles) / 1000));
+            auto slices = [&](int s) {
+                const int ctas = tiles * s, above = ctas > 48 ? ctas - 48 : 0;
+                const long cost = 3800 + 8 * mt + ctas * (440 + 62 * mt / 10) / 100 + 79 * s +
+                                  (G + s - 1) / s * (451L + mt * 6 / 10 + above * (31 + mt * 4 / 10) / 100);
+                take(s, cost > kTwoLaunches ? cost : kTwoLaunches);
+            };
+            // as many as there are SMs, or as many as pay for being added
+            const int most = sms / tiles < G ? sms / tiles : G;
+            if (most >= 2) slices(most);
+            if (most > 2) {
+                const int s = (int)(sqrtf((float)G * (451 + mt * 6 / 10) / (79 + tiles * (440 + 62 * mt / 10) / 100)) + 0.5f);
+                if (s >= 2 && s < most) slices(s);
+            }
+            if (8 * tiles >= sms) take(0, (6000 + 26 * mt + balanced * (466 + mt * 11 / 10)) * dearer / 100);     // (fewer: slices do as well)
         } else {
-            classic = busy(sms, g.tiles / sms * G) + (g.tiles % sms != 0 ? busy(g.tiles % sms, G) : 0) + 3500;
+            const long waves = (g.tiles + sms - 1) / sms;
+            take(1, 1350 - mt + waves * (981 + 10 * mt) + waves * G * (398 + mt / 2) + g.tiles * G / sms * (96 + mt * 4 / 10));
+            if (g.tiles < 3 * sms) take(0, (5540 + 61 * mt + balanced * (459 + mt)) * dearer / 100);
         }
-        const bool waves = classic <= balanced || g.tiles >= 2 * sms;
-        if (waves) split_k = s0;
-        g.cost = waves ? classic : balanced;
     }
     g.split_k = split_k;
     if (split_k == 0) {
@@ -401,13 +423,24 @@ const int* mid_max_clusters() {     // [size]
     return d->mid_clusters;
 }
 
-// mtc: most batch rows of a tile, 64 or 128.  Cost model in ns, fitted to the figures below: a unit takes a CTA 400 + 0.7 mt
-// ns when it has the SM to itself and 470 + 1.6 mt when two share it (64-row build), 500 + 2 mt and 560 + 2.8 mt (128 rows);
-// a launch 4 us beside its units, and 0.7 us more where more than half of the slots are taken, so that the next launch's
-// CTAs do not find room before this one ends; the exchange inside a cluster of s 600 + 150 s (4300 + 300 s).
+// mtc: most batch rows of a tile, 64 or 128.  Cost model in ns, fitted like the wide-tile kernel's.  A unit takes a CTA of the
+// 64-row build 0.34 us with 16 rows and 0.40 with 64 while it has the SM to itself, 0.50 and 0.52 where two share it (whole
+// tiles from the first on: 1 / 16 / 32 / 64 of 16 rows 0.34 / 0.39 / 0.44 / 0.47; clusters from 56 CTAs on), more with
+// three quarters of the slots taken (64 rows: 256 / 280 / 296 CTAs 0.57 / 0.62 / 0.66).  The exchange inside a cluster grows with
+// the rows that a CTA finishes and with the CTAs at it; sizes that are not a power of two and slices of a single unit cost
+// a little more, the last cluster that fits finds its place late (16 rows, K = 5120: 91 / 92 / 93 tiles in three slices
+// 11.3 / 11.4 / 12.4 us).  Slices beyond a cluster pay for the second kernel and 63 ns each (K = 24960, two tiles, 32 rows: eight
+// slices 12.2 us, 16 / 24 / 32 / 74 through the workspace 9.9 / 9.4 / 8.8 / 11.9).
 // Measured (us), M = 32: K = N = 4096 four slices 7.09, eight 7.44; K = 11008 / N = 4096 8 / 6 / 4 slices 11.0 / 11.6 /
 // 13.8; K = 18432 / N = 7168 5 / 4 21.8 / 22.9; K = 4096 / N = 12288 2 / 1 12.2 / 17.3, three no longer fit at once: 17.5;
 // K = 4096 / N = 22016 1 / 2 18.7 / 22.6; K = 1024 / N = 3136 4 / 8 4.18 / 5.10.
+// Whole tiles that leave SMs free take one SM each, by asking for more than half of its shared memory: beside the CTAs of the
+// launch in front, which are still there when this one starts early, they would come to sit in pairs, and a pair takes 0.45 to
+// 0.53 us a unit instead of 0.35 to 0.41.  us in pairs / spread, 32 rows: K = 4096: 64 tiles 17.6 / 14.6, 114 18.5 / 15.0, 140
+// 18.6 / 15.3, 148 15.6 / 15.6; K = 1280: 75 6.9 / 6.6, 130 7.5 / 7.1, 148 6.8 / 7.4; K = 640: 130 5.0 / 5.3 (the next launch
+// cannot start beside this one).  With one CTA per SM and the kernel before this one: 75 tiles of K = 1280, 64 rows, 7.3.
+bool mid_spread(long tiles, int G, int sms) { return tiles <= sms - 8 && G >= 8; }
+
 MidGeom mid_geom(int mtc, int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg) {
     MidGeom g;
     g.mtc = mtc;
@@ -421,15 +454,55 @@ MidGeom mid_geom(int mtc, int M, int N, int G, int split_k, int sms, bool allow_
     if (split_k == 0) {
         const int* max_clusters = mid_max_clusters();
         const bool wide = mtc > 64;
-        const long alone = wide ? 500 + 2 * g.mt : 400 + g.mt * 7 / 10, shared = wide ? 560 + g.mt * 14 / 5 : 470 + g.mt * 8 / 5;
-        for (int s = 1; s <= kMidMaxCluster && s <= G; ++s) {
-            if (s > 1 && (!allow_cluster || g.tiles > max_clusters[s] || !fits(s))) continue;
-            const long ctas = g.tiles * s;
-            const long units = ((ctas + slots - 1) / slots) * ((G + s - 1) / s);
-            const long cost = 4000 + units * (ctas > sms ? shared : alone) + (ctas > sms ? 700 : 0) +
-                              (s > 1 ? (wide ? 4300 + 300 * s : 600 + 150 * s) : 0);
+        const int mt = g.mt, tiles = (int)(g.tiles < slots ? g.tiles : slots);
+        auto take = [&](int s, long cost) {
             if (g.cost == 0 || cost < g.cost) { g.cost = cost; split_k = s; }
+        };
+        const int rows_ns = sg / 2;     // more scale rows a unit: felt where two CTAs share an SM
+        auto sharing = [](int ctas) { return ctas <= 56 ? 0 : ctas >= 104 ? 48 : ctas - 56; };        // of 48
+        auto crowd = [&](int ctas) { return ctas > slots * 3 / 4 ? ctas - slots * 3 / 4 : 0; };      // of 74
+        if (g.tiles > slots) {
+            const long waves = (g.tiles + slots - 1) / slots;
+            take(1, wide ? 39 * mt - 670 + waves * (3300 + G * (800L + mt * 4 / 10)) : 600 + waves * (2900 + G * 520L));
+        } else if (mid_spread(g.tiles, G, sms)) {
+            take(1, wide ? 1620 + 23 * mt + tiles * 285 / 100 + G * (677L - mt / 2 + mt * 3 * tiles / 1000)
+                         : 1850 + 16 * mt + tiles * 555 / 100 + G * (330L + mt * 11 / 10 + mt * 7 * tiles / 1000 + 14 * rows_ns * sharing(tiles) / 48));
+        } else {
+            const int pairs = tiles < 80 ? tiles : 80;
+            take(1, wide ? 1740 + 22 * mt + tiles * 514 / 100 + G * (587L + mt * 4 / 10 + 161 * sharing(tiles) / 48)
+                         : 1900 + 22 * mt + 2 * tiles + G * (320L + mt * 13 / 10 + (170 - mt * 8 / 10 + 34 * rows_ns) * pairs / 80 + crowd(tiles) * mt * 14 / 740));
         }
+        if (allow_cluster)
+#pragma unroll
+            for (int s = 2; s <= kMidMaxCluster; ++s) {
+                if (s > G || tiles > max_clusters[s] || !fits(s)) continue;
+                const int ctas = tiles * s, rows = (mt / 4 + s - 1) / s, u = (G + s - 1) / s;
+                const bool odd = (s & (s - 1)) != 0, last = s > 2 && tiles == max_clusters[s];
+                take(s, wide ? 2230 + 33 * mt + ctas * (15 * mt - 104) / 100 + 99 * s + 26 * rows + u * (644L + 164 * sharing(ctas) / 48 - crowd(ctas) * mt * 9 / 740) +
+                                   (odd ? 201 : 0) + (last ? 1613 : 0)
+                             : 2550 + 17 * mt + ctas * (280 + 55 * mt / 10) / 100 + 63 * s + 96 * rows +
+                                   u * (316L + mt * 15 / 10 + (109 + 34 * rows_ns) * sharing(ctas) / 48 + crowd(ctas) * (178 - mt * 3 / 4 + 50 * rows_ns) / 100) +
+                                   (odd ? 107 : 0) + (last ? 513 : 0) + (u == 1 ? 493 : 0) +
+                                   (sg > 1 && mt < 64 && mid_smem_bytes(mtc, mt, sg, 3, s) > kMidSmemBudget ? 400 : 0));   // (two-stage weight ring)
+            }
+        // through the workspace: as many slices as there are SMs or slots, or as many as pay for being added
+        // (with few slices only where their exchange buffer leaves no room for a cluster: groups of 32, 64 rows)
+        if (3 * tiles <= slots * 7 / 8) {
+            const int unit = wide ? 697 + mt / 2 : 224 + mt * 29 / 10, more = wide ? 19 * mt - 364 : 15 * mt - 234;
+            const int add = (wide ? 62 : 63) + tiles * more / 100;
+            const int pays = (int)(sqrtf((float)G * unit / (add > 20 ? add : 20)) + 0.5f);
+            for (int cap : {sms / tiles, slots * 7 / 8 / tiles}) {
+                int s = cap < pays ? cap : pays;
+                if (s > G) s = G;
+                if (s < 2 || (s <= kMidMaxCluster && allow_cluster && fits(s))) continue;
+                const int ctas = tiles * s;
+                const long cost = (wide ? 4350 + mt : 5200 - 13 * mt) + ctas * more / 100 + (wide ? 62 : 63) * s +
+                                  (G + s - 1) / s * (unit + (wide ? -23L : 104L + 28 * rows_ns) * sharing(ctas) / 48);
+                take(s, cost > kTwoLaunches ? cost : kTwoLaunches);
+            }
+        }
+        // (large activations, which every column tile reads again, do not stay in L2: M = 1968, K = 15616 / N = 2432 174 us)
+        if ((long)M * G * (2 * kGroup) > (40l << 20)) g.cost += g.cost / 4;
     }
     g.split_k = split_k;
     g.cluster = allow_cluster && split_k >= 2 && split_k <= kMidMaxCluster && fits(split_k);
@@ -442,6 +515,7 @@ MidGeom mid_geom(int mtc, int M, int N, int G, int split_k, int sms, bool allow_
     // A CTA takes half of the SM's tensor memory: ask for enough shared memory that no third one, and no CTA of the
     // wide-tile kernel (which takes all of it), ever shares the SM, so that the allocation never has to wait.
     if (g.smem_bytes < 108 * 1024) g.smem_bytes = 108 * 1024;
+    if (split_k == 1 && mid_spread(g.tiles, G, sms) && g.smem_bytes < 120 * 1024) g.smem_bytes = 120 * 1024;
     return g;
 }
 size_t mid_workspace_bytes(const MidGeom& g) {
@@ -466,7 +540,7 @@ struct WidePlan {
     TileGeom tile;
     size_t workspace_bytes() const { return use_mid ? mid_workspace_bytes(mid) : tile_workspace_bytes(tile); }
 };
-WidePlan wide_plan(int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg) {
+WidePlan wide_plan(int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg, bool epi) {
     WidePlan w;
     w.use_mid = true;
     if (M <= 64) {
@@ -477,6 +551,8 @@ WidePlan wide_plan(int M, int N, int G, int split_k, int sms, bool allow_cluster
     const MidGeom m128 = mid_geom(128, M, N, G, 0, sms, allow_cluster, sg);
     if (m128.cost < w.mid.cost) w.mid = m128;
     w.tile = tile_geom(M, N, G, 0, sms);
+    // (bias or activation in that kernel's own epilogue: K = 512, 80 / 208 rows 1.9 / 2.9 us more; in the other one 0.3)
+    if (epi && w.tile.split_k == 1) w.tile.cost += (w.tile.tiles + sms - 1) / sms * (1200 + 8 * w.tile.mt);
     w.use_mid = w.mid.cost < w.tile.cost;
     if (split_k != 0) {
         if (w.use_mid) w.mid = mid_geom(w.mid.mtc, M, N, G, split_k, sms, allow_cluster, sg);
@@ -486,22 +562,27 @@ WidePlan wide_plan(int M, int N, int G, int split_k, int sms, bool allow_cluster
 }
 
 // 9 to 16 rows with path and split_k left open: the warp-MMA kernel runs its 16-row build, which converts every weight for
-// two MMAs; the two-CTA tcgen05 kernel is ahead on long shapes and level on short ones.  Its cost model, fitted to 32 and 64
-// rows, is 1.7 us too high here.  us, warp-MMA / tcgen05, M = 16: K = 28672 / N = 8192 38.6 / 32.1, K = 18432 / N = 7168 26.4 /
-// 21.3, K = 4096 / N = 12288 12.7 / 11.1, N = 22016 18.8 / 18.0, K = 8192 / N = 8192 13.3 / 12.5, K = 1024 / N = 3136 5.0 /
-// 3.9, K = 11008 / N = 4096 10.9 / 10.4; K = N = 4096 6.1 / 6.8, K = 2048 / N = 8192 5.9 / 6.5, K = 6144 / N = 1536 6.0 / 6.0.
+// two MMAs; the two-CTA tcgen05 kernel is ahead on long shapes and level on short ones (calls of less than 4.6 us are the host's, and
+// its own is shorter).  us, warp-MMA / tcgen05, M = 16: K = 28672 / N = 8192 38.6 / 32.1, K = 18432 / N = 7168 26.4 / 21.3, K = 4096 /
+// N = 12288 12.7 / 11.1, K = 8192 / N = 8192 13.3 / 12.5, K = 27648 / N = 1024 15.2 / 10.5, K = 1024 / N = 3136 5.0 / 3.9, K = 11008 /
+// N = 4096 10.9 / 10.4; K = N = 4096 6.1 / 6.8, K = 2048 / N = 8192 5.9 / 6.5, K = 6144 / N = 1536 6.0 / 6.0.
 bool small_batch_takes_mid(int M, int N, int G, int sms, bool allow_cluster, int sg) {
     if (M < 9 || M > 16) return false;
-    // (more 64-column tiles than CTA slots: K = 4096 / N = 22016 18.8 / 18.0 by itself, and behind or in front of a cluster
-    // launch, as between a block's projections, 23.4 / 18.0: some SMs get four tiles)
-    if (N / kTileN > 2 * sms) return true;
-    const long mid = mid_geom(64, M, N, G, 0, sms, allow_cluster, sg).cost - 1700;
-    return mid * 20 < decode_geom(M, N, G, 0, sms, allow_cluster, sg).cost * 19;
+    const DecodeGeom d = decode_geom(M, N, G, 0, sms, allow_cluster, sg);
+    if (d.cost < 4600) return false;
+    // Whole tiles, and more of them than CTA slots: level by itself, but in front of or behind another launch, as between a
+    // block's projections, some SMs get four (us, K = 4096 / N = 22016: 18.8 / 18.5, and with K = N = 4096 in front 30.2 / 25.4).
+    // Groups of 32 cost this kernel more (18.9 / 21.1 by itself): by cost, like balanced chunks (K = 8192 / N = 20224 31.4 / 35.1
+    // and 40.7 / 43.7).
+    if (sg < 4 && d.split_k == 1 && N / kTileN >= 2 * sms + 8) return true;
+    // (with an SM to itself a CTA of the warp-MMA kernel is faster than its model says: 256 columns of K = 13952 6.8 us)
+    const long dec = d.cluster && d.nchunks <= 36 ? d.cost - 100 * ((G + d.split_k - 1) / d.split_k) : d.cost;
+    return mid_geom(64, M, N, G, 0, sms, allow_cluster, sg).cost * 100 < dec * 93;
 }
 
 // Nominal split factor of the tcgen05 path's schedule: how many chunks share one tile's K range.
 int choose_split_tile(int M, int N, int G, int sms, bool allow_cluster, int sg) {
-    const WidePlan w = wide_plan(M, N, G, 0, sms, allow_cluster, sg);
+    const WidePlan w = wide_plan(M, N, G, 0, sms, allow_cluster, sg, false);
     if (w.use_mid) return w.mid.split_k;
     if (w.tile.split_k >= 1) return w.tile.split_k;
     long s = (w.tile.nchunks + w.tile.tiles - 1) / w.tile.tiles;
@@ -601,7 +682,7 @@ struct GemmPlan {
 };
 // An explicit split_k > 1 asks for its workspace on every kernel, used or not.  With split_k == 0 slices that meet in a cluster
 // ask for none, and balanced chunks, which cross tile boundaries, give way to whole tiles where `ws_bytes` does not hold them.
-GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, int sms, bool allow_cluster, size_t ws_bytes = SIZE_MAX) {
+GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, bool epi, int sms, bool allow_cluster, size_t ws_bytes) {
     GemmPlan p;
     int path = resolve_path(M, path_asked);
     if (path_asked == W4A16_PATH_AUTO && split_k == 0 && path == W4A16_PATH_DECODE &&
@@ -620,7 +701,7 @@ GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, int
             p.workspace = 0;
         }
     } else {
-        p.wide = wide_plan(M, N, G, split_k, sms, allow_cluster, sg);
+        p.wide = wide_plan(M, N, G, split_k, sms, allow_cluster, sg, epi);
         p.kernel = !p.wide.use_mid ? W4A16_KERNEL_TILE : p.wide.mid.mtc <= 64 ? W4A16_KERNEL_MID64 : W4A16_KERNEL_MID128;
         p.workspace = split_k == 0 && p.wide.use_mid && p.wide.mid.cluster ? 0 : p.wide.workspace_bytes();
         if (p.workspace > ws_bytes && !p.wide.use_mid && p.wide.tile.split_k == 0) {
@@ -706,14 +787,15 @@ size_t w4a16_workspace_bytes(int M, int N, int K, int group, int split_k) {
     const size_t whole = decode_partial_bytes(decode_geom(M, N, G, split_k, sms, true, sg));   // (asked for by whole tiles too)
     if (whole > need) need = whole;
     for (bool clusters : {true, false})
-        for (int path : {W4A16_PATH_AUTO, W4A16_PATH_SIMPLE, W4A16_PATH_DECODE, W4A16_PATH_TILE}) {
-            const size_t n = gemm_plan(M, N, G, sg, split_k, path, sms, clusters).workspace;
-            if (n > need) need = n;
-        }
+        for (bool epi : {false, true})
+            for (int path : {W4A16_PATH_AUTO, W4A16_PATH_SIMPLE, W4A16_PATH_DECODE, W4A16_PATH_TILE}) {
+                const size_t n = gemm_plan(M, N, G, sg, split_k, path, epi, sms, clusters, SIZE_MAX).workspace;
+                if (n > need) need = n;
+            }
     return kWsFullHeaderBytes + need;
 }
 
-int w4a16_gemm_plan(int M, int N, int K, int group, int split_k, int path, w4a16_plan* out) {
+int w4a16_gemm_plan(int M, int N, int K, int group, int split_k, int path, int with_epilogue, w4a16_plan* out) {
     std::lock_guard<std::mutex> lock(g_mu);
     if (!out) return W4A16_ERR_NULL;
     const int rc = check_weight_shape(N, K, group);
@@ -721,7 +803,7 @@ int w4a16_gemm_plan(int M, int N, int K, int group, int split_k, int path, w4a16
     if (M < 1) return W4A16_ERR_SHAPE;
     if (split_k < 0 || split_k > K / kGroup) return W4A16_ERR_SPLITK;
     if (path < W4A16_PATH_AUTO || path > W4A16_PATH_TILE) return W4A16_ERR_PATH;
-    const GemmPlan g = gemm_plan(M, N, K / kGroup, kGroup / group, split_k, path, sm_count_or_default(), clusters_ok());
+    const GemmPlan g = gemm_plan(M, N, K / kGroup, kGroup / group, split_k, path, with_epilogue != 0, sm_count_or_default(), clusters_ok(), SIZE_MAX);
     out->kernel = g.kernel;
     out->workspace_bytes = g.workspace == 0 ? 0 : kWsFullHeaderBytes + g.workspace;
     switch (g.kernel) {
@@ -968,7 +1050,7 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
     // registered workspace: [small-M tickets and reserve: the documented header][partial results]
     unsigned char* ws_body = d->ws ? static_cast<unsigned char*>(d->ws) + kWsFullHeaderBytes : nullptr;
     const size_t ws_body_bytes = d->ws_bytes > kWsFullHeaderBytes ? d->ws_bytes - kWsFullHeaderBytes : 0;
-    const GemmPlan plan = gemm_plan(M, N, G, sg, split_k, path, d->sm_count, d->cluster_ok, ws_body_bytes);
+    const GemmPlan plan = gemm_plan(M, N, G, sg, split_k, path, bias != nullptr || act != W4A16_ACT_NONE, d->sm_count, d->cluster_ok, ws_body_bytes);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint32_t* Zw = sym ? nullptr : static_cast<const uint32_t*>(Z);
     Epilogue epi;

@@ -145,6 +145,7 @@ def test_workspace_query_covers_what_every_call_asks_for(lib):
                 for path in (0, 1, 2, 3):
                     p = B.w4a16_gemm_plan(M, N, K, group, split, path)
                     assert p.workspace_bytes <= size, (M, N, K, group, split, path)
+                    assert B.w4a16_gemm_plan(M, N, K, group, split, path, True).workspace_bytes <= size, (M, N, K, group, split, path)
                     if split != 0:
                         assert p.split_k == split
                     elif path != B.PATH_SIMPLE and p.split_k != 0:
@@ -159,6 +160,24 @@ def test_slices_of_few_column_tiles_meet_in_a_cluster(lib):
         p = B.w4a16_gemm_plan(M, N, K, group, 0, B.PATH_DECODE)
         assert (p.split_k, p.cluster) == (6, 1), (M, N, K, group)
     assert B.w4a16_gemm_plan(2, 640, 19072, 64).split_k == 25        # 7.9 us; six in a cluster 9.3
+
+
+def test_schedules_of_few_or_whole_column_tiles_above_16_rows(lib):
+    """tcgen05 path, us of the schedule taken once / of the one asked for here.  Few column tiles and a long K: as many slices
+    as pay for being added, more than a cluster holds for the two-CTA kernel and not one per SM for the wide one (M = 51,
+    K = 19712, N = 128: 8 slices 11.9 / 25 9.1; M = 240, K = 21760, N = 128: 74 slices 25.6 / 24 11.0).  One wave of whole tiles
+    where slices do not fit well (M = 45, K = 1408, N = 11904: three slices 9.6 / 8.0)."""
+    p = B.w4a16_gemm_plan(51, 128, 19712)
+    assert (p.kernel, p.cluster) == (B.KERNEL_MID64, 0) and 16 <= p.split_k <= 32
+    for M, N, K in [(240, 128, 21760), (89, 128, 22784), (256, 128, 17152), (177, 64, 13312), (71, 320, 6016)]:
+        p = B.w4a16_gemm_plan(M, N, K)
+        assert 2 <= p.split_k <= 30, (M, N, K, p.split_k)
+    assert B.w4a16_gemm_plan(45, 11904, 1408, 64).split_k <= 2
+    # 9 to 16 rows: long shapes of few tiles go to the tcgen05 kernel, groups of 32 and more tiles than CTA slots do not
+    assert B.w4a16_gemm_plan(16, 1024, 27648).kernel == B.KERNEL_MID64
+    assert B.w4a16_gemm_plan(16, 22016, 4096).kernel == B.KERNEL_MID64
+    assert B.w4a16_gemm_plan(16, 22016, 4096, 32).kernel == B.KERNEL_DECODE
+    assert B.w4a16_gemm_plan(16, 20224, 8192).kernel == B.KERNEL_DECODE
 
 
 def test_argument_errors_are_reported_before_any_device_work(lib):

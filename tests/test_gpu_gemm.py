@@ -128,8 +128,8 @@ def test_workspace_errors():
 # Schedules that the library picks itself where whole tiles would leave SMs idle: slices that meet in a cluster (each kernel)
 # never touch the workspace; balanced chunks give way to whole tiles when there is none.
 @pytest.mark.parametrize("M,K,N,kernel,cluster", [
-    (4, 1792, 8576, B.KERNEL_DECODE, 1), (16, 4096, 12288, B.KERNEL_MID64, 1), (32, 1280, 12288, B.KERNEL_MID64, 1),
-    (65, 5632, 6464, B.KERNEL_MID128, 1), (129, 6016, 9984, B.KERNEL_TILE, 0)])
+    (4, 1792, 8576, B.KERNEL_DECODE, 1), (16, 4096, 12288, B.KERNEL_MID64, 1), (32, 4096, 4096, B.KERNEL_MID64, 1),
+    (112, 9216, 6528, B.KERNEL_MID128, 1), (129, 6016, 9984, B.KERNEL_TILE, 0)])
 def test_automatic_schedules_without_a_workspace(M, K, N, kernel, cluster):
     plan = B.w4a16_gemm_plan(M, N, K)
     assert (plan.kernel, plan.cluster) == (kernel, cluster) and (cluster or plan.split_k == 0)
