@@ -10,6 +10,7 @@
 #include <string.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels_basic.cuh"
@@ -112,15 +113,29 @@ bool flags_ok(int flags) { return (flags & ~(W4A16_FLAG_SYMMETRIC | W4A16_FLAG_B
 
 size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 
+// What the schedules are planned for.  Made once per call and passed on: asking for the device costs 30 ns each time.
+struct Chip {
+    int sms;
+    bool clusters;               // a launch with clusters has not been refused
+    const int* max_clusters;     // [size]: clusters of two-per-SM CTAs that run at the same time
+};
+const int* mid_max_clusters(DeviceState* d);
+Chip chip_of(DeviceState* d) { return {d->sm_count, d->cluster_ok, mid_max_clusters(d)}; }
 // For the size and schedule queries, which also answer on a host without a device.
-int sm_count_or_default() {
+Chip chip_or_default() {
     DeviceState* d = nullptr;
-    if (current_device(&d) == W4A16_OK) return d->sm_count;
-    return 148;
+    if (current_device(&d) == W4A16_OK) return chip_of(d);
+    return {148, true, mid_max_clusters(nullptr)};
 }
-bool clusters_ok() {
-    DeviceState* d = nullptr;
-    return current_device(&d) != W4A16_OK || d->cluster_ok;
+Chip without_clusters(Chip chip) { chip.clusters = false; return chip; }
+
+// f(2), f(3) ... with the sizes as constants.
+template <int kFrom, int kTo, typename F>
+void for_each_size(const F& f) {
+    if constexpr (kFrom <= kTo) {
+        f(std::integral_constant<int, kFrom>{});
+        for_each_size<kFrom + 1, kTo>(f);
+    }
 }
 
 // ---- decode-path launch geometry ------------------------------------------------
@@ -147,20 +162,19 @@ struct DecodeGeom {
 // N = 22016: the box takes 8 KiB of a slot whatever M is, and long shapes want the ring stage that costs).
 constexpr int kDecABoxMinRows = 2;
 
-const int* mid_max_clusters();
-
-DecodeGeom decode_geom(int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg) {
+DecodeGeom decode_geom(int M, int N, int G, int split_k, const Chip& chip, int sg) {
     DecodeGeom g;
     g.mb = decode_mb(M);
     g.mchunks = (M + 8 * g.mb - 1) / (8 * g.mb);
     const int T = N / kTileN;
     const long units = (long)T * G;
+    const bool allow_cluster = chip.clusters;
     // Two CTAs per SM.  (Three, with a two-stage ring and 72 registers, were ahead on long launches
     // while every exchange went through the workspace; with the cluster exchange two are ahead again
     // everywhere but K = 4096 / N = 12288, by 3 %: 33.8 against 34.8 us at K = 28672 / N = 8192, 15.0
     // against 15.8 at N = 22016.  The kernel keeps the template parameter.)
     g.cps = 2;
-    long slots = (long)g.cps * sms;
+    long slots = (long)g.cps * chip.sms;
     g.cost = 0;
     if (split_k == 0) {
         // How the unit range is cut when the caller leaves it open.  Balanced chunks use every CTA slot, but a chunk that
@@ -178,7 +192,7 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, int sms, bool allow_clu
         // through the workspace 6.5; K = 28672 / N = 8192 two 31.2, balanced 32.4; K = 4096 / N = 22016 (344 whole tiles on
         // 296 CTAs, whose pairs share the SM's issue slots: 15 % over the mean, with 16 rows 30) 14.4, balanced 18.4.
         const long unit_ns = g.mb == 1 ? 288 : 330, wide = g.mb == 1 ? 0 : 700, add_ns = ((M < 8 * g.mb ? M : 8 * g.mb) + 3) / 4 * 80;
-        const int* max_clusters = mid_max_clusters();      // (two CTAs per SM, like that kernel)
+        const int* max_clusters = chip.max_clusters;
         auto take = [&](int s, long cost) {
             if (g.cost == 0 || cost < g.cost) { g.cost = cost; split_k = s; }
         };
@@ -191,10 +205,11 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, int sms, bool allow_clu
             // 69 / 70 in four 4.0 / 4.4 / 4.9 / 5.1, in two 4.2; 41 / 42 / 43 / 44 in six 3.8 / 4.0 / 4.4 / 4.8, in five 3.5), not
             // with 2.  A long launch hardly notices (K = 28672: 50 in five 14.9; K = 10880: 42 in six 7.0, in five 7.7).  Of equal
             // slices the even count is ahead (20 tiles of K = 3200, M = 16: 4.4 in six, 4.9 in five).
-            for (int s = 2; s <= kDecMaxCluster && s <= G; ++s) {
+            for_each_size<2, kDecMaxCluster>([&](auto size) {
+                constexpr int s = decltype(size)::value;
                 const int room = max_clusters[s];
-                if (T + 2 > room) continue;
-                const long u = (G + s - 1) / s, ctas = (long)T * s;
+                if (s > G || T + 2 > room) return;
+                const int u = (G + s - 1) / s, ctas = T * s;
                 long wait = 0;
                 if (s == 3 || s == 5) {
                     const int over = s == 3 ? T - room * 8 / 9 : T - room * 7 / 8;
@@ -208,7 +223,7 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, int sms, bool allow_clu
                 }
                 if (wait < 0) wait = 0;
                 take(s, (s == 2 ? 1700 : 2150) + (s % 2 != 0 && u > 3 ? 150 : 0) + wide * 7 / 4 + unit_ns * u + (10 * ctas > 9 * slots ? 500 : 0) + wait);
-            }
+            });
         }
         const int s0 = (int)(slots * 7 / 8 / T < G ? slots * 7 / 8 / T : G);
         if (s0 > kDecMaxCluster || (s0 >= 2 && !(allow_cluster && g.mchunks == 1)))
@@ -258,8 +273,8 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, int sms, bool allow_clu
 }
 
 // Nominal split factor of the balanced schedule: how many CTAs share one column tile's K range.
-int choose_split_decode(int M, int N, int G, int sms, bool allow_cluster, int sg) {
-    DecodeGeom g = decode_geom(M, N, G, 0, sms, allow_cluster, sg);
+int choose_split_decode(int M, int N, int G, const Chip& chip, int sg) {
+    DecodeGeom g = decode_geom(M, N, G, 0, chip, sg);
     if (g.split_k >= 1) return g.split_k;
     const int T = N / kTileN;
     int s = (g.ctas + T - 1) / T;
@@ -393,10 +408,9 @@ __global__ void __launch_bounds__(kMidThreads, 2) mid_shape_probe_kernel(float* 
     extern __shared__ float probe_smem[];
     out[threadIdx.x] = probe_smem[threadIdx.x];
 }
-const int* mid_max_clusters() {     // [size]
+const int* mid_max_clusters(DeviceState* d) {     // [size]
     static const int without_device[kMidMaxCluster + 1] = {0, 296, 148, 93, 71, 56, 45, 37, 33};   // (size queries on a host)
-    DeviceState* d = nullptr;
-    if (current_device(&d) != W4A16_OK || !d->is_sm100) return without_device;
+    if (d == nullptr || !d->is_sm100) return without_device;
     if (d->mid_clusters[1] != 0) return d->mid_clusters;
     const bool ok = cudaFuncSetAttribute(mid_shape_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          d->max_smem_optin) == cudaSuccess;
@@ -441,8 +455,10 @@ const int* mid_max_clusters() {     // [size]
 // cannot start beside this one).  With one CTA per SM and the kernel before this one: 75 tiles of K = 1280, 64 rows, 7.3.
 bool mid_spread(long tiles, int G, int sms) { return tiles <= sms - 8 && G >= 8; }
 
-MidGeom mid_geom(int mtc, int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg) {
+MidGeom mid_geom(int mtc, int M, int N, int G, int split_k, const Chip& chip, int sg) {
     MidGeom g;
+    const int sms = chip.sms;
+    const bool allow_cluster = chip.clusters;
     g.mtc = mtc;
     g.m_tiles = (M + g.mtc - 1) / g.mtc;
     g.mt = ((M + g.m_tiles - 1) / g.m_tiles + 15) / 16 * 16;
@@ -452,7 +468,7 @@ MidGeom mid_geom(int mtc, int M, int N, int G, int split_k, int sms, bool allow_
     auto fits = [&](int s) { return mid_smem_bytes(g.mtc, g.mt, sg, 2, s) <= kMidSmemBudget; };
     g.cost = 0;
     if (split_k == 0) {
-        const int* max_clusters = mid_max_clusters();
+        const int* max_clusters = chip.max_clusters;
         const bool wide = mtc > 64;
         const int mt = g.mt, tiles = (int)(g.tiles < slots ? g.tiles : slots);
         auto take = [&](int s, long cost) {
@@ -472,19 +488,19 @@ MidGeom mid_geom(int mtc, int M, int N, int G, int split_k, int sms, bool allow_
             take(1, wide ? 1740 + 22 * mt + tiles * 514 / 100 + G * (587L + mt * 4 / 10 + 161 * sharing(tiles) / 48)
                          : 1900 + 22 * mt + 2 * tiles + G * (320L + mt * 13 / 10 + (170 - mt * 8 / 10 + 34 * rows_ns) * pairs / 80 + crowd(tiles) * mt * 14 / 740));
         }
-        if (allow_cluster)
-#pragma unroll
-            for (int s = 2; s <= kMidMaxCluster; ++s) {
-                if (s > G || tiles > max_clusters[s] || !fits(s)) continue;
-                const int ctas = tiles * s, rows = (mt / 4 + s - 1) / s, u = (G + s - 1) / s;
-                const bool odd = (s & (s - 1)) != 0, last = s > 2 && tiles == max_clusters[s];
-                take(s, wide ? 2230 + 33 * mt + ctas * (15 * mt - 104) / 100 + 99 * s + 26 * rows + u * (644L + 164 * sharing(ctas) / 48 - crowd(ctas) * mt * 9 / 740) +
-                                   (odd ? 201 : 0) + (last ? 1613 : 0)
-                             : 2550 + 17 * mt + ctas * (280 + 55 * mt / 10) / 100 + 63 * s + 96 * rows +
-                                   u * (316L + mt * 15 / 10 + (109 + 34 * rows_ns) * sharing(ctas) / 48 + crowd(ctas) * (178 - mt * 3 / 4 + 50 * rows_ns) / 100) +
-                                   (odd ? 107 : 0) + (last ? 513 : 0) + (u == 1 ? 493 : 0) +
-                                   (sg > 1 && mt < 64 && mid_smem_bytes(mtc, mt, sg, 3, s) > kMidSmemBudget ? 400 : 0));   // (two-stage weight ring)
-            }
+        auto cluster = [&](auto size) {        // (sizes as constants: three divisions by each)
+            constexpr int s = decltype(size)::value;
+            if (s > G || tiles > max_clusters[s] || !fits(s)) return;
+            const int ctas = tiles * s, rows = (mt / 4 + s - 1) / s, u = (G + s - 1) / s;
+            const bool odd = (s & (s - 1)) != 0, last = s > 2 && tiles == max_clusters[s];
+            take(s, wide ? 2230 + 33 * mt + ctas * (15 * mt - 104) / 100 + 99 * s + 26 * rows + u * (644L + 164 * sharing(ctas) / 48 - crowd(ctas) * mt * 9 / 740) +
+                               (odd ? 201 : 0) + (last ? 1613 : 0)
+                         : 2550 + 17 * mt + ctas * (280 + 55 * mt / 10) / 100 + 63 * s + 96 * rows +
+                               u * (316L + mt * 15 / 10 + (109 + 34 * rows_ns) * sharing(ctas) / 48 + crowd(ctas) * (178 - mt * 3 / 4 + 50 * rows_ns) / 100) +
+                               (odd ? 107 : 0) + (last ? 513 : 0) + (u == 1 ? 493 : 0) +
+                               (sg > 1 && mt < 64 && mid_smem_bytes(mtc, mt, sg, 3, s) > kMidSmemBudget ? 400 : 0));   // (two-stage weight ring)
+        };
+        if (allow_cluster) for_each_size<2, kMidMaxCluster>(cluster);
         // through the workspace: as many slices as there are SMs or slots, or as many as pay for being added
         // (with few slices only where their exchange buffer leaves no room for a cluster: groups of 32, 64 rows)
         if (3 * tiles <= slots * 7 / 8) {
@@ -540,23 +556,23 @@ struct WidePlan {
     TileGeom tile;
     size_t workspace_bytes() const { return use_mid ? mid_workspace_bytes(mid) : tile_workspace_bytes(tile); }
 };
-WidePlan wide_plan(int M, int N, int G, int split_k, int sms, bool allow_cluster, int sg, bool epi) {
+WidePlan wide_plan(int M, int N, int G, int split_k, const Chip& chip, int sg, bool epi) {
     WidePlan w;
     w.use_mid = true;
     if (M <= 64) {
-        w.mid = mid_geom(64, M, N, G, split_k, sms, allow_cluster, sg);
+        w.mid = mid_geom(64, M, N, G, split_k, chip, sg);
         return w;
     }
-    w.mid = mid_geom(64, M, N, G, 0, sms, allow_cluster, sg);
-    const MidGeom m128 = mid_geom(128, M, N, G, 0, sms, allow_cluster, sg);
+    w.mid = mid_geom(64, M, N, G, 0, chip, sg);
+    const MidGeom m128 = mid_geom(128, M, N, G, 0, chip, sg);
     if (m128.cost < w.mid.cost) w.mid = m128;
-    w.tile = tile_geom(M, N, G, 0, sms);
+    w.tile = tile_geom(M, N, G, 0, chip.sms);
     // (bias or activation in that kernel's own epilogue: K = 512, 80 / 208 rows 1.9 / 2.9 us more; in the other one 0.3)
-    if (epi && w.tile.split_k == 1) w.tile.cost += (w.tile.tiles + sms - 1) / sms * (1200 + 8 * w.tile.mt);
+    if (epi && w.tile.split_k == 1) w.tile.cost += (w.tile.tiles + chip.sms - 1) / chip.sms * (1200 + 8 * w.tile.mt);
     w.use_mid = w.mid.cost < w.tile.cost;
     if (split_k != 0) {
-        if (w.use_mid) w.mid = mid_geom(w.mid.mtc, M, N, G, split_k, sms, allow_cluster, sg);
-        else w.tile = tile_geom(M, N, G, split_k, sms);
+        if (w.use_mid) w.mid = mid_geom(w.mid.mtc, M, N, G, split_k, chip, sg);
+        else w.tile = tile_geom(M, N, G, split_k, chip.sms);
     }
     return w;
 }
@@ -566,23 +582,21 @@ WidePlan wide_plan(int M, int N, int G, int split_k, int sms, bool allow_cluster
 // its own is shorter).  us, warp-MMA / tcgen05, M = 16: K = 28672 / N = 8192 38.6 / 32.1, K = 18432 / N = 7168 26.4 / 21.3, K = 4096 /
 // N = 12288 12.7 / 11.1, K = 8192 / N = 8192 13.3 / 12.5, K = 27648 / N = 1024 15.2 / 10.5, K = 1024 / N = 3136 5.0 / 3.9, K = 11008 /
 // N = 4096 10.9 / 10.4; K = N = 4096 6.1 / 6.8, K = 2048 / N = 8192 5.9 / 6.5, K = 6144 / N = 1536 6.0 / 6.0.
-bool small_batch_takes_mid(int M, int N, int G, int sms, bool allow_cluster, int sg) {
-    if (M < 9 || M > 16) return false;
-    const DecodeGeom d = decode_geom(M, N, G, 0, sms, allow_cluster, sg);
-    if (d.cost < 4600) return false;
+bool small_batch_takes_mid(const DecodeGeom& d, int M, int N, int G, const Chip& chip, int sg, MidGeom* mid) {
+    if (M < 9 || M > 16 || d.cost < 4600) return false;
+    *mid = mid_geom(64, M, N, G, 0, chip, sg);
     // Whole tiles, and more of them than CTA slots: level by itself, but in front of or behind another launch, as between a
     // block's projections, some SMs get four (us, K = 4096 / N = 22016: 18.8 / 18.5, and with K = N = 4096 in front 30.2 / 25.4).
     // Groups of 32 cost this kernel more (18.9 / 21.1 by itself): by cost, like balanced chunks (K = 8192 / N = 20224 31.4 / 35.1
     // and 40.7 / 43.7).
-    if (sg < 4 && d.split_k == 1 && N / kTileN >= 2 * sms + 8) return true;
+    if (sg < 4 && d.split_k == 1 && N / kTileN >= 2 * chip.sms + 8) return true;
     // (with an SM to itself a CTA of the warp-MMA kernel is faster than its model says: 256 columns of K = 13952 6.8 us)
     const long dec = d.cluster && d.nchunks <= 36 ? d.cost - 100 * ((G + d.split_k - 1) / d.split_k) : d.cost;
-    return mid_geom(64, M, N, G, 0, sms, allow_cluster, sg).cost * 100 < dec * 93;
+    return mid->cost * 100 < dec * 93;
 }
 
 // Nominal split factor of the tcgen05 path's schedule: how many chunks share one tile's K range.
-int choose_split_tile(int M, int N, int G, int sms, bool allow_cluster, int sg) {
-    const WidePlan w = wide_plan(M, N, G, 0, sms, allow_cluster, sg, false);
+int nominal_split(const WidePlan& w, int G) {
     if (w.use_mid) return w.mid.split_k;
     if (w.tile.split_k >= 1) return w.tile.split_k;
     long s = (w.tile.nchunks + w.tile.tiles - 1) / w.tile.tiles;
@@ -682,32 +696,35 @@ struct GemmPlan {
 };
 // An explicit split_k > 1 asks for its workspace on every kernel, used or not.  With split_k == 0 slices that meet in a cluster
 // ask for none, and balanced chunks, which cross tile boundaries, give way to whole tiles where `ws_bytes` does not hold them.
-GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, bool epi, int sms, bool allow_cluster, size_t ws_bytes) {
+GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, bool epi, const Chip& chip, size_t ws_bytes) {
     GemmPlan p;
-    int path = resolve_path(M, path_asked);
-    if (path_asked == W4A16_PATH_AUTO && split_k == 0 && path == W4A16_PATH_DECODE &&
-        small_batch_takes_mid(M, N, G, sms, allow_cluster, sg))
-        path = W4A16_PATH_TILE;
+    const int path = resolve_path(M, path_asked);
     if (path == W4A16_PATH_SIMPLE) {
         p.kernel = W4A16_KERNEL_SIMPLE;
-        p.split_simple = split_k == 0 ? choose_split_decode(M, N, G, sms, true, sg) : split_k;
+        p.split_simple = split_k == 0 ? choose_split_decode(M, N, G, chip, sg) : split_k;
         p.workspace = p.split_simple > 1 ? simple_partial_bytes(M, N, p.split_simple) : 0;
-    } else if (path == W4A16_PATH_DECODE) {
+        return p;
+    }
+    if (path == W4A16_PATH_DECODE) {
         p.kernel = W4A16_KERNEL_DECODE;
-        p.dec = decode_geom(M, N, G, split_k, sms, allow_cluster, sg);
-        p.workspace = decode_scratch(p.dec, split_k);
-        if (p.workspace > ws_bytes && p.dec.split_k == 0) {
-            p.dec = decode_geom(M, N, G, 1, sms, allow_cluster, sg);
-            p.workspace = 0;
+        p.dec = decode_geom(M, N, G, split_k, chip, sg);
+        p.wide.use_mid = path_asked == W4A16_PATH_AUTO && split_k == 0 && small_batch_takes_mid(p.dec, M, N, G, chip, sg, &p.wide.mid);
+        if (!p.wide.use_mid) {
+            p.workspace = decode_scratch(p.dec, split_k);
+            if (p.workspace > ws_bytes && p.dec.split_k == 0) {
+                p.dec = decode_geom(M, N, G, 1, chip, sg);
+                p.workspace = 0;
+            }
+            return p;
         }
     } else {
-        p.wide = wide_plan(M, N, G, split_k, sms, allow_cluster, sg, epi);
-        p.kernel = !p.wide.use_mid ? W4A16_KERNEL_TILE : p.wide.mid.mtc <= 64 ? W4A16_KERNEL_MID64 : W4A16_KERNEL_MID128;
-        p.workspace = split_k == 0 && p.wide.use_mid && p.wide.mid.cluster ? 0 : p.wide.workspace_bytes();
-        if (p.workspace > ws_bytes && !p.wide.use_mid && p.wide.tile.split_k == 0) {
-            p.wide.tile = tile_geom(M, N, G, 1, sms);
-            p.workspace = 0;
-        }
+        p.wide = wide_plan(M, N, G, split_k, chip, sg, epi);
+    }
+    p.kernel = !p.wide.use_mid ? W4A16_KERNEL_TILE : p.wide.mid.mtc <= 64 ? W4A16_KERNEL_MID64 : W4A16_KERNEL_MID128;
+    p.workspace = split_k == 0 && p.wide.use_mid && p.wide.mid.cluster ? 0 : p.wide.workspace_bytes();
+    if (p.workspace > ws_bytes && !p.wide.use_mid && p.wide.tile.split_k == 0) {
+        p.wide.tile = tile_geom(M, N, G, 1, chip.sms);
+        p.workspace = 0;
     }
     return p;
 }
@@ -755,17 +772,11 @@ size_t w4a16_packed_z_bytes(int N, int K, int group) {   // asymmetric formats; 
 
 int w4a16_choose_split_k_ex(int M, int N, int K, int group, int path) {
     std::lock_guard<std::mutex> lock(g_mu);
-    if (check_weight_shape(N, K, group) != W4A16_OK || M < 1) return 1;
-    const int G = K / kGroup, sg = kGroup / group, sms = sm_count_or_default();
-    const bool clusters = clusters_ok();
-    switch (resolve_path(M, path)) {
-        case W4A16_PATH_DECODE:
-            if (path == W4A16_PATH_AUTO && small_batch_takes_mid(M, N, G, sms, clusters, sg))
-                return choose_split_tile(M, N, G, sms, clusters, sg);
-            return choose_split_decode(M, N, G, sms, clusters, sg);
-        case W4A16_PATH_TILE: return choose_split_tile(M, N, G, sms, clusters, sg);
-        default: return 1;
-    }
+    if (check_weight_shape(N, K, group) != W4A16_OK || M < 1 || path < W4A16_PATH_AUTO || path > W4A16_PATH_TILE || path == W4A16_PATH_SIMPLE) return 1;
+    const int G = K / kGroup, sg = kGroup / group;
+    const Chip chip = chip_or_default();
+    const GemmPlan p = gemm_plan(M, N, G, sg, 0, path, false, chip, SIZE_MAX);
+    return p.kernel == W4A16_KERNEL_DECODE ? choose_split_decode(M, N, G, chip, sg) : nominal_split(p.wide, G);
 }
 int w4a16_choose_path(int M, int N, int K, int group) {
     std::lock_guard<std::mutex> lock(g_mu);
@@ -782,14 +793,16 @@ size_t w4a16_workspace_bytes(int M, int N, int K, int group, int split_k) {
     if (split_k == 1) return 0;
     // enough for whichever path w4a16_gemm / w4a16_gemm_ex may take with this split_k, on a device that places clusters
     // and on one that refused them (the schedule differs)
-    const int G = K / kGroup, sg = kGroup / group, sms = sm_count_or_default();
-    size_t need = simple_partial_bytes(M, N, split_k == 0 ? choose_split_decode(M, N, G, sms, true, sg) : split_k);
-    const size_t whole = decode_partial_bytes(decode_geom(M, N, G, split_k, sms, true, sg));   // (asked for by whole tiles too)
+    const int G = K / kGroup, sg = kGroup / group;
+    Chip chip = chip_or_default();
+    chip.clusters = true;
+    size_t need = simple_partial_bytes(M, N, split_k == 0 ? choose_split_decode(M, N, G, chip, sg) : split_k);
+    const size_t whole = decode_partial_bytes(decode_geom(M, N, G, split_k, chip, sg));   // (asked for by whole tiles too)
     if (whole > need) need = whole;
-    for (bool clusters : {true, false})
+    for (const Chip& c : {chip, without_clusters(chip)})
         for (bool epi : {false, true})
             for (int path : {W4A16_PATH_AUTO, W4A16_PATH_SIMPLE, W4A16_PATH_DECODE, W4A16_PATH_TILE}) {
-                const size_t n = gemm_plan(M, N, G, sg, split_k, path, epi, sms, clusters, SIZE_MAX).workspace;
+                const size_t n = gemm_plan(M, N, G, sg, split_k, path, epi, c, SIZE_MAX).workspace;
                 if (n > need) need = n;
             }
     return kWsFullHeaderBytes + need;
@@ -803,7 +816,7 @@ int w4a16_gemm_plan(int M, int N, int K, int group, int split_k, int path, int w
     if (M < 1) return W4A16_ERR_SHAPE;
     if (split_k < 0 || split_k > K / kGroup) return W4A16_ERR_SPLITK;
     if (path < W4A16_PATH_AUTO || path > W4A16_PATH_TILE) return W4A16_ERR_PATH;
-    const GemmPlan g = gemm_plan(M, N, K / kGroup, kGroup / group, split_k, path, with_epilogue != 0, sm_count_or_default(), clusters_ok(), SIZE_MAX);
+    const GemmPlan g = gemm_plan(M, N, K / kGroup, kGroup / group, split_k, path, with_epilogue != 0, chip_or_default(), SIZE_MAX);
     out->kernel = g.kernel;
     out->workspace_bytes = g.workspace == 0 ? 0 : kWsFullHeaderBytes + g.workspace;
     switch (g.kernel) {
@@ -1050,7 +1063,7 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
     // registered workspace: [small-M tickets and reserve: the documented header][partial results]
     unsigned char* ws_body = d->ws ? static_cast<unsigned char*>(d->ws) + kWsFullHeaderBytes : nullptr;
     const size_t ws_body_bytes = d->ws_bytes > kWsFullHeaderBytes ? d->ws_bytes - kWsFullHeaderBytes : 0;
-    const GemmPlan plan = gemm_plan(M, N, G, sg, split_k, path, bias != nullptr || act != W4A16_ACT_NONE, d->sm_count, d->cluster_ok, ws_body_bytes);
+    const GemmPlan plan = gemm_plan(M, N, G, sg, split_k, path, bias != nullptr || act != W4A16_ACT_NONE, chip_of(d), ws_body_bytes);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint32_t* Zw = sym ? nullptr : static_cast<const uint32_t*>(Z);
     Epilogue epi;
@@ -1348,10 +1361,10 @@ int w4a16_gemm_static_ws(const uint16_t* A, const void* Wq, const void* S, const
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return W4A16_ERR_CUDA;
 
-    DecodeGeom g = decode_geom(M, N, G, split_k, d->sm_count, false, sg);   // no clusters here: this entry point keeps the path it was built with
+    DecodeGeom g = decode_geom(M, N, G, split_k, without_clusters(chip_of(d)), sg);   // no clusters here: this entry point keeps the path it was built with
     // (balanced chunks give way to whole tiles, as in gemm_plan)
     if (g.split_k == 0 && kWsHeaderBytes + decode_partial_bytes(g) > (size_t)W4A16_STATIC_WS_BYTES)
-        g = decode_geom(M, N, G, 1, d->sm_count, false, sg);
+        g = decode_geom(M, N, G, 1, without_clusters(chip_of(d)), sg);
     if (g.mchunks > 65535 || (long)g.mchunks * (N / kTileN) > kMaxTickets) return W4A16_ERR_PATH;
     if (g.smem_bytes > d->max_smem_optin) return W4A16_ERR_PATH;
     // the whole scratch need of this shape must fit the built-in array, or nothing is launched (a schedule of
