@@ -38,7 +38,13 @@ SWEEP_K, SWEEP_N, SWEEP_M = 11008, 4096, (1, 2, 4, 8, 16)
 WORKLOAD = "config2_down_proj_decode_K11008_N4096_M1-2-4-8-16"
 MIN_ROTATION_BYTES = 512 << 20
 E2E_STREAMS = 2
-PATH_NAMES = {1: "gemm_simple_kernel", 2: "gemm_decode_kernel", 3: "gemm_tile_kernel"}
+KERNEL_NAMES = {1: "gemm_simple_kernel", 2: "gemm_decode_kernel", 3: "gemm_tile_kernel", 4: "gemm_mid_kernel<64>",
+                5: "gemm_mid_kernel<128>"}
+
+
+def _kernel_name(B, M, K, N, split_k=0):
+    return KERNEL_NAMES.get(B.w4a16_gemm_plan(M, N, K, split_k=split_k).kernel, "?")
+
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, from the ncu captures summarised under profiles/
 # (None = not captured since that kernel last changed).  Decode kernel: the mean of the five launches of a
@@ -387,7 +393,7 @@ def run_ours(args):
         med, mn = _time_calls(lambda: B.w4a16_gemm(acts[i], layer.take(), outs[i], split_k=splits[i]),
                               20, args.case_calls, torch)
         per_call[M] = med
-        rec = _case_record(2, "down_proj", M, K, N, med, mn, PATH_NAMES.get(B.w4a16_choose_path(M, N, K), "?"),
+        rec = _case_record(2, "down_proj", M, K, N, med, mn, _kernel_name(B, M, K, N, splits[i]),
                            peaks, wl)
         rec["split_k"] = splits[i]
         rec["chosen_split_k"] = B.w4a16_choose_split_k(M, N, K)
@@ -457,7 +463,7 @@ def run_ours(args):
                 med, mn = _time_calls(lambda: B.w4a16_gemm(A, cur.take(), C, split_k=0), 10,
                                       max(20, args.case_calls // 4), torch)
                 rec = _case_record(c.config, c.name, c.M, c.K, c.N, med, mn,
-                                   PATH_NAMES.get(B.w4a16_choose_path(c.M, c.N, c.K), "?"), peaks, wl)
+                                   _kernel_name(B, c.M, c.K, c.N), peaks, wl)
                 rec["split_k"] = 0
                 rec["chosen_split_k"] = B.w4a16_choose_split_k(c.M, c.N, c.K)
                 if c.config in (3, 6):
@@ -532,7 +538,7 @@ def run_ours(args):
     # ---- roofline of the dominant kernel.  Every launch of the timed region is gemm_decode_kernel (one
     # per GEMM), so its average launch duration over the region is region time / launches, and the
     # algorithmic bytes of an average launch are step bytes / launches per step.
-    dom_kernel = PATH_NAMES.get(B.w4a16_choose_path(SWEEP_M[0], N, K), "?")
+    dom_kernel = _kernel_name(B, SWEEP_M[0], K, N, splits[0])
     launch_us = elapsed / (args.steps * launches_per_step) * 1e6
     bytes_per_launch = step_bytes / launches_per_step
     achieved = bytes_per_launch / launch_us / 1e3
@@ -546,7 +552,7 @@ def run_ours(args):
                 "launch_us_by_M": {str(M): _r(per_call[M] * 1e6, 3) for M in SWEEP_M},
                 "frac_by_M": {str(M): _r(wl.algorithmic_bytes(M, K, N) / per_call[M] / 1e9 / hbm_peak)
                               for M in SWEEP_M},
-                "heaviest_launch": "M=%d: %s" % (heavy, PATH_NAMES.get(B.w4a16_choose_path(heavy, N, K), "?"))}
+                "heaviest_launch": "M=%d: %s" % (heavy, _kernel_name(B, heavy, K, N, splits[-1]))}
 
     # ---- CPU baseline: the oracle on whole steps (rank 0, N = 1 only)
     cpu = None

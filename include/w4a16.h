@@ -110,9 +110,8 @@ int w4a16_set_workspace(void *dev_ptr, size_t bytes);
  * w4a16_gemm accepts; >= 1.  `path` as in w4a16_gemm_ex. */
 int w4a16_choose_split_k(int M, int N, int K, int group);
 int w4a16_choose_split_k_ex(int M, int N, int K, int group, int path);
-/* The kernel path (W4A16_PATH_*) w4a16_gemm takes for a shape, or a negative error code.  (W4A16_PATH_DECODE
- * for every M <= 16, also where w4a16_gemm with split_k == 0 hands 9 to 16 rows of a long shape to the tcgen05
- * kernel; forcing the path forces the kernel.) */
+/* The kernel path (W4A16_PATH_*) w4a16_gemm takes for a shape with split_k == 0, or a negative error code.  (9 to 16
+ * rows of a long shape go to W4A16_PATH_TILE; with an explicit split_k every M <= 16 runs on W4A16_PATH_DECODE.) */
 int w4a16_choose_path(int M, int N, int K, int group);
 
 /* What w4a16_gemm_fmt runs for these arguments on the current device (on a host without one: what a B200 would run),

@@ -781,7 +781,8 @@ int w4a16_choose_split_k_ex(int M, int N, int K, int group, int path) {
 int w4a16_choose_path(int M, int N, int K, int group) {
     std::lock_guard<std::mutex> lock(g_mu);
     if (check_weight_shape(N, K, group) != W4A16_OK || M < 1) return W4A16_ERR_SHAPE;
-    return resolve_path(M, W4A16_PATH_AUTO);
+    const GemmPlan p = gemm_plan(M, N, K / kGroup, kGroup / group, 0, W4A16_PATH_AUTO, false, chip_or_default(), SIZE_MAX);
+    return p.kernel == W4A16_KERNEL_DECODE ? W4A16_PATH_DECODE : W4A16_PATH_TILE;
 }
 int w4a16_choose_split_k(int M, int N, int K, int group) {
     return w4a16_choose_split_k_ex(M, N, K, group, W4A16_PATH_AUTO);

@@ -107,11 +107,17 @@ def test_path_and_schedule_rules_at_the_benchmark_shapes(lib):
     DECODE, TILE = 2, 3
     path = lambda M, N, K: lib.w4a16_choose_path(M, N, K, 128)
     split = lambda M, N, K: lib.w4a16_choose_split_k(M, N, K, 128)
-    # up to 16 rows (one pass of the warp-MMA kernel over the weights): always that kernel
+    # up to 16 rows (one pass of the warp-MMA kernel over the weights): that kernel, but for long shapes from 9 rows on
     for N, K in [(4096, 4096), (4096, 11008), (8192, 28672), (22016, 4096), (1536, 6144), (12288, 4096)]:
         for M in (1, 4, 8, 9, 16):
-            assert path(M, N, K) == DECODE
+            assert path(M, N, K) == (TILE if M > 8 and (N, K) in [(8192, 28672), (22016, 4096), (12288, 4096)] else DECODE)
     assert split(16, 4096, 11008) == 4
+    # path and split are those of the plan that the call itself makes, and forcing them gives the same plan
+    for M, N, K in [(9, 22016, 4096), (16, 12288, 4096), (16, 4096, 11008), (8, 8192, 28672), (32, 4096, 4096), (600, 8192, 8192)]:
+        plan = B.w4a16_gemm_plan(M, N, K)
+        assert path(M, N, K) == (DECODE if plan.kernel == B.KERNEL_DECODE else TILE)
+        forced = B.w4a16_gemm_plan(M, N, K, path=path(M, N, K))
+        assert (forced.kernel, forced.tile_rows, forced.split_k) == (plan.kernel, plan.tile_rows, plan.split_k)
     # above 16 rows: tcgen05
     for M in (17, 32, 64, 256, 4096):
         assert path(M, 4096, 11008) == TILE
