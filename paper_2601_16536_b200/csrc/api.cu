@@ -684,10 +684,14 @@ size_t decode_scratch(const DecodeGeom& g, int split_k) {
     return g.split_k == 1 || (split_k == 0 && g.cluster) ? 0 : decode_partial_bytes(g);
 }
 
+// Can the warp-MMA kernel number this launch's batch chunks and tickets?
+bool decode_runs(const DecodeGeom& g, int N) { return g.mchunks <= 65535 && (long)g.mchunks * (N / kTileN) <= kMaxTickets; }
+
 // What a GEMM call runs: kernel, schedule and the workspace behind the header that it asks for (0: none).  The entry points
 // and the queries all come here, with the group's scale rows per block (sg): whether a cluster's exchange buffer fits, and
 // with it the number of slices, depends on them.
 struct GemmPlan {
+    int rc;              // W4A16_OK, or why the kernel cannot run the shape
     int kernel;          // W4A16_KERNEL_*
     int split_simple;
     DecodeGeom dec;
@@ -698,11 +702,13 @@ struct GemmPlan {
 // ask for none, and balanced chunks, which cross tile boundaries, give way to whole tiles where `ws_bytes` does not hold them.
 GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, bool epi, const Chip& chip, size_t ws_bytes) {
     GemmPlan p;
+    p.rc = W4A16_OK;
     const int path = resolve_path(M, path_asked);
     if (path == W4A16_PATH_SIMPLE) {
         p.kernel = W4A16_KERNEL_SIMPLE;
         p.split_simple = split_k == 0 ? choose_split_decode(M, N, G, chip, sg) : split_k;
         p.workspace = p.split_simple > 1 ? simple_partial_bytes(M, N, p.split_simple) : 0;
+        if ((M + kSimpleMB - 1) / kSimpleMB > 65535) p.rc = W4A16_ERR_PATH;
         return p;
     }
     if (path == W4A16_PATH_DECODE) {
@@ -715,6 +721,7 @@ GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, boo
                 p.dec = decode_geom(M, N, G, 1, chip, sg);
                 p.workspace = 0;
             }
+            if (!decode_runs(p.dec, N)) p.rc = W4A16_ERR_PATH;
             return p;
         }
     } else {
@@ -726,6 +733,12 @@ GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, boo
         p.wide.tile = tile_geom(M, N, G, 1, chip.sms);
         p.workspace = 0;
     }
+    // 32-bit arithmetic: the kernels count units and chunks, the kernel that sums slices the rows of all tiles
+    const bool mid = p.wide.use_mid;
+    const long long tiles = mid ? p.wide.mid.tiles : p.wide.tile.tiles;
+    const bool summed = mid ? p.wide.mid.split_k != 1 && !p.wide.mid.cluster : p.wide.tile.split_k != 1;
+    const int units = mid ? p.wide.mid.split_k : G, rows = !summed ? 0 : mid ? p.wide.mid.mt : p.wide.tile.mt;
+    if (tiles * (units > rows ? units : rows) >= (1ll << 31)) p.rc = W4A16_ERR_SHAPE;
     return p;
 }
 
@@ -818,6 +831,7 @@ int w4a16_gemm_plan(int M, int N, int K, int group, int split_k, int path, int w
     if (split_k < 0 || split_k > K / kGroup) return W4A16_ERR_SPLITK;
     if (path < W4A16_PATH_AUTO || path > W4A16_PATH_TILE) return W4A16_ERR_PATH;
     const GemmPlan g = gemm_plan(M, N, K / kGroup, kGroup / group, split_k, path, with_epilogue != 0, chip_or_default(), SIZE_MAX);
+    if (g.rc != W4A16_OK) return g.rc;
     out->kernel = g.kernel;
     out->workspace_bytes = g.workspace == 0 ? 0 : kWsFullHeaderBytes + g.workspace;
     switch (g.kernel) {
@@ -1065,6 +1079,7 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
     unsigned char* ws_body = d->ws ? static_cast<unsigned char*>(d->ws) + kWsFullHeaderBytes : nullptr;
     const size_t ws_body_bytes = d->ws_bytes > kWsFullHeaderBytes ? d->ws_bytes - kWsFullHeaderBytes : 0;
     const GemmPlan plan = gemm_plan(M, N, G, sg, split_k, path, bias != nullptr || act != W4A16_ACT_NONE, chip_of(d), ws_body_bytes);
+    if (plan.rc != W4A16_OK) return plan.rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint32_t* Zw = sym ? nullptr : static_cast<const uint32_t*>(Z);
     Epilogue epi;
@@ -1074,7 +1089,6 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         split_k = plan.split_simple;
         if (ws_body_bytes < plan.workspace) return W4A16_ERR_WORKSPACE;
         int mchunks = (M + kSimpleMB - 1) / kSimpleMB;
-        if (mchunks > 65535) return W4A16_ERR_PATH;
         float* partials = reinterpret_cast<float*>(ws_body);
         dim3 grid(N / kTileN, mchunks, split_k);
         if (bf)
@@ -1100,7 +1114,6 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         const MidGeom& g = plan.wide.mid;
         if (g.smem_bytes > d->max_smem_optin) return W4A16_ERR_PATH;
         if (ws_body_bytes < plan.workspace) return W4A16_ERR_WORKSPACE;
-        if ((long long)g.tiles * (g.split_k > g.mt ? g.split_k : g.mt) >= (1ll << 31)) return W4A16_ERR_SHAPE;   // (32-bit chunk arithmetic)
         CUtensorMap tmap;
         if (!make_act_tensor_map(&tmap, A, M, K, g.mt, mid_stage_k(g.mtc))) return W4A16_ERR_CUDA;
         MidParams p;
@@ -1168,8 +1181,6 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         const TileGeom& g = plan.wide.tile;
         if (g.smem_bytes > d->max_smem_optin) return W4A16_ERR_PATH;
         if (ws_body_bytes < plan.workspace) return W4A16_ERR_WORKSPACE;
-        // (the kernel's chunk arithmetic is 32-bit)
-        if ((long long)g.tiles * G >= (1ll << 31)) return W4A16_ERR_SHAPE;
         CUtensorMap tmap;
         if (!make_act_tensor_map(&tmap, A, M, K, g.mt, kTileStageK)) return W4A16_ERR_CUDA;
         TileParams p;
@@ -1224,7 +1235,6 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
 
     // W4A16_KERNEL_DECODE
     const DecodeGeom& g = plan.dec;
-    if (g.mchunks > 65535 || (long)g.mchunks * (N / kTileN) > kMaxTickets) return W4A16_ERR_PATH;
     if (g.smem_bytes > d->max_smem_optin) return W4A16_ERR_PATH;
     if (ws_body_bytes < plan.workspace) return W4A16_ERR_WORKSPACE;
     DecodeParams p;
@@ -1366,7 +1376,7 @@ int w4a16_gemm_static_ws(const uint16_t* A, const void* Wq, const void* S, const
     // (balanced chunks give way to whole tiles, as in gemm_plan)
     if (g.split_k == 0 && kWsHeaderBytes + decode_partial_bytes(g) > (size_t)W4A16_STATIC_WS_BYTES)
         g = decode_geom(M, N, G, 1, without_clusters(chip_of(d)), sg);
-    if (g.mchunks > 65535 || (long)g.mchunks * (N / kTileN) > kMaxTickets) return W4A16_ERR_PATH;
+    if (!decode_runs(g, N)) return W4A16_ERR_PATH;
     if (g.smem_bytes > d->max_smem_optin) return W4A16_ERR_PATH;
     // the whole scratch need of this shape must fit the built-in array, or nothing is launched (a schedule of
     // whole tiles, split_k == 1, leaves no partial tiles and draws no tickets: it needs none)

@@ -336,7 +336,7 @@ tile_splitk_reduce_kernel(const float* __restrict__ ws, uint16_t* __restrict__ C
     __shared__ int chunks[3];                           // first and last contributor, slot of the first
     // the next kernel of the stream may start its prologue; the partial tiles are the previous kernel's output
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int r = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5);   // (tiles * mt < 2^31: the caller checks)
+    const int r = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5);   // (tiles * mt < 2^31: gemm_plan)
     const int T = fast_div(r, p.div_mt);                // tile = batch tile * n_tiles + column tile; mt % 16 == 0: one per block
     if (threadIdx.x == 0) {
         if (p.split_k > 0) {
