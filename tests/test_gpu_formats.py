@@ -126,9 +126,9 @@ def test_bias_and_activation_are_applied_before_the_final_rounding(path, M, act)
 
 @pytest.mark.parametrize("bf16", [False, True])
 def test_bias_and_activation_after_the_second_kernels_sum(bf16):
-    """256-row tiles in K slices: the partial tiles are summed by a kernel of their own, which then also adds
+    """Wide tiles in K slices: the partial tiles are summed by a kernel of their own, which then also adds
     the bias and applies the activation before the one rounding."""
-    M, K, N = 150, 1024, 1536
+    M, K, N = 200, 2048, 4224
     d = wl.make_problem(M, K, N, seed=911, bf16=bf16)
     pw = _pack(d, N, K, 128, False, bf16=bf16)
     r = np.random.Generator(np.random.PCG64(5))
@@ -142,6 +142,8 @@ def test_bias_and_activation_after_the_second_kernels_sum(bf16):
     ws = ensure_ws(M, N, K, (0, 4))
     ref = oracle.epilogue(oracle.gemm(d["A"], d["Wq"], d["S"], d["Z"], M, N, K, 128, bf16=bf16), bias, "silu")
     for split_k in (0, 4):
+        plan = B.w4a16_gemm_plan(M, N, K, split_k=split_k, path=B.PATH_TILE, with_epilogue=True)
+        assert plan.kernel == B.KERNEL_TILE and plan.split_k >= 2
         C = B.w4a16_gemm(_dev16(d["A"], bf16), pw, split_k=split_k, path=B.PATH_TILE, bias=_dev16(bias_bits, bf16), act=B.ACT_SILU)
         torch.cuda.synchronize()
         assert B.w4a16_device_status() == 0

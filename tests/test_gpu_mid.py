@@ -33,12 +33,18 @@ def test_exact_inputs_bit_equal_for_every_schedule(M, K, N, splits):
     del ws
 
 
-@pytest.mark.parametrize("M,K,N,splits", [
+@pytest.mark.parametrize("M,K,N,splits,kernel,rows", [
     # batch tiles of 96, 112, 128 rows in the two-CTA kernel (exchange on top of its rings), several of them, a ragged last one
-    (96, 640, 21952, (0, 1, 2)), (128, 1152, 11072, (0, 3)), (300, 1024, 12288, (0, 2)), (128, 384, 22016, (0, 3)),
-    # batch tiles of the wide-tile kernel that are not a power of two: 176, 208, 240 rows, whole tiles, slices, balanced chunks
-    (176, 2048, 3200, (0, 1, 3)), (777, 512, 5696, (0, 1, 2)), (470, 1536, 8256, (0, 1, 4)), (600, 1024, 8192, (0, 1))])
-def test_batch_tiles_above_64_rows_bit_equal(M, K, N, splits):
+    (96, 640, 21952, (0, 1, 2), B.KERNEL_MID128, 96), (300, 1024, 12288, (0, 2), B.KERNEL_MID128, 112),
+    (128, 384, 22016, (0, 3), B.KERNEL_MID128, 128),
+    # several batch tiles of the 64-row build
+    (128, 1152, 11072, (0, 3), B.KERNEL_MID64, 64), (176, 2048, 3200, (0, 1, 3), B.KERNEL_MID64, 64), (777, 512, 5696, (0, 1, 2), B.KERNEL_MID64, 64),
+    # batch tiles of the wide-tile kernel: ragged last ones, whole tiles and slices (balanced chunks: test_gpu_builds.py)
+    (470, 1536, 8256, (0, 1, 4), B.KERNEL_TILE, 240), (600, 1024, 8192, (0, 1), B.KERNEL_TILE, 160), (200, 2048, 4224, (0, 1, 3), B.KERNEL_TILE, 208)])
+def test_batch_tiles_above_64_rows_bit_equal(M, K, N, splits, kernel, rows):
+    for split_k in splits:
+        plan = B.w4a16_gemm_plan(M, N, K, split_k=split_k, path=B.PATH_TILE)
+        assert (plan.kernel, plan.tile_rows) == (kernel, rows)
     d = wl.make_exact_problem(M, K, N, seed=8100 + M)
     n0 = N - 192        # the last columns: a 64-column tail tile where there is one
     want = oracle.gemm_int(d["A_int"], d["Wq"][:, n0:].copy(), d["E"][:, n0:].copy(), d["Z"][:, n0:].copy(), M, 192, K, 128)

@@ -23,14 +23,14 @@ def _run(d, M, N, K, split_k, path=B.PATH_TILE):
     return C
 
 
-# (M, K, N): batch tiles of 16 / 32 / 64 / 128 / 256 rows with ragged tails, one and several column
-# tiles, a 64-column tail tile (N = 192, 320), one to many groups
+# (M, K, N): one and several batch tiles with ragged tails, one and several column tiles, a 64-column tail tile (N = 192, 320),
+# one to many groups.  (Which kernel a shape goes to is the plan's choice: test_gpu_builds.py and test_gpu_mid.py ask for it.)
 SHAPES = [(32, 128, 128), (1, 256, 128), (9, 640, 192), (16, 1152, 256), (17, 640, 192), (33, 384, 256), (64, 1152, 128),
           (100, 896, 320), (128, 512, 256), (129, 768, 128), (256, 2048, 384), (300, 1280, 192),
           (700, 640, 256),
-          # wide enough (twelve column tiles and more) for the 128- and 256-row batch tiles themselves
+          # more column tiles
           (120, 512, 1536), (300, 384, 1600),
-          # wide enough for 64-row batch tiles (more than 24 column tiles), with a 64-column tail tile
+          # more than 24 column tiles, with a 64-column tail tile
           (64, 640, 3328), (40, 1152, 3392)]
 
 
@@ -67,15 +67,17 @@ def test_tile_path_exact_inputs_bit_equal_for_every_split():
 
 
 def test_wide_batch_tiles_with_slices_bit_equal_for_every_split():
-    # Twelve column tiles keep the 256-row batch tile, and its K slices are summed by the second kernel
-    # (tile_splitk_reduce_kernel) instead of inside the GEMM kernel: same order, so with exact inputs the same
-    # bits as one slice, for a ragged batch (200 of 256 rows) and a ragged slice count (8 groups in 3 slices).
-    M, K, N = 200, 1024, 1536
-    d = wl.make_exact_problem(M, K, N, seed=7250)
-    want = oracle.gemm_int(d["A_int"], d["Wq"], d["E"], d["Z"], M, N, K, 128)
-    for split_k in (1, 0, 2, 3, 4, 8):
-        C = _run(d, M, N, K, split_k)
-        assert np.array_equal(c_bits(C), want), "split_k=%d" % split_k
+    # The K slices of the wide-tile kernel are summed by the second kernel (tile_splitk_reduce_kernel) in ascending order, so
+    # with exact inputs they give the same bits as one slice, for a ragged batch (200 of 208 rows) and ragged slice counts
+    # (16 blocks in 3 and 5 slices).  The first shape runs the two-CTA kernel, whose slices meet in a cluster.
+    for M, K, N, kernel, splits in ((200, 1024, 1536, B.KERNEL_MID64, (1, 0, 2, 3, 4, 8)), (200, 2048, 4224, B.KERNEL_TILE, (1, 0, 2, 3, 4, 5, 8))):
+        d = wl.make_exact_problem(M, K, N, seed=7250)
+        want = oracle.gemm_int(d["A_int"], d["Wq"], d["E"], d["Z"], M, N, K, 128)
+        for split_k in splits:
+            plan = B.w4a16_gemm_plan(M, N, K, split_k=split_k, path=B.PATH_TILE)
+            assert plan.kernel == kernel and plan.cluster == (kernel == B.KERNEL_MID64 and plan.split_k > 1)
+            C = _run(d, M, N, K, split_k)
+            assert np.array_equal(c_bits(C), want), "split_k=%d" % split_k
 
 
 def test_tile_path_bit_identical_run_to_run():
