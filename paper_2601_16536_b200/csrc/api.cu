@@ -928,16 +928,10 @@ int w4a16_dequant_fmt(const void* Wq, const void* S, const void* Z, uint16_t* W1
     DeviceState* d = nullptr;
     if ((rc = current_device(&d)) != W4A16_OK) return rc;
     if (!d->is_sm100) return W4A16_ERR_ARCH;
-    const int blocks = (int)((long long)(K / kGroup) * (N / kTileN)), per = kBlockKernelThreads / 32;
-    const unsigned grid = (unsigned)((blocks + per - 1) / per);
-    const uint32_t* z = sym ? nullptr : static_cast<const uint32_t*>(Z);
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (bf)
-        dequant_kernel<true><<<grid, kBlockKernelThreads, 0, st>>>(static_cast<const uint32_t*>(Wq), static_cast<const uint16_t*>(S),
-                                                                   z, W16, N, K / kGroup, kGroup / group, blocks);
-    else
-        dequant_kernel<false><<<grid, kBlockKernelThreads, 0, st>>>(static_cast<const uint32_t*>(Wq), static_cast<const uint16_t*>(S),
-                                                                    z, W16, N, K / kGroup, kGroup / group, blocks);
+    const unsigned blocks = (unsigned)((long long)(K / kGroup) * (N / kTileN));
+    (bf ? dequant_kernel<true> : dequant_kernel<false>)<<<blocks, kBlockKernelThreads, 0, static_cast<cudaStream_t>(stream)>>>(
+        static_cast<const uint32_t*>(Wq), static_cast<const uint16_t*>(S), sym ? nullptr : static_cast<const uint32_t*>(Z), W16, N,
+        K / kGroup, kGroup / group);
     return cudaGetLastError() == cudaSuccess ? W4A16_OK : W4A16_ERR_CUDA;
 }
 

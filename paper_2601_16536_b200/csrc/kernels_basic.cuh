@@ -7,7 +7,7 @@
 namespace w4a16 {
 
 // The three kernels below work on whole blocks (64 columns x 128 k), numbered with the column tile fastest, so that the
-// CTAs that run together touch neighbouring columns of the same rows.  They are bound by HBM.
+// CTAs that run together touch neighbouring columns of the same rows.
 constexpr int kBlockKernelThreads = 128;
 struct BlockPos {
     int t, g;        // column tile, k block
@@ -194,21 +194,21 @@ quantize_kernel(const uint16_t* __restrict__ W16, uint32_t* __restrict__ Wq, uin
 // ------------------------------------------------------------------ dequant
 // Algorithm 1, Phase 1 as a standalone kernel: w16 = rn((q - z) * s) in the 16-bit format: (q - z) is formed exactly and
 // multiplied by s with one multiply (round-to-nearest-even, subnormals kept).  Z == nullptr: symmetric format, z = 8.
-// One warp per block: a lane takes 8 neighbouring columns x 32 k (eight 16-byte loads in flight), swaps the halves of
-// neighbouring columns' registers and stores 16 bytes of a row at a time, eight lanes one 128-byte line of the row.
-// K = N = 8192: a thread per word with 2-byte stores 68 us, this form 31 us (HBM floor 25.6).
+// One CTA per block, a warp for 32 k of it: a lane takes 8 neighbouring columns x 8 k (a word of each column; four lanes read
+// a column's 16 bytes), swaps the halves of neighbouring columns' registers and stores 16 bytes of a row at a time, eight
+// lanes one 128-byte line of the row.  us, a thread per word with 2-byte stores / a warp per block with 16-byte loads / this
+// form: K = N = 8192 68 / 31.8 / 31.4 (HBM floor 25.6), K = N = 4096 18.7 / 10.5 / 8.5, K = 128 / N = 8192 4.2 / 5.1 / 4.1: one
+// warp's way through a whole block was too long for a matrix of few.
 template <bool BF>
 __global__ void __launch_bounds__(kBlockKernelThreads)
 dequant_kernel(const uint32_t* __restrict__ Wq, const uint16_t* __restrict__ S, const uint32_t* __restrict__ Z,
-               uint16_t* __restrict__ W16, int N, int G, int sg, int blocks) {
-    const int b = blockIdx.x * (kBlockKernelThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (b >= blocks) return;
-    const BlockPos pos(b, N / kTileN, G);
-    const int rb = lane & 7, kq = lane >> 3;      // columns 8 rb .. + 7, k = 32 kq .. + 31 of the block
-    const uint4* src = reinterpret_cast<const uint4*>(Wq + pos.blk * kBlockWords);
-    uint4 w[8];
+               uint16_t* __restrict__ W16, int N, int G, int sg) {
+    const BlockPos pos(blockIdx.x, N / kTileN, G);
+    const int kq = threadIdx.x >> 5, kw = (threadIdx.x >> 3) & 3, rb = threadIdx.x & 7;   // columns 8 rb .. + 7, k = 32 kq + 8 kw .. + 7
+    const uint32_t* src = Wq + pos.blk * kBlockWords + kw;
+    uint32_t w[8];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) w[c] = __ldg(src + block_word_index(8 * rb + c, 4 * kq) / 4);
+    for (int c = 0; c < 8; ++c) w[c] = __ldg(src + block_word_index(8 * rb + c, 4 * kq));
     const size_t row = pos.blk * sg + kq * sg / 4;
     // column 8 rb + c sits at position p0 + 4 c of a row of scales / zero points
     const int p0 = sz_perm(8 * rb);
@@ -223,23 +223,17 @@ dequant_kernel(const uint32_t* __restrict__ Wq, const uint16_t* __restrict__ S, 
         zlo[c] = zconst_lo<BF>(z);
         zhi[c] = zconst_hi<BF>(z);
     }
-    uint16_t* dst = W16 + (size_t)(pos.g * kGroup + 32 * kq) * N + (size_t)pos.t * kTileN + 8 * rb;
+    uint16_t* dst = W16 + (size_t)(pos.g * kGroup + 32 * kq + 8 * kw) * N + (size_t)pos.t * kTileN + 8 * rb;
+    Pack8 f[8];
 #pragma unroll
-    for (int kw = 0; kw < 4; ++kw) {
-        Pack8 f[8];
+    for (int c = 0; c < 8; ++c) f[c] = dequant_word<BF>(w[c], zlo[c], zhi[c], s2[c]);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const uint32_t word = kw == 0 ? w[c].x : kw == 1 ? w[c].y : kw == 2 ? w[c].z : w[c].w;
-            f[c] = dequant_word<BF>(word, zlo[c], zhi[c], s2[c]);
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            uint16_t* p = dst + (size_t)(8 * kw + 2 * j) * N;
-            *reinterpret_cast<uint4*>(p) = make_uint4(__byte_perm(f[0].h[j], f[1].h[j], 0x5410), __byte_perm(f[2].h[j], f[3].h[j], 0x5410),
-                                                      __byte_perm(f[4].h[j], f[5].h[j], 0x5410), __byte_perm(f[6].h[j], f[7].h[j], 0x5410));
-            *reinterpret_cast<uint4*>(p + N) = make_uint4(__byte_perm(f[0].h[j], f[1].h[j], 0x7632), __byte_perm(f[2].h[j], f[3].h[j], 0x7632),
-                                                          __byte_perm(f[4].h[j], f[5].h[j], 0x7632), __byte_perm(f[6].h[j], f[7].h[j], 0x7632));
-        }
+    for (int j = 0; j < 4; ++j) {
+        uint16_t* p = dst + (size_t)(2 * j) * N;
+        *reinterpret_cast<uint4*>(p) = make_uint4(__byte_perm(f[0].h[j], f[1].h[j], 0x5410), __byte_perm(f[2].h[j], f[3].h[j], 0x5410),
+                                                  __byte_perm(f[4].h[j], f[5].h[j], 0x5410), __byte_perm(f[6].h[j], f[7].h[j], 0x5410));
+        *reinterpret_cast<uint4*>(p + N) = make_uint4(__byte_perm(f[0].h[j], f[1].h[j], 0x7632), __byte_perm(f[2].h[j], f[3].h[j], 0x7632),
+                                                      __byte_perm(f[4].h[j], f[5].h[j], 0x7632), __byte_perm(f[6].h[j], f[7].h[j], 0x7632));
     }
 }
 
