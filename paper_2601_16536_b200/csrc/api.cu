@@ -196,7 +196,9 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, const Chip& chip, int s
         auto take = [&](int s, long cost) {
             if (g.cost == 0 || cost < g.cost) { g.cost = cost; split_k = s; }
         };
-        if (T > slots) take(1, g.mb == 1 ? 1500 + unit_ns * ((units * 23 / 20 + slots - 1) / slots) : 4000 + unit_ns * units * 13 / (10 * slots));
+        // (several batch chunks, which only a forced path has, fill the SMs as few rows do)
+        const bool few = g.mb == 1 || g.mchunks > 1;
+        if (T > slots) take(1, few ? 1500 + wide + unit_ns * ((units * 23 / 20 + slots - 1) / slots) : 4000 + unit_ns * units * 13 / (10 * slots));
         else take(1, 1500 + wide + unit_ns * G);
         if (allow_cluster && g.mchunks == 1) {
             // The last clusters that fit find a place late, while the launch in front still holds its SMs: from 7/8 or 8/9 of them
@@ -229,7 +231,7 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, const Chip& chip, int s
         if (s0 > kDecMaxCluster || (s0 >= 2 && !(allow_cluster && g.mchunks == 1)))
             take(s0, 4000 + wide + add_ns * s0 + unit_ns * ((G + s0 - 1) / s0));
         const long share = slots / T > 3 ? slots / T - 3 : 0;      // (contributors of a tile, beyond what the constant holds)
-        take(0, (g.mb == 1 ? 5700 : 7500) + add_ns * share + unit_ns * ((units * 27 / 25 + slots - 1) / slots));
+        take(0, (g.mb == 1 ? 5700 : few ? 6400 : 7500) + add_ns * share + unit_ns * ((units * 27 / 25 + slots - 1) / slots));
     }
     g.split_k = split_k;
     if (split_k == 0) {
