@@ -231,7 +231,7 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, const Chip& chip, int s
         if (s0 > kDecMaxCluster || (s0 >= 2 && !(allow_cluster && g.mchunks == 1)))
             take(s0, 4000 + wide + add_ns * s0 + unit_ns * ((G + s0 - 1) / s0));
         const long share = slots / T > 3 ? slots / T - 3 : 0;      // (contributors of a tile, beyond what the constant holds)
-        take(0, (g.mb == 1 ? 5700 : few ? 6400 : 7500) + add_ns * share + unit_ns * ((units * 27 / 25 + slots - 1) / slots));
+        take(0, (g.mb == 1 ? 5700 : 7500) + add_ns * share + unit_ns * ((units * 27 / 25 + slots - 1) / slots));
     }
     g.split_k = split_k;
     if (split_k == 0) {
