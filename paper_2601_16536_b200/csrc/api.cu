@@ -210,7 +210,10 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, const Chip& chip, int s
             for_each_size<2, kDecMaxCluster>([&](auto size) {
                 constexpr int s = decltype(size)::value;
                 const int room = max_clusters[s];
-                if (s > G || T + 2 > room) return;
+                // Every place for pairs (us, M = 4, 147 tiles: K = 2048 5.0, whole tiles 6.1; K = 7168 10.3, balanced 14.4; K = 14336
+                // 17.5 and 21.5; 148: 10.3 and 12.4, but one whole tile per SM 4.95 to 5.0 at K = 2048, M = 16 5.9 to 6.2).  Of the
+                // larger ones the last two cost the time below and more (M = 4, K = 7168: 72 in four 10.7, in three 8.0).
+                if (s > G || T + (s > 2 ? 2 : G < 24 ? 1 : 0) > room) return;
                 const int u = (G + s - 1) / s, ctas = T * s;
                 long wait = 0;
                 if (s == 3 || s == 5) {

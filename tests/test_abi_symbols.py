@@ -170,6 +170,10 @@ def test_slices_of_few_column_tiles_meet_in_a_cluster(lib):
         p = B.w4a16_gemm_plan(M, N, K, group, 0, B.PATH_DECODE)
         assert (p.split_k, p.cluster) == (6, 1), (M, N, K, group)
     assert B.w4a16_gemm_plan(2, 640, 19072, 64).split_k == 25        # 7.9 us; six in a cluster 9.3
+    # pairs of CTAs up to the last two places (147 tiles 10.3 us, balanced 14.4; 148 10.3 and 12.4), but one tile per SM
+    # of a short K stays whole (K = 2048: 5.9, pairs 6.2)
+    for M, N, K, split in [(4, 64 * 147, 7168, 2), (16, 64 * 148, 7168, 2), (16, 64 * 147, 2048, 2), (16, 64 * 148, 2048, 1)]:
+        assert B.w4a16_gemm_plan(M, N, K, 128, 0, B.PATH_DECODE).split_k == split, (M, N, K)
 
 
 def test_schedules_of_few_or_whole_column_tiles_above_16_rows(lib):
