@@ -101,7 +101,7 @@ size_t w4a16_packed_z_bytes(int N, int K, int group);
  * owned by the caller and must outlive every gemm call enqueued while it is registered.  The
  * call zeroes that header (the kernels' ticket counters) on the default stream and waits.  gemm calls that need the workspace and overlap on
  * the GPU (different streams) race on it; serialise them or use split_k = 1. */
-#define W4A16_WORKSPACE_HEADER_BYTES (16384u + 131072u)
+#define W4A16_WORKSPACE_HEADER_BYTES (16384u + 131072u)   /* ticket counters; 128 KiB that no kernel uses, kept for the buffers of existing callers */
 size_t w4a16_workspace_bytes(int M, int N, int K, int group, int split_k);
 int w4a16_set_workspace(void *dev_ptr, size_t bytes);
 
@@ -258,9 +258,11 @@ int w4a16_gemm_static_ws(const uint16_t *A, const void *Wq, const void *S, const
 /* Every wait inside the kernels on a barrier or on another CTA has a limit (two seconds): a
  * wait that runs out records a code in a status word on the device, the kernel releases what
  * it holds and returns.  (The one instruction that can block without a limit is the tensor-
- * memory allocation of the tile kernel; it cannot wait on another CTA of this library because
- * the kernel asks for more than half of an SM's shared memory, so two of its CTAs never share
- * an SM, and each frees its columns before it returns.)
+ * memory allocation of the two tcgen05 kernels.  Two CTAs of the wide one never share an SM, by
+ * their shared memory, and two of the other take half of the columns each; but a CTA of one may
+ * find the columns held by one of the other.  That one frees them before it returns, and cannot
+ * itself be waiting for the blocked one: every CTA of a launch allocates before it lets the next
+ * launch of its stream start, so a holder waits only for launches that have all their columns.)
  * w4a16_device_status synchronises the current device, copies the word to *status_out
  * (0 = no kernel gave up since the last call; bit 0 = a barrier wait ran out) and clears it.
  * If it was nonzero the call also zeroes the ticket counters of the registered workspace (a

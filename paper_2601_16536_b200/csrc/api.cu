@@ -141,15 +141,16 @@ void for_each_size(const F& f) {
 // ---- decode-path launch geometry ------------------------------------------------
 int decode_mb(int M) { return M <= 8 ? 1 : 2; }
 
-// The decode kernel is persistent: `ctas` CTAs per batch chunk (two per SM with about 100 KiB of
-// shared memory each, or three with about 60 KiB; 9 warps), `nchunks` chunks of work units dealt to
-// them.
+// The decode kernel is persistent: `ctas` CTAs per batch chunk (9 warps, about 100 KiB of shared
+// memory), `nchunks` chunks of work units dealt to them.  Two CTAs per SM: three, with a two-stage ring
+// and 72 registers, are behind everywhere but at K = 4096 / N = 12288, by 3 % (33.8 against 34.8 us at
+// K = 28672 / N = 8192, 15.0 against 15.8 at N = 22016).
+constexpr int kDecCtasPerSm = 2;
 struct DecodeGeom {
     int mb, mchunks, stages, smem_bytes, ctas, nchunks;
     int stage_bytes;   // ring stride for the batch rows a CTA has
     int prefetch;      // stages whose weights are requested before the wait for the previous kernel
     bool a_box;        // activation rows of a stage as one tensor copy (kernel_decode.cuh)
-    int cps;       // CTAs per SM the launch is sized for (2 or 3)
     long cost;     // ns by the cost model (automatic schedules)
     bool cluster;  // one thread-block cluster of split_k CTAs per tile: partial tiles meet in shared memory
     int split_k;   // what the kernel runs: 0 = balanced chunks, S >= 1 = S slices per tile
@@ -169,12 +170,7 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, const Chip& chip, int s
     const int T = N / kTileN;
     const long units = (long)T * G;
     const bool allow_cluster = chip.clusters;
-    // Two CTAs per SM.  (Three, with a two-stage ring and 72 registers, were ahead on long launches
-    // while every exchange went through the workspace; with the cluster exchange two are ahead again
-    // everywhere but K = 4096 / N = 12288, by 3 %: 33.8 against 34.8 us at K = 28672 / N = 8192, 15.0
-    // against 15.8 at N = 22016.  The kernel keeps the template parameter.)
-    g.cps = 2;
-    long slots = (long)g.cps * chip.sms;
+    const long slots = (long)kDecCtasPerSm * chip.sms;
     g.cost = 0;
     if (split_k == 0) {
         // How the unit range is cut when the caller leaves it open.  Balanced chunks use every CTA slot, but a chunk that
@@ -250,7 +246,7 @@ DecodeGeom decode_geom(int M, int N, int G, int split_k, const Chip& chip, int s
     // S slices per tile, every slice on a CTA of its own, one batch chunk: the S CTAs of a tile form a
     // cluster and exchange their partial tiles through distributed shared memory
     g.cluster = allow_cluster && split_k >= 2 && split_k <= kDecMaxCluster && g.nchunks == g.ctas && g.mchunks == 1;
-    const int budget = (227 * 1024) / g.cps - 1024;   // per CTA
+    const int budget = (227 * 1024) / kDecCtasPerSm - 1024;   // per CTA
     const int xs = g.cluster ? split_k : 0;   // slices that meet in the exchange buffer
     const int rows = M < 8 * g.mb ? M : 8 * g.mb;   // batch rows of a CTA (the last chunk of a large M may have fewer)
     // (the box is 8 chunks of 64 k long: K >= 512)
@@ -377,7 +373,8 @@ TileGeom tile_geom_rows(int mt, int M, int N, int G, int split_k, int sms) {
     st -= st % 2;
     g.stages = st;
     g.smem_bytes = kTileBarBytes + 1024 + st * tile_stage_bytes(mt);
-    // each CTA takes the SM's whole tensor memory: ask for enough shared memory that two never share an SM
+    // each CTA takes the SM's whole tensor memory: ask for enough shared memory that two never share an SM (beside
+    // one of the kernel for small batch tiles its allocation waits until that one ends: see w4a16_device_status in the header)
     if (g.smem_bytes < 120 * 1024) g.smem_bytes = 120 * 1024;
     return g;
 }

@@ -24,7 +24,7 @@
 // casts to FP16 and writes C (Algorithm 1, Phase 3, inside the same launch).  No CTA
 // waits for another one, and the order of the sum does not depend on which CTA comes
 // last, so results are bit-identical from run to run.  Where the S slices of a tile each
-// have a CTA and S <= 4, the launch is made of clusters of S CTAs and the partial tiles go
+// have a CTA and S <= 6, the launch is made of clusters of S CTAs and the partial tiles go
 // through the first CTA's shared memory instead (template parameter CL below): same order
 // of the sum, same bits, about half the latency.
 #pragma once
@@ -149,15 +149,6 @@ template <int OFF>
 __device__ __forceinline__ uint2 lds64(uint32_t addr) {
     uint2 v;
     asm volatile("ld.shared.v2.u32 {%0, %1}, [%2 + %3];" : "=r"(v.x), "=r"(v.y) : "r"(addr), "n"(OFF) : "memory");
-    return v;
-}
-template <int OFF>
-__device__ __forceinline__ uint4 lds128(uint32_t addr) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4 + %5];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "r"(addr), "n"(OFF)
-                 : "memory");
     return v;
 }
 template <int OFF>

@@ -91,16 +91,6 @@ struct MidChunk {
     }
 };
 
-template <int OFF>
-__device__ __forceinline__ uint4 mid_lds128(uint32_t addr) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4 + %5];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "r"(addr), "n"(OFF)
-                 : "memory");
-    return v;
-}
-
 template <int MTC, int SG, bool BF, bool SYM>
 __global__ void __launch_bounds__(kMidThreads, 2)
 gemm_mid_kernel(const __grid_constant__ CUtensorMap tmap_a, const MidParams p) {
@@ -110,6 +100,11 @@ gemm_mid_kernel(const __grid_constant__ CUtensorMap tmap_a, const MidParams p) {
     constexpr int kStageK = mid_stage_k(MTC);
     constexpr int kSPU = kGroup / kStageK;            // operand slots per unit
     constexpr int R = mid_slots(MTC);
+    // A set does not visit every ring turn of a slot (three slots, two sets; odd segments), so its wait for "retired" may
+    // skip a phase, and a parity wait cannot tell a phase from the one two turns back.  That one is over all the same: the
+    // one issuer's commits complete in order, the set's stage before this one (at most kSPU + 1 stages back) has waited for
+    // that commit or a later one, and earlier segments' commits are behind the epilogue's wait for d_full.
+    static_assert(R >= kSPU + 1, "a slot's retired barrier");
     constexpr int kSlotCols = kStageK / 2;
     constexpr bool kOverlay = MTC > 64;               // exchange buffer on top of the rings
     constexpr int kWStage = mid_wstage_bytes(SG);
@@ -300,10 +295,10 @@ gemm_mid_kernel(const __grid_constant__ CUtensorMap tmap_a, const MidParams p) {
                 if (!mbar_wait(w0 + woff + kWFull, wph)) { ok = false; break; }
                 uint4 w[4];
                 uint32_t s[SG], zw[SG];
-                w[0] = mid_lds128<0>(w_a0 + woff);
-                w[1] = mid_lds128<0>(w_a1 + woff);
-                w[2] = mid_lds128<2048>(w_a0 + woff);
-                w[3] = mid_lds128<2048>(w_a1 + woff);
+                w[0] = lds128<0>(w_a0 + woff);
+                w[1] = lds128<0>(w_a1 + woff);
+                w[2] = lds128<2048>(w_a0 + woff);
+                w[3] = lds128<2048>(w_a1 + woff);
 #pragma unroll
                 for (int i = 0; i < SG; ++i) {
                     asm volatile("{\n\t.reg .b16 t;\n\tld.shared.u16 t, [%1];\n\tcvt.u32.u16 %0, t;\n\t}"
@@ -446,7 +441,7 @@ gemm_mid_kernel(const __grid_constant__ CUtensorMap tmap_a, const MidParams p) {
                 const uint32_t src = xch + (uint32_t)(((q - rank * per) * kTileCols + row) * 16);
                 for (int s = 0; s < S; ++s) {
                     uint4 x = make_uint4(own[0], own[1], own[2], own[3]);
-                    if (s != rank) x = mid_lds128<0>(src + (uint32_t)((s - (s > rank ? 1 : 0)) * xslot));
+                    if (s != rank) x = lds128<0>(src + (uint32_t)((s - (s > rank ? 1 : 0)) * xslot));
                     if (s == 0) {
                         acc = make_float4(__uint_as_float(x.x), __uint_as_float(x.y), __uint_as_float(x.z), __uint_as_float(x.w));
                     } else {

@@ -53,6 +53,7 @@ namespace w4a16 {
 constexpr int kTileCols = 128;                      // n per CTA tile = UMMA M
 constexpr int kTileBoxK = 64;                       // k per activation TMA box (one 128-byte swizzle row)
 constexpr int kTileStageK = 64;                     // k per pipeline stage
+constexpr int kTileSPU = kGroup / kTileStageK;      // stages per unit
 constexpr int kTileDequantWarps = 16;               // four sets of four (one warp per TMEM lane quarter)
 constexpr int kTileSets = kTileDequantWarps / 4;
 constexpr int kTileThreads = (2 + kTileDequantWarps) * 32;   // producer, issuer, dequant / epilogue warps
@@ -207,9 +208,8 @@ struct SegWalk {
     int left;          // units of the chunk after this segment
     bool first;        // first segment of its chunk
     uint32_t n0;       // stages of this CTA before the segment (ring positions derive from it)
-    const int spu;     // stages per unit (group): 1 or 2
-    __device__ __forceinline__ SegWalk(const TileParams& p_, int spu_)
-        : p(p_), ci((int)blockIdx.x), t(0), g0(0), units(0), left(0), first(true), n0(0), spu(spu_) {
+    __device__ __forceinline__ explicit SegWalk(const TileParams& p_)
+        : p(p_), ci((int)blockIdx.x), t(0), g0(0), units(0), left(0), first(true), n0(0) {
         load_chunk();
     }
     __device__ __forceinline__ void load_chunk() {
@@ -224,7 +224,7 @@ struct SegWalk {
     }
     __device__ __forceinline__ bool valid() const { return ci < p.nchunks; }
     __device__ __forceinline__ void next() {
-        n0 += (uint32_t)(spu * units);
+        n0 += (uint32_t)(kTileSPU * units);
         if (left == 0) {
             ci += (int)gridDim.x;
             load_chunk();
@@ -239,7 +239,7 @@ struct SegWalk {
     // (batch tile and column tile: asked once per segment, and two registers fewer than kept)
     __device__ __forceinline__ int mt_i() const { return fast_div(t, p.div_ntiles); }
     __device__ __forceinline__ int nt() const { return t - mt_i() * p.n_tiles; }
-    __device__ __forceinline__ int stages_in_seg() const { return spu * units; }
+    __device__ __forceinline__ int stages_in_seg() const { return kTileSPU * units; }
     __device__ __forceinline__ bool whole_tile() const { return g0 == 0 && units == p.G; }
 };
 
@@ -293,7 +293,7 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
     const int mt = p.mt;
     const int stage_bytes = tile_stage_bytes(mt);
     constexpr int kStageK = kTileStageK;                 // k per ring slot
-    constexpr int kSPU = kGroup / kStageK;               // stages per unit
+    constexpr int kSPU = kTileSPU;
     constexpr int kSlotCols = kStageK / 2;               // TMEM columns of one operand slot
     constexpr int kACol = kTileACol;
     constexpr int kNW = kStageK / 32;                    // 16-byte chunks of a thread's column per stage
@@ -345,7 +345,7 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
         bool ok = true;
         RingPos r{0, 0u, 0u};
         uint32_t n = 0;
-        for (SegWalk w(p, kSPU); w.valid() && ok; w.next()) {
+        for (SegWalk w(p); w.valid() && ok; w.next()) {
             int kb = w.g0 * (kGroup / kTileBoxK);            // 64-k box index along K
             const int m = w.mt_i() * mt;
             const int nst = w.stages_in_seg();
@@ -372,7 +372,7 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
         uint32_t n_seg = 0;
         bool ok = true;
         RingPos r{0, 0u, 0u};
-        for (SegWalk w(p, kSPU); w.valid() && ok; w.next(), ++n_seg) {
+        for (SegWalk w(p); w.valid() && ok; w.next(), ++n_seg) {
             // the epilogue of the segment before must have drained the accumulator
             if (!mbar_wait(d_empty, (n_seg & 1u) ^ 1u)) { ok = false; break; }
             const int nst = w.stages_in_seg();
@@ -414,7 +414,7 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
         // set's stages are kTileSets apart, so its position steps; it is recomputed only when the cursor enters a new
         // segment.  (One 32-bit position instead of three pointers: the loop runs at the register limit.)
         static_assert(kSPU == 2, "a stage is one 64-k half of a packed block");
-        SegWalk wl(p, kSPU);
+        SegWalk wl(p);
         int jl = 0;
         bool l_in = false;                      // this thread's column exists (not past the matrix edge)
         uint32_t hb = 0u;                       // 64-k half block: 2 * packed block + half
@@ -502,7 +502,7 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
             }
             return true;
         };
-        for (SegWalk w(p, kSPU); w.valid() && ok; w.next(), ++n_seg) {
+        for (SegWalk w(p); w.valid() && ok; w.next(), ++n_seg) {
             const int nst = w.stages_in_seg();
             for (int j = first_own(w); j < nst; j += kTileSets) {
                 const uint32_t n = w.n0 + (uint32_t)j;

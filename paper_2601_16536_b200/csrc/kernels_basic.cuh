@@ -66,10 +66,10 @@ __device__ __forceinline__ void load_sz(const uint16_t* __restrict__ S, const ui
 }
 
 // ------------------------------------------------------------------ quantize (the step before the path)
-// Eq. 1, x_q = round(x / s) + z, per group of `group` consecutive k of one column: one thread per (group,
-// column).  Asymmetric: s = (max - min) / 15 rounded to the 16-bit format, z = clamp(round(-min / s), 0, 15);
-// symmetric: s = max|x| / 7, z = 8; a zero or non-finite s becomes 1; q = clamp(round(x / s) + z, 0, 15),
-// ties to even.  Every operation is one IEEE binary32 operation in this order, because the results are
+// Eq. 1, x_q = round(x / s) + z, per group of `group` consecutive k of one column.  Asymmetric:
+// s = (max - min) / 15 rounded to the 16-bit format, z = clamp(round(-min / s), 0, 15); symmetric:
+// s = max|x| / 7, z = 8; a zero or non-finite s becomes 1; q = clamp(round(x / s) + z, 0, 15), ties to
+// even.  Every operation is one IEEE binary32 operation in this order, because the results are
 // integers decided by floating point.  Output in the raw layout that w4a16_pack consumes.
 template <bool BF>
 __device__ __forceinline__ float group_scale(float num, float den, uint16_t& bits) {
@@ -105,8 +105,7 @@ __device__ __forceinline__ uint32_t quantize_exact(float x, float s, int z) {
 
 // One CTA per 64 columns x 128 k, each of its four warps 32 k: a lane keeps its two columns' 32 rows in registers (128
 // bytes a row and warp, every weight read once), warps of the same group exchange minimum and maximum through shared
-// memory.  Codes
-// without a division: u = x * (1 / s) + 768 in one FMA is the quotient rounded to a multiple of 2^-14 (where it is below
+// memory.  Codes without a division: u = x * (1 / s) + 768 in one FMA is the quotient rounded to a multiple of 2^-14 (where it is below
 // 256; beyond 16 every code is clamped anyway), and that has the same nearest integer, ties to even, as the definition's
 // fl(x / s): x = X 2^a and s = T 2^b have 11-bit significands, so x - h s for a half-integer h is zero or at least
 // 2^min(a, b - 1), which with |h| >= 1/2 (hence a >= b - 2) is more than 2^-13 of s.  The reciprocal, the FMA and the
