@@ -50,7 +50,7 @@ def _kernel_name(B, M, K, N, split_k=0):
 # (None = not captured since that kernel last changed).  Decode kernel: the mean of the five launches of a
 # step, M = 1 / 2 / 4 / 8 / 16 at K = 11008, N = 4096: 23.482 / 23.505 / 23.549 / 23.636 / 23.813 MB read, 0 written.
 NCU_TRAFFIC_BYTES = {"gemm_decode_kernel": 23597000}
-NCU_TRAFFIC_BYTES_TILE = 189215000    # gemm_tile_kernel<256>, M=4096 K=N=8192 (read 135.2 MB + write 54.0 MB, mean of two launches)
+NCU_TRAFFIC_BYTES_TILE = 172179000    # gemm_tile_kernel, M=4096 K=N=8192 (read 120.1 MB + write 52.0 MB, one launch)
 
 
 def _peaks():
