@@ -744,6 +744,26 @@ GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, boo
     return p;
 }
 
+// Quantizer and pack: set up while the kernel in front runs, and ordered behind it by the kernels themselves (in a row, as a
+// model load calls them, a gap between two launches costs about 2 us).
+template <typename... P, typename... A>
+int launch_block_kernel(void (*kern)(P...), unsigned blocks, cudaStream_t st, A... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks, 1, 1);
+    cfg.blockDim = dim3(kBlockKernelThreads, 1, 1);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...) != cudaSuccess) {
+        cudaGetLastError();
+        return W4A16_ERR_CUDA;
+    }
+    return W4A16_OK;
+}
+
 // ---- built-in scratch for w4a16_gemm_static_ws -------------------------------------
 // Lives in the library's device image: every GPU that loads the library holds these bytes until
 // the process exits.  In host code `g_static_ws` is only a handle for cudaGetSymbolAddress; the
@@ -883,9 +903,7 @@ int w4a16_quantize(const uint16_t* W16, uint32_t* Wq_raw, uint16_t* S_raw, uint8
     const unsigned blocks = (unsigned)((long long)G * (N / kTileN));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     uint8_t* z = sym ? nullptr : Z_raw;
-    if (bf) quantize_kernel<true><<<blocks, kBlockKernelThreads, 0, st>>>(W16, Wq_raw, S_raw, z, N, G, sg, sym ? 1 : 0);
-    else quantize_kernel<false><<<blocks, kBlockKernelThreads, 0, st>>>(W16, Wq_raw, S_raw, z, N, G, sg, sym ? 1 : 0);
-    return cudaGetLastError() == cudaSuccess ? W4A16_OK : W4A16_ERR_CUDA;
+    return launch_block_kernel(bf ? quantize_kernel<true> : quantize_kernel<false>, blocks, st, W16, Wq_raw, S_raw, z, N, G, sg, sym ? 1 : 0);
 }
 
 int w4a16_pack_fmt(const uint32_t* Wq_raw, const uint16_t* S_raw, const uint8_t* Z_raw, void* Wq, void* S, void* Z,
@@ -904,12 +922,10 @@ int w4a16_pack_fmt(const uint32_t* Wq_raw, const uint16_t* S_raw, const uint8_t*
     if (!d->is_sm100) return W4A16_ERR_ARCH;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int G = K / kGroup, sg = kGroup / group;
-    const int blocks = (int)((long long)G * (N / kTileN)), per = kBlockKernelThreads / 32;
-    pack_kernel<<<(unsigned)((blocks + per - 1) / per), kBlockKernelThreads, 0, st>>>(
-        Wq_raw, S_raw, sym ? nullptr : Z_raw, static_cast<uint32_t*>(Wq), static_cast<uint16_t*>(S),
-        sym ? nullptr : static_cast<uint8_t*>(Z), N, G, sg, blocks);
+    const int blocks = (int)((long long)G * (N / kTileN)), per = kBlockKernelThreads / 64;   // half a block a warp
     ++d->pack_epoch;
-    return cudaGetLastError() == cudaSuccess ? W4A16_OK : W4A16_ERR_CUDA;
+    return launch_block_kernel(pack_kernel, (unsigned)((blocks + per - 1) / per), st, Wq_raw, S_raw, sym ? nullptr : Z_raw,
+                               static_cast<uint32_t*>(Wq), static_cast<uint16_t*>(S), sym ? nullptr : static_cast<uint8_t*>(Z), N, G, sg, blocks);
 }
 
 int w4a16_pack(const uint32_t* Wq_raw, const uint16_t* S_raw, const uint8_t* Z_raw, void* Wq, void* S, void* Z,

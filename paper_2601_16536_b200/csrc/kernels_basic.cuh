@@ -15,6 +15,13 @@ struct BlockPos {
     __device__ __forceinline__ BlockPos(int b, int T, int G) : t(b % T), g(b / T), blk((size_t)t * G + g) {}
 };
 
+// Programmatic dependent launch: the kernel behind this one may be set up while this one runs, and this one was set up while
+// the kernel in front of it ran.  Every CTA of a kernel launched that way waits, also one without work: what comes behind
+// counts on this grid not ending before the one in front of it.  (Their inputs are read past the L1 cache: the kernel in front
+// may have written them while this one was already on the SM.)
+__device__ __forceinline__ void next_launch_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_launch_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------ pack
 // Raw word (nibble i = k + i) -> packed word (even k in the low half, odd k in the high half, ascending).
 __device__ __forceinline__ uint32_t pack_word(uint32_t r) {
@@ -22,36 +29,36 @@ __device__ __forceinline__ uint32_t pack_word(uint32_t r) {
     return __byte_perm(e | (e >> 4), o | (o >> 4), 0x6420);
 }
 
-// One warp per block.  A lane reads four consecutive k-words of one column (32 columns: 128 bytes a row) and writes them
-// as the column's 16-byte chunk: eight columns make up a 128-byte line.  Scales and zero points of the block go along in
-// the same launch.  K = 11008 / N = 4096: three kernels with a thread per word 36 us together, this one
-// 12.4 us (HBM floor 6.9).
+// One warp per half block (32 columns x 128 k).  A lane reads four consecutive k-words of one column (32 columns: 128 bytes a
+// row) and writes them as the column's 16-byte chunk: eight columns make up a 128-byte line.  Scales and zero points of the
+// half block go along in the same launch.  The launch is latency: a warp's loads, then its stores.  K = 11008 / N = 4096: a
+// warp per block, plain launch 12.5 us, this form 10.6 (HBM floor 7.2), 8.5 behind the quantizer.
 __global__ void __launch_bounds__(kBlockKernelThreads)
 pack_kernel(const uint32_t* __restrict__ Wq_raw, const uint16_t* __restrict__ S_raw, const uint8_t* __restrict__ Z_raw,
             uint32_t* __restrict__ Wq, uint16_t* __restrict__ S, uint8_t* __restrict__ Z, int N, int G, int sg, int blocks) {
-    const int b = blockIdx.x * (kBlockKernelThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    next_launch_may_start();
+    wait_for_launch_before();            // (every warp: see there)
+    const int i = blockIdx.x * (kBlockKernelThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int b = i >> 1, h = i & 1;
     if (b >= blocks) return;
     const BlockPos pos(b, N / kTileN, G);
-    const uint32_t* src = Wq_raw + (size_t)pos.g * (kGroup / 8) * N + (size_t)pos.t * kTileN + lane;
-    uint32_t r[2][16];
+    const uint32_t* src = Wq_raw + (size_t)pos.g * (kGroup / 8) * N + (size_t)pos.t * kTileN + 32 * h + lane;
+    uint32_t r[16];
 #pragma unroll
-    for (int kw = 0; kw < 16; ++kw)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) r[h][kw] = __ldg(src + (size_t)kw * N + 32 * h);
-    __syncwarp();                        // (all 32 loads stay ahead of the first store)
+    for (int kw = 0; kw < 16; ++kw) r[kw] = __ldcg(src + (size_t)kw * N);
+    __syncwarp();                        // (all 16 loads stay ahead of the first store)
     uint4* dst = reinterpret_cast<uint4*>(Wq + pos.blk * kBlockWords);
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int q = 0; q < 4; ++q)      // k-words 4 q .. 4 q + 3
-            dst[block_word_index(32 * h + lane, 4 * q) / 4] = make_uint4(pack_word(r[h][4 * q]), pack_word(r[h][4 * q + 1]),
-                                                                         pack_word(r[h][4 * q + 2]), pack_word(r[h][4 * q + 3]));
-    // positions 2 lane, 2 lane + 1 of a row of scales / zero points belong to columns c0, c0 + 8 (sz_perm)
-    const int c0 = (lane & 16) * 2 + ((lane >> 1) & 7) + (lane & 1) * 16;
+    for (int q = 0; q < 4; ++q)          // k-words 4 q .. 4 q + 3
+        dst[block_word_index(32 * h + lane, 4 * q) / 4] =
+            make_uint4(pack_word(r[4 * q]), pack_word(r[4 * q + 1]), pack_word(r[4 * q + 2]), pack_word(r[4 * q + 3]));
+    if (lane >= 16) return;
+    // positions 32 h + 2 lane, + 1 of a row of scales / zero points belong to columns c0, c0 + 8 (sz_perm)
+    const int c0 = 32 * h + (lane >> 1) + (lane & 1) * 16;
     for (int j = 0; j < sg; ++j) {
         const size_t in = (size_t)(pos.g * sg + j) * N + (size_t)pos.t * kTileN + c0, row = pos.blk * sg + j;
-        reinterpret_cast<uint32_t*>(S + row * kSBlockHalves)[lane] = (uint32_t)S_raw[in] | ((uint32_t)S_raw[in + 8] << 16);
-        if (Z_raw != nullptr) Z[row * (kZBlockWords * 4) + lane] = (uint8_t)((Z_raw[in] & 15u) | (Z_raw[in + 8] << 4));
+        reinterpret_cast<uint32_t*>(S + row * kSBlockHalves)[16 * h + lane] = (uint32_t)__ldcg(S_raw + in) | ((uint32_t)__ldcg(S_raw + in + 8) << 16);
+        if (Z_raw != nullptr) Z[row * (kZBlockWords * 4) + 16 * h + lane] = (uint8_t)((__ldcg(Z_raw + in) & 15u) | (__ldcg(Z_raw + in + 8) << 4));
     }
 }
 
@@ -97,21 +104,51 @@ __device__ __forceinline__ uint32_t max2(uint32_t a, uint32_t b) {
     return r;
 }
 
-// One code of the definition above.
+// One code of the definition above, and eight of a column as a raw word (out of line: groups whose scale has no normal
+// reciprocal hardly ever come, and in line the divisions were four fifths of the kernel's code).
 __device__ __forceinline__ uint32_t quantize_exact(float x, float s, int z) {
     const float r = __fadd_rn(rintf(__fdiv_rn(x, s)), (float)z);
     return (uint32_t)(r < 0.0f ? 0 : r > 15.0f ? 15 : (int)r);
+}
+template <bool BF>
+__device__ __noinline__ uint32_t quantize_word_exact(const uint16_t* x, int N, float s, int z) {
+    uint32_t w = 0u;
+#pragma unroll 1
+    for (int i = 0; i < 8; ++i) w |= quantize_exact(widen<BF>(__ldcg(x + (size_t)i * N)), s, z) << (4 * i);
+    return w;
+}
+
+// Two FP32 operations in one instruction.
+__device__ __forceinline__ uint64_t pair_f32(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
 }
 
 // One CTA per 64 columns x 128 k, each of its four warps 32 k: a lane keeps its two columns' 32 rows in registers (128
 // bytes a row and warp, every weight read once), warps of the same group exchange minimum and maximum through shared
 // memory.  Codes without a division: u = x * (1 / s) + 768 in one FMA is the quotient rounded to a multiple of 2^-14 (where it is below
-// 256; beyond 16 every code is clamped anyway), and that has the same nearest integer, ties to even, as the definition's
+// 256), and that has the same nearest integer, ties to even, as the definition's
 // fl(x / s): x = X 2^a and s = T 2^b have 11-bit significands, so x - h s for a half-integer h is zero or at least
 // 2^min(a, b - 1), which with |h| >= 1/2 (hence a >= b - 2) is more than 2^-13 of s.  The reciprocal, the FMA and the
 // definition's own division are off by less than 2^-19, the grid by at most 2^-15: a tie lands on the half exactly,
-// anything else stays on its side of it.  (Scales whose reciprocal is not a normal number take the divisions.)
-// K = 11008 / N = 4096: a thread per (group, column), two passes and a division per weight 96 us, this form 29 us (HBM floor 17).
+// anything else stays on its side of it.  (Scales whose reciprocal is not a normal number take the divisions.)  The clamp to
+// 0 .. 15 comes first, on the 16-bit weights, two at a time: x between -z s and (15 - z) s, each rounded to 16 bits.  Those
+// bounds are within 2^-9 of themselves, so their own codes are 0 and 15, and what lies beyond them has no other code.
+// What bounds it: memory while a CTA loads, instructions while it computes (13 a pair of weights), overlapped only between
+// CTAs.  K = 11008 / N = 4096: a thread per (group, column), two passes and a division per weight 96 us; FP32 clamps, one
+// column at a time and the divisions in line (25 % of the warp time went into fetching instructions) 28.9; this form 23.4
+// (HBM floor 17.4).  Held to 48 registers for ten CTAs an SM it spills.
 template <bool BF>
 __global__ void __launch_bounds__(kBlockKernelThreads)
 quantize_kernel(const uint16_t* __restrict__ W16, uint32_t* __restrict__ Wq, uint16_t* __restrict__ S,
@@ -119,11 +156,13 @@ quantize_kernel(const uint16_t* __restrict__ W16, uint32_t* __restrict__ Wq, uin
     __shared__ uint32_t part_lo[4][32], part_hi[4][32];
     const BlockPos pos(blockIdx.x, N / kTileN, G);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    next_launch_may_start();
+    wait_for_launch_before();
     const size_t n = (size_t)pos.t * kTileN + 2 * lane;
     const uint16_t* src = W16 + (size_t)(pos.g * kGroup + warp * 32) * N + n;
     uint32_t v[32];
 #pragma unroll
-    for (int k = 0; k < 32; ++k) v[k] = __ldg(reinterpret_cast<const uint32_t*>(src + (size_t)k * N));
+    for (int k = 0; k < 32; ++k) v[k] = __ldcg(reinterpret_cast<const uint32_t*>(src + (size_t)k * N));
     uint32_t lo = BF ? 0x7f807f80u : 0x7c007c00u, hi = lo | 0x80008000u;     // +inf, -inf
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
@@ -141,7 +180,8 @@ quantize_kernel(const uint16_t* __restrict__ W16, uint32_t* __restrict__ Wq, uin
     constexpr float kGrid = 768.0f;                      // 1.5 * 2^9: neighbours 2^-14 apart
     constexpr float kMagic = 12582912.0f;                // 1.5 * 2^23, bits 0x4b400000: neighbours 1 apart
     uint16_t sb[2];
-    float s[2], rinv[2], least[2], most[2];
+    float s[2], rinv[2];
+    uint32_t least = 0u, most = 0u;
     int z[2];
     bool slow[2];
 #pragma unroll
@@ -156,8 +196,8 @@ quantize_kernel(const uint16_t* __restrict__ W16, uint32_t* __restrict__ Wq, uin
             z[c] = zf < 0.0f ? 0 : zf > 15.0f ? 15 : (int)zf;
         }
         rinv[c] = __frcp_rn(s[c]);
-        least[c] = kMagic - (float)z[c];                 // codes 0 and 15
-        most[c] = kMagic + (float)(15 - z[c]);
+        least |= (uint32_t)cast_out<BF>(-(float)z[c] * s[c]) << (16 * c);          // codes 0 and 15
+        most |= (uint32_t)cast_out<BF>((float)(15 - z[c]) * s[c]) << (16 * c);
         slow[c] = !(s[c] > 1e-30f && s[c] < 1e30f);
     }
     const size_t out = (size_t)(pos.g * sg + warp / wpg) * N + n;
@@ -165,27 +205,25 @@ quantize_kernel(const uint16_t* __restrict__ W16, uint32_t* __restrict__ Wq, uin
         *reinterpret_cast<uint32_t*>(S + out) = (uint32_t)sb[0] | ((uint32_t)sb[1] << 16);
         if (Z != nullptr) *reinterpret_cast<uint16_t*>(Z + out) = (uint16_t)(z[0] | (z[1] << 8));
     }
+    const uint64_t rinv2 = pair_f32(rinv[0], rinv[1]), grid2 = pair_f32(kGrid, kGrid), magic2 = pair_f32(kMagic - kGrid, kMagic - kGrid);
+    const uint32_t zw[2] = {((uint32_t)z[0] - 0x4b400000u) * 0x11111111u, ((uint32_t)z[1] - 0x4b400000u) * 0x11111111u};
     uint32_t* dst = Wq + (size_t)(pos.g * (kGroup / 8) + warp * 4) * N + n;
 #pragma unroll
     for (int kw = 0; kw < 4; ++kw) {
-        uint32_t w[2];
+        uint32_t w[2] = {0u, 0u};
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            uint32_t acc = 0u;
-#pragma unroll
-            for (int i = 7; i >= 0; --i) {
-                const float u = __fmaf_rn(widen<BF>((uint16_t)(v[8 * kw + i] >> (16 * c))), rinv[c], kGrid);
-                const float y = __fadd_rn(u, kMagic - kGrid);          // low bits: round(x / s)
-                acc = acc * 16u + __float_as_uint(fminf(fmaxf(y, least[c]), most[c]));
-            }
-            w[c] = acc + ((uint32_t)z[c] - 0x4b400000u) * 0x11111111u; // + z in each digit, the constant's copies out again
-            if (slow[c]) {
-                w[c] = 0u;
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    w[c] |= quantize_exact(widen<BF>((uint16_t)(v[8 * kw + i] >> (16 * c))), s[c], z[c]) << (4 * i);
-            }
+        for (int i = 7; i >= 0; --i) {
+            const uint32_t x = min2<BF>(max2<BF>(v[8 * kw + i], least), most);
+            const uint64_t u = fma_f32x2(pair_f32(widen<BF>((uint16_t)x), widen<BF>((uint16_t)(x >> 16))), rinv2, grid2);
+            const uint64_t y = add_f32x2(u, magic2);     // low bits: round(x / s)
+            w[0] = w[0] * 16u + (uint32_t)y;
+            w[1] = w[1] * 16u + (uint32_t)(y >> 32);
         }
+        // + z in each digit, the constant's copies out again
+        w[0] += zw[0];
+        w[1] += zw[1];
+        if (slow[0]) w[0] = quantize_word_exact<BF>(src + (size_t)(8 * kw) * N, N, s[0], z[0]);
+        if (slow[1]) w[1] = quantize_word_exact<BF>(src + (size_t)(8 * kw) * N + 1, N, s[1], z[1]);
         *reinterpret_cast<uint2*>(dst + (size_t)kw * N) = make_uint2(w[0], w[1]);
     }
 }

@@ -85,3 +85,25 @@ def test_quantize_pack_gemm_chain(M, symmetric):
     full = A_bits.view(np.float16).astype(np.float64) @ bits.view(np.float16).astype(np.float64)
     assert np.linalg.norm(ref - full) / np.linalg.norm(full) < 0.2
     del ws
+
+
+@pytest.mark.parametrize("K,N", [(128, 64), (1024, 960), (4096, 4096)])
+def test_a_row_of_quantize_and_pack_calls_is_ordered(K, N):
+    """Eight matrices through one set of raw buffers without a synchronisation in between: each launch is set up while the
+    one in front of it runs, so a pack that read too early, or a quantizer that wrote too early, would mix two matrices."""
+    Ws = [(torch.randn(K, N, device="cuda") * 0.04 * (1 + i)).half() for i in range(8)]
+    Wq = torch.empty((K // 8, N), dtype=torch.int32, device="cuda")
+    S = torch.empty((K // 128, N), dtype=torch.float16, device="cuda")
+    Z = torch.empty((K // 128, N), dtype=torch.uint8, device="cuda")
+    L, st = B.load(), torch.cuda.current_stream().cuda_stream
+    packed = []
+    for W in Ws:
+        assert L.w4a16_quantize(W.data_ptr(), Wq.data_ptr(), S.data_ptr(), Z.data_ptr(), N, K, 128, 0, st) == 0
+        packed.append(B.w4a16_pack(Wq, S, Z, N, K))
+    torch.cuda.synchronize()
+    for W, pw in zip(Ws, packed):
+        q, s, z = B.w4a16_quantize(W)
+        torch.cuda.synchronize()
+        one = B.w4a16_pack(q, s, z, N, K)
+        torch.cuda.synchronize()
+        assert torch.equal(pw.Wq, one.Wq) and torch.equal(pw.S, one.S) and torch.equal(pw.Z, one.Z)
