@@ -187,6 +187,21 @@ __device__ __forceinline__ bool mbar_wait_inline(uint32_t addr, uint32_t parity)
     return ok != 0;
 }
 
+// Has the phase completed?  (No wait.)
+__device__ __forceinline__ bool mbar_test(uint32_t addr, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t"
+        "}"
+        : "=r"(ok)
+        : "r"(addr), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // The same bounded wait with cluster-scope acquire: for a barrier that CTAs of the cluster arrive on
 // after writing this CTA's shared memory.
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity) {

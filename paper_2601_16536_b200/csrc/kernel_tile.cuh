@@ -115,6 +115,17 @@ __device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// The same with the descriptor as two words, of which only the low one (the address) changes from one MMA to the next.
+__device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
+                                          uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 b, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
 // 16 consecutive 32-bit TMEM columns of this thread's lane <- registers.
 __device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16]) {
     asm volatile(
@@ -368,30 +379,68 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
         asm volatile("griddepcontrol.wait;" ::: "memory");
+        // What the loop needs of a stage steps by constants and is kept as 32-bit shared addresses, tensor-memory columns and
+        // the low word of the box's descriptor: the warp's own scalar code, not the tensor pipe, sets the time of a stage.
+        // With barriers as 64-bit pointers and the ring position worked out for each stage the issuer always found its stage
+        // ready and took 620 clocks for it with 208 rows and 680 with 256; the MMAs alone take 419 and 514.  us, that form /
+        // this one one stage at a time / two at a time: M = 777, K = 4096 / N = 22016 117 / 110 / 109; M = 1024, K = N = 8192
+        // 100.1 / 99.0 / 98.7, M = 4096 368 / 368 / 362; M = 300, K = N = 4096 24.8 / 23.2 / 23.5.  Not faster: both stages'
+        // waits ahead of the first MMA (112.5 at M = 777), the next stage's barrier tested ahead of this one's MMAs (112.6).
         const uint32_t idesc = tile_idesc(mt, BF);
+        const uint32_t full0 = smem_u32(full), full_end = full0 + 8u * R, retired0 = smem_u32(retired);
+        const uint32_t d_full_a = smem_u32(d_full), d_empty_a = smem_u32(d_empty);
+        const uint64_t box0 = smem_desc_sw128(smem_u32(stage0));
+        const uint32_t box_lo0 = (uint32_t)box0, box_hi = (uint32_t)(box0 >> 32), box_step = (uint32_t)stage_bytes >> 4;
+        uint32_t bar = full0, ret = retired0, box = box_lo0, a_t = tmem_base + kACol, ph = 0u;
+        auto half_unit = [&](uint32_t a, uint32_t b, uint32_t first) {
+#pragma unroll
+            for (int kk = 0; kk < kStageK / 16; ++kk)            // 16 k: 8 TMEM columns of A, 32 bytes along B's swizzled rows
+                tc_mma_ts(tmem_base, a + kk * 8, b + kk * 2, box_hi, idesc, kk == 0 ? first : 1u);
+        };
         uint32_t n_seg = 0;
         bool ok = true;
-        RingPos r{0, 0u, 0u};
         for (SegWalk w(p); w.valid() && ok; w.next(), ++n_seg) {
             // the epilogue of the segment before must have drained the accumulator
-            if (!mbar_wait(d_empty, (n_seg & 1u) ^ 1u)) { ok = false; break; }
-            const int nst = w.stages_in_seg();
+            if (!mbar_wait(d_empty_a, (n_seg & 1u) ^ 1u)) { ok = false; break; }
             uint32_t acc = 0u;                                   // the segment's first MMA overwrites
-            for (int j = 0; j < nst; ++j) {
-                if (!mbar_wait(&full[r.slot], r.ph)) { ok = false; break; }
+            for (int left = w.units; left > 0; --left) {
+                // Two stages a turn (a unit; the ring has an even number of slots): their MMAs in one go if the second one
+                // is there already, as it mostly is.
+                if (!mbar_wait(bar, ph)) { ok = false; break; }
+                const bool both = mbar_test(bar + 8u, ph);
                 tc_fence_after();
                 if (elect_one()) {
-                    const uint64_t bdesc = smem_desc_sw128(smem_u32(stage0 + r.slot * stage_bytes));
-                    const uint32_t a_t = tmem_base + kACol + r.slot * kSlotCols;
-#pragma unroll
-                    for (int kk = 0; kk < kStageK / 16; ++kk)    // 16 k: 8 TMEM columns of A, 32 bytes along B's swizzled rows
-                        tc_mma_ts(tmem_base, a_t + kk * 8, bdesc + (uint64_t)(kk * 2), idesc, kk == 0 ? acc : 1u);
-                    tc_commit(retired_bar(retired, r));
-                    if (j + 1 == nst) tc_commit(d_full);
+                    half_unit(a_t, box, acc);
+                    tc_commit(ret);
+                    if (both) {
+                        half_unit(a_t + kSlotCols, box + box_step, 1u);
+                        tc_commit(ret + 8u);
+                        if (left == 1) tc_commit(d_full_a);
+                    }
                 }
                 __syncwarp();
+                if (!both) {
+                    if (!mbar_wait(bar + 8u, ph)) { ok = false; break; }
+                    tc_fence_after();
+                    if (elect_one()) {
+                        half_unit(a_t + kSlotCols, box + box_step, 1u);
+                        tc_commit(ret + 8u);
+                        if (left == 1) tc_commit(d_full_a);
+                    }
+                    __syncwarp();
+                }
                 acc = 1u;
-                r.advance(1, R);
+                bar += 16u;
+                ret += 16u;
+                box += 2u * box_step;
+                a_t += 2u * kSlotCols;
+                if (bar == full_end) {                           // next turn: the other set of "retired" barriers
+                    ph ^= 1u;
+                    bar = full0;
+                    ret = retired0 + ph * (8u * kTileMaxStages);
+                    box = box_lo0;
+                    a_t = tmem_base + kACol;
+                }
             }
         }
         if (!ok && lane == 0) *abort_flag = 1;
