@@ -377,13 +377,13 @@ gemm_mid_kernel(const __grid_constant__ CUtensorMap tmap_a, const MidParams p) {
                     tc_ld16(d_t + c0, v);
                     tc_wait_ld();
                     if (p.split_k == 1) {
-                        if (n < p.N) {
+                        uint16_t y[16];
+                        finish_column<BF>(v, y, has_bias, bias, p.epi.act);
+                        const int rows = n < p.N ? p.M - (m_base + c0) : 0;
+                        uint16_t* dst = p.C + (size_t)(m_base + c0) * p.N + n;
 #pragma unroll
-                            for (int q = 0; q < 16; ++q) {
-                                const int m = m_base + c0 + q;
-                                if (m < p.M) p.C[(size_t)m * p.N + n] = finish_col<BF>(__uint_as_float(v[q]), has_bias, bias, p.epi.act);
-                            }
-                        }
+                        for (int q = 0; q < 16; ++q, dst += p.N)
+                            if (q < rows) *dst = y[q];
                     } else {
 #pragma unroll
                         for (int q = 0; q < 16; ++q) part[(size_t)(c0 + q) * kTileCols] = __uint_as_float(v[q]);
@@ -449,14 +449,14 @@ gemm_mid_kernel(const __grid_constant__ CUtensorMap tmap_a, const MidParams p) {
                         acc.z += __uint_as_float(x.z); acc.w += __uint_as_float(x.w);
                     }
                 }
-                if (n < p.N) {
-                    const float a[4] = {acc.x, acc.y, acc.z, acc.w};
+                const uint32_t a[4] = {__float_as_uint(acc.x), __float_as_uint(acc.y), __float_as_uint(acc.z), __float_as_uint(acc.w)};
+                uint16_t y[4];
+                finish_column<BF>(a, y, has_bias, bias, p.epi.act);
+                const int rows = n < p.N ? p.M - (m_base + 4 * q) : 0;
+                uint16_t* dst = p.C + (size_t)(m_base + 4 * q) * p.N + n;
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int m = m_base + 4 * q + e;
-                        if (m < p.M) p.C[(size_t)m * p.N + n] = finish_col<BF>(a[e], has_bias, bias, p.epi.act);
-                    }
-                }
+                for (int e = 0; e < 4; ++e, dst += p.N)
+                    if (e < rows) *dst = y[e];
             }
         }
         if (!ok && lane == 0) flags[0] = 1;

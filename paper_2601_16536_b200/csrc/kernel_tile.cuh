@@ -590,13 +590,13 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
                 tc_ld16(d_t + cc, v);
                 tc_wait_ld();
                 if (whole) {
-                    if (n < p.N) {
+                    uint16_t c[kStep];
+                    finish_column<BF>(v, c, has_bias, bias, EPI ? p.epi.act : kActNone);
+                    const int rows = n < p.N ? p.M - (m_base + cc) : 0;
+                    uint16_t* dst = p.C + (size_t)(m_base + cc) * p.N + n;
 #pragma unroll
-                        for (int q = 0; q < kStep; ++q) {
-                            const int m = m_base + cc + q;
-                            if (m < p.M) p.C[(size_t)m * p.N + n] = EPI ? finish_col<BF>(__uint_as_float(v[q]), has_bias, bias, p.epi.act) : cast_out<BF>(__uint_as_float(v[q]));
-                        }
-                    }
+                    for (int q = 0; q < kStep; ++q, dst += p.N)
+                        if (q < rows) *dst = c[q];
                 } else {
 #pragma unroll
                     for (int q = 0; q < kStep; ++q) part[(size_t)(cc + q) * kTileCols] = __uint_as_float(v[q]);
