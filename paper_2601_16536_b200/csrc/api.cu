@@ -744,7 +744,7 @@ GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, boo
     return p;
 }
 
-// Quantizer and pack: set up while the kernel in front runs, and ordered behind it by the kernels themselves (in a row, as a
+// Quantizer, pack and dequantization: set up while the kernel in front runs, and ordered behind it by the kernels themselves (in a row, as a
 // model load calls them, a gap between two launches costs about 2 us).
 template <typename... P, typename... A>
 int launch_block_kernel(void (*kern)(P...), unsigned blocks, cudaStream_t st, A... args) {
@@ -947,10 +947,9 @@ int w4a16_dequant_fmt(const void* Wq, const void* S, const void* Z, uint16_t* W1
     if ((rc = current_device(&d)) != W4A16_OK) return rc;
     if (!d->is_sm100) return W4A16_ERR_ARCH;
     const unsigned blocks = (unsigned)((long long)(K / kGroup) * (N / kTileN));
-    (bf ? dequant_kernel<true> : dequant_kernel<false>)<<<blocks, kBlockKernelThreads, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const uint32_t*>(Wq), static_cast<const uint16_t*>(S), sym ? nullptr : static_cast<const uint32_t*>(Z), W16, N,
-        K / kGroup, kGroup / group);
-    return cudaGetLastError() == cudaSuccess ? W4A16_OK : W4A16_ERR_CUDA;
+    return launch_block_kernel(bf ? dequant_kernel<true> : dequant_kernel<false>, blocks, static_cast<cudaStream_t>(stream),
+                               static_cast<const uint32_t*>(Wq), static_cast<const uint16_t*>(S),
+                               sym ? nullptr : static_cast<const uint32_t*>(Z), W16, N, K / kGroup, kGroup / group);
 }
 
 int w4a16_dequant(const void* Wq, const void* S, const void* Z, uint16_t* W16, int N, int K, int group,

@@ -231,31 +231,45 @@ quantize_kernel(const uint16_t* __restrict__ W16, uint32_t* __restrict__ Wq, uin
 // ------------------------------------------------------------------ dequant
 // Algorithm 1, Phase 1 as a standalone kernel: w16 = rn((q - z) * s) in the 16-bit format: (q - z) is formed exactly and
 // multiplied by s with one multiply (round-to-nearest-even, subnormals kept).  Z == nullptr: symmetric format, z = 8.
-// One CTA per block, a warp for 32 k of it: a lane takes 8 neighbouring columns x 8 k (a word of each column; four lanes read
-// a column's 16 bytes), swaps the halves of neighbouring columns' registers and stores 16 bytes of a row at a time, eight
-// lanes one 128-byte line of the row.  us, a thread per word with 2-byte stores / a warp per block with 16-byte loads / this
-// form: K = N = 8192 68 / 31.8 / 31.4 (HBM floor 25.6), K = N = 4096 18.7 / 10.5 / 8.5, K = 128 / N = 8192 4.2 / 5.1 / 4.1: one
-// warp's way through a whole block was too long for a matrix of few.
+// One CTA per block, a warp for 32 k of it: a lane takes 8 neighbouring columns x 8 k (a word of each column), swaps the halves
+// of neighbouring columns' registers and stores 16 bytes of a row at a time, eight lanes one 128-byte line of the row.  The
+// packed words come through shared memory, 16 bytes a load: fetched word by word a warp's load touches eight lines, and the
+// L1 was the busiest unit (75 %).  The 256-byte sub-blocks lie 272 bytes apart, so that the words a warp reads at a time come from
+// 32 banks.  Bound by HBM, most of it the stores.  us, a thread per word with 2-byte stores / word loads, plain launch / this form:
+// K = N = 8192 68 / 31.2 / 28.5 (HBM floor 26.3, a device copy of as many bytes 28.8), K = 11008 / N = 4096 - / 22.8 / 19.7 (17.6).
 template <bool BF>
 __global__ void __launch_bounds__(kBlockKernelThreads)
 dequant_kernel(const uint32_t* __restrict__ Wq, const uint16_t* __restrict__ S, const uint32_t* __restrict__ Z,
                uint16_t* __restrict__ W16, int N, int G, int sg) {
+    constexpr int kSub = 64, kSubStride = 68;           // words
+    __shared__ __align__(16) uint32_t packed[kBlockWords / kSub * kSubStride];
+    next_launch_may_start();
+    wait_for_launch_before();
     const BlockPos pos(blockIdx.x, N / kTileN, G);
     const int kq = threadIdx.x >> 5, kw = (threadIdx.x >> 3) & 3, rb = threadIdx.x & 7;   // columns 8 rb .. + 7, k = 32 kq + 8 kw .. + 7
-    const uint32_t* src = Wq + pos.blk * kBlockWords + kw;
-    uint32_t w[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) w[c] = __ldg(src + block_word_index(8 * rb + c, 4 * kq));
+    const uint4* src = reinterpret_cast<const uint4*>(Wq + pos.blk * kBlockWords) + threadIdx.x;
+    const uint4 lo = __ldcg(src), hi = __ldcg(src + kBlockKernelThreads);
     const size_t row = pos.blk * sg + kq * sg / 4;
     // column 8 rb + c sits at position p0 + 4 c of a row of scales / zero points
     const int p0 = sz_perm(8 * rb);
     uint4 zz = make_uint4(0u, 0u, 0u, 0u);
-    if (Z != nullptr) zz = __ldg(reinterpret_cast<const uint4*>(Z + row * kZBlockWords) + (p0 >> 5));
+    if (Z != nullptr) zz = __ldcg(reinterpret_cast<const uint4*>(Z + row * kZBlockWords) + (p0 >> 5));
     const uint32_t zw[4] = {zz.x, zz.y, zz.z, zz.w};
     uint32_t s2[8], zlo[8], zhi[8];
 #pragma unroll
+    for (int c = 0; c < 8; ++c) s2[c] = (uint32_t)__ldcg(S + row * kSBlockHalves + p0 + 4 * c) * 0x00010001u;
+    uint4* dst4 = reinterpret_cast<uint4*>(packed) + threadIdx.x + threadIdx.x / (kSub / 4);    // (a sub-block is 16 pieces, 17 with its gap)
+    dst4[0] = lo;
+    dst4[kBlockKernelThreads / (kSub / 4) * (kSubStride / 4)] = hi;
+    __syncthreads();
+    uint32_t w[8];
+#pragma unroll
     for (int c = 0; c < 8; ++c) {
-        s2[c] = (uint32_t)__ldg(S + row * kSBlockHalves + p0 + 4 * c) * 0x00010001u;
+        const int at = block_word_index(c, 4 * kq) + kw;       // of column c; sub-block rb of that half is rb further
+        w[c] = packed[(at / kSub + rb) * kSubStride + at % kSub];
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
         const uint32_t z = Z == nullptr ? (uint32_t)kSymZero : ((zw[c >> 1] >> (16 * (c & 1) + 4 * (p0 & 3))) & 15u);
         zlo[c] = zconst_lo<BF>(z);
         zhi[c] = zconst_hi<BF>(z);

@@ -68,3 +68,20 @@ def test_pack_rejects_bad_shapes():
     x = torch.zeros(4096, dtype=torch.uint8, device="cuda")
     with pytest.raises(B.W4A16Error):
         B.w4a16_pack(x, x, x, 100, 128)
+
+
+@pytest.mark.parametrize("K,N", [(128, 64), (1152, 320), (4096, 4096)])
+def test_a_row_of_pack_and_dequant_calls_is_ordered(K, N):
+    # eight matrices through the same raw and packed buffers without a synchronisation in between: every launch is set up
+    # while the one in front of it runs
+    probs = [wl.draw_weights(K, N, seed=i) for i in range(8)]
+    dev = [tuple(to_dev(d[k]) for k in ("Wq", "S", "Z")) for d in probs]
+    pw = B.w4a16_pack(*dev[0], N, K)
+    L, st = B.load(), torch.cuda.current_stream().cuda_stream
+    outs = []
+    for Wq, S, Z in dev:
+        assert L.w4a16_pack(Wq.data_ptr(), S.data_ptr(), Z.data_ptr(), pw.Wq.data_ptr(), pw.S.data_ptr(), pw.Z.data_ptr(), N, K, 128, st) == 0
+        outs.append(B.w4a16_dequant(pw))
+    torch.cuda.synchronize()
+    for d, out in zip(probs, outs):
+        assert np.array_equal(out.cpu().numpy().view(np.uint16), oracle.dequant(d["Wq"], d["S"], d["Z"], K, N, 128))
