@@ -407,7 +407,8 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
                 // Two stages a turn (a unit; the ring has an even number of slots): their MMAs in one go if the second one
                 // is there already, as it mostly is.
                 if (!mbar_wait(bar, ph)) { ok = false; break; }
-                const bool both = mbar_test(bar + 8u, ph);
+                // (by vote: the other warps may complete the barrier between the answers of two lanes)
+                const bool both = __all_sync(0xffffffffu, mbar_test(bar + 8u, ph));
                 tc_fence_after();
                 if (elect_one()) {
                     half_unit(a_t, box, acc);

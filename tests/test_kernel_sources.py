@@ -27,3 +27,17 @@ def test_kernels_that_let_the_next_launch_start_wait_for_the_one_in_front_before
             seen.append(name)
             assert not re.search(r"\breturn\b", body[:body.index("griddepcontrol.wait")]), name
     assert sorted(seen) == ["stage_activations_kernel", "tile_splitk_reduce_kernel"]
+
+
+def test_a_barrier_tested_without_waiting_steers_a_warp_only_by_vote():
+    """Each lane gets its own answer from a test of a barrier that other warps complete meanwhile.  What comes behind it is
+    for the whole warp (elect.sync, __syncwarp, which MMAs go out), so that the lanes have to agree first."""
+    uses = 0
+    for name in sorted(os.listdir(CSRC)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+        for m in re.finditer(r"(\S*\s*\S*)\bmbar_test\(", text):
+            if "bool" in m.group(1):                     # the definition
+                continue
+            uses += 1
+            assert re.search(r"__(all|any)_sync\(0xffffffffu,\s*$", m.group(1)), (name, m.group(0))
+    assert uses == 1
