@@ -15,6 +15,7 @@
 #include "common.cuh"
 #include "kernels_basic.cuh"
 #include "kernel_tables.h"
+#include "pack_order.cuh"
 
 using namespace w4a16;
 
@@ -35,42 +36,8 @@ struct DeviceState {
     int mid_clusters[16] = {};         // mid_max_clusters, 0 = not asked yet
     bool mid_attr_set[2][3][2][2] = {};   // [64 / 128 rows][log2 SG][bf16][symmetric]
     bool tile_attr_set[3][2][2][2] = {};   // [log2 SG][bf16][symmetric][epilogue]
-    // Programmatic dependent launch lets a GEMM kernel prefetch packed weights before the previous
-    // kernel in its stream has finished.  The previous kernel of a stream may be a w4a16_pack that
-    // writes those weights, so the first GEMM launched on a stream after any pack on the device is a
-    // plain, fully ordered launch, and only the launches after it on that stream overlap their
-    // predecessor again.  pack_epoch counts the packs; the table remembers, per stream, the epoch of
-    // its last GEMM launch (a stream that is not in the table gets a plain launch).
-    unsigned long long pack_epoch = 1;
-    struct StreamEpoch { cudaStream_t stream; unsigned long long epoch; };
-    static constexpr int kStreamSlots = 32;
-    StreamEpoch streams[kStreamSlots] = {};
-    int stream_evict = 0;
+    PackOrder order;          // which GEMM launches may overlap the kernel in front of them
     bool cluster_ok = true;   // cleared when a cluster launch is refused (fewer SMs than usual, MPS limits ...)
-
-    // Has a GEMM been launched on `st` since the last pack?
-    bool packs_seen(cudaStream_t st) const {
-        for (int i = 0; i < kStreamSlots; ++i)
-            if (streams[i].epoch != 0 && streams[i].stream == st) return streams[i].epoch == pack_epoch;
-        return false;
-    }
-    // May this launch on `st` overlap the previous kernel of the stream?  Records the launch.
-    bool pdl_allowed(cudaStream_t st) {
-        for (int i = 0; i < kStreamSlots; ++i) {
-            if (streams[i].epoch != 0 && streams[i].stream == st) {
-                const bool ok = streams[i].epoch == pack_epoch;
-                streams[i].epoch = pack_epoch;
-                return ok;
-            }
-        }
-        int slot = -1;
-        for (int i = 0; i < kStreamSlots; ++i)
-            if (streams[i].epoch == 0) { slot = i; break; }
-        if (slot < 0) { slot = stream_evict; stream_evict = (stream_evict + 1) % kStreamSlots; }
-        streams[slot].stream = st;
-        streams[slot].epoch = pack_epoch;
-        return false;
-    }
 };
 DeviceState g_dev[kMaxDevices];
 // One lock for the per-device records above (workspace registration, attribute flags, stream table):
@@ -923,7 +890,7 @@ int w4a16_pack_fmt(const uint32_t* Wq_raw, const uint16_t* S_raw, const uint8_t*
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int G = K / kGroup, sg = kGroup / group;
     const int blocks = (int)((long long)G * (N / kTileN)), per = kBlockKernelThreads / 64;   // half a block a warp
-    ++d->pack_epoch;
+    d->order.pack_issued();
     return launch_block_kernel(pack_kernel, (unsigned)((blocks + per - 1) / per), st, Wq_raw, S_raw, sym ? nullptr : Z_raw,
                                static_cast<uint32_t*>(Wq), static_cast<uint16_t*>(S), sym ? nullptr : static_cast<uint8_t*>(Z), N, G, sg, blocks);
 }
@@ -971,6 +938,34 @@ TileKernel tile_kernel(int sg, bool bf, bool sym, bool epi) {
                                                                                 : tile_kernel_bf16_sg4(sym, epi);
     return sg == 1 ? tile_kernel_f16_sg1(sym, epi) : sg == 2 ? tile_kernel_f16_sg2(sym, epi)
                                                                        : tile_kernel_f16_sg4(sym, epi);
+}
+
+// Launches a GEMM kernel.  Programmatic dependent launch where the order allows it: its prologue and its requests for packed weights
+// overlap the tail of the previous kernel of the stream, and it orders itself with griddepcontrol.wait.
+// `cluster` CTAs with consecutive blockIdx.x form a thread-block cluster.
+template <typename Params>
+bool launch_gemm_kernel(DeviceState* d, cudaLaunchConfig_t cfg, int cluster, void (*kern)(CUtensorMap, Params), const CUtensorMap& tmap, const Params& p) {
+    cudaLaunchAttribute attr[2];
+    int n_attr = 0;
+    if (cluster > 1) {
+        attr[n_attr].id = cudaLaunchAttributeClusterDimension;
+        attr[n_attr].val.clusterDim.x = (unsigned)cluster;
+        attr[n_attr].val.clusterDim.y = 1;
+        attr[n_attr].val.clusterDim.z = 1;
+        ++n_attr;
+    }
+    return d->order.launch(reinterpret_cast<uintptr_t>(cfg.stream), [&](bool overlap) {
+        if (overlap) {
+            attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
+            ++n_attr;
+        }
+        cfg.attrs = attr;
+        cfg.numAttrs = n_attr;
+        if (cudaLaunchKernelEx(&cfg, kern, tmap, p) == cudaSuccess) return true;
+        cudaGetLastError();
+        return false;
+    });
 }
 
 // Split-K sum behind a tcgen05 kernel that stored its partial tiles: S slices per tile, or (split_k == 0) balanced chunks.
@@ -1058,7 +1053,7 @@ int stage_activations(const void* host, void* dev, int n16, cudaStream_t st) {
     cfg.stream = st;
     cfg.attrs = attr;
     // (behind a pack a plain launch: the GEMM that follows asks for packed weights while this kernel runs)
-    cfg.numAttrs = d->packs_seen(st) ? 1 : 0;
+    cfg.numAttrs = d->order.may_overlap(reinterpret_cast<uintptr_t>(st)) ? 1 : 0;
     if (cudaLaunchKernelEx(&cfg, stage_activations_kernel, static_cast<const uint4*>(host), static_cast<uint4*>(dev), n16) != cudaSuccess) {
         cudaGetLastError();
         return W4A16_ERR_CUDA;
@@ -1159,24 +1154,7 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         cfg.blockDim = dim3(kMidThreads, 1, 1);
         cfg.dynamicSmemBytes = (size_t)g.smem_bytes;
         cfg.stream = st;
-        cudaLaunchAttribute attr[2];
-        int n_attr = 0;
-        if (g.cluster) {   // the slices of a tile are one cluster (consecutive blockIdx.x)
-            attr[n_attr].id = cudaLaunchAttributeClusterDimension;
-            attr[n_attr].val.clusterDim.x = (unsigned)g.split_k;
-            attr[n_attr].val.clusterDim.y = 1;
-            attr[n_attr].val.clusterDim.z = 1;
-            ++n_attr;
-        }
-        if (d->pdl_allowed(st)) {
-            attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
-            ++n_attr;
-        }
-        cfg.attrs = attr;
-        cfg.numAttrs = n_attr;
-        if (cudaLaunchKernelEx(&cfg, kern, tmap, p) != cudaSuccess) {
-            cudaGetLastError();
+        if (!launch_gemm_kernel(d, cfg, g.cluster ? g.split_k : 1, kern, tmap, p)) {   // (the slices of a tile are one cluster)
             if (g.cluster) {   // (see the warp-MMA kernel below)
                 d->cluster_ok = false;
                 return gemm_locked(A, Wq, S, Z, bias, C, M, N, K, group, split_k, path, flags, act, stream);
@@ -1223,22 +1201,12 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
             }
             attr_set = true;
         }
-        // programmatic dependent launch: this kernel's prologue and weight prefetch may overlap the
-        // tail of the previous kernel in the stream; it orders itself with griddepcontrol.wait
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(g.ctas, 1, 1);
         cfg.blockDim = dim3(kTileThreads, 1, 1);
         cfg.dynamicSmemBytes = (size_t)g.smem_bytes;
         cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = d->pdl_allowed(st) ? 1 : 0;
-        if (cudaLaunchKernelEx(&cfg, kern, tmap, p) != cudaSuccess) {
-            cudaGetLastError();
-            return W4A16_ERR_CUDA;
-        }
+        if (!launch_gemm_kernel(d, cfg, 1, kern, tmap, p)) return W4A16_ERR_CUDA;
         if (g.split_k != 1)
             return launch_tile_reduce(p.ws, C, M, N, G, g.mt, g.n_tiles, g.tiles, g.split_k, g.nchunks, bf, epi, st);
         return W4A16_OK;
@@ -1280,31 +1248,12 @@ int gemm_locked(const uint16_t* A, const void* Wq, const void* S, const void* Z,
         }
         attr_set = true;
     }
-    // programmatic dependent launch (see the tile path above): prologue and weight prefetch may overlap
-    // the tail of the previous kernel in the stream
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(g.ctas, g.mchunks, 1);
     cfg.blockDim = dim3(kDecThreads, 1, 1);
     cfg.dynamicSmemBytes = (size_t)g.smem_bytes;
     cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    int n_attr = 0;
-    if (g.cluster) {   // the split_k CTAs of a column tile are one cluster (consecutive blockIdx.x)
-        attr[n_attr].id = cudaLaunchAttributeClusterDimension;
-        attr[n_attr].val.clusterDim.x = (unsigned)g.split_k;
-        attr[n_attr].val.clusterDim.y = 1;
-        attr[n_attr].val.clusterDim.z = 1;
-        ++n_attr;
-    }
-    if (d->pdl_allowed(st)) {
-        attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
-        ++n_attr;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = n_attr;
-    if (cudaLaunchKernelEx(&cfg, kern, tmap_a, p) != cudaSuccess) {
-        cudaGetLastError();
+    if (!launch_gemm_kernel(d, cfg, g.cluster ? g.split_k : 1, kern, tmap_a, p)) {   // (the split_k CTAs of a column tile are one cluster)
         if (g.cluster) {
             // the device would not place the clusters: from now on the workspace exchange (and the path
             // rule that goes with it), starting with this call

@@ -1,0 +1,59 @@
+// Which GEMM launches may begin before the previous kernel of their stream has ended.  Host code without CUDA calls.
+//
+// Programmatic dependent launch lets a GEMM kernel request packed weights while the previous kernel of its stream still runs.
+// That kernel may be a w4a16_pack that writes those weights (pack_kernel lets the next launch start as soon as all of its CTAs
+// are there), or may itself have started before such a pack ended.  So the first GEMM launched on a stream after any pack on
+// the device is a plain, fully ordered launch; behind a GEMM that was itself ordered behind the pack, the next ones may
+// overlap their predecessor again.
+#pragma once
+
+#include <stdint.h>
+
+namespace w4a16 {
+
+class PackOrder {
+public:
+    void pack_issued() { ++epoch_; }
+
+    // Has a GEMM been launched on `stream` since the last pack?
+    bool may_overlap(uintptr_t stream) const {
+        for (const Slot& s : slots_)
+            if (s.epoch != 0 && s.stream == stream) return s.epoch == epoch_;
+        return false;
+    }
+
+    // f(overlap) launches a GEMM kernel and tells whether it got onto the stream.  A launch that was refused orders nothing:
+    // only one that is there stands between the pack and what comes behind.
+    template <typename F>
+    bool launch(uintptr_t stream, const F& f) {
+        const bool overlap = may_overlap(stream);
+        const bool ok = f(overlap);
+        if (ok && !overlap) launched(stream);
+        return ok;
+    }
+
+private:
+    // The epoch counts the packs; a slot holds the epoch of its stream's last GEMM launch.  (A stream without a slot gets a
+    // plain launch, so that what is evicted costs no more than that.)
+    struct Slot { uintptr_t stream; unsigned long long epoch; };
+    static constexpr int kSlots = 32;
+
+    void launched(uintptr_t stream) {
+        Slot* slot = nullptr;
+        for (Slot& s : slots_)
+            if (s.epoch != 0 && s.stream == stream) { slot = &s; break; }
+        for (int i = 0; slot == nullptr && i < kSlots; ++i)
+            if (slots_[i].epoch == 0) slot = &slots_[i];
+        if (slot == nullptr) {
+            slot = &slots_[evict_];
+            evict_ = (evict_ + 1) % kSlots;
+        }
+        *slot = {stream, epoch_};
+    }
+
+    unsigned long long epoch_ = 1;
+    Slot slots_[kSlots] = {};
+    int evict_ = 0;
+};
+
+}  // namespace w4a16
