@@ -11,12 +11,16 @@
 
 namespace w4a16 {
 
+// Takes streams by their handles (cudaStream_t).
+constexpr uintptr_t kPerThreadStream = 0x2;          // cudaStreamPerThread: one handle for a stream of each host thread
+
 class PackOrder {
 public:
     void pack_issued() { ++epoch_; }
 
     // Has a GEMM been launched on `stream` since the last pack?
     bool may_overlap(uintptr_t stream) const {
+        stream = own(stream);
         for (const Slot& s : slots_)
             if (s.epoch != 0 && s.stream == stream) return s.epoch == epoch_;
         return false;
@@ -28,7 +32,7 @@ public:
     bool launch(uintptr_t stream, const F& f) {
         const bool overlap = may_overlap(stream);
         const bool ok = f(overlap);
-        if (ok && !overlap) launched(stream);
+        if (ok && !overlap) launched(own(stream));
         return ok;
     }
 
@@ -37,6 +41,13 @@ private:
     // plain launch, so that what is evicted costs no more than that.)
     struct Slot { uintptr_t stream; unsigned long long epoch; };
     static constexpr int kSlots = 32;
+
+    // The calling thread's own stream of that handle.  (An address is no handle of another stream; the next thread that gets
+    // it inherits a record like the one that a new stream inherits with a handle: older than any pack still to come.)
+    static uintptr_t own(uintptr_t stream) {
+        static thread_local char thread;
+        return stream == kPerThreadStream ? reinterpret_cast<uintptr_t>(&thread) : stream;
+    }
 
     void launched(uintptr_t stream) {
         Slot* slot = nullptr;

@@ -6,6 +6,7 @@ after a w4a16_pack enqueued on that stream.  The status path (a bounded wait tha
 exercised with the library's diagnostic kernel: nothing faults, the context stays usable.
 """
 import mmap
+import threading
 
 import numpy as np
 import pytest
@@ -52,6 +53,37 @@ def test_pack_then_gemm_on_a_side_stream_with_another_stream_in_between():
             first = c_bits(C).copy()
         assert np.array_equal(c_bits(C), first)
         del pw, filler
+    del ws
+
+
+def test_pack_then_gemm_on_the_per_thread_stream_with_another_thread_in_between():
+    """cudaStreamPerThread names a stream of each thread: a GEMM of another thread under the same handle, between this
+    thread's pack and GEMM, must not count as the first one behind the pack."""
+    M, K, N, per_thread = 4, 11008, 4096, 2
+    probs = [wl.make_problem(M, K, N, seed=3110 + i) for i in range(3)]
+    raw = [[to_dev(d[k]) for k in ("Wq", "S", "Z")] for d in probs]
+    pw, ws = pack_problem(probs[0], N, K), ensure_ws(M, N, K, 0)
+    other = wl.make_problem(M, 1024, 256, seed=3120)
+    other_pw, A_other, A = pack_problem(other, 256, 1024), to_dev(other["A"]), [to_dev(d["A"]) for d in probs]
+    C, C_other = [torch.empty((M, N), dtype=torch.float16, device="cuda") for _ in probs], torch.empty((M, 256), dtype=torch.float16, device="cuda")
+    L, dev = B.load(), torch.cuda.current_device()
+    torch.cuda.synchronize()
+
+    def gemm(a, w, c, split_k):
+        torch.cuda.set_device(dev)
+        assert L.w4a16_gemm(a.data_ptr(), w.Wq.data_ptr(), w.S.data_ptr(), w.Z.data_ptr(), c.data_ptr(), M, w.N, w.K, 128, split_k, per_thread) == 0
+
+    for r, a, c in zip(raw, A, C):
+        for _ in range(4):                       # (several, so that the last is still to come when the GEMM is enqueued)
+            assert L.w4a16_pack(r[0].data_ptr(), r[1].data_ptr(), r[2].data_ptr(), pw.Wq.data_ptr(), pw.S.data_ptr(), pw.Z.data_ptr(), N, K, 128, per_thread) == 0
+        t = threading.Thread(target=gemm, args=(A_other, other_pw, C_other, 1))
+        t.start()
+        t.join()
+        gemm(a, pw, c, 0)
+    torch.cuda.synchronize()
+    assert B.w4a16_device_status() == 0
+    for d, c in zip(probs, C):
+        assert_close(c_f64(c), oracle.gemm(d["A"], d["Wq"], d["S"], d["Z"], M, N, K, 128), "per-thread stream")
     del ws
 
 

@@ -3,6 +3,7 @@ compiler and driven through a small C interface."""
 import ctypes
 import os
 import subprocess
+import threading
 
 import pytest
 
@@ -78,3 +79,20 @@ def test_a_refused_launch_orders_nothing(lib):
     assert [o.gemm(A, accepted=False), o.gemm(A, accepted=False), o.gemm(A), o.gemm(A)] == ["plain", "plain", "plain", "overlapped"]
     # one that is refused where overlap was allowed takes nothing away
     assert [o.gemm(A, accepted=False), o.gemm(A)] == ["overlapped", "overlapped"]
+
+
+def test_the_per_thread_handle_is_a_stream_of_each_thread(lib):
+    """A GEMM on another thread's stream of the same handle stands behind nothing of this thread's."""
+    per_thread, o = 2, Order(lib)
+
+    def on_another_thread(f):
+        got = []
+        t = threading.Thread(target=lambda: got.append(f()))
+        t.start()
+        t.join()
+        return got[0]
+
+    assert [o.gemm(per_thread), o.gemm(per_thread)] == ["plain", "overlapped"]
+    o.pack()
+    assert on_another_thread(lambda: [o.gemm(per_thread), o.gemm(per_thread)]) == ["plain", "overlapped"]
+    assert [o.gemm(per_thread), o.gemm(per_thread)] == ["plain", "overlapped"]
