@@ -68,6 +68,18 @@ int current_device(DeviceState** out) {
     return W4A16_OK;
 }
 
+PackOrder::Queue queue_of(cudaStream_t st) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) {
+        cudaGetLastError();    // (the default stream while another one is captured: the launch will be refused)
+        id = ~0ull;
+    } else if (status == cudaStreamCaptureStatusNone) {
+        id = 0;
+    }
+    return {reinterpret_cast<uintptr_t>(st), id};
+}
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 int check_weight_shape(int N, int K, int group) {
@@ -954,7 +966,7 @@ bool launch_gemm_kernel(DeviceState* d, cudaLaunchConfig_t cfg, int cluster, voi
         attr[n_attr].val.clusterDim.z = 1;
         ++n_attr;
     }
-    return d->order.launch(reinterpret_cast<uintptr_t>(cfg.stream), [&](bool overlap) {
+    return d->order.launch(queue_of(cfg.stream), [&](bool overlap) {
         if (overlap) {
             attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
             attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
@@ -1053,7 +1065,7 @@ int stage_activations(const void* host, void* dev, int n16, cudaStream_t st) {
     cfg.stream = st;
     cfg.attrs = attr;
     // (behind a pack a plain launch: the GEMM that follows asks for packed weights while this kernel runs)
-    cfg.numAttrs = d->order.may_overlap(reinterpret_cast<uintptr_t>(st)) ? 1 : 0;
+    cfg.numAttrs = d->order.may_overlap(queue_of(st)) ? 1 : 0;
     if (cudaLaunchKernelEx(&cfg, stage_activations_kernel, static_cast<const uint4*>(host), static_cast<uint4*>(dev), n16) != cudaSuccess) {
         cudaGetLastError();
         return W4A16_ERR_CUDA;

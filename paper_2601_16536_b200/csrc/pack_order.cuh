@@ -11,55 +11,63 @@
 
 namespace w4a16 {
 
-// Takes streams by their handles (cudaStream_t).
 constexpr uintptr_t kPerThreadStream = 0x2;          // cudaStreamPerThread: one handle for a stream of each host thread
 
 class PackOrder {
 public:
+    // What launches are ordered in: a stream by its handle (cudaStream_t), or a capture of it by the capture's id.  What is
+    // captured does not run on the stream, so that neither says anything about the other.
+    struct Queue { uintptr_t stream; unsigned long long capture; };
+
     void pack_issued() { ++epoch_; }
 
-    // Has a GEMM been launched on `stream` since the last pack?
-    bool may_overlap(uintptr_t stream) const {
-        stream = own(stream);
+    // Has a GEMM been launched in `queue` since the last pack?
+    bool may_overlap(Queue queue) const {
+        queue = own(queue);
         for (const Slot& s : slots_)
-            if (s.epoch != 0 && s.stream == stream) return s.epoch == epoch_;
+            if (s.of(queue)) return s.epoch == epoch_;
         return false;
     }
 
-    // f(overlap) launches a GEMM kernel and tells whether it got onto the stream.  A launch that was refused orders nothing:
+    // f(overlap) launches a GEMM kernel and tells whether it got into the queue.  A launch that was refused orders nothing:
     // only one that is there stands between the pack and what comes behind.
     template <typename F>
-    bool launch(uintptr_t stream, const F& f) {
-        const bool overlap = may_overlap(stream);
+    bool launch(Queue queue, const F& f) {
+        const bool overlap = may_overlap(queue);
         const bool ok = f(overlap);
-        if (ok && !overlap) launched(own(stream));
+        if (ok && !overlap) launched(own(queue));
         return ok;
     }
 
 private:
-    // The epoch counts the packs; a slot holds the epoch of its stream's last GEMM launch.  (A stream without a slot gets a
+    // The epoch counts the packs; a slot holds the epoch of its queue's last GEMM launch.  (A queue without a slot gets a
     // plain launch, so that what is evicted costs no more than that.)
-    struct Slot { uintptr_t stream; unsigned long long epoch; };
+    struct Slot {
+        Queue queue;
+        unsigned long long epoch;
+        bool of(const Queue& q) const { return epoch != 0 && queue.stream == q.stream && queue.capture == q.capture; }
+    };
     static constexpr int kSlots = 32;
 
     // The calling thread's own stream of that handle.  (An address is no handle of another stream; the next thread that gets
     // it inherits a record like the one that a new stream inherits with a handle: older than any pack still to come.)
-    static uintptr_t own(uintptr_t stream) {
+    static Queue own(Queue queue) {
         static thread_local char thread;
-        return stream == kPerThreadStream ? reinterpret_cast<uintptr_t>(&thread) : stream;
+        if (queue.stream == kPerThreadStream) queue.stream = reinterpret_cast<uintptr_t>(&thread);
+        return queue;
     }
 
-    void launched(uintptr_t stream) {
+    void launched(const Queue& queue) {
         Slot* slot = nullptr;
         for (Slot& s : slots_)
-            if (s.epoch != 0 && s.stream == stream) { slot = &s; break; }
+            if (s.of(queue)) { slot = &s; break; }
         for (int i = 0; slot == nullptr && i < kSlots; ++i)
             if (slots_[i].epoch == 0) slot = &slots_[i];
         if (slot == nullptr) {
             slot = &slots_[evict_];
             evict_ = (evict_ + 1) % kSlots;
         }
-        *slot = {stream, epoch_};
+        *slot = {queue, epoch_};
     }
 
     unsigned long long epoch_ = 1;

@@ -87,6 +87,47 @@ def test_pack_then_gemm_on_the_per_thread_stream_with_another_thread_in_between(
     del ws
 
 
+@pytest.mark.parametrize("M", [1, 64, 300])
+def test_pack_then_a_captured_gemm_then_gemm_on_the_same_stream(M):
+    """The captured GEMM does not run on the stream, so the next one there still is the first behind the pack.  Replayed
+    behind another pack, the graph has the new weights."""
+    K, N = 4096, 2048
+    probs = [wl.make_problem(M, K, N, seed=3130 + i) for i in range(3)]
+    raw = [[to_dev(d[k]) for k in ("Wq", "S", "Z")] for d in probs]
+    A = to_dev(probs[0]["A"])
+    pw, ws, L = pack_problem(probs[0], N, K), ensure_ws(M, N, K, 0), B.load()
+    want = []
+    for r in raw:
+        want.append(c_bits(B.w4a16_gemm(A, B.w4a16_pack(*r, N, K))).copy())
+        torch.cuda.synchronize()
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    outs = [torch.empty((M, N), dtype=torch.float16, device="cuda") for _ in range(4)]
+    captured = torch.empty((M, N), dtype=torch.float16, device="cuda")
+    filler = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+
+    def pack(r):
+        filler.fill_(1)                          # the pack is still to come when what is behind it is enqueued
+        assert L.w4a16_pack(r[0].data_ptr(), r[1].data_ptr(), r[2].data_ptr(), pw.Wq.data_ptr(), pw.S.data_ptr(), pw.Z.data_ptr(), N, K, 128, side.cuda_stream) == 0
+
+    with torch.cuda.stream(side):
+        B.w4a16_gemm(A, pw, C=outs[3])
+        pack(raw[1])
+        graph.capture_begin()
+        B.w4a16_gemm(A, pw, C=captured)
+        graph.capture_end()
+        B.w4a16_gemm(A, pw, C=outs[0])
+        pack(raw[2])
+        graph.replay()
+        outs[1].copy_(captured)
+        B.w4a16_gemm(A, pw, C=outs[2])
+    torch.cuda.synchronize()
+    assert B.w4a16_device_status() == 0
+    for c, w in zip(outs, (want[1], want[2], want[2], want[0])):
+        assert np.array_equal(c_bits(c), w)
+    del ws
+
+
 @pytest.mark.parametrize("path,M", [(B.PATH_DECODE, 8), (B.PATH_TILE, 32)])
 def test_gemm_on_a_non_default_stream_matches_the_default_stream(path, M):
     K, N = 2304, 512

@@ -16,9 +16,9 @@ void* order_new() { return new PackOrder; }
 void order_delete(void* o) { delete static_cast<PackOrder*>(o); }
 void order_pack(void* o) { static_cast<PackOrder*>(o)->pack_issued(); }
 // returns whether the launch was allowed to overlap; `accepted`: whether it got onto the stream
-int order_launch(void* o, unsigned long long stream, int accepted) {
+int order_launch(void* o, unsigned long long stream, unsigned long long capture, int accepted) {
     bool overlapped = false;
-    static_cast<PackOrder*>(o)->launch((uintptr_t)stream, [&](bool overlap) { overlapped = overlap; return accepted != 0; });
+    static_cast<PackOrder*>(o)->launch({(uintptr_t)stream, capture}, [&](bool overlap) { overlapped = overlap; return accepted != 0; });
     return overlapped ? 1 : 0;
 }
 }
@@ -35,7 +35,7 @@ def lib(tmp_path_factory):
     L = ctypes.CDLL(so)
     L.order_new.restype = ctypes.c_void_p
     L.order_delete.argtypes = L.order_pack.argtypes = [ctypes.c_void_p]
-    L.order_launch.argtypes = [ctypes.c_void_p, ctypes.c_ulonglong, ctypes.c_int]
+    L.order_launch.argtypes = [ctypes.c_void_p, ctypes.c_ulonglong, ctypes.c_ulonglong, ctypes.c_int]
     return L
 
 
@@ -49,8 +49,8 @@ class Order:
     def pack(self):
         self.L.order_pack(self.o)
 
-    def gemm(self, stream, accepted=True):
-        return "overlapped" if self.L.order_launch(self.o, stream, int(accepted)) else "plain"
+    def gemm(self, stream, accepted=True, capture=0):
+        return "overlapped" if self.L.order_launch(self.o, stream, capture, int(accepted)) else "plain"
 
 
 A, B = 0x5000, 0x6000
@@ -96,3 +96,16 @@ def test_the_per_thread_handle_is_a_stream_of_each_thread(lib):
     o.pack()
     assert on_another_thread(lambda: [o.gemm(per_thread), o.gemm(per_thread)]) == ["plain", "overlapped"]
     assert [o.gemm(per_thread), o.gemm(per_thread)] == ["plain", "overlapped"]
+
+
+def test_a_captured_gemm_orders_nothing_on_its_stream(lib):
+    """Pack on a stream, a GEMM captured from that stream into a graph that is not replayed, then a GEMM on the stream: the
+    last one stands directly behind the pack.  And a capture begins like a stream that nothing is known of."""
+    o = Order(lib)
+    assert [o.gemm(A), o.gemm(A)] == ["plain", "overlapped"]
+    o.pack()
+    assert [o.gemm(A, capture=7), o.gemm(A, capture=7)] == ["plain", "overlapped"]
+    assert [o.gemm(A), o.gemm(A)] == ["plain", "overlapped"]
+    assert [o.gemm(A, capture=8), o.gemm(A, capture=8)] == ["plain", "overlapped"]
+    o.pack()                                             # captured or not
+    assert [o.gemm(A, capture=8), o.gemm(A)] == ["plain", "plain"]
