@@ -724,9 +724,9 @@ GemmPlan gemm_plan(int M, int N, int G, int sg, int split_k, int path_asked, boo
 }
 
 // Quantizer, pack and dequantization: set up while the kernel in front runs, and ordered behind it by the kernels themselves (in a row, as a
-// model load calls them, a gap between two launches costs about 2 us).
+// model load calls them, a gap between two launches costs about 2 us).  In a graph plain launches, with a pack that releases nothing.
 template <typename... P, typename... A>
-int launch_block_kernel(void (*kern)(P...), unsigned blocks, cudaStream_t st, A... args) {
+int launch_block_kernel(void (*kern)(P...), unsigned blocks, cudaStream_t st, bool early, A... args) {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -735,7 +735,7 @@ int launch_block_kernel(void (*kern)(P...), unsigned blocks, cudaStream_t st, A.
     cfg.blockDim = dim3(kBlockKernelThreads, 1, 1);
     cfg.stream = st;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     if (cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...) != cudaSuccess) {
         cudaGetLastError();
         return W4A16_ERR_CUDA;
@@ -882,7 +882,7 @@ int w4a16_quantize(const uint16_t* W16, uint32_t* Wq_raw, uint16_t* S_raw, uint8
     const unsigned blocks = (unsigned)((long long)G * (N / kTileN));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     uint8_t* z = sym ? nullptr : Z_raw;
-    return launch_block_kernel(bf ? quantize_kernel<true> : quantize_kernel<false>, blocks, st, W16, Wq_raw, S_raw, z, N, G, sg, sym ? 1 : 0);
+    return launch_block_kernel(bf ? quantize_kernel<true> : quantize_kernel<false>, blocks, st, PackOrder::may_release(queue_of(st)), W16, Wq_raw, S_raw, z, N, G, sg, sym ? 1 : 0);
 }
 
 int w4a16_pack_fmt(const uint32_t* Wq_raw, const uint16_t* S_raw, const uint8_t* Z_raw, void* Wq, void* S, void* Z,
@@ -902,9 +902,10 @@ int w4a16_pack_fmt(const uint32_t* Wq_raw, const uint16_t* S_raw, const uint8_t*
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int G = K / kGroup, sg = kGroup / group;
     const int blocks = (int)((long long)G * (N / kTileN)), per = kBlockKernelThreads / 64;   // half a block a warp
+    const bool early = PackOrder::may_release(queue_of(st));
     d->order.pack_issued();
-    return launch_block_kernel(pack_kernel, (unsigned)((blocks + per - 1) / per), st, Wq_raw, S_raw, sym ? nullptr : Z_raw,
-                               static_cast<uint32_t*>(Wq), static_cast<uint16_t*>(S), sym ? nullptr : static_cast<uint8_t*>(Z), N, G, sg, blocks);
+    return launch_block_kernel(pack_kernel, (unsigned)((blocks + per - 1) / per), st, early, Wq_raw, S_raw, sym ? nullptr : Z_raw,
+                               static_cast<uint32_t*>(Wq), static_cast<uint16_t*>(S), sym ? nullptr : static_cast<uint8_t*>(Z), N, G, sg, blocks, early);
 }
 
 int w4a16_pack(const uint32_t* Wq_raw, const uint16_t* S_raw, const uint8_t* Z_raw, void* Wq, void* S, void* Z,
@@ -926,7 +927,8 @@ int w4a16_dequant_fmt(const void* Wq, const void* S, const void* Z, uint16_t* W1
     if ((rc = current_device(&d)) != W4A16_OK) return rc;
     if (!d->is_sm100) return W4A16_ERR_ARCH;
     const unsigned blocks = (unsigned)((long long)(K / kGroup) * (N / kTileN));
-    return launch_block_kernel(bf ? dequant_kernel<true> : dequant_kernel<false>, blocks, static_cast<cudaStream_t>(stream),
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    return launch_block_kernel(bf ? dequant_kernel<true> : dequant_kernel<false>, blocks, st, PackOrder::may_release(queue_of(st)),
                                static_cast<const uint32_t*>(Wq), static_cast<const uint16_t*>(S),
                                sym ? nullptr : static_cast<const uint32_t*>(Z), W16, N, K / kGroup, kGroup / group);
 }

@@ -35,8 +35,8 @@ __device__ __forceinline__ uint32_t pack_word(uint32_t r) {
 // warp per block, plain launch 12.5 us, this form 10.6 (HBM floor 7.2), 8.5 behind the quantizer.
 __global__ void __launch_bounds__(kBlockKernelThreads)
 pack_kernel(const uint32_t* __restrict__ Wq_raw, const uint16_t* __restrict__ S_raw, const uint8_t* __restrict__ Z_raw,
-            uint32_t* __restrict__ Wq, uint16_t* __restrict__ S, uint8_t* __restrict__ Z, int N, int G, int sg, int blocks) {
-    next_launch_may_start();
+            uint32_t* __restrict__ Wq, uint16_t* __restrict__ S, uint8_t* __restrict__ Z, int N, int G, int sg, int blocks, bool release) {
+    if (release) next_launch_may_start();
     wait_for_launch_before();            // (every warp: see there)
     const int i = blockIdx.x * (kBlockKernelThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int b = i >> 1, h = i & 1;

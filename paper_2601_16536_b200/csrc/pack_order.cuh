@@ -21,6 +21,10 @@ public:
 
     void pack_issued() { ++epoch_; }
 
+    // May a pack, or a kernel that may come behind one, start early in `queue` and let the next launch start early?  Not in a
+    // capture: the replays of a graph are not counted, so that a GEMM behind one may be allowed to overlap.
+    static bool may_release(const Queue& queue) { return queue.capture == 0; }
+
     // Has a GEMM been launched in `queue` since the last pack?
     bool may_overlap(Queue queue) const {
         queue = own(queue);

@@ -107,3 +107,42 @@ def test_a_row_of_quantize_and_pack_calls_is_ordered(K, N):
         one = B.w4a16_pack(q, s, z, N, K)
         torch.cuda.synchronize()
         assert torch.equal(pw.Wq, one.Wq) and torch.equal(pw.S, one.S) and torch.equal(pw.Z, one.Z)
+
+
+@pytest.mark.parametrize("M", [1, 64, 300])
+def test_quantize_pack_dequantize_in_a_graph_in_front_of_gemms(M):
+    """The three kernels captured and replayed on new weights, with two GEMMs on the stream behind every replay: what they
+    request early is what the replay has packed."""
+    K, N = 2048, 1024
+    Ws = [(torch.randn(K, N, device="cuda") * 0.04 * (1 + i)).half() for i in range(4)]
+    W, A = Ws[0].clone(), torch.randn(M, K, device="cuda").half()
+    ws, want = ensure_ws(M, N, K, 0), []
+    for w in Ws:
+        pw = B.w4a16_pack(*B.w4a16_quantize(w), N, K)
+        torch.cuda.synchronize()
+        want.append((B.w4a16_dequant(pw), B.w4a16_gemm(A, pw)))
+        torch.cuda.synchronize()
+    L, side, graph = B.load(), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    Wq, S, Z = B.w4a16_quantize(W)
+    pw = B.w4a16_pack(Wq, S, Z, N, K)
+    W16 = torch.empty((K, N), dtype=torch.float16, device="cuda")
+    got = [(torch.empty_like(W16), *(torch.empty((M, N), dtype=torch.float16, device="cuda") for _ in range(2))) for _ in Ws]
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        graph.capture_begin()
+        st = side.cuda_stream
+        assert L.w4a16_quantize(W.data_ptr(), Wq.data_ptr(), S.data_ptr(), Z.data_ptr(), N, K, 128, 0, st) == 0
+        assert L.w4a16_pack(Wq.data_ptr(), S.data_ptr(), Z.data_ptr(), pw.Wq.data_ptr(), pw.S.data_ptr(), pw.Z.data_ptr(), N, K, 128, st) == 0
+        B.w4a16_dequant(pw, out=W16)
+        graph.capture_end()
+        for w, (d, c0, c1) in zip(Ws, got):
+            W.copy_(w)
+            graph.replay()
+            B.w4a16_gemm(A, pw, C=c0)
+            B.w4a16_gemm(A, pw, C=c1)
+            d.copy_(W16)
+    torch.cuda.synchronize()
+    assert B.w4a16_device_status() == 0
+    for (d, c), (gd, g0, g1) in zip(want, got):
+        assert torch.equal(d, gd) and torch.equal(c, g0) and torch.equal(c, g1)
+    del ws

@@ -15,6 +15,7 @@ extern "C" {
 void* order_new() { return new PackOrder; }
 void order_delete(void* o) { delete static_cast<PackOrder*>(o); }
 void order_pack(void* o) { static_cast<PackOrder*>(o)->pack_issued(); }
+int order_may_release(unsigned long long stream, unsigned long long capture) { return PackOrder::may_release({(uintptr_t)stream, capture}); }
 // returns whether the launch was allowed to overlap; `accepted`: whether it got onto the stream
 int order_launch(void* o, unsigned long long stream, unsigned long long capture, int accepted) {
     bool overlapped = false;
@@ -35,6 +36,7 @@ def lib(tmp_path_factory):
     L = ctypes.CDLL(so)
     L.order_new.restype = ctypes.c_void_p
     L.order_delete.argtypes = L.order_pack.argtypes = [ctypes.c_void_p]
+    L.order_may_release.argtypes = [ctypes.c_ulonglong, ctypes.c_ulonglong]
     L.order_launch.argtypes = [ctypes.c_void_p, ctypes.c_ulonglong, ctypes.c_ulonglong, ctypes.c_int]
     return L
 
@@ -109,3 +111,11 @@ def test_a_captured_gemm_orders_nothing_on_its_stream(lib):
     assert [o.gemm(A, capture=8), o.gemm(A, capture=8)] == ["plain", "overlapped"]
     o.pack()                                             # captured or not
     assert [o.gemm(A, capture=8), o.gemm(A)] == ["plain", "plain"]
+
+
+def test_a_pack_in_a_graph_releases_nothing(lib):
+    """A replay is no call of the library: a GEMM behind one goes by what was launched before."""
+    assert lib.order_may_release(A, 0) and not lib.order_may_release(A, 7)
+    o = Order(lib)
+    o.pack()                                             # captured
+    assert [o.gemm(A), o.gemm(A)] == ["plain", "overlapped"]   # ... and the second may stand directly behind a replay
