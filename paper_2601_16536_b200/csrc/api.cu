@@ -68,16 +68,15 @@ int current_device(DeviceState** out) {
     return W4A16_OK;
 }
 
-PackOrder::Queue queue_of(cudaStream_t st) {
+// The capture that `st` is in; 0 = none.
+unsigned long long capture_of(cudaStream_t st) {
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
     unsigned long long id = 0;
     if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) {
         cudaGetLastError();    // (the default stream while another one is captured: the launch will be refused)
-        id = ~0ull;
-    } else if (status == cudaStreamCaptureStatusNone) {
-        id = 0;
+        return ~0ull;
     }
-    return {reinterpret_cast<uintptr_t>(st), id};
+    return status == cudaStreamCaptureStatusNone ? 0 : id;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -882,7 +881,7 @@ int w4a16_quantize(const uint16_t* W16, uint32_t* Wq_raw, uint16_t* S_raw, uint8
     const unsigned blocks = (unsigned)((long long)G * (N / kTileN));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     uint8_t* z = sym ? nullptr : Z_raw;
-    return launch_block_kernel(bf ? quantize_kernel<true> : quantize_kernel<false>, blocks, st, PackOrder::may_release(queue_of(st)), W16, Wq_raw, S_raw, z, N, G, sg, sym ? 1 : 0);
+    return launch_block_kernel(bf ? quantize_kernel<true> : quantize_kernel<false>, blocks, st, PackOrder::may_release(capture_of(st)), W16, Wq_raw, S_raw, z, N, G, sg, sym ? 1 : 0);
 }
 
 int w4a16_pack_fmt(const uint32_t* Wq_raw, const uint16_t* S_raw, const uint8_t* Z_raw, void* Wq, void* S, void* Z,
@@ -902,7 +901,7 @@ int w4a16_pack_fmt(const uint32_t* Wq_raw, const uint16_t* S_raw, const uint8_t*
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int G = K / kGroup, sg = kGroup / group;
     const int blocks = (int)((long long)G * (N / kTileN)), per = kBlockKernelThreads / 64;   // half a block a warp
-    const bool early = PackOrder::may_release(queue_of(st));
+    const bool early = PackOrder::may_release(capture_of(st));
     d->order.pack_issued();
     return launch_block_kernel(pack_kernel, (unsigned)((blocks + per - 1) / per), st, early, Wq_raw, S_raw, sym ? nullptr : Z_raw,
                                static_cast<uint32_t*>(Wq), static_cast<uint16_t*>(S), sym ? nullptr : static_cast<uint8_t*>(Z), N, G, sg, blocks, early);
@@ -928,7 +927,7 @@ int w4a16_dequant_fmt(const void* Wq, const void* S, const void* Z, uint16_t* W1
     if (!d->is_sm100) return W4A16_ERR_ARCH;
     const unsigned blocks = (unsigned)((long long)(K / kGroup) * (N / kTileN));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    return launch_block_kernel(bf ? dequant_kernel<true> : dequant_kernel<false>, blocks, st, PackOrder::may_release(queue_of(st)),
+    return launch_block_kernel(bf ? dequant_kernel<true> : dequant_kernel<false>, blocks, st, PackOrder::may_release(capture_of(st)),
                                static_cast<const uint32_t*>(Wq), static_cast<const uint16_t*>(S),
                                sym ? nullptr : static_cast<const uint32_t*>(Z), W16, N, K / kGroup, kGroup / group);
 }
@@ -968,7 +967,7 @@ bool launch_gemm_kernel(DeviceState* d, cudaLaunchConfig_t cfg, int cluster, voi
         attr[n_attr].val.clusterDim.z = 1;
         ++n_attr;
     }
-    return d->order.launch(queue_of(cfg.stream), [&](bool overlap) {
+    return d->order.launch(reinterpret_cast<uintptr_t>(cfg.stream), [&] { return capture_of(cfg.stream); }, [&](bool overlap) {
         if (overlap) {
             attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
             attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
@@ -1067,7 +1066,7 @@ int stage_activations(const void* host, void* dev, int n16, cudaStream_t st) {
     cfg.stream = st;
     cfg.attrs = attr;
     // (behind a pack a plain launch: the GEMM that follows asks for packed weights while this kernel runs)
-    cfg.numAttrs = d->order.may_overlap(queue_of(st)) ? 1 : 0;
+    cfg.numAttrs = d->order.may_overlap(reinterpret_cast<uintptr_t>(st), [&] { return capture_of(st); }) ? 1 : 0;
     if (cudaLaunchKernelEx(&cfg, stage_activations_kernel, static_cast<const uint4*>(host), static_cast<uint4*>(dev), n16) != cudaSuccess) {
         cudaGetLastError();
         return W4A16_ERR_CUDA;

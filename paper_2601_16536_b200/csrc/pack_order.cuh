@@ -15,37 +15,38 @@ constexpr uintptr_t kPerThreadStream = 0x2;          // cudaStreamPerThread: one
 
 class PackOrder {
 public:
-    // What launches are ordered in: a stream by its handle (cudaStream_t), or a capture of it by the capture's id.  What is
-    // captured does not run on the stream, so that neither says anything about the other.
-    struct Queue { uintptr_t stream; unsigned long long capture; };
-
     void pack_issued() { ++epoch_; }
 
-    // May a pack, or a kernel that may come behind one, start early in `queue` and let the next launch start early?  Not in a
-    // capture: the replays of a graph are not counted, so that a GEMM behind one may be allowed to overlap.
-    static bool may_release(const Queue& queue) { return queue.capture == 0; }
+    // May a pack, or a kernel that may come behind one, start early and let the next launch start early?  Not in a capture (id
+    // `capture`, 0 = none): the replays of a graph are not counted, so that a GEMM behind one may be allowed to overlap.
+    static bool may_release(unsigned long long capture) { return capture == 0; }
 
-    // Has a GEMM been launched in `queue` since the last pack?
-    bool may_overlap(Queue queue) const {
-        queue = own(queue);
-        for (const Slot& s : slots_)
-            if (s.of(queue)) return s.epoch == epoch_;
-        return false;
+    // Has a GEMM been launched on `stream` (a cudaStream_t) since the last pack, or captured since then in the capture that the
+    // stream is in?  capture_of() tells its id, and is asked only where the stream's own record does not allow the overlap,
+    // because asking the runtime costs 50 to 100 ns of a call's 3.5 us: with no pack since then there is none in the capture
+    // either, and the graph's replays are ordered behind whatever is on their stream.
+    template <typename Capture>
+    bool may_overlap(uintptr_t stream, const Capture& capture_of) const {
+        if (current({own(stream), 0})) return true;
+        const unsigned long long capture = capture_of();
+        return capture != 0 && current({own(stream), capture});
     }
 
-    // f(overlap) launches a GEMM kernel and tells whether it got into the queue.  A launch that was refused orders nothing:
-    // only one that is there stands between the pack and what comes behind.
-    template <typename F>
-    bool launch(Queue queue, const F& f) {
-        const bool overlap = may_overlap(queue);
+    // f(overlap) launches a GEMM kernel and tells whether it got onto the stream.  A launch that was refused orders nothing:
+    // only one that is there stands between the pack and what comes behind.  Nor does a captured one on the stream: it does
+    // not run there.
+    template <typename Capture, typename F>
+    bool launch(uintptr_t stream, const Capture& capture_of, const F& f) {
+        const bool overlap = may_overlap(stream, capture_of);
         const bool ok = f(overlap);
-        if (ok && !overlap) launched(own(queue));
+        if (ok && !overlap) launched({own(stream), capture_of()});
         return ok;
     }
 
 private:
-    // The epoch counts the packs; a slot holds the epoch of its queue's last GEMM launch.  (A queue without a slot gets a
-    // plain launch, so that what is evicted costs no more than that.)
+    // The epoch counts the packs; a slot holds the epoch of its queue's last GEMM launch: a stream, or a capture of it.  (A
+    // queue without a slot gets a plain launch, so that what is evicted costs no more than that.)
+    struct Queue { uintptr_t stream; unsigned long long capture; };
     struct Slot {
         Queue queue;
         unsigned long long epoch;
@@ -55,10 +56,15 @@ private:
 
     // The calling thread's own stream of that handle.  (An address is no handle of another stream; the next thread that gets
     // it inherits a record like the one that a new stream inherits with a handle: older than any pack still to come.)
-    static Queue own(Queue queue) {
+    static uintptr_t own(uintptr_t stream) {
         static thread_local char thread;
-        if (queue.stream == kPerThreadStream) queue.stream = reinterpret_cast<uintptr_t>(&thread);
-        return queue;
+        return stream == kPerThreadStream ? reinterpret_cast<uintptr_t>(&thread) : stream;
+    }
+
+    bool current(const Queue& queue) const {
+        for (const Slot& s : slots_)
+            if (s.of(queue)) return s.epoch == epoch_;
+        return false;
     }
 
     void launched(const Queue& queue) {

@@ -15,11 +15,11 @@ extern "C" {
 void* order_new() { return new PackOrder; }
 void order_delete(void* o) { delete static_cast<PackOrder*>(o); }
 void order_pack(void* o) { static_cast<PackOrder*>(o)->pack_issued(); }
-int order_may_release(unsigned long long stream, unsigned long long capture) { return PackOrder::may_release({(uintptr_t)stream, capture}); }
+int order_may_release(unsigned long long capture) { return PackOrder::may_release(capture); }
 // returns whether the launch was allowed to overlap; `accepted`: whether it got onto the stream
 int order_launch(void* o, unsigned long long stream, unsigned long long capture, int accepted) {
     bool overlapped = false;
-    static_cast<PackOrder*>(o)->launch({(uintptr_t)stream, capture}, [&](bool overlap) { overlapped = overlap; return accepted != 0; });
+    static_cast<PackOrder*>(o)->launch((uintptr_t)stream, [&] { return capture; }, [&](bool overlap) { overlapped = overlap; return accepted != 0; });
     return overlapped ? 1 : 0;
 }
 }
@@ -36,7 +36,7 @@ def lib(tmp_path_factory):
     L = ctypes.CDLL(so)
     L.order_new.restype = ctypes.c_void_p
     L.order_delete.argtypes = L.order_pack.argtypes = [ctypes.c_void_p]
-    L.order_may_release.argtypes = [ctypes.c_ulonglong, ctypes.c_ulonglong]
+    L.order_may_release.argtypes = [ctypes.c_ulonglong]
     L.order_launch.argtypes = [ctypes.c_void_p, ctypes.c_ulonglong, ctypes.c_ulonglong, ctypes.c_int]
     return L
 
@@ -102,20 +102,21 @@ def test_the_per_thread_handle_is_a_stream_of_each_thread(lib):
 
 def test_a_captured_gemm_orders_nothing_on_its_stream(lib):
     """Pack on a stream, a GEMM captured from that stream into a graph that is not replayed, then a GEMM on the stream: the
-    last one stands directly behind the pack.  And a capture begins like a stream that nothing is known of."""
+    last one stands directly behind the pack."""
     o = Order(lib)
     assert [o.gemm(A), o.gemm(A)] == ["plain", "overlapped"]
     o.pack()
     assert [o.gemm(A, capture=7), o.gemm(A, capture=7)] == ["plain", "overlapped"]
-    assert [o.gemm(A), o.gemm(A)] == ["plain", "overlapped"]
     assert [o.gemm(A, capture=8), o.gemm(A, capture=8)] == ["plain", "overlapped"]
+    assert [o.gemm(A), o.gemm(A)] == ["plain", "overlapped"]
+    assert o.gemm(A, capture=9) == "overlapped"          # no pack since the stream's last GEMM, hence none in this capture
     o.pack()                                             # captured or not
     assert [o.gemm(A, capture=8), o.gemm(A)] == ["plain", "plain"]
 
 
 def test_a_pack_in_a_graph_releases_nothing(lib):
     """A replay is no call of the library: a GEMM behind one goes by what was launched before."""
-    assert lib.order_may_release(A, 0) and not lib.order_may_release(A, 7)
+    assert lib.order_may_release(0) and not lib.order_may_release(7)
     o = Order(lib)
     o.pack()                                             # captured
     assert [o.gemm(A), o.gemm(A)] == ["plain", "overlapped"]   # ... and the second may stand directly behind a replay
