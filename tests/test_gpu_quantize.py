@@ -65,6 +65,50 @@ def test_quantize_is_bit_exact_on_ties_and_extreme_scales(group, symmetric, bf16
     assert symmetric or np.array_equal(Z.cpu().numpy(), z)
 
 
+@pytest.mark.parametrize("group", [32, 64, 128])
+@pytest.mark.parametrize("symmetric", [False, True])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_quantize_infinities_and_nans(group, symmetric, bf16):
+    """A group with an infinity has scale 1 (the definition's rule for a scale that is not finite), the infinities codes 15 and
+    0.  A NaN takes no part in a group's minimum and maximum and gets code 0; what is beside it has the codes it would have
+    without it (the oracle, whose conversion of a NaN to an integer is not defined, gets another number of the group in its
+    place)."""
+    K, N = 256, 128
+    r = np.random.Generator(np.random.PCG64([group, 31]))
+    x = (r.standard_normal((K, N)) * 2.0 ** r.integers(-9, 3, size=(1, N))).astype(np.float32)
+    x[r.random((K, N)) < 0.02] = np.inf
+    x[r.random((K, N)) < 0.02] = -np.inf
+    x[:, 5] = np.inf
+    x[:, 6] = -np.inf
+    x[:, 7] = np.where(r.random(K) < 0.5, np.inf, -np.inf)
+    x[:, 64:] = np.where(np.isinf(x[:, 64:]), np.float32(0.5), x[:, 64:])          # the second tile: NaN only
+    bits = wl._bits16(x, bf16)
+    exp = 0x7F80 if bf16 else 0x7C00
+    nan = r.random((K, N)) < 0.05
+    nan[:group, 9] = True                                                          # a group of nothing else
+    nan[:, 10] = np.arange(K) % group != 3                                         # one number a group
+    poisoned = bits.copy()
+    poisoned[nan] = r.choice(np.array([exp | 1, exp | 0x40, exp | 0x8001, 0xFFFF], dtype=np.uint16), size=int(nan.sum()))
+    # oracle's weights: in place of a NaN a number that its group has anyway, or, in a group of NaN alone, 0: there scale 1 and
+    # zero point 0 are what the definition gives for the empty minimum and maximum (+inf, -inf) and for zeros alike
+    clean = bits.copy()
+    for g in range(K // group):
+        rows = slice(g * group, (g + 1) * group)
+        for n in range(N):
+            bad = nan[rows, n]
+            clean[rows, n][bad] = 0 if bad.all() else bits[rows, n][~bad][0]
+    flags = (B.FLAG_SYMMETRIC if symmetric else 0) | (B.FLAG_BF16 if bf16 else 0)
+    W = torch.from_numpy(poisoned.view(np.int16)).cuda().view(torch.bfloat16 if bf16 else torch.float16)
+    Wq, S, Z = B.w4a16_quantize(W, group, flags)
+    torch.cuda.synchronize()
+    wq, s, z = oracle.quantize(clean, K, N, group, symmetric=symmetric, bf16=bf16)
+    assert np.array_equal(S.view(torch.int16).cpu().numpy().view(np.uint16), s)
+    assert symmetric or np.array_equal(Z.cpu().numpy(), z)
+    want = oracle.unpack(wq, K, N)
+    want[nan] = 0
+    assert np.array_equal(oracle.unpack(Wq.cpu().numpy().view(np.uint32), K, N), want)
+
+
 @pytest.mark.parametrize("M,symmetric", [(4, False), (4, True), (48, False)])
 def test_quantize_pack_gemm_chain(M, symmetric):
     K, N, group = 2048, 512, 128

@@ -128,6 +128,46 @@ def test_pack_then_a_captured_gemm_then_gemm_on_the_same_stream(M):
     del ws
 
 
+@pytest.mark.parametrize("M", [1, 64, 300])
+@pytest.mark.parametrize("side", [False, True])
+def test_pack_dequantize_gemm_rows_through_one_set_of_packed_buffers(M, side):
+    """Per matrix: pack, dequantization, two GEMMs, and the quantizer on other weights in front of a third, all enqueued without
+    a synchronisation into the same buffers.  Each of these lets the next launch start early, so that it is not the GEMM's
+    direct predecessor alone that has to have ended before packed words are read."""
+    K, N = 4096, 2048
+    probs = [wl.make_problem(M, K, N, seed=3140 + i) for i in range(4)]
+    raw = [[to_dev(d[k]) for k in ("Wq", "S", "Z")] for d in probs]
+    A, W16 = to_dev(probs[0]["A"]), torch.randn(K, N, device="cuda").half()
+    ws, want = ensure_ws(M, N, K, 0), []
+    for r in raw:
+        w = B.w4a16_pack(*r, N, K)
+        torch.cuda.synchronize()
+        want.append((B.w4a16_dequant(w), B.w4a16_gemm(A, w)))
+        torch.cuda.synchronize()
+    raw16 = B.w4a16_quantize(W16)
+    pw, L = pack_problem(probs[0], N, K), B.load()
+    outs = [(torch.empty((K, N), dtype=torch.float16, device="cuda"),
+             [torch.empty((M, N), dtype=torch.float16, device="cuda") for _ in range(3)]) for _ in raw]
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream() if side else torch.cuda.current_stream()
+    with torch.cuda.stream(stream):
+        st = stream.cuda_stream
+        for r, (w16, c) in zip(raw, outs):
+            assert L.w4a16_pack(r[0].data_ptr(), r[1].data_ptr(), r[2].data_ptr(), pw.Wq.data_ptr(), pw.S.data_ptr(), pw.Z.data_ptr(), N, K, 128, st) == 0
+            B.w4a16_dequant(pw, out=w16)
+            B.w4a16_gemm(A, pw, C=c[0])
+            B.w4a16_gemm(A, pw, C=c[1])
+            assert L.w4a16_quantize(W16.data_ptr(), raw16[0].data_ptr(), raw16[1].data_ptr(), raw16[2].data_ptr(), N, K, 128, 0, st) == 0
+            B.w4a16_gemm(A, pw, C=c[2])
+    torch.cuda.synchronize()
+    assert B.w4a16_device_status() == 0
+    for (w16, c), (gw16, gc) in zip(want, outs):
+        assert torch.equal(w16, gw16) and all(torch.equal(c, g) for g in gc)
+    for a, b in zip(raw16, B.w4a16_quantize(W16)):
+        assert torch.equal(a, b)
+    del ws
+
+
 @pytest.mark.parametrize("path,M", [(B.PATH_DECODE, 8), (B.PATH_TILE, 32)])
 def test_gemm_on_a_non_default_stream_matches_the_default_stream(path, M):
     K, N = 2304, 512

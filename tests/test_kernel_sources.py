@@ -23,10 +23,11 @@ def test_kernels_that_let_the_next_launch_start_wait_for_the_one_in_front_before
     the next kernel would run beside the one in front of it."""
     seen = []
     for name, body in _kernels(open(os.path.join(CSRC, "kernels_basic.cuh")).read()):
+        body = body.replace("next_launch_may_start()", "griddepcontrol.launch_dependents").replace("wait_for_launch_before()", "griddepcontrol.wait")
         if "griddepcontrol.launch_dependents" in body:
             seen.append(name)
             assert not re.search(r"\breturn\b", body[:body.index("griddepcontrol.wait")]), name
-    assert sorted(seen) == ["stage_activations_kernel", "tile_splitk_reduce_kernel"]
+    assert sorted(seen) == ["dequant_kernel", "pack_kernel", "quantize_kernel", "stage_activations_kernel", "tile_splitk_reduce_kernel"]
 
 
 def test_a_barrier_tested_without_waiting_steers_a_warp_only_by_vote():
