@@ -108,9 +108,10 @@ __device__ __forceinline__ void mbar_arrive_lane0(uint32_t bar, int lane) {
                  "r"(lane)
                  : "memory");
 }
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) { mbar_arrive(smem_u32(bar)); }
 // Bounded wait: returns false (after recording the status code) if the phase does not complete
 // within about two seconds.  Fast path, inlined: one try_wait (about 40 clocks when the phase is
 // already complete).  Slow path, a function of its own so that the many waits of a kernel do not
