@@ -282,10 +282,13 @@ constexpr long kTwoLaunches = 6300;
 
 // What a launch costs, in ns, and how its units are cut.  Here and below the constants are least-squares fits of the relative
 // error to calls timed back to back, 12,700 schedules of 840 shapes drawn over M = 17 to 1500 (FP16, groups of 128): 3 to 6 %
-// off; the schedules they choose take 1.4 % longer than the best ones timed.  A unit takes a CTA 0.50 us with 80 rows and 0.57 with
-// 256 while few SMs are busy (the ring's hand-offs) and up to 0.79 with all of them (the L2 that brings the activations); the
-// rest is what a launch shows beside its units, the epilogue's rows among it, and for slices the second kernel, the partial
-// tiles and 79 ns for every slice that it adds.
+// off; the schedules they choose take 1.4 % longer than the best ones timed.  (Fitted before the issuer's loop of kernel_tile.cuh took
+// 5 to 20 % off a unit of that kernel.  Timed again with it, 90 shapes drawn over M = 65 to 1500, with and without bias and SiLU:
+// the choice is 0.9 % behind the best by the geometric mean and 5 to 13 % in seven of them, mostly where few column tiles would now
+// rather go to that kernel: M = 96, K = 9472 / N = 1408, eight of its slices 9.9 us, eleven of the other kernel's 11.2.)  A unit took
+// a CTA 0.50 us with 80 rows and 0.57 with 256 while few SMs are busy (the ring's hand-offs) and up to 0.79 with all of them (the L2
+// that brings the activations); the rest is what a launch shows beside its units, the epilogue's rows among it, and for slices the
+// second kernel, the partial tiles and 79 ns for every slice that it adds.
 TileGeom tile_geom_rows(int mt, int M, int N, int G, int split_k, int sms) {
     TileGeom g;
     g.mt = mt;
@@ -296,18 +299,18 @@ TileGeom tile_geom_rows(int mt, int M, int N, int G, int split_k, int sms) {
     if (split_k == 0) {
         // Balanced chunks use every SM to the end, but a chunk that starts or ends inside a tile leaves an FP32 partial tile
         // behind, whose store stalls the pipeline in mid-stream; dearer from two waves on (the CTAs no longer read the same
-        // activations at the same time) and never from three (M = 2787, K = 4224 / N = 13824 319 us, in waves 290; but 2.2 waves of
-        // 256 rows, M = 1454, K = 13056 / N = 6912 205 us, in waves 240).  S slices per tile (tiles <= SMs)
+        // activations at the same time) and never from three (M = 2787, K = 4224 / N = 13824 332 us, in waves 275; but 2.2 waves of
+        // 256 rows, M = 1454, K = 13056 / N = 6912 227 us, in waves 270).  S slices per tile (tiles <= SMs)
         // or whole tiles in waves (tiles > SMs) avoid that at the price of idle SMs.
-        // us, slices or waves / balanced: M = 256: K = 16384 / N = 4096 30.5 / 32.1, K = N = 8192 29.6 / 32.0; M = 600, K = N =
-        // 8192 83.3 / 82.7; M = 777, K = 4096 / N = 22016 119 / 140; M = 1024, K = N = 8192 99 / 112; M = 256, K = 8192 /
-        // N = 20480 (160 tiles) 86.5 / 78.8.
+        // us after a second of load (power-capped), slices or waves / balanced: M = 256: K = 16384 / N = 4096 31.1 / 33.5, K = N =
+        // 8192 34.7 / 38.0; M = 600, K = N = 8192 93.8 / 81.6; M = 777, K = 4096 / N = 22016 137 / 160; M = 1024, K = N = 8192
+        // 119 / 129; M = 256, K = 8192 / N = 20480 (160 tiles) 107 / 83.
         auto take = [&](int s, long cost) {
             if (g.cost == 0 || cost < g.cost) { g.cost = cost; split_k = s; }
         };
         const long balanced = (g.tiles * G + sms - 1) / sms;
         // percent; activations of half the L2 and more do not stay in it when the CTAs read different parts of them (M = 2509,
-        // K = 22144 / N = 3392, 111 MB: 370 us, in waves 290)
+        // K = 22144 / N = 3392, 111 MB: 397 us, in waves 370)
         const int dearer = ((long)M * G * (2 * kGroup) > (56l << 20) ? 113 : 100) * (g.tiles < 2 * sms ? 100 : 113) / 100;
         if (g.tiles <= sms) {
             const int tiles = (int)g.tiles;
@@ -347,7 +350,7 @@ TileGeom tile_geom_rows(int mt, int M, int N, int G, int split_k, int sms) {
     if (st > kTileMaxStages) st = kTileMaxStages;
     if (st > kTileSlots) st = kTileSlots;               // the ring also lives in tensor memory
     // parity waits tell a barrier phase only from its neighbour: every dequant set has to come back to a slot on
-    // every turn or every second one (kernel_tile.cuh)
+    // every turn or every second one, and the issuer takes two slots a turn of its loop (kernel_tile.cuh)
     st -= st % 2;
     g.stages = st;
     g.smem_bytes = kTileBarBytes + 1024 + st * tile_stage_bytes(mt);
@@ -358,7 +361,8 @@ TileGeom tile_geom_rows(int mt, int M, int N, int G, int split_k, int sms) {
 }
 
 // Batch rows per tile (the MMA's N): M in equal parts of at most 256 rows, rounded up to 16 -- the fewest parts, or one or
-// two more where that fills the last wave of tiles better.  M = 777, N = 22016: 4 x 208 rows 126 us, 4 x 256 131.
+// two more where that fills the last wave of tiles better.  M = 777, K = 4096 / N = 22016, us
+// after a second of load: 4 x 208 rows 131, 4 x 256 152, 5 x 160 139.
 TileGeom tile_geom(int M, int N, int G, int split_k, int sms) {
     const int least = (M + 255) / 256;
     TileGeom best = {};
@@ -526,10 +530,10 @@ size_t tile_workspace_bytes(const TileGeom& g) {
 }
 
 // The tcgen05 path's kernel for a shape: up to 64 rows the 64-row build of kernel_mid.cuh; above, the cheapest by the cost
-// models of it (several batch tiles), its 128-row build and kernel_tile.cuh.  Measured (us, in that order), the first column
-// decides: M = 128: K = N = 4096 10.4 / 14.8 / 13.0, K = 11008 / N = 4096 17.6 / 21.0 / 20.8, K = N = 8192 23.5 / 24.4 /
-// 26.6, K = 4096 / N = 22016 38.5 / 33.3 / 35.8; M = 256: K = N = 2048 8.0 / 12.2 / 11.7, K = 16384 / N = 4096 40.6 / 38.3 /
-// 32.9; M = 300, K = 4096 / N = 12288 - / 33.5 / 45.0; M = 512 - / 62.7 / 48.5; M = 1024, K = N = 8192 - / 128 / 102.
+// models of it (several batch tiles), its 128-row build and kernel_tile.cuh.  us in that order, after a second of load: M = 128:
+// K = N = 4096 14.2 / 20.2 / 15.0, K = 11008 / N = 4096 16.9 / 19.6 / 17.7, K = N = 8192 24.3 / 24.4 / 24.7, K = 4096 / N = 22016
+// 36.4 / 31.4 / 32.8; M = 256: K = N = 2048 8.4 / 13.4 / 9.5, K = 16384 / N = 4096 46.5 / 41.7 / 35.4; M = 300, K = 4096 / N =
+// 12288 45.6 / 34.4 / 43.7; M = 512 69.6 / 66.7 / 48.1; M = 1024, K = N = 8192 181 / 132 / 110.
 struct WidePlan {
     bool use_mid;
     MidGeom mid;
@@ -547,7 +551,8 @@ WidePlan wide_plan(int M, int N, int G, int split_k, const Chip& chip, int sg, b
     const MidGeom m128 = mid_geom(128, M, N, G, 0, chip, sg);
     if (m128.cost < w.mid.cost) w.mid = m128;
     w.tile = tile_geom(M, N, G, 0, chip.sms);
-    // (bias or activation in that kernel's own epilogue: K = 512, 80 / 208 rows 1.9 / 2.9 us more; in the other one 0.3)
+    // (bias and SiLU in that kernel's own epilogue: K = 512 / N = 12288, 80 / 208 rows 1.9 / 2.9 us more, bias and ReLU 0.7 / 0.8;
+    // in the other one 1.2 / 2.1 and 0.4 / 0.6)
     if (epi && w.tile.split_k == 1) w.tile.cost += (w.tile.tiles + chip.sms - 1) / chip.sms * (1200 + 8 * w.tile.mt);
     w.use_mid = w.mid.cost < w.tile.cost;
     if (split_k != 0) {

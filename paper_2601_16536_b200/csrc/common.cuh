@@ -401,8 +401,8 @@ __device__ __forceinline__ float widen(uint16_t v) {
 }
 
 // x / (1 + exp(-x)) by the hardware reciprocal (1 ulp; exp(-x) = inf gives 0): the result is rounded to 16 bits next, and
-// __expf's own error (2 ulp and more) is the larger one.  With the IEEE division M = 777, K = 4096 / N = 22016 took 12 us more;
-// M = 128 38.3 and 34.7, M = 64 23.4 and 21.9.
+// __expf's own error (2 ulp and more) is the larger one.  us, K = 4096 / N = 22016, FP16, bias and SiLU, IEEE division / this:
+// M = 777 163 / 150, M = 128 35.4 / 33.2, M = 64 23.0 / 22.1.
 __device__ __forceinline__ float silu(float x) {
     float r;
     asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(1.f + __expf(-x)));
@@ -418,10 +418,10 @@ __device__ __forceinline__ uint16_t finish(float v, int n, const Epilogue& e) {
     return cast_out<BF>(v);
 }
 
-// The same for several rows of one column, the column's bias at hand.  The activation is chosen once, not for each value: with
-// the branch inside, the exponential and the reciprocal of one value had to end before the next one's began (M = 777,
-// K = 4096 / N = 22016 with bias and SiLU: 12.8 thousand clocks for a tile's epilogue, three quarters of them that chain; the
-// call 130.9 us and now 121.7).
+// The same for several rows of one column, the column's bias at hand.  The activation is chosen and the rows are checked once, not
+// for each value: with a check, a branch and a store for each, the exponential and the reciprocal of one value had to end before
+// the next one's began.  us, M = 777, K = 4096 / N = 22016 with bias and SiLU, after a second of load, that form / this: FP16 in
+// groups of 128 173.7 / 150.2 (without bias and SiLU 128.7 / 131.3), symmetric BF16 in groups of 64 166.4 / 144.2 (124.4 / 125.6).
 template <bool BF, int R>
 __device__ __forceinline__ void finish_column(const uint32_t (&v)[R], uint16_t (&c)[R], bool has_bias, float bias, int act) {
     float x[R];

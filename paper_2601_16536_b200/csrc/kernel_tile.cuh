@@ -271,11 +271,9 @@ struct RingPos {
 // set takes every fourth stage, and with six slots it comes back to a slot only every second turn;
 // with one barrier per slot it would skip a phase each time, and nothing but a single in-order issuer
 // would keep the skipped phase from still being open.  With one barrier per slot and turn parity the
-// set meets the same barrier on every visit and that barrier completes exactly one phase in between.
-__device__ __forceinline__ uint64_t* retired_bar(uint64_t* retired, const RingPos& r) {
-    return retired + (r.turn & 1u) * kTileMaxStages + r.slot;      // the stage at r commits here
-}
-// until the stage that used r's slot one ring turn earlier has retired (r.turn >= 1)
+// set meets the same barrier on every visit and that barrier completes exactly one phase in between.  (The stage in slot s of
+// turn t commits to retired[(t & 1) * kTileMaxStages + s]: the issuer steps through them.)
+// Until the stage that used r's slot one ring turn earlier has retired (r.turn >= 1)
 __device__ __forceinline__ bool wait_slot_free(uint64_t* retired, const RingPos& r) {
     const uint32_t t = r.turn - 1u;
     return mbar_wait(retired + (t & 1u) * kTileMaxStages + r.slot, (t >> 1) & 1u);
@@ -435,7 +433,7 @@ gemm_tile_kernel(const __grid_constant__ CUtensorMap tmap_a, const TileParams p)
                 ret += 16u;
                 box += 2u * box_step;
                 a_t += 2u * kSlotCols;
-                if (bar == full_end) {                           // next turn: the other set of "retired" barriers
+                if (bar == full_end) {                           // next turn (t & 1 = ph): the other set of "retired" barriers
                     ph ^= 1u;
                     bar = full0;
                     ret = retired0 + ph * (8u * kTileMaxStages);
