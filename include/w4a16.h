@@ -18,6 +18,13 @@
  *   - Calls enqueue work on `stream` (a cudaStream_t passed as void*; NULL = the
  *     default stream) and return without waiting.  Argument errors are detected on the
  *     host, returned at once, and launch nothing.
+ *   - Order: every kernel touches the caller's buffers in stream order (for the packed weights of a
+ *     GEMM see w4a16_gemm).  Most of them let the next launch of their stream be set up while they
+ *     still run: the GEMMs, w4a16_dequant, w4a16_quantize and, outside of stream capture,
+ *     w4a16_pack.  Copies, events and ordinary launches behind a call notice nothing of that.
+ *     A caller's own kernel launched with programmatic stream serialization directly behind one
+ *     may start before the call's kernel has ended, and has to wait for it (griddepcontrol.wait,
+ *     cudaGridDependencySynchronize) before it touches what the call reads or writes.
  *   - Return value: W4A16_OK (0) or a negative W4A16_ERR_* code; w4a16_strerror()
  *     names it.  Nothing is printed, nothing throws, nothing exits.
  *   - FP16 values cross the boundary as their 16-bit patterns (uint16_t).
@@ -162,11 +169,15 @@ int w4a16_dequant(const void *Wq, const void *S, const void *Z, uint16_t *W16,
  * K slices that meet in the workspace (slices that meet in a cluster need none, and chunks that
  * cross tile boundaries give way to whole tiles).
  * Ordering: A, C and the workspace are touched in stream order.  The packed buffers Wq, S, Z
- * may be read (prefetched) while the previous kernel of the stream is still running, so
- * they must not be written by in-flight work other than a w4a16_pack enqueued earlier on the
- * same stream (the library makes the first GEMM launch on each stream after a pack a fully
- * ordered one; a pack on ANOTHER stream needs the caller's own event or synchronisation before
- * the GEMM, as for any cross-stream dependency); pack weights once, at load. */
+ * may be read (prefetched) while the previous kernels of the stream are still running (the one in
+ * front may itself have been let start before the one in front of it ended), so they must not be
+ * written by in-flight work other than a w4a16_pack enqueued earlier on the same stream: the
+ * library makes the first GEMM launch on each stream after a pack a fully ordered one, whatever
+ * stands between the two.  (A launch that the device refused, or one captured into a graph, is not
+ * the first; cudaStreamPerThread is a stream of each host thread.  A pack captured into a graph is
+ * ordered in front of the GEMMs captured behind it, and a replayed one in front of what is enqueued
+ * behind the replay.)  A pack on ANOTHER stream needs the caller's own event or synchronisation
+ * before the GEMM, as for any cross-stream dependency; pack weights once, at load. */
 int w4a16_gemm(const uint16_t *A, const void *Wq, const void *S, const void *Z, uint16_t *C,
                int M, int N, int K, int group, int split_k, w4a16_stream_t stream);
 
