@@ -31,8 +31,10 @@ __device__ __forceinline__ uint32_t pack_word(uint32_t r) {
 
 // One warp per half block (32 columns x 128 k).  A lane reads four consecutive k-words of one column (32 columns: 128 bytes a
 // row) and writes them as the column's 16-byte chunk: eight columns make up a 128-byte line.  Scales and zero points of the
-// half block go along in the same launch.  The launch is latency: a warp's loads, then its stores.  K = 11008 / N = 4096: a
-// warp per block, plain launch 12.5 us, this form 10.6 (HBM floor 7.2), 8.5 behind the quantizer.
+// half block go along in the same launch, half a warp per row.  The launch is latency: a warp's loads, all of them ahead of its first
+// store.  us, K = 11008 / N = 4096, a row of calls / one by itself: a warp per block, plain launch 12.4 / 15.2, in groups of 32
+// 12.4 / 15.8; half a block, the rows of scales one after the other behind the words 10.6 / 16.2 and 12.7 / 18.2; this form
+// 9.6 / 14.7 and 10.6 / 16.0 (HBM floor 7.2).
 __global__ void __launch_bounds__(kBlockKernelThreads)
 pack_kernel(const uint32_t* __restrict__ Wq_raw, const uint16_t* __restrict__ S_raw, const uint8_t* __restrict__ Z_raw,
             uint32_t* __restrict__ Wq, uint16_t* __restrict__ S, uint8_t* __restrict__ Z, int N, int G, int sg, int blocks, bool release) {
@@ -46,19 +48,33 @@ pack_kernel(const uint32_t* __restrict__ Wq_raw, const uint16_t* __restrict__ S_
     uint32_t r[16];
 #pragma unroll
     for (int kw = 0; kw < 16; ++kw) r[kw] = __ldcg(src + (size_t)kw * N);
-    __syncwarp();                        // (all 16 loads stay ahead of the first store)
+    // Half a warp per row of scales / zero points: rows lane / 16 and that + 2.  Positions 32 h + 2 p, + 1 (p = lane & 15) of a
+    // row belong to columns c0, c0 + 8 (sz_perm).
+    const int p = lane & 15, c0 = 32 * h + (p >> 1) + (p & 1) * 16;
+    uint32_t s[2], z[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int j = (lane >> 4) + 2 * i;
+        if (j < sg) {
+            const size_t in = (size_t)(pos.g * sg + j) * N + (size_t)pos.t * kTileN + c0;
+            s[i] = (uint32_t)__ldcg(S_raw + in) | ((uint32_t)__ldcg(S_raw + in + 8) << 16);
+            if (Z_raw != nullptr) z[i] = (__ldcg(Z_raw + in) & 15u) | ((uint32_t)__ldcg(Z_raw + in + 8) << 4);
+        }
+    }
+    __syncwarp();                        // (all loads stay ahead of the first store)
     uint4* dst = reinterpret_cast<uint4*>(Wq + pos.blk * kBlockWords);
 #pragma unroll
     for (int q = 0; q < 4; ++q)          // k-words 4 q .. 4 q + 3
         dst[block_word_index(32 * h + lane, 4 * q) / 4] =
             make_uint4(pack_word(r[4 * q]), pack_word(r[4 * q + 1]), pack_word(r[4 * q + 2]), pack_word(r[4 * q + 3]));
-    if (lane >= 16) return;
-    // positions 32 h + 2 lane, + 1 of a row of scales / zero points belong to columns c0, c0 + 8 (sz_perm)
-    const int c0 = 32 * h + (lane >> 1) + (lane & 1) * 16;
-    for (int j = 0; j < sg; ++j) {
-        const size_t in = (size_t)(pos.g * sg + j) * N + (size_t)pos.t * kTileN + c0, row = pos.blk * sg + j;
-        reinterpret_cast<uint32_t*>(S + row * kSBlockHalves)[16 * h + lane] = (uint32_t)__ldcg(S_raw + in) | ((uint32_t)__ldcg(S_raw + in + 8) << 16);
-        if (Z_raw != nullptr) Z[row * (kZBlockWords * 4) + 16 * h + lane] = (uint8_t)((__ldcg(Z_raw + in) & 15u) | (__ldcg(Z_raw + in + 8) << 4));
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int j = (lane >> 4) + 2 * i;
+        if (j < sg) {
+            const size_t row = pos.blk * sg + j;
+            reinterpret_cast<uint32_t*>(S + row * kSBlockHalves)[16 * h + p] = s[i];
+            if (Z_raw != nullptr) Z[row * (kZBlockWords * 4) + 16 * h + p] = (uint8_t)z[i];
+        }
     }
 }
 
@@ -147,7 +163,7 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
 // bounds are within 2^-9 of themselves, so their own codes are 0 and 15, and what lies beyond them has no other code.
 // What bounds it: memory while a CTA loads, instructions while it computes (13 a pair of weights), overlapped only between
 // CTAs.  K = 11008 / N = 4096: a thread per (group, column), two passes and a division per weight 96 us; FP32 clamps, one
-// column at a time and the divisions in line (25 % of the warp time went into fetching instructions) 28.9; this form 23.4
+// column at a time and the divisions in line (25 % of the warp time went into fetching instructions, now 7) 28.9; this form 23.4
 // (HBM floor 17.4).  Held to 48 registers for ten CTAs an SM it spills.
 template <bool BF>
 __global__ void __launch_bounds__(kBlockKernelThreads)
@@ -234,7 +250,7 @@ quantize_kernel(const uint16_t* __restrict__ W16, uint32_t* __restrict__ Wq, uin
 // One CTA per block, a warp for 32 k of it: a lane takes 8 neighbouring columns x 8 k (a word of each column), swaps the halves
 // of neighbouring columns' registers and stores 16 bytes of a row at a time, eight lanes one 128-byte line of the row.  The
 // packed words come through shared memory, 16 bytes a load: fetched word by word a warp's load touches eight lines, and the
-// L1 was the busiest unit (75 %).  The 256-byte sub-blocks lie 272 bytes apart, so that the words a warp reads at a time come from
+// L1 was the busiest unit (75 %; it still is, 73 % of a shorter time, the stores' part).  The 256-byte sub-blocks lie 272 bytes apart, so that the words a warp reads at a time come from
 // 32 banks.  Bound by HBM, most of it the stores.  us, a thread per word with 2-byte stores / word loads, plain launch / this form:
 // K = N = 8192 68 / 31.2 / 28.5 (HBM floor 26.3, a device copy of as many bytes 28.8), K = 11008 / N = 4096 - / 22.8 / 19.7 (17.6).
 template <bool BF>
