@@ -48,9 +48,9 @@ def _kernel_name(B, M, K, N, split_k=0):
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, from the ncu captures summarised under profiles/
 # (None = not captured since that kernel last changed).  Decode kernel: the mean of the five launches of a
-# step, M = 1 / 2 / 4 / 8 / 16 at K = 11008, N = 4096: 23.482 / 23.505 / 23.549 / 23.636 / 23.813 MB read, 0 written.
-NCU_TRAFFIC_BYTES = {"gemm_decode_kernel": 23597000}
-NCU_TRAFFIC_BYTES_TILE = 172179000    # gemm_tile_kernel, M=4096 K=N=8192 (read 120.1 MB + write 52.0 MB, one launch)
+# step, M = 1 / 2 / 4 / 8 / 16 at K = 11008, N = 4096: 23.478 / 23.501 / 23.545 / 23.632 / 23.809 MB read, 0 written.
+NCU_TRAFFIC_BYTES = {"gemm_decode_kernel": 23593000}
+NCU_TRAFFIC_BYTES_TILE = 170608000    # gemm_tile_kernel, M=4096 K=N=8192 (read 118.5 MB + write 52.1 MB, one launch)
 
 
 def _peaks():
