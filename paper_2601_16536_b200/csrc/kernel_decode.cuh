@@ -459,7 +459,8 @@ __global__ void __launch_bounds__(kDecThreads, 2) gemm_decode_kernel(const __gri
     // whose slices meet in a cluster: the counter gains 1 to 3 % in some builds and loses as much in others, which take one stage
     // at a time (M = 8, K = 11008 / N = 4096, one counter / a stage at a time: FP16 8.90 / 8.79, symmetric BF16 8.85 / 8.66, BF16
     // 8.79 / 9.09; K = 28672 / N = 8192, symmetric FP16 in groups of 32 33.3 / 33.9.  K = 12800 / N = 5632, whose last clusters
-    // find their place late, FP16 in groups of 32 16.7 / 15.7).
+    // find their place late, FP16 in groups of 32 16.7 / 15.7).  (One body for both: as a function called from two loops it cost
+    // builds that this is not about 1 to 2 %.)
     constexpr bool kCounted = !(CL && ABOX && MB == 1 && (SYM ? SG == 1 : !BF));
     const uint32_t full0 = smem_u32(full);
     constexpr uint32_t kEmptyOff = 8u * kDecMaxStages;
@@ -467,74 +468,6 @@ __global__ void __launch_bounds__(kDecThreads, 2) gemm_decode_kernel(const __gri
     uint32_t bar = full0;
     uint32_t st_addr = stage0_addr;
     uint32_t sa_addr = a_slot0;
-    auto multiply = [&](int left) {                          // the stage in the current slot, which holds at most `left` units
-        if (us < left) {
-            const uint32_t wa = st_addr + w_off, aa = sa_addr + a_off, aa1 = sa_addr + a_off1;
-            if constexpr (SG == 1) load_consts(st_addr, 0);
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                if constexpr (SG == 2) load_consts(st_addr, c);
-                if constexpr (SG == 4) load_consts(st_addr, 2 * c);
-                // B fragments: batch row 8 mb + gq, 16 consecutive k per lane
-                uint32_t bw[MB][8];
-#pragma unroll
-                for (int mb = 0; mb < MB; ++mb) {
-                    uint4 x, y;
-                    const uint32_t ab = mb == 0 ? aa : aa1;
-                    if constexpr (a_box) {
-                        if (c == 0) {
-                            x = lds128<0>(ab);
-                            y = lds128<0>(ab ^ 16u);
-                        } else {
-                            x = lds128<kADc>(ab);
-                            y = lds128<kADc>(ab ^ 16u);
-                        }
-                    } else if (c == 0) {
-                        x = lds128<0>(ab);
-                        y = lds128<16>(ab);
-                    } else {
-                        x = lds128<128>(ab);
-                        y = lds128<128 + 16>(ab);
-                    }
-                    bw[mb][0] = x.x; bw[mb][1] = x.y; bw[mb][2] = x.z; bw[mb][3] = x.w;
-                    bw[mb][4] = y.x; bw[mb][5] = y.y; bw[mb][6] = y.z; bw[mb][7] = y.w;
-                }
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    // sub-block (c, 2 (2 hh + r)) holds columns 16 rr + gq, the next one columns + 8
-                    uint2 va, vb;
-                    if (c == 0 && r == 0) { va = lds64<0>(wa); vb = lds64<256>(wa); }
-                    else if (c == 0)      { va = lds64<512>(wa); vb = lds64<512 + 256>(wa); }
-                    else if (r == 0)      { va = lds64<2048>(wa); vb = lds64<2048 + 256>(wa); }
-                    else                  { va = lds64<2048 + 512>(wa); vb = lds64<2048 + 512 + 256>(wa); }
-                    const uint32_t wwa[2] = {va.x, va.y}, wwb[2] = {vb.x, vb.y};
-#pragma unroll
-                    for (int wi = 0; wi < 2; ++wi) {
-                        const Pack8 fa = dequant_word<BF>(wwa[wi], zlo[2 * r], zhi[2 * r], s2[2 * r]);
-                        const Pack8 fb = dequant_word<BF>(wwb[wi], zlo[2 * r + 1], zhi[2 * r + 1], s2[2 * r + 1]);
-#pragma unroll
-                        for (int mb = 0; mb < MB; ++mb) {
-                            mma_m16n8k16<BF>(acc[r][mb], fa.h[0], fb.h[0], fa.h[1], fb.h[1], bw[mb][4 * wi],
-                                             bw[mb][4 * wi + 1]);
-                            mma_m16n8k16<BF>(acc[r][mb], fa.h[2], fb.h[2], fa.h[3], fb.h[3], bw[mb][4 * wi + 2],
-                                             bw[mb][4 * wi + 3]);
-                        }
-                    }
-                }
-            }
-        }
-    };
-    auto next_slot = [&] {
-        st_addr += (uint32_t)stage_bytes;
-        sa_addr += a_step;
-        bar += 8u;
-        if (bar == full0 + 8u * (uint32_t)p.stages) {
-            bar = full0;
-            phase ^= 1u;
-            st_addr = stage0_addr;
-            sa_addr = a_slot0;
-        }
-    };
     for (int ci = blockIdx.x; ci < p.nchunks; ci += gridDim.x) {
         const int u0 = chunk_begin(p, ci);
         const int u1 = chunk_begin(p, ci + 1);
@@ -544,23 +477,82 @@ __global__ void __launch_bounds__(kDecThreads, 2) gemm_decode_kernel(const __gri
         int tile_end = (t + 1) * p.G;
         int seg_start = u0;
         while (u < u1) {
-            if constexpr (kCounted) {
-                const int seg_end = min(u1, tile_end);
-                for (int left = seg_end - u; left > 0; left -= kDecUnitsPerStage) {
-                    if (!mbar_wait(bar, phase)) return;      // status recorded; every consumer warp sees it
-                    multiply(left);
-                    __syncwarp();
-                    mbar_arrive_lane0(bar + kEmptyOff, lane);
-                    next_slot();
+            const int seg_end = min(u1, tile_end);
+            int left = kCounted ? seg_end - u : min(kDecUnitsPerStage, seg_end - u);
+            do {
+                if (!mbar_wait(bar, phase)) return;          // status recorded; every consumer warp sees it
+                if (us < left) {
+                    const uint32_t wa = st_addr + w_off, aa = sa_addr + a_off, aa1 = sa_addr + a_off1;
+                    if constexpr (SG == 1) load_consts(st_addr, 0);
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        if constexpr (SG == 2) load_consts(st_addr, c);
+                        if constexpr (SG == 4) load_consts(st_addr, 2 * c);
+                        // B fragments: batch row 8 mb + gq, 16 consecutive k per lane
+                        uint32_t bw[MB][8];
+#pragma unroll
+                        for (int mb = 0; mb < MB; ++mb) {
+                            uint4 x, y;
+                            const uint32_t ab = mb == 0 ? aa : aa1;
+                            if constexpr (a_box) {
+                                if (c == 0) {
+                                    x = lds128<0>(ab);
+                                    y = lds128<0>(ab ^ 16u);
+                                } else {
+                                    x = lds128<kADc>(ab);
+                                    y = lds128<kADc>(ab ^ 16u);
+                                }
+                            } else if (c == 0) {
+                                x = lds128<0>(ab);
+                                y = lds128<16>(ab);
+                            } else {
+                                x = lds128<128>(ab);
+                                y = lds128<128 + 16>(ab);
+                            }
+                            bw[mb][0] = x.x; bw[mb][1] = x.y; bw[mb][2] = x.z; bw[mb][3] = x.w;
+                            bw[mb][4] = y.x; bw[mb][5] = y.y; bw[mb][6] = y.z; bw[mb][7] = y.w;
+                        }
+#pragma unroll
+                        for (int r = 0; r < 2; ++r) {
+                            // sub-block (c, 2 (2 hh + r)) holds columns 16 rr + gq, the next one columns + 8
+                            uint2 va, vb;
+                            if (c == 0 && r == 0) { va = lds64<0>(wa); vb = lds64<256>(wa); }
+                            else if (c == 0)      { va = lds64<512>(wa); vb = lds64<512 + 256>(wa); }
+                            else if (r == 0)      { va = lds64<2048>(wa); vb = lds64<2048 + 256>(wa); }
+                            else                  { va = lds64<2048 + 512>(wa); vb = lds64<2048 + 512 + 256>(wa); }
+                            const uint32_t wwa[2] = {va.x, va.y}, wwb[2] = {vb.x, vb.y};
+#pragma unroll
+                            for (int wi = 0; wi < 2; ++wi) {
+                                const Pack8 fa = dequant_word<BF>(wwa[wi], zlo[2 * r], zhi[2 * r], s2[2 * r]);
+                                const Pack8 fb = dequant_word<BF>(wwb[wi], zlo[2 * r + 1], zhi[2 * r + 1], s2[2 * r + 1]);
+#pragma unroll
+                                for (int mb = 0; mb < MB; ++mb) {
+                                    mma_m16n8k16<BF>(acc[r][mb], fa.h[0], fb.h[0], fa.h[1], fb.h[1], bw[mb][4 * wi],
+                                                     bw[mb][4 * wi + 1]);
+                                    mma_m16n8k16<BF>(acc[r][mb], fa.h[2], fb.h[2], fa.h[3], fb.h[3], bw[mb][4 * wi + 2],
+                                                     bw[mb][4 * wi + 3]);
+                                }
+                            }
+                        }
+                    }
                 }
+                __syncwarp();
+                if constexpr (kCounted) mbar_arrive_lane0(bar + kEmptyOff, lane);
+                else if (lane == 0) mbar_arrive(bar + kEmptyOff);
+                st_addr += (uint32_t)stage_bytes;
+                sa_addr += a_step;
+                bar += 8u;
+                if (bar == full0 + 8u * (uint32_t)p.stages) {
+                    bar = full0;
+                    phase ^= 1u;
+                    st_addr = stage0_addr;
+                    sa_addr = a_slot0;
+                }
+                if constexpr (kCounted) left -= kDecUnitsPerStage;
+            } while (kCounted && left > 0);
+            if constexpr (kCounted) {
                 u = seg_end;
             } else {
-                const int left = min(kDecUnitsPerStage, min(u1, tile_end) - u);
-                if (!mbar_wait(bar, phase)) return;
-                multiply(left);
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar + kEmptyOff);
-                next_slot();
                 u += left;
                 if (u != tile_end && u != u1) continue;
             }
